@@ -3,6 +3,7 @@
 //   blocks (Sec. 5.2) -> density rho by the H^2 sweep (Sec. 6.2) + tail
 //   (Sec. 7.1.1) -> singular near field B (Sec. 4) -> weighted mass M (Sec. 6.1).
 #include "device_common.cuh"
+#include "gamma_fixed.cuh"
 
 namespace vfd {
 
@@ -12,7 +13,7 @@ namespace vfd {
 __global__ void k_fields_points(int d, int nQ, const double *__restrict__ qx, const int *__restrict__ qcell,
                                 const double *__restrict__ qbary, const int *__restrict__ cells, DField Fs, DField Fk,
                                 double *__restrict__ out_s, double *__restrict__ out_lk, double smin, double smax,
-                                int *err)
+                                int *err, const long long *__restrict__ lw, int w, long long *__restrict__ ab)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nQ) return;
@@ -24,6 +25,13 @@ __global__ void k_fields_points(int d, int nQ, const double *__restrict__ qx, co
     out_s[i] = s;
     out_lk[i] = lk;
     if (!(s >= smin && s <= smax)) atomicOr(err, 1);
+    if (ab) {   // exponent terms of the fixed-point evaluations: a, b, a + log2 of the weight
+        i64 A, B;
+        if (!fx_terms(d, w, s, lk, A, B)) atomicOr(err + 1, 1);
+        ab[i] = A;
+        ab[nQ + i] = B;
+        ab[2 * (size_t)nQ + i] = A + lw[i];
+    }
 }
 
 // lcell, lbary (nodal fields): the node's closest cell and the barycentric
@@ -31,7 +39,7 @@ __global__ void k_fields_points(int d, int nQ, const double *__restrict__ qx, co
 __global__ void k_fields_nodes(int d, int n, const double *__restrict__ pts, DField Fs, DField Fk,
                                const int *__restrict__ lcell, const double *__restrict__ lbary,
                                const int *__restrict__ cells, double *__restrict__ out_s, double *__restrict__ out_lk,
-                               double smin, double smax, int *err)
+                               double smin, double smax, int *err, int w, long long *__restrict__ ab)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -43,6 +51,12 @@ __global__ void k_fields_nodes(int d, int n, const double *__restrict__ pts, DFi
     out_s[i] = s;
     out_lk[i] = lk;
     if (!(s >= smin && s <= smax)) atomicOr(err, 2);
+    if (ab) {
+        i64 A, B;
+        if (!fx_terms(d, w, s, lk, A, B)) atomicOr(err + 1, 2);
+        ab[i] = A;
+        ab[n + i] = B;
+    }
 }
 
 void launch_field_points(const MeshData &m, OpData &op, cudaStream_t st)
@@ -52,27 +66,31 @@ void launch_field_points(const MeshData &m, OpData &op, cudaStream_t st)
     double smin = chk ? 0.0 : -1e300, smax = chk ? op.s_bar : 1e300;
     op.q_s.alloc(m.nQ);
     op.q_lk.alloc(m.nQ);
+    if (m.fx_ok) op.q_ab.alloc(3 * (size_t)m.nQ);
     k_fields_points<<<cdiv(m.nQ, 256), 256, 0, st>>>(d, m.nQ, m.qx.p, m.qcell.p, m.qbary.p, m.cells.p, op.fs, op.fk,
-                                                     op.q_s.p, op.q_lk.p, smin, smax, op.errflag.p);
+                                                     op.q_s.p, op.q_lk.p, smin, smax, op.errflag.p, m.fx_lw.p, m.fx_w,
+                                                     op.q_ab.p);
     VFD_CUDA(cudaGetLastError());
     const bool nodal = op.fs.nodal || op.fk.nodal;
-    auto nodes = [&](const DBuf<double> &pts, int n, const NodeLoc &loc, DBuf<double> &os, DBuf<double> &ol) {
+    auto nodes = [&](const DBuf<double> &pts, int n, const NodeLoc &loc, DBuf<double> &os, DBuf<double> &ol,
+                     DBuf<long long> &ab) {
         os.alloc(n);
         ol.alloc(n);
+        if (m.fx_ok) ab.alloc(2 * (size_t)n);
         VFD_REQUIRE(!nodal || loc.done, VFD_ECUDA, "Chebyshev nodes not located for a nodal field");
         if (n)
             k_fields_nodes<<<cdiv(n, 256), 256, 0, st>>>(d, n, pts.p, op.fs, op.fk, nodal ? loc.cell.p : nullptr,
                                                           nodal ? loc.bary.p : nullptr, m.cells.p, os.p, ol.p, smin,
-                                                          smax, op.errflag.p);
+                                                          smax, op.errflag.p, m.fx_w, ab.p);
         VFD_CUDA(cudaGetLastError());
     };
-    if (m.nfar) nodes(m.kt_cheb, m.kt.nnode * k, m.kt_loc, op.kc_s, op.kc_lk);
+    if (m.nfar) nodes(m.kt_cheb, m.kt.nnode * k, m.kt_loc, op.kc_s, op.kc_lk, op.kc_ab);
     // the inner operator's nodes (k_in per box)
     if (m.nfar && m.k_in && op.precision != VFD_FP64)
-        nodes(m.kt_cheb_in, m.kt.nnode * m.k_in, m.kt_in_loc, op.kc_s_in, op.kc_lk_in);
+        nodes(m.kt_cheb_in, m.kt.nnode * m.k_in, m.kt_in_loc, op.kc_s_in, op.kc_lk_in, op.kc_ab_in);
     if (m.nrfar) {
-        nodes(m.tt_cheb, m.tt.nnode * k, m.tt_loc, op.tc_s, op.tc_lk);
-        nodes(m.st_cheb, m.st.nnode * k, m.st_loc, op.sc_s, op.sc_lk);
+        nodes(m.tt_cheb, m.tt.nnode * k, m.tt_loc, op.tc_s, op.tc_lk, op.tc_ab);
+        nodes(m.st_cheb, m.st.nnode * k, m.st_loc, op.sc_s, op.sc_lk, op.sc_ab);
     }
 }
 
@@ -389,6 +407,7 @@ struct RhoParams {
     const int *rnear_ptr, *rnear_col;
     const double *qx, *qw, *qs, *qlk;
     const int *qcell, *cells;
+    int near_done;                   // rho holds the near sums already
     int tail;
     double R;
     const double *g9x, *g9w;
@@ -424,9 +443,9 @@ __global__ void __launch_bounds__(128) k_rho_points(RhoParams P)
             int cell = P.qcell[id];
             for (int a = 0; a < P.nv; ++a) cv[a] = P.cells[(size_t)cell * P.nv + a];
         }
-        double acc = 0.0;
+        double acc = P.near_done && act ? P.rho[id] : 0.0;
         // near sources: masked direct sum
-        for (int ne = P.rnear_ptr[leaf]; ne < P.rnear_ptr[leaf + 1]; ++ne) {
+        for (int ne = P.rnear_ptr[leaf]; !P.near_done && ne < P.rnear_ptr[leaf + 1]; ++ne) {
             int sn = P.rnear_col[ne];
             int sb = P.st_begin[sn], se = P.st_end[sn];
             for (int j0 = sb; j0 < se; j0 += CH) {
@@ -534,7 +553,10 @@ void launch_density(const MeshData &m, OpData &op, cudaStream_t st)
     DBuf<double> yt;
     yt.alloc((size_t)m.tt.nnode * k);
     yt.zero(st);
-    if (m.nrfar) {
+    if (op.fx) launch_rho_near_fixed(m, op, st);
+    if (m.nrfar && op.fx) {
+        launch_rho_coupling_fixed(m, op, yt.p, st);
+    } else if (m.nrfar) {
         int n = m.tt.nnode * k;
         k_rho_coupling<<<cdiv(n, 128), 128, 0, st>>>(d, k, m.tt.nnode, m.rfar_ptr.p, m.rfar_col.p, m.tt_cheb.p,
                                                       op.tc_s.p, op.tc_lk.p, m.st_cheb.p, op.sc_s.p, op.sc_lk.p,
@@ -575,6 +597,7 @@ void launch_density(const MeshData &m, OpData &op, cudaStream_t st)
     P.qlk = op.q_lk.p;
     P.qcell = m.qcell.p;
     P.cells = m.cells.p;
+    P.near_done = op.fx ? 1 : 0;
     P.tail = m.opts.tail_mode;
     P.R = m.opts.tail_R;
     P.g9x = m.gl9_x.p;
@@ -622,6 +645,11 @@ void launch_coupling_build(const MeshData &m, OpData &op, cudaStream_t st)
     const long long n = (long long)m.nfar * m.k * m.k;
     op.S64.alloc(n);
     if (!n) return;
+    if (op.fx) {
+        if (m.k_in && op.precision != VFD_FP64) op.S64_in.alloc((long long)m.nfar * m.k_in * m.k_in);
+        launch_coupling_fixed(m, op, st);
+        return;
+    }
     k_coupling<<<cdiv(n, 256), 256, 0, st>>>(m.d, m.k, m.kt.nnode, m.far_ptr.p, m.far_col.p, m.kt_cheb.p, op.kc_s.p,
                                              op.kc_lk.p, m.mtab.p, op.S64.p);
     VFD_CUDA(cudaGetLastError());
@@ -874,6 +902,13 @@ __global__ void k_near_transpose(int nnear, const int *__restrict__ src, const i
     }
 }
 
+void launch_near_transpose(const MeshData &m, OpData &op, cudaStream_t st)
+{
+    k_near_transpose<<<m.nnear, 256, 0, st>>>(m.nnear, m.near_src.p, m.near_pair_row.p, m.near_col.p, m.kt_begin.p,
+                                              m.kt_end.p, m.kt.first_leaf(), m.near_off.p, m.panel_w.p, op.D64.p);
+    VFD_CUDA(cudaGetLastError());
+}
+
 void launch_near_build(const MeshData &m, OpData &op, cudaStream_t st)
 {
     op.D64.alloc(m.near_entries);
@@ -914,24 +949,27 @@ void launch_near_build(const MeshData &m, OpData &op, cudaStream_t st)
     int TQ = 32;
     while (TQ > 1 && shm_for(TQ) > 200 * 1024) TQ /= 2;
     size_t shm = shm_for(TQ);
-    if (shm <= 200 * 1024 && TQ >= 8) {
+    const bool whole = shm <= 200 * 1024 && TQ >= 8;
+    // with the column points tiled too (large leaf point sets, e.g. tetrahedra)
+    const size_t tshm = (size_t)32 * NB_TC * 8 + (size_t)32 * P.maxleaf * 8 + (size_t)P.maxleaf * P.maxleaf * 8 +
+                        (size_t)NB_TC * (m.d + 2) * 8 + (size_t)32 * (m.d + 2) * 8 + (size_t)NB_TC * 4 * 4 +
+                        (size_t)32 * 4 * 4;
+    VFD_REQUIRE(whole || tshm <= 220 * 1024, VFD_EUNSUPPORTED, "leaves too large for the near-block kernel");
+    if (op.fx) {
+        launch_near_build_fixed(m, op, st);
+        return;
+    }
+    if (whole) {
         P.TQ = TQ;
         VFD_CUDA(cudaFuncSetAttribute(k_near_build, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
         k_near_build<<<m.nnear, 256, shm, st>>>(P);
     } else {
-        // the column points tiled too (large leaf point sets, e.g. tetrahedra)
         P.TQ = 32;
-        const size_t tshm = (size_t)P.TQ * NB_TC * 8 + (size_t)P.TQ * P.maxleaf * 8 + (size_t)P.maxleaf * P.maxleaf * 8 +
-                            (size_t)NB_TC * (m.d + 2) * 8 + (size_t)P.TQ * (m.d + 2) * 8 + (size_t)NB_TC * 4 * 4 +
-                            (size_t)P.TQ * 4 * 4;
-        VFD_REQUIRE(tshm <= 220 * 1024, VFD_EUNSUPPORTED, "leaves too large for the near-block kernel");
         VFD_CUDA(cudaFuncSetAttribute(k_near_build_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tshm));
         k_near_build_tiled<<<m.nnear, 256, tshm, st>>>(P);
     }
     VFD_CUDA(cudaGetLastError());
-    k_near_transpose<<<m.nnear, 256, 0, st>>>(m.nnear, m.near_src.p, m.near_pair_row.p, m.near_col.p, m.kt_begin.p,
-                                              m.kt_end.p, P.fl, m.near_off.p, m.panel_w.p, op.D64.p);
-    VFD_CUDA(cudaGetLastError());
+    launch_near_transpose(m, op, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -279,9 +279,10 @@ vfd_status vfd_assemble(vfd_mesh_t mesh, const vfd_field *s, const vfd_field *lo
     launch_field_points(m, *op, st);
     mark();
     int herr[2] = {0, 0};
-    VFD_CUDA(cudaMemcpyAsync(herr, op->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+    VFD_CUDA(cudaMemcpyAsync(herr, op->errflag.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
     VFD_CUDA(cudaStreamSynchronize(st));
     VFD_REQUIRE(herr[0] == 0, VFD_EINVAL, "s(x) outside [0, s_bar] at some evaluation point");
+    op->fx = m.fx_ok && herr[1] == 0;   // else the FP64 kernel evaluations
     // a3: coupling blocks (and their algebraic recompression, FP64 operators)
     launch_coupling_build(m, *op, st);
     if (m.opts.recompress_tol > 0.0) recompress_far(m, *op, m.opts.recompress_tol, st);

@@ -12,6 +12,7 @@
 #include <thread>
 #include <vector>
 
+#include "gamma_fixed.cuh"
 #include "vfd_internal.h"
 
 namespace vfd {
@@ -251,6 +252,86 @@ void csr_from_lists(const std::vector<std::vector<T>> &lists, std::vector<int> &
 
 }  // namespace
 
+namespace {
+
+std::vector<unsigned long long> make_fixed_tables()
+{
+    // layout and formats in gamma_fixed.cuh, computed in extended precision
+    std::vector<unsigned long long> t(FX_WORDS);
+    for (int j = 0; j < FX_LOGN; ++j) {
+        const long double one = 2147483648.0L;   // 2^31
+        const unsigned long long c = (unsigned long long)std::ceil(one / (1.0L + j / (long double)FX_LOGN));
+        t[2 * j] = c;
+        t[2 * j + 1] = (unsigned long long)std::llround(std::ldexp(-std::log((long double)c / one), 56));
+    }
+    for (int j = 0; j < FX_EXPN; ++j)
+        t[2 * FX_LOGN + j] =
+            (unsigned long long)std::floor(std::ldexp(std::exp2(j / (long double)FX_EXPN), 63) + 0.5L) + 896ULL;
+    return t;
+}
+
+// coordinates in the fixed-point format of gamma_fixed.cuh: x - o split into a
+// sum of two doubles (exact), each rounded to the grid
+void fixed_coords(const std::vector<double> &x, int d, bool soa, const double *o, int w, DBuf<long long> &out)
+{
+    std::vector<long long> h(x.size());
+    const size_t n = x.size() / (d ? d : 1);
+    for (size_t i = 0; i < x.size(); ++i) {
+        const int c = soa ? (int)(i / n) : (int)(i % d);
+        const double hi = x[i] - o[c], bb = hi - x[i], lo = (x[i] - (hi - bb)) + (-o[c] - bb);
+        h[i] = std::llrint(std::ldexp(hi, 62 - w)) + std::llrint(std::ldexp(lo, 62 - w));
+    }
+    out.upload(h);
+}
+
+// Scale and origin of the fixed-point coordinates, and whether the mesh fits
+// the format: the rounding of a coordinate, 2^-62 W, has to be small against
+// the distances of points in cells that do not touch.  A cell's measure over
+// its largest facet's bound diam^(d-1) is a lower bound of its height up to a
+// factor d; at 2^-15 W it bounds the relative error of a distance by about
+// 2^-46, which is what FP64 leaves of an exponent of that size.
+void setup_fixed(MeshData &m, const std::vector<double> &qx, const std::vector<double> &qw,
+                 const std::vector<double> &meas, const std::vector<double> &diam)
+{
+    const int d = m.d;
+    double lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0}, o[3] = {0, 0, 0}, diag2 = 0.0;
+    for (int c = 0; c < d; ++c) {
+        lo[c] = 1e300;
+        hi[c] = -1e300;
+        for (int v = 0; v < m.M; ++v) {
+            lo[c] = std::min(lo[c], m.X[(size_t)v * d + c]);
+            hi[c] = std::max(hi[c], m.X[(size_t)v * d + c]);
+        }
+        o[c] = 0.5 * (lo[c] + hi[c]);
+        diag2 += (hi[c] - lo[c]) * (hi[c] - lo[c]);
+    }
+    m.fx_ok = false;
+    const double diag = 1.01 * std::sqrt(diag2);   // the boxes of the trees reach a little past the points
+    if (!std::isfinite(diag) || !(diag > 0.0)) return;
+    const int w = std::ilogb(diag) + 1;
+    if (w < -30 || w > 30) return;
+    const double W = std::ldexp(1.0, w);
+    for (size_t c = 0; c < meas.size(); ++c)
+        if (!(meas[c] >= std::ldexp(W, -15) * std::pow(diam[c], d - 1))) return;
+    std::vector<long long> lw(qw.size());
+    for (size_t i = 0; i < qw.size(); ++i) {
+        const double l = std::log2(qw[i]);
+        if (!(std::fabs(l) < 100.0)) return;
+        lw[i] = (long long)std::llround(std::ldexp(std::log2((long double)qw[i]), 53));
+    }
+    m.fx_w = w;
+    m.fx_lw.upload(lw);
+    m.fx_tab.upload(make_fixed_tables());
+    fixed_coords(qx, d, true, o, w, m.fx_qX);
+    fixed_coords(m.kt_cheb_h, d, false, o, w, m.fx_ktX);
+    fixed_coords(m.kt_cheb_in_h, d, false, o, w, m.fx_ktX_in);
+    fixed_coords(m.tt_cheb_h, d, false, o, w, m.fx_ttX);
+    fixed_coords(m.st_cheb_h, d, false, o, w, m.fx_stX);
+    m.fx_ok = true;
+}
+
+}  // namespace
+
 MeshData *build_mesh(int d, int64_t n_vert, const double *coords, int64_t n_cell, const int32_t *cells,
                      const uint8_t *inter, const vfd_mesh_opts &opts)
 {
@@ -287,7 +368,7 @@ MeshData *build_mesh(int d, int64_t n_vert, const double *coords, int64_t n_cell
             VFD_REQUIRE(m->T[i] >= 0 && m->T[i] < M, VFD_EINVAL, "cell vertex id out of range");
 
         // ---- cell measures, h_max
-        std::vector<double> meas(C);
+        std::vector<double> meas(C), cdiam(C);
         for (int c = 0; c < C; ++c) {
             const int *t = &m->T[(size_t)c * nv];
             double mu, diam = 0.0;
@@ -319,6 +400,7 @@ MeshData *build_mesh(int d, int64_t n_vert, const double *coords, int64_t n_cell
             }
             VFD_REQUIRE(mu > 0.0, VFD_EINVAL, "degenerate cell " + std::to_string(c));
             meas[c] = mu;
+            cdiam[c] = diam;
             m->h_max = std::max(m->h_max, diam);
         }
 
@@ -1060,6 +1142,7 @@ MeshData *build_mesh(int d, int64_t n_vert, const double *coords, int64_t n_cell
             m->gl9_x.upload(gx);
             m->gl9_w.upload(gw);
             m->mtab.upload(make_math_tables());
+            setup_fixed(*m, qx, qw, meas, cdiam);
         }
     } catch (...) {
         delete m;

@@ -206,6 +206,12 @@ struct MeshData {
     DBuf<double> gl_x, gl_w;            // Gauss-Legendre on [0,1], n_sing points
     DBuf<double> gl9_x, gl9_w;          // 9-point rule for the tail
     DBuf<double> mtab;                  // tables of the table-driven FP64 log/exp
+    // fixed-point kernel evaluations (gamma_fixed.cuh): scale 2^fx_w, coordinates of the
+    // rule points (SoA) and of the Chebyshev nodes (node-major), log2 of the rule weights (Q53)
+    bool fx_ok = false;
+    int fx_w = 0;
+    DBuf<unsigned long long> fx_tab;
+    DBuf<long long> fx_qX, fx_lw, fx_ktX, fx_ktX_in, fx_ttX, fx_stX;
 
     DBuf<int> rfarT_ptr, rfarT_col;     // transposed: source node -> target nodes
     DBuf<int> rnearT_ptr, rnearT_col;   // transposed: source leaf index -> target leaf indices
@@ -244,6 +250,10 @@ struct OpData {
     DBuf<double> kc_s_in, kc_lk_in;    // at the inner operator's Chebyshev nodes (low-precision operators)
     DBuf<double> S64_in;               // the inner operator's coupling blocks, nfar x k_in x k_in
     DBuf<double> tc_s, tc_lk, sc_s, sc_lk;  // density trees' Chebyshev nodes
+    // exponent terms of the fixed-point kernel evaluations, (a, b) per point; q_ab ends with a
+    // third array, a + log2 of the rule weight.  fx: every point fits the formats
+    bool fx = false;
+    DBuf<long long> q_ab, kc_ab, kc_ab_in, tc_ab, sc_ab;
     DBuf<double> valB, valM, valBM;    // CSR values
     DBuf<double> rho;                  // interior points, canonical order
     DBuf<double> S64;                  // nfar * k * k
@@ -386,6 +396,12 @@ void launch_coupling_build(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_near_build(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_convert_fp32(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_load(const MeshData &m, const double *f, double *F, cudaStream_t st);
+// assemble_fixed.cu: the same with fixed-point kernel evaluations (operators with fx set)
+void launch_near_build_fixed(const MeshData &m, OpData &op, cudaStream_t st);
+void launch_near_transpose(const MeshData &m, OpData &op, cudaStream_t st);
+void launch_coupling_fixed(const MeshData &m, OpData &op, cudaStream_t st);
+void launch_rho_coupling_fixed(const MeshData &m, OpData &op, double *yt, cudaStream_t st);
+void launch_rho_near_fixed(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_selftest_math(const MeshData &m, int which, long long n, const double *x, double *out, cudaStream_t st);
 // apply.cu
 void apply_parts_ex(const MeshData &m, OpData &op, int parts, const double *X, double *Y, int nrhs, int64_t ld,
