@@ -18,7 +18,7 @@
 #include <algorithm>
 #include <mutex>
 
-#include "device_common.cuh"
+#include "apply_common.cuh"
 
 namespace vfd {
 
@@ -421,6 +421,26 @@ static FarView make_far_view(const MeshData &m, const OpData &op, bool use, bool
     return F;
 }
 
+// the node sums of columns [c0, c0 + cols) for the fixed-point apply (apply_fixed.cu)
+void launch_far_sum(const MeshData &m, OpData &op, int c0, int cols, cudaStream_t st, const int *skip)
+{
+    const FarView F = make_far_view(m, op, true, false);
+    const int64_t hs = (int64_t)m.kt.nnode * m.k;
+    const size_t ps = (size_t)F.nlev * m.kt.nleaf * m.k;
+    k_far_sum<double><<<dim3(m.kt.nnode - ((1 << F.lmin) - 1), cols), 128, 0, st>>>(
+        F, m.kt.nleaf, op.P64.p + c0 * ps, op.xhat.p + c0 * hs, hs, skip);
+    VFD_CUDA(cudaGetLastError());
+}
+
+void launch_far_couple_sum(const MeshData &m, OpData &op, int c0, int cols, cudaStream_t st, const int *skip)
+{
+    const FarView F = make_far_view(m, op, true, false);
+    const int64_t hs = (int64_t)m.kt.nnode * m.k;
+    k_far_couple_sum<double><<<dim3(cdiv(hs, 256), cols), 256, 0, st>>>(
+        F, m.nfar, m.kt.nnode, m.far_ptr.p, op.ye64.p + (size_t)c0 * m.nfar * m.k, op.yhat.p + c0 * hs, hs, skip);
+    VFD_CUDA(cudaGetLastError());
+}
+
 template <class T, class A>
 static void apply_impl(const MeshData &m, OpData &op, int parts, const double *X, double *Y, int nrhs, int64_t ld,
                        const T *Ul, const T *S, const T *D, A *xhat, A *yhat, A *part, A *ye, bool rc, cudaStream_t st,
@@ -516,6 +536,10 @@ void apply_parts_ex(const MeshData &m, OpData &op, int parts, const double *X, d
             op.yhat.alloc(need);
             op.P64.alloc(needp);
             op.ye64.alloc(needy);
+        }
+        if (parts == VFD_PART_ALL && op.fa && m.nnear > 0) {
+            apply_fixed(m, op, X, Y, nrhs, ld, st, skip);
+            return;
         }
         const bool rc = op.rc_on;   // the recompressed far field of the FP64 operator
         apply_impl<double, double>(m, op, parts, X, Y, nrhs, ld, rc ? op.Ulc64.p : m.Ul64.p, rc ? op.Sc64.p : op.S64.p,

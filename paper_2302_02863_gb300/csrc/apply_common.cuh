@@ -1,0 +1,16 @@
+// Declarations shared by the FP64 apply (apply.cu) and its fixed-point form
+// (apply_fixed.cu).
+#pragma once
+
+#include "device_common.cuh"
+
+namespace vfd {
+
+// apply.cu: node sums of columns [c0, c0 + cols), P64 -> xhat and ye64 -> yhat
+void launch_far_sum(const MeshData &m, OpData &op, int c0, int cols, cudaStream_t st, const int *skip);
+void launch_far_couple_sum(const MeshData &m, OpData &op, int c0, int cols, cudaStream_t st, const int *skip);
+// apply_fixed.cu: Y = A X with the FP64 operator (OpData::fa)
+void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st,
+                 const int *skip);
+
+}  // namespace vfd

@@ -1,0 +1,1076 @@
+// The FP64 operator apply in fixed-point arithmetic.
+//
+// One FP64 multiply-add takes a warp 16 cycles of an SM on this part, so the
+// FP64 kernels of apply.cu are bound by the FP64 pipe at any number of columns
+// (98M multiply-adds a column at 27k DoFs and rank 64: 156 us at the pipe's
+// rate, against 115 us for the bytes of one pass over the operator).  Here the
+// operator's entries and the vectors are 61-bit integers, scaled by a power of
+// two per panel row (near entries, B + M added to them), coupling block or leaf
+// (flattened bases), and per gathered piece of a vector:
+//   v = (hi 2^30 + lo) 2^(E - 60), |v| < 2^E, lo in [-2^29, 2^29), |hi| <= 2^30
+// and a product takes three 32 x 32 + 64 bit multiply-adds,
+//   hh += a.hi x.hi,   mid += a.hi x.lo + a.lo x.hi
+// (3 cycles a warp; a.lo x.lo is below the last place kept).  Every fourth product
+// the bits of hh and mid from 2^40 on move to 32-bit counters, so that nothing
+// overflows (2^60 a product).  Rounding to 2^-61 of the largest entry of a row or
+// block replaces rounding to 2^-53 of every partial sum: measured errors are at
+// the end of the comment.  The sums are exact in the integers, so their order
+// does not matter.
+//
+// Non-finite or nearly denormal vectors (a piece whose largest entry is Inf,
+// NaN or below 2^-895) take plain FP64 sums over the FP64 operator instead, so
+// that Inf, NaN and denormals come out as they do there.
+//
+//   1. k_fa_proj    per leaf: Ul^T x of every far level
+//   2. k_fa_couple  a warp per admissible block: S_e xhat, xhat summed over the
+//                   column node's leaves while it is gathered
+//   3. k_fa_near    per row, the near panel row (concurrently with 1-2)
+//   4. k_fa_expand  Y[i] += sum over levels of Ul[i] . yhat, yhat summed over the
+//                   node's blocks while it is gathered
+// With 4 or more columns the two sums are kernels of their own (apply.cu): a
+// gather that repeats them for every block or leaf then costs more than it saves.
+// Columns go in groups of NC = 8 (4, 2, 1 for the remainder): an entry is loaded
+// once for NC products.
+//
+// Measured at 27k DoFs, rank 64 (FP64 kernels first): one column 243 -> 150 us,
+// 64 columns 11.87 -> 5.27 ms.  Error against extended precision with the same
+// FP64 operator, relative 2-norm, normal x on 400 to 1000 DoFs: 1.2e-16 to
+// 1.3e-16 (FP64 kernels), 5.8e-17 to 7.8e-17 here; x = 1: 5.9e-16 to 3.3e-15 and
+// 1.5e-16 to 6.3e-16; x spread over six decades: 1.1e-16 to 1.4e-16 and 5.9e-17
+// to 7.8e-17.
+#include <algorithm>
+
+#include "apply_common.cuh"
+
+namespace vfd {
+
+typedef long long i64;
+typedef unsigned long long u64;
+
+namespace {
+
+constexpr int FA_LO = 30, FA_TOP = 40;
+
+// exponent key of a value: 0 for zero, else its biased exponent (denormals 1)
+__device__ __forceinline__ unsigned fa_key(double v)
+{
+    // the exponent field is masked after the shift: a mask of the sign bit alone becomes
+    // an FP64 absolute value, which leaves the sign of a NaN
+    const unsigned h = (unsigned)__double2hiint(v);
+    return (h << 1 | (unsigned)__double2loint(v)) == 0 ? 0u : max(1u, (h >> 20) & 0x7ffu);
+}
+// keys of a piece that the fixed-point products cannot take
+__device__ __forceinline__ bool fa_slow(unsigned key) { return key == 0x7ffu || (key && key < 128u); }
+
+// v 2^(60 - E) rounded, E = key - 1022 with key the largest of the piece
+__device__ __forceinline__ i64 fa_round(double v, int key)
+{
+    const u64 b = (u64)__double_as_longlong(v);
+    const int e = (int)((b >> 52) & 0x7ff), s = e - key + 7;
+    const u64 m = (b & 0xfffffffffffffULL) | (e ? 1ULL << 52 : 0ULL);
+    const u64 r = s >= 0 ? m << s : (s > -64 ? (m + (1ULL << (-s - 1))) >> -s : 0ULL);
+    return (i64)b < 0 ? -(i64)r : (i64)r;
+}
+__device__ __forceinline__ int2 fa_split(i64 v)
+{
+    const int lo = (int)((unsigned)v << (32 - FA_LO)) >> (32 - FA_LO);
+    return make_int2(lo, (int)((v - lo) >> FA_LO));
+}
+// 2^k as FP64, -1022 <= k <= 1023
+__device__ __forceinline__ double fa_pow2(int k) { return __longlong_as_double((i64)(k + 1023) << 52); }
+// scale of a piece: 2^(E - 30), E = key - 1022 (any for a piece of zeros)
+__device__ __forceinline__ double fa_scale(unsigned key) { return fa_pow2(key ? (int)key - 1022 - 30 : 0); }
+// sums of products: carry() after every fourth mac at most (seven fit)
+struct FaAcc {
+    i64 hh = 0, mid = 0;
+    int th = 0, tm = 0;   // what hh and mid have passed on, weight 2^FA_TOP
+    __device__ __forceinline__ void mac(int2 a, int2 x)
+    {
+        hh += (i64)a.y * x.y;
+        mid += (i64)a.y * x.x;
+        mid += (i64)a.x * x.y;
+    }
+    __device__ __forceinline__ void carry()
+    {
+        th += (int)(hh >> FA_TOP);
+        hh &= (1LL << FA_TOP) - 1;
+        tm += (int)(mid >> FA_TOP);
+        mid &= (1LL << FA_TOP) - 1;
+    }
+    // after carry: hh takes mid, rounded (the sum is th 2^FA_TOP + hh in units of 2^60)
+    __device__ __forceinline__ void fold()
+    {
+        hh += ((mid + (1LL << (FA_LO - 1))) >> FA_LO) + ((i64)tm << (FA_TOP - FA_LO));
+    }
+    __device__ __forceinline__ double value() const { return fma((double)th, 1099511627776.0, (double)hh); }
+};
+
+// products of a column: out_a = sum_b M[b stride + a] x[b], thread per a, x in
+// shared memory [b][NC]
+template <int NC>
+__device__ __forceinline__ void fa_column(const int2 *__restrict__ M, size_t stride, int n, int step, const int2 *x,
+                                          double *out)
+{
+    FaAcc s[NC];
+    int b = 0;
+#pragma unroll 2
+    for (; b + 3 * step < n; b += 4 * step) {
+        int2 m[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) m[q] = M[(size_t)(b + q * step) * stride];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) s[c].mac(m[q], x[(b + q * step) * NC + c]);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[c].carry();
+    }
+    for (; b < n; b += step) {
+        const int2 m = M[(size_t)b * stride];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[c].mac(m, x[b * NC + c]);
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        s[c].carry();
+        s[c].fold();
+        out[c] = s[c].value();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// 1. projections: CTA per (leaf, 128 of the nlev k columns, group of columns)
+// ---------------------------------------------------------------------------
+struct FaFar {
+    int fl, nleaf, lmin, L, nlev, k, nnode, nfar, nrhs, c0;   // c0: first column of this launch
+    int kp, wp;   // row strides of a coupling block and of the bases (even: 16-byte rows)
+    const int *kb, *ke, *fptr, *fcol;
+    const int2 *U, *S;
+    const int *ue, *se;
+    const double *Ud, *Sd;   // FP64: [level][N][k], blocks
+    int N;
+};
+
+template <int NC>
+__global__ void __launch_bounds__(128) k_fa_proj(FaFar P, const double *__restrict__ X, int64_t ld,
+                                                 double *__restrict__ part, const int *skip)
+{
+    extern __shared__ __align__(16) unsigned char fa_sm[];
+    __shared__ unsigned key[NC];
+    if (skip && *skip) return;
+    const int leaf = blockIdx.x, w = P.nlev * P.k, r0 = P.c0 + blockIdx.z * NC;
+    const int b = P.kb[P.fl + leaf], n = P.ke[P.fl + leaf] - b;
+    double *raw = (double *)fa_sm;   // [i][NC]
+    int2 *xs = (int2 *)fa_sm;
+    if (threadIdx.x < NC) key[threadIdx.x] = 0;
+    __syncthreads();
+    for (int t = threadIdx.x; t < n * NC; t += blockDim.x) {
+        const int c = t / n, i = t - c * n;
+        const double v = r0 + c < P.nrhs ? X[(size_t)(r0 + c) * ld + b + i] : 0.0;
+        raw[i * NC + c] = v;
+        atomicMax(&key[c], fa_key(v));
+    }
+    __syncthreads();
+    bool slow = false;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) slow |= fa_slow(key[c]);
+    if (!slow) {
+        for (int t = threadIdx.x; t < n * NC; t += blockDim.x) xs[t] = fa_split(fa_round(raw[t], key[t % NC]));
+        __syncthreads();
+    }
+    const int col = blockIdx.y * blockDim.x + threadIdx.x;
+    if (col >= w) return;
+    const int2 *M = P.U + (size_t)b * P.wp + col;
+    const int eu = P.ue[leaf], lv = col / P.k, a = col - lv * P.k;
+    double out[NC];
+    if (!slow) {
+        fa_column<NC>(M, P.wp, n, 1, xs, out);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) out[c] = out[c] * fa_pow2(eu - 30) * fa_scale(key[c]);
+    } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) out[c] = 0.0;
+        for (int i = 0; i < n; ++i) {
+            const double m = P.Ud[((size_t)lv * P.N + b + i) * P.k + a];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) out[c] = fma(m, raw[i * NC + c], out[c]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+        if (r0 + c < P.nrhs) part[(((size_t)(r0 + c) * P.nlev + lv) * P.nleaf + leaf) * P.k + a] = out[c];
+}
+
+// ---------------------------------------------------------------------------
+// 2. coupling: warp per admissible block; k <= 16 columns: 32/k' groups of lanes
+//    share the rows
+// ---------------------------------------------------------------------------
+constexpr int FC_WARPS = 4;
+
+template <int NC>
+__global__ void __launch_bounds__(32 * FC_WARPS)
+k_fa_couple(FaFar P, const double *__restrict__ part, const double *__restrict__ xhat, double *__restrict__ ye,
+            const int *skip)
+{
+    __shared__ int2 xs_[FC_WARPS][KMAX * NC];
+    if (skip && *skip) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int e = blockIdx.x * FC_WARPS + warp, r0 = P.c0 + blockIdx.y * NC, k = P.k;
+    if (e >= P.nfar) return;
+    int2 *xs = xs_[warp];
+    double *raw = (double *)xs;
+    const int node = P.fcol[e], l = 31 - __clz(node + 1), sh = P.L - l;
+    const int leaf0 = ((node + 1) << sh) - (1 << P.L);
+    unsigned key[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const int r = r0 + c;
+        unsigned mk = 0;
+        for (int b = lane; b < k; b += 32) {
+            double v = 0.0;
+            if (r < P.nrhs) {
+                if (xhat) {
+                    v = xhat[((size_t)r * P.nnode + node) * k + b];
+                } else {
+                    const double *p = part + (((size_t)r * P.nlev + l - P.lmin) * P.nleaf + leaf0) * k + b;
+#pragma unroll 8
+                    for (int j = 0; j < (1 << sh); ++j) v += p[(size_t)j * k];
+                }
+            }
+            raw[b * NC + c] = v;
+            mk = max(mk, fa_key(v));
+        }
+        key[c] = __reduce_max_sync(0xffffffffu, mk);
+    }
+    bool slow = false;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) slow |= fa_slow(key[c]);
+    __syncwarp();
+    const int2 *S = P.S + (size_t)e * k * P.kp;
+    const int es = P.se[e];
+    if (slow) {
+        for (int a = lane; a < k; a += 32)
+            for (int c = 0; c < NC && r0 + c < P.nrhs; ++c) {
+                double v = 0.0;
+                for (int b = 0; b < k; ++b) v = fma(P.Sd[((size_t)e * k + b) * k + a], raw[b * NC + c], v);
+                ye[((size_t)(r0 + c) * P.nfar + e) * k + a] = v;
+            }
+        return;
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+        for (int b = lane; b < k; b += 32) xs[b * NC + c] = fa_split(fa_round(raw[b * NC + c], key[c]));
+    __syncwarp();
+    // lanes over a; with k <= 16 the groups of ga lanes take every (32 / ga)-th row
+    const int ga = k > 16 ? 32 : k > 8 ? 16 : 8, gb = 32 / ga, la = lane & (ga - 1), lb = lane / ga;
+    for (int a0 = 0; a0 < k; a0 += ga) {
+        const int a = a0 + la;
+        double out[NC];
+        if (a < k) {
+            fa_column<NC>(S + a + (size_t)lb * P.kp, P.kp, max(0, k - lb), gb, xs + lb * NC, out);
+        } else {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) out[c] = 0.0;
+        }
+        for (int o = ga; o < 32; o <<= 1) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) out[c] += __shfl_xor_sync(0xffffffffu, out[c], o);
+        }
+        if (a < k && lb == 0) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (r0 + c < P.nrhs)
+                    ye[((size_t)(r0 + c) * P.nfar + e) * k + a] =
+                        out[c] * fa_pow2(es - 30) * fa_scale(key[c]);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// rows: sums over the entries of matrix rows, 8 lanes to a row and four rows to
+// a warp, x in shared memory: [j] for one column, else [pair of columns][j]
+// ---------------------------------------------------------------------------
+template <int NC>
+__device__ __forceinline__ void fa_row(const int2 *__restrict__ row, int w, int l8, const int4 *xs, int ws, FaAcc *s)
+{
+    if (NC == 1) {
+        const int4 *r4 = (const int4 *)row, *x4 = xs;
+        const int nv = w >> 1;
+        int v = l8;
+#pragma unroll 2
+        for (; v + 8 < nv; v += 16) {
+            const int4 a = r4[v], b = r4[v + 8], x = x4[v], y = x4[v + 8];
+            s[0].mac(make_int2(a.x, a.y), make_int2(x.x, x.y));
+            s[0].mac(make_int2(a.z, a.w), make_int2(x.z, x.w));
+            s[0].mac(make_int2(b.x, b.y), make_int2(y.x, y.y));
+            s[0].mac(make_int2(b.z, b.w), make_int2(y.z, y.w));
+            s[0].carry();
+        }
+        if (v < nv) {
+            const int4 a = r4[v], x = x4[v];
+            s[0].mac(make_int2(a.x, a.y), make_int2(x.x, x.y));
+            s[0].mac(make_int2(a.z, a.w), make_int2(x.z, x.w));
+        }
+    } else {
+        auto term = [&](int2 a, int j) {
+#pragma unroll
+            for (int p = 0; p < NC / 2; ++p) {
+                const int4 x = xs[(size_t)p * ws + j];
+                s[2 * p].mac(a, make_int2(x.x, x.y));
+                s[2 * p + 1].mac(a, make_int2(x.z, x.w));
+            }
+        };
+        int j = l8;
+#pragma unroll 1
+        for (; j + 24 < w; j += 32) {
+            int2 a[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) a[q] = row[j + 8 * q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) term(a[q], j + 8 * q);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) s[c].carry();
+        }
+        for (; j < w; j += 8) term(row[j], j);
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        s[c].carry();
+        s[c].fold();
+    }
+}
+
+// sum over the 8 lanes of a row (th and hh); every lane ends with one column,
+// returned, and its sum in s[0]
+template <int NC>
+__device__ __forceinline__ int fa_sum8(FaAcc *s, int l8)
+{
+    int n = NC, col = 0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = l8 & o;
+#pragma unroll
+            for (int q = 0; q < NC / 2; ++q)
+                if (q < n) {
+                    const int st = up ? s[q].th : s[q + n].th, kt = up ? s[q + n].th : s[q].th;
+                    const i64 sl = up ? s[q].hh : s[q + n].hh, kl = up ? s[q + n].hh : s[q].hh;
+                    s[q].th = kt + __shfl_xor_sync(0xffffffffu, st, o);
+                    s[q].hh = kl + __shfl_xor_sync(0xffffffffu, sl, o);
+                }
+            col += up ? n : 0;
+        } else {
+            s[0].th += __shfl_xor_sync(0xffffffffu, s[0].th, o);
+            s[0].hh += __shfl_xor_sync(0xffffffffu, s[0].hh, o);
+        }
+    }
+    return col;
+}
+
+// convert the gathered piece (raw FP64 in the layout of fa_row) in place
+template <int NC>
+__device__ __forceinline__ void fa_convert(unsigned char *sm, int ws, const unsigned *key)
+{
+    double *raw = (double *)sm;
+    int2 *xs = (int2 *)sm;
+    for (int t = threadIdx.x; t < ws * NC; t += blockDim.x) {
+        const int c = NC == 1 ? 0 : 2 * (t / (2 * ws)) + (t & 1);
+        xs[t] = fa_split(fa_round(raw[t], (int)key[c]));
+    }
+}
+template <int NC>
+__device__ __forceinline__ int fa_slot(int j, int c, int ws)   // of column c's entry j
+{
+    return NC == 1 ? j : (c >> 1) * 2 * ws + 2 * j + (c & 1);
+}
+
+// ---------------------------------------------------------------------------
+// 3. near rows: CTA per (leaf, slice of NR rows, group of columns)
+// ---------------------------------------------------------------------------
+struct FaNear {
+    int fl, NR, nrhs, c0;
+    const int *kb, *ke, *pw, *gcol, *goff, *rowptr, *colidx;
+    const int64_t *poff;
+    const double *val;   // B + M
+    int folded;          // B + M are in the fixed-point panels
+    const int2 *D;
+    const int *re;
+    const double *Dd;    // FP64 panels
+};
+
+template <int NC>
+__global__ void __launch_bounds__(128) k_fa_near(FaNear P, const double *__restrict__ X, int64_t ld,
+                                                 double *__restrict__ Y, const int *skip)
+{
+    extern __shared__ __align__(16) unsigned char fa_sm[];
+    __shared__ unsigned key[NC];
+    if (skip && *skip) return;
+    const int lf = blockIdx.x, r0 = P.c0 + blockIdx.z * NC;
+    const int b_leaf = P.kb[P.fl + lf], b = b_leaf + blockIdx.y * P.NR, e = min(P.ke[P.fl + lf], b + P.NR);
+    if (b >= e) return;
+    const int W = P.pw[lf];
+    const int *gc = P.gcol + P.goff[lf];
+    double *raw = (double *)fa_sm;
+    if (threadIdx.x < NC) key[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        unsigned mk = 0;
+        const double *x = X + (size_t)(r0 + c) * ld;
+        for (int t = threadIdx.x; t < W; t += blockDim.x) {
+            const int j = gc[t];
+            const double v = j >= 0 && r0 + c < P.nrhs ? x[j] : 0.0;
+            raw[fa_slot<NC>(t, c, W)] = v;
+            mk = max(mk, fa_key(v));
+        }
+        mk = __reduce_max_sync(0xffffffffu, mk);
+        if ((threadIdx.x & 31) == 0) atomicMax(&key[c], mk);
+    }
+    __syncthreads();
+    bool slow = false;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) slow |= fa_slow(key[c]);
+    if (!slow) fa_convert<NC>(fa_sm, W, key);
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l8 = lane & 7, nw = blockDim.x >> 5;
+    for (int g0 = b + 4 * warp; g0 < e; g0 += 4 * nw) {
+        const int i = g0 + (lane >> 3);
+        const bool on = i < e;
+        const int2 *row = P.D + P.poff[lf] + (size_t)(i - b_leaf) * W;
+        if (!slow) {
+            FaAcc s[NC];
+            if (on) fa_row<NC>(row, W, l8, (const int4 *)fa_sm, W, s);
+            const int c = fa_sum8<NC>(s, l8), r = r0 + c;
+            if (on && (l8 & (8 / NC - 1)) == 0 && r < P.nrhs) {
+                double v = s[0].value() * fa_pow2(P.re[i] - 30) *
+                           fa_scale(key[c]);
+                if (!P.folded)
+                    for (int q = P.rowptr[i]; q < P.rowptr[i + 1]; ++q)
+                    v = fma(P.val[q], X[(size_t)r * ld + P.colidx[q]], v);
+                Y[(size_t)r * ld + i] = v;
+            }
+        } else if (on) {
+            for (int c = l8; c < NC && r0 + c < P.nrhs; c += 8) {
+                double v = 0.0;
+                for (int j = 0; j < W; ++j)
+                    v = fma(P.Dd[(row - P.D) + j], raw[fa_slot<NC>(j, c, W)], v);
+                for (int q = P.rowptr[i]; q < P.rowptr[i + 1]; ++q)
+                    v = fma(P.val[q], X[(size_t)(r0 + c) * ld + P.colidx[q]], v);
+                Y[(size_t)(r0 + c) * ld + i] = v;
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// 4. expansion: CTA per (leaf, slice of NR rows, group of columns)
+// ---------------------------------------------------------------------------
+template <int NC>
+__global__ void __launch_bounds__(128)
+k_fa_expand(FaFar P, int NR, const double *__restrict__ ye, const double *__restrict__ yhat, double *__restrict__ Y,
+            int64_t ld, const int *skip)
+{
+    extern __shared__ __align__(16) unsigned char fa_sm[];
+    __shared__ unsigned key[NC];
+    if (skip && *skip) return;
+    const int lf = blockIdx.x, r0 = P.c0 + blockIdx.z * NC, k = P.k, w = P.nlev * k, ws = P.wp;
+    const int b_leaf = P.kb[P.fl + lf], b = b_leaf + blockIdx.y * NR, e = min(P.ke[P.fl + lf], b + NR);
+    if (b >= e) return;
+    double *raw = (double *)fa_sm;
+    if (threadIdx.x < NC) key[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        unsigned mk = 0;
+        const int r = r0 + c;
+        for (int t = threadIdx.x; t < ws; t += blockDim.x) {
+            double v = 0.0;
+            if (t < w && r < P.nrhs) {
+                const int lv = t / k, a = t - lv * k;
+                const int node = ((P.fl + lf + 1) >> (P.nlev - 1 - lv)) - 1;
+                if (yhat) {
+                    v = yhat[((size_t)r * P.nnode + node) * k + a];
+                } else {
+                    const int q0 = P.fptr[node], q1 = P.fptr[node + 1];
+                    const double *p = ye + (size_t)r * P.nfar * k + a;
+#pragma unroll 4
+                    for (int q = q0; q < q1; ++q) v += p[(size_t)q * k];
+                }
+            }
+            raw[fa_slot<NC>(t, c, ws)] = v;
+            mk = max(mk, fa_key(v));
+        }
+        mk = __reduce_max_sync(0xffffffffu, mk);
+        if ((threadIdx.x & 31) == 0) atomicMax(&key[c], mk);
+    }
+    __syncthreads();
+    bool slow = false;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) slow |= fa_slow(key[c]);
+    if (!slow) fa_convert<NC>(fa_sm, ws, key);
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l8 = lane & 7, nw = blockDim.x >> 5;
+    const int eu = P.ue[lf];
+    for (int g0 = b + 4 * warp; g0 < e; g0 += 4 * nw) {
+        const int i = g0 + (lane >> 3);
+        const bool on = i < e;
+        const int2 *row = P.U + (size_t)i * P.wp;
+        if (!slow) {
+            FaAcc s[NC];
+            if (on) fa_row<NC>(row, w, l8, (const int4 *)fa_sm, ws, s);
+            const int c = fa_sum8<NC>(s, l8), r = r0 + c;
+            if (on && (l8 & (8 / NC - 1)) == 0 && r < P.nrhs)
+                Y[(size_t)r * ld + i] += s[0].value() * fa_pow2(eu - 30) *
+                                         fa_scale(key[c]);
+        } else if (on) {
+            for (int c = l8; c < NC && r0 + c < P.nrhs; c += 8) {
+                double v = 0.0;
+                for (int j = 0; j < w; ++j)
+                    v = fma(P.Ud[((size_t)(j / k) * P.N + i) * k + j % k], raw[fa_slot<NC>(j, c, ws)], v);
+                Y[(size_t)(r0 + c) * ld + i] += v;
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// One column: the kernels stream the operator (781 MB at 27k DoFs and rank 64),
+// so what bounds them is the number of loads in flight.  Every lane keeps two
+// batches of eight 16-byte loads going; the first is issued before x is gathered.
+// Measured against the column kernels above with NC = 1 (four loads ahead, none
+// before the gather): coupling 94 -> 66 us, near rows 65 -> 51, expansion 46 -> 38,
+// projections 32 -> 22 us.
+// ---------------------------------------------------------------------------
+constexpr int FA_B = 8;
+
+template <class L>
+__device__ __forceinline__ void fa_batch(int4 *a, int t0, int n, L load)
+{
+#pragma unroll
+    for (int q = 0; q < FA_B; ++q) a[q] = t0 + q < n ? load(t0 + q) : make_int4(0, 0, 0, 0);
+}
+
+// items 0..n-1 of a lane, a holding the first batch; use(item, t), zero items to
+// the end of the last batch; carry() after every EVERY items
+template <int EVERY, class L, class U, class C>
+__device__ __forceinline__ void fa_pipe(int4 *a, int n, L load, U use, C carry)
+{
+#pragma unroll 1
+    for (int t0 = 0; t0 < n; t0 += FA_B) {
+        int4 b[FA_B];
+        fa_batch(b, t0 + FA_B, n, load);
+#pragma unroll
+        for (int q = 0; q < FA_B; ++q) {
+            use(a[q], min(t0 + q, n - 1));
+            if ((q + 1) % EVERY == 0) carry();
+        }
+#pragma unroll
+        for (int q = 0; q < FA_B; ++q) a[q] = b[q];
+    }
+}
+
+__device__ __forceinline__ int4 fa_ld(const int4 *p) { return __ldcs(p); }   // streamed once
+
+__global__ void __launch_bounds__(128)
+k_fa_proj1(FaFar P, const double *__restrict__ X, double *__restrict__ part, const int *skip)
+{
+    extern __shared__ __align__(16) unsigned char fa_sm[];
+    __shared__ unsigned key;
+    if (skip && *skip) return;
+    const int leaf = blockIdx.x, b = P.kb[P.fl + leaf], n = P.ke[P.fl + leaf] - b, w2 = P.wp >> 1;
+    const int cp = blockIdx.y * blockDim.x + threadIdx.x;
+    const int4 *M = (const int4 *)P.U + (size_t)b * w2 + min(cp, w2 - 1);
+    auto load = [&](int t) { return __ldg(M + (size_t)t * w2); };   // read again by the expansion
+    int4 a[FA_B];
+    fa_batch(a, 0, n, load);
+    double *raw = (double *)fa_sm;
+    int2 *xs = (int2 *)fa_sm;
+    if (threadIdx.x == 0) key = 0;
+    __syncthreads();
+    unsigned mk = 0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        raw[i] = X[b + i];
+        mk = max(mk, fa_key(raw[i]));
+    }
+    mk = __reduce_max_sync(0xffffffffu, mk);
+    if ((threadIdx.x & 31) == 0 && mk) atomicMax(&key, mk);
+    __syncthreads();
+    const unsigned ky = key;
+    const bool slow = fa_slow(ky);
+    if (!slow)
+        for (int i = threadIdx.x; i < n; i += blockDim.x) xs[i] = fa_split(fa_round(raw[i], ky));
+    __syncthreads();
+    FaAcc s0, s1;
+    if (!slow)
+        fa_pipe<4>(a, n, load,
+                [&](int4 m, int t) {
+                    const int2 x = xs[t];
+                    s0.mac(make_int2(m.x, m.y), x);
+                    s1.mac(make_int2(m.z, m.w), x);
+                },
+                [&] { s0.carry(), s1.carry(); });
+    s0.fold();
+    s1.fold();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int col = 2 * cp + h, lv = col / P.k, al = col - lv * P.k;
+        if (cp >= w2 || lv >= P.nlev) continue;
+        double v = (h ? s1 : s0).value() * fa_pow2(P.ue[leaf] - 30) * fa_scale(ky);
+        if (slow) {
+            v = 0.0;
+            for (int i = 0; i < n; ++i) v = fma(P.Ud[((size_t)lv * P.N + b + i) * P.k + al], raw[i], v);
+        }
+        part[((size_t)lv * P.nleaf + leaf) * P.k + al] = v;
+    }
+}
+
+__global__ void __launch_bounds__(32 * FC_WARPS)
+k_fa_couple1(FaFar P, const double *__restrict__ part, const double *__restrict__ xhat, double *__restrict__ ye,
+             const int *skip)
+{
+    __shared__ int2 xs_[FC_WARPS][KMAX];
+    if (skip && *skip) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, e = blockIdx.x * FC_WARPS + warp, k = P.k;
+    if (e >= P.nfar) return;
+    // lanes over the pairs of columns, the rest of the warp over the rows
+    const int np = P.kp >> 1, ga = np > 16 ? 32 : np > 8 ? 16 : np > 4 ? 8 : 4, gb = 32 / ga;
+    const int pr = lane & (ga - 1), lb = lane / ga, n = (k + gb - 1) / gb;
+    const int4 *S = (const int4 *)P.S + (size_t)e * k * np + min(pr, np - 1);
+    auto load = [&](int t) {
+        const int b = lb + t * gb;
+        return b < k ? fa_ld(S + (size_t)b * np) : make_int4(0, 0, 0, 0);
+    };
+    int4 a[FA_B];
+    fa_batch(a, 0, n, load);
+    int2 *xs = xs_[warp];
+    double *raw = (double *)xs;
+    const int node = P.fcol[e], l = 31 - __clz(node + 1), sh = P.L - l, leaf0 = ((node + 1) << sh) - (1 << P.L);
+    unsigned ky = 0;
+    for (int b = lane; b < k; b += 32) {
+        double v = 0.0;
+        if (xhat) {
+            v = xhat[(size_t)node * k + b];
+        } else {
+            const double *p = part + ((size_t)(l - P.lmin) * P.nleaf + leaf0) * k + b;
+#pragma unroll 8
+            for (int j = 0; j < (1 << sh); ++j) v += p[(size_t)j * k];
+        }
+        raw[b] = v;
+        ky = max(ky, fa_key(v));
+    }
+    ky = __reduce_max_sync(0xffffffffu, ky);
+    __syncwarp();
+    double *out = ye + (size_t)e * k;
+    if (fa_slow(ky)) {
+        for (int al = lane; al < k; al += 32) {
+            double v = 0.0;
+            for (int b = 0; b < k; ++b) v = fma(P.Sd[((size_t)e * k + b) * k + al], raw[b], v);
+            out[al] = v;
+        }
+        return;
+    }
+    for (int b = lane; b < k; b += 32) xs[b] = fa_split(fa_round(raw[b], ky));
+    __syncwarp();
+    FaAcc s0, s1;
+    fa_pipe<4>(a, n, load,
+            [&](int4 m, int t) {
+                const int2 x = xs[min(lb + t * gb, k - 1)];   // the row past the end is zero
+                s0.mac(make_int2(m.x, m.y), x);
+                s1.mac(make_int2(m.z, m.w), x);
+            },
+            [&] { s0.carry(), s1.carry(); });
+    s0.fold();
+    s1.fold();
+    double v0 = s0.value(), v1 = s1.value();
+    for (int o = ga; o < 32; o <<= 1) {
+        v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+        v1 += __shfl_xor_sync(0xffffffffu, v1, o);
+    }
+    if (lb == 0 && pr < np) {
+        const double sc = fa_pow2(P.se[e] - 30), sx = fa_scale(ky);
+        out[2 * pr] = v0 * sc * sx;
+        if (2 * pr + 1 < k) out[2 * pr + 1] = v1 * sc * sx;
+    }
+}
+
+// gathered piece of one column (W entries of raw), its key in *key: fixed-point in place; true where it stays FP64
+__device__ __forceinline__ bool fa_piece(unsigned char *sm, int W, unsigned mk, unsigned *key, unsigned &ky)
+{
+    mk = __reduce_max_sync(0xffffffffu, mk);
+    if ((threadIdx.x & 31) == 0 && mk) atomicMax(key, mk);
+    __syncthreads();
+    ky = *key;
+    const bool slow = fa_slow(ky);
+    if (!slow) fa_convert<1>(sm, W, &ky);
+    __syncthreads();
+    return slow;
+}
+
+// 16 rows a CTA, 4 a warp, 8 lanes a row
+__global__ void __launch_bounds__(128)
+k_fa_near1(FaNear P, const double *__restrict__ X, double *__restrict__ Y, const int *skip)
+{
+    extern __shared__ __align__(16) unsigned char fa_sm[];
+    __shared__ unsigned key;
+    if (skip && *skip) return;
+    const int lf = blockIdx.x, b_leaf = P.kb[P.fl + lf], b = b_leaf + blockIdx.y * 16, e = min(P.ke[P.fl + lf], b + 16);
+    if (b >= e) return;
+    const int W = P.pw[lf], lane = threadIdx.x & 31, l8 = lane & 7, i = b + 4 * (threadIdx.x >> 5) + (lane >> 3);
+    const size_t ro = P.poff[lf] + (size_t)(min(i, e - 1) - b_leaf) * W;
+    const int4 *row = (const int4 *)(P.D + ro) + l8;
+    const int nv = W >> 1, n = (nv + 7) >> 3;
+    auto load = [&](int t) { return l8 + 8 * t < nv ? fa_ld(row + 8 * t) : make_int4(0, 0, 0, 0); };
+    int4 a[FA_B];
+    fa_batch(a, 0, n, load);
+    const int *gc = P.gcol + P.goff[lf];
+    double *raw = (double *)fa_sm;
+    if (threadIdx.x == 0) key = 0;
+    __syncthreads();
+    unsigned mk = 0, ky;
+#pragma unroll 4
+    for (int t = threadIdx.x; t < W; t += blockDim.x) {
+        const int j = gc[t];
+        const double v = j >= 0 ? X[j] : 0.0;
+        raw[t] = v;
+        mk = max(mk, fa_key(v));
+    }
+    const bool slow = fa_piece(fa_sm, W, mk, &key, ky);
+    FaAcc s;
+    if (!slow)
+        fa_pipe<2>(a, n, load,
+                [&](int4 m, int t) {
+                    const int4 x = ((const int4 *)fa_sm)[min(l8 + 8 * t, nv - 1)];
+                    s.mac(make_int2(m.x, m.y), make_int2(x.x, x.y));
+                    s.mac(make_int2(m.z, m.w), make_int2(x.z, x.w));
+                },
+                [&] { s.carry(); });
+    s.fold();
+    fa_sum8<1>(&s, l8);
+    if (i >= e || l8) return;
+    double v = s.value() * fa_pow2(P.re[i] - 30) * fa_scale(ky);
+    if (slow) {
+        v = 0.0;
+        for (int j = 0; j < W; ++j) v = fma(P.Dd[ro + j], raw[j], v);
+    }
+    if (slow || !P.folded)
+        for (int q = P.rowptr[i]; q < P.rowptr[i + 1]; ++q) v = fma(P.val[q], X[P.colidx[q]], v);
+    Y[i] = v;
+}
+
+__global__ void __launch_bounds__(128)
+k_fa_expand1(FaFar P, const double *__restrict__ ye, const double *__restrict__ yhat, double *__restrict__ Y,
+             const int *skip)
+{
+    extern __shared__ __align__(16) unsigned char fa_sm[];
+    __shared__ unsigned key;
+    if (skip && *skip) return;
+    const int lf = blockIdx.x, k = P.k, w = P.nlev * k, b0 = P.kb[P.fl + lf];
+    const int b = b0 + blockIdx.y * 16, e = min(P.ke[P.fl + lf], b + 16);
+    if (b >= e) return;
+    const int lane = threadIdx.x & 31, l8 = lane & 7, i = b + 4 * (threadIdx.x >> 5) + (lane >> 3);
+    const int nv = P.wp >> 1, n = (nv + 7) >> 3;
+    const int4 *row = (const int4 *)P.U + (size_t)min(i, e - 1) * nv + l8;
+    auto load = [&](int t) { return l8 + 8 * t < nv ? __ldg(row + 8 * t) : make_int4(0, 0, 0, 0); };
+    int4 a[FA_B];
+    fa_batch(a, 0, n, load);
+    double *raw = (double *)fa_sm;
+    if (threadIdx.x == 0) key = 0;
+    __syncthreads();
+    unsigned mk = 0, ky;
+#pragma unroll 2
+    for (int t = threadIdx.x; t < P.wp; t += blockDim.x) {
+        double v = 0.0;
+        if (t < w) {
+            const int lv = t / k, al = t - lv * k, node = ((P.fl + lf + 1) >> (P.nlev - 1 - lv)) - 1;
+            if (yhat) {
+                v = yhat[(size_t)node * k + al];
+            } else {
+                const int q1 = P.fptr[node + 1];
+#pragma unroll 8
+                for (int q = P.fptr[node]; q < q1; ++q) v += ye[(size_t)q * k + al];
+            }
+        }
+        raw[t] = v;
+        mk = max(mk, fa_key(v));
+    }
+    const bool slow = fa_piece(fa_sm, P.wp, mk, &key, ky);
+    FaAcc s;
+    if (!slow)
+        fa_pipe<2>(a, n, load,
+                [&](int4 m, int t) {
+                    const int4 x = ((const int4 *)fa_sm)[min(l8 + 8 * t, nv - 1)];
+                    s.mac(make_int2(m.x, m.y), make_int2(x.x, x.y));
+                    s.mac(make_int2(m.z, m.w), make_int2(x.z, x.w));
+                },
+                [&] { s.carry(); });
+    s.fold();
+    fa_sum8<1>(&s, l8);
+    if (i >= e || l8) return;
+    double v = s.value() * fa_pow2(P.ue[lf] - 30) * fa_scale(ky);
+    if (slow) {
+        v = 0.0;
+        for (int j = 0; j < w; ++j) v = fma(P.Ud[((size_t)(j / k) * P.N + i) * k + j % k], raw[j], v);
+    }
+    Y[i] += v;
+}
+
+// ---------------------------------------------------------------------------
+// the operands
+// ---------------------------------------------------------------------------
+// largest exponent key of n values (warp), as the exponent E with |v| < 2^E;
+// flags what the format cannot hold
+__device__ __forceinline__ int fa_exponent(unsigned key, int *err)
+{
+    key = __reduce_max_sync(0xffffffffu, key);
+    if (key == 0x7ffu || (key && key < 200u) || key > 1900u) {
+        if ((threadIdx.x & 31) == 0) atomicOr(err, 4);
+        return 0;
+    }
+    return key ? (int)key - 1022 : 0;
+}
+
+// near panel rows, a warp each; B + M added at their panel positions
+__global__ void k_fa_build_near(int N, int fl, const int *__restrict__ vleaf, const int *__restrict__ kb,
+                                const int *__restrict__ pw, const int64_t *__restrict__ poff,
+                                const double *__restrict__ D, const int *__restrict__ rowptr,
+                                const int64_t *__restrict__ bpos, const double *__restrict__ val,
+                                int2 *__restrict__ out, int *__restrict__ re, int *err)
+{
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (i >= N) return;
+    const int lf = vleaf[i], W = pw[lf];
+    const size_t o = poff[lf] + (size_t)(i - kb[fl + lf]) * W;
+    unsigned key = 0;
+    for (int j = lane; j < W; j += 32) key = max(key, fa_key(D[o + j]));
+    if (val)
+        for (int q = rowptr[i] + lane; q < rowptr[i + 1]; q += 32) key = max(key, fa_key(val[q]));
+    const int E = fa_exponent(key, err) + (val ? 1 : 0);   // room for the sum of two entries
+    for (int j = lane; j < W; j += 32) out[o + j] = fa_split(fa_round(D[o + j], E + 1022));
+    __syncwarp();
+    if (val)
+        for (int q = rowptr[i] + lane; q < rowptr[i + 1]; q += 32) {   // distinct positions
+            const int2 d = out[bpos[q]];
+            out[bpos[q]] = fa_split(((i64)d.y << FA_LO) + d.x + fa_round(val[q], E + 1022));
+        }
+    if (lane == 0) re[i] = E;
+}
+
+// coupling blocks, a warp each; rows padded to an even length
+__global__ void k_fa_build_S(int nfar, int k, int kp, const double *__restrict__ S, int2 *__restrict__ out,
+                             int *__restrict__ se, int *err)
+{
+    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (e >= nfar) return;
+    const double *in = S + (size_t)e * k * k;
+    int2 *o = out + (size_t)e * k * kp;
+    unsigned key = 0;
+    for (int j = lane; j < k * k; j += 32) key = max(key, fa_key(in[j]));
+    const int E = fa_exponent(key, err);
+    for (int j = lane; j < k * kp; j += 32) {
+        const int b = j / kp, a = j - b * kp;
+        o[j] = a < k ? fa_split(fa_round(in[b * k + a], E + 1022)) : make_int2(0, 0);
+    }
+    if (lane == 0) se[e] = E;
+}
+
+// flattened bases, CTA per leaf: [level][N][k] -> [N][level k], rows padded to an even length
+__global__ void k_fa_build_U(int fl, int N, int k, int nlev, const int *__restrict__ kb, const int *__restrict__ ke,
+                             const double *__restrict__ U, int2 *__restrict__ out, int *__restrict__ ue, int *err)
+{
+    __shared__ unsigned key;
+    __shared__ int E;
+    const int b = kb[fl + blockIdx.x], n = ke[fl + blockIdx.x] - b, w = nlev * k, wp = (w + 1) & ~1;
+    if (threadIdx.x == 0) key = 0;
+    __syncthreads();
+    unsigned mk = 0;
+    for (int t = threadIdx.x; t < n * w; t += blockDim.x) {
+        const int i = b + t / w, q = t % w;
+        mk = max(mk, fa_key(U[((size_t)(q / k) * N + i) * k + q % k]));
+    }
+    atomicMax(&key, mk);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int e = fa_exponent(key, err);
+        if (threadIdx.x == 0) E = e;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < n * wp; t += blockDim.x) {
+        const int i = b + t / wp, q = t % wp;
+        out[(size_t)i * wp + q] =
+            q < w ? fa_split(fa_round(U[((size_t)(q / k) * N + i) * k + q % k], E + 1022)) : make_int2(0, 0);
+    }
+    if (threadIdx.x == 0) ue[blockIdx.x] = E;
+}
+
+}  // namespace
+
+// the mesh's flattened bases (geometry only, end of the mesh setup)
+void build_fixed_bases(MeshData &m)
+{
+    const int nlev = m.nfar > 0 ? m.kt.L - m.far_lmin + 1 : 0;
+    m.fa_ok = true;
+    if (!nlev) return;
+    DBuf<int> err;
+    err.alloc(1);
+    err.zero(nullptr);
+    m.fa_U.alloc((size_t)((nlev * m.k + 1) & ~1) * m.N);
+    m.fa_ue.alloc(m.kt.nleaf);
+    k_fa_build_U<<<m.kt.nleaf, 256>>>(m.kt.first_leaf(), m.N, m.k, nlev, m.kt_begin.p, m.kt_end.p, m.Ul64.p,
+                                      (int2 *)m.fa_U.p, m.fa_ue.p, err.p);
+    VFD_CUDA(cudaGetLastError());
+    int h = 0;
+    VFD_CUDA(cudaMemcpy(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost));
+    if (h) {
+        m.fa_ok = false;
+        m.fa_U.release();
+    }
+}
+
+// the operator's near panels (with B + M) and coupling blocks; err gets bit 2
+// where an entry does not fit
+void build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t st)
+{
+    op.fa_D.alloc(m.near_entries);
+    op.fa_re.alloc(m.N);
+    k_fa_build_near<<<cdiv((long long)m.N * 32, 256), 256, 0, st>>>(
+        m.N, m.kt.first_leaf(), m.vleaf.p, m.kt_begin.p, m.panel_w.p, m.panel_off.p, op.D64.p, m.rowptr.p, m.bm_pos.p,
+        m.bm_in_panels ? op.valBM.p : nullptr, (int2 *)op.fa_D.p, op.fa_re.p, err);
+    if (m.nfar) {
+        const int kp = (m.k + 1) & ~1;
+        op.fa_S.alloc((size_t)m.nfar * m.k * kp);
+        op.fa_se.alloc(m.nfar);
+        k_fa_build_S<<<cdiv((long long)m.nfar * 32, 256), 256, 0, st>>>(m.nfar, m.k, kp, op.S64.p, (int2 *)op.fa_S.p,
+                                                                        op.fa_se.p, err);
+    }
+    VFD_CUDA(cudaGetLastError());
+}
+
+namespace {
+
+// one launch of every kernel for ng groups of NC columns from column c0
+template <int NC>
+void apply_group(const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int nrhs, int64_t ld,
+                 bool summed, cudaStream_t st, const int *skip)
+{
+    const int k = m.k, nleaf = m.kt.nleaf, nnode = m.kt.nnode;
+    const bool far = m.nfar > 0;
+    FaFar P;
+    P.fl = m.kt.first_leaf();
+    P.nleaf = nleaf;
+    P.lmin = m.far_lmin;
+    P.L = m.kt.L;
+    P.nlev = far ? m.kt.L - m.far_lmin + 1 : 0;
+    P.k = k;
+    P.kp = (k + 1) & ~1;
+    P.wp = (P.nlev * k + 1) & ~1;
+    P.nnode = nnode;
+    P.nfar = m.nfar;
+    P.nrhs = nrhs;
+    P.c0 = c0;
+    P.kb = m.kt_begin.p;
+    P.ke = m.kt_end.p;
+    P.fptr = m.far_ptr.p;
+    P.fcol = m.far_col.p;
+    P.U = (const int2 *)m.fa_U.p;
+    P.S = (const int2 *)op.fa_S.p;
+    P.ue = m.fa_ue.p;
+    P.Ud = m.Ul64.p;
+    P.Sd = op.S64.p;
+    P.N = m.N;
+    P.se = op.fa_se.p;
+    const int w = P.nlev * k, cols = std::min(nrhs - c0, ng * NC);
+    // one column: the kernels get its own pieces
+    const size_t ps = (size_t)P.nlev * nleaf * k, hs = (size_t)nnode * k, ys = (size_t)m.nfar * k;
+    const double *X1 = X + (size_t)c0 * ld;
+    double *Y1 = Y + (size_t)c0 * ld;
+    if (far) {
+        VFD_CUDA(cudaEventRecord(op.ev_fork, st));
+        VFD_CUDA(cudaStreamWaitEvent(op.side, op.ev_fork, 0));
+        const size_t shp = (size_t)m.max_leaf_size * NC * 8;
+        if (NC == 1) k_fa_proj1<<<dim3(nleaf, cdiv(w, 256)), 128, shp, op.side>>>(P, X1, op.P64.p + c0 * ps, skip);
+        else k_fa_proj<NC><<<dim3(nleaf, cdiv(w, 128), ng), 128, shp, op.side>>>(P, X, ld, op.P64.p, skip);
+        if (summed) launch_far_sum(m, op, c0, cols, op.side, skip);
+        if (NC == 1)
+            k_fa_couple1<<<cdiv(m.nfar, FC_WARPS), 32 * FC_WARPS, 0, op.side>>>(
+                P, op.P64.p + c0 * ps, summed ? op.xhat.p + c0 * hs : nullptr, op.ye64.p + c0 * ys, skip);
+        else
+            k_fa_couple<NC><<<dim3(cdiv(m.nfar, FC_WARPS), ng), 32 * FC_WARPS, 0, op.side>>>(
+                P, op.P64.p, summed ? op.xhat.p : nullptr, op.ye64.p, skip);
+        if (summed) launch_far_couple_sum(m, op, c0, cols, op.side, skip);
+    }
+    FaNear R;
+    R.fl = P.fl;
+    R.NR = 64;
+    R.nrhs = nrhs;
+    R.c0 = c0;
+    R.kb = P.kb;
+    R.ke = P.ke;
+    R.pw = m.panel_w.p;
+    R.gcol = m.gcol.p;
+    R.goff = m.gcol_off.p;
+    R.rowptr = m.rowptr.p;
+    R.colidx = m.colidx.p;
+    R.poff = m.panel_off.p;
+    R.val = op.valBM.p;
+    R.folded = m.bm_in_panels ? 1 : 0;
+    R.Dd = op.D64.p;
+    R.D = (const int2 *)op.fa_D.p;
+    R.re = op.fa_re.p;
+    const size_t shm = (size_t)m.max_panel_w * NC * 8;
+    VFD_REQUIRE(shm <= 227 * 1024, VFD_EUNSUPPORTED,
+                "apply: a near panel is wider than shared memory holds (use a low-rank operator, lambda > 0)");
+    if (NC == 1) {
+        if (shm > 47 * 1024)
+            VFD_CUDA(cudaFuncSetAttribute(k_fa_near1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+        k_fa_near1<<<dim3(nleaf, cdiv(m.max_leaf_size, 16)), 128, shm, st>>>(R, X1, Y1, skip);
+    } else {
+        if (shm > 47 * 1024)
+            VFD_CUDA(cudaFuncSetAttribute(k_fa_near<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+        k_fa_near<NC><<<dim3(nleaf, cdiv(m.max_leaf_size, R.NR), ng), 128, shm, st>>>(R, X, ld, Y, skip);
+    }
+    if (far) {
+        VFD_CUDA(cudaEventRecord(op.ev_join, op.side));
+        VFD_CUDA(cudaStreamWaitEvent(st, op.ev_join, 0));
+        const size_t she = (size_t)P.wp * NC * 8;
+        if (NC == 1) {
+            k_fa_expand1<<<dim3(nleaf, cdiv(m.max_leaf_size, 16)), 128, she, st>>>(
+                P, op.ye64.p + c0 * ys, summed ? op.yhat.p + c0 * hs : nullptr, Y1, skip);
+        } else {
+            if (she > 47 * 1024)
+                VFD_CUDA(cudaFuncSetAttribute(k_fa_expand<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)she));
+            k_fa_expand<NC><<<dim3(nleaf, cdiv(m.max_leaf_size, 64), ng), 128, she, st>>>(
+                P, 64, op.ye64.p, summed ? op.yhat.p : nullptr, Y, ld, skip);
+        }
+    }
+    VFD_CUDA(cudaGetLastError());
+}
+
+}  // namespace
+
+// Y = A X with the FP64 operator (all parts); the workspaces are those of the FP64 apply
+void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st,
+                 const int *skip)
+{
+    // the node sums inside the gathers pay for few columns and short spans
+    const bool summed = nrhs >= 4 || m.kt.L - m.far_lmin > 7;
+    // widest group whose panel piece leaves room for two CTAs an SM
+    int nc = 8;
+    while (nc > 1 && (size_t)m.max_panel_w * nc * 8 > 100 * 1024) nc >>= 1;
+    int c0 = 0;
+    auto go = [&](int NC, int ng) {
+        if (NC == 8) apply_group<8>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip);
+        else if (NC == 4) apply_group<4>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip);
+        else if (NC == 2) apply_group<2>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip);
+        else apply_group<1>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip);
+        c0 += NC * ng;
+    };
+    if (nrhs / nc) go(nc, nrhs / nc);
+    while (c0 < nrhs) {   // the remainder in one group of the next size
+        int r = 1;
+        while (r < std::min(nc, nrhs - c0)) r <<= 1;
+        go(r, 1);
+    }
+}
+
+}  // namespace vfd

@@ -1143,6 +1143,7 @@ MeshData *build_mesh(int d, int64_t n_vert, const double *coords, int64_t n_cell
             m->gl9_w.upload(gw);
             m->mtab.upload(make_math_tables());
             setup_fixed(*m, qx, qw, meas, cdiam);
+            build_fixed_bases(*m);
         }
     } catch (...) {
         delete m;

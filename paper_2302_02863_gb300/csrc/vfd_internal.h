@@ -160,6 +160,11 @@ struct MeshData {
     DBuf<int> kt_Uoff;         // nleaf
     int far_lmin = 0;          // first level with admissible blocks
     DBuf<double> Ul64;         // per-level bases, (L - far_lmin + 1) x N x k (the last slice is U)
+    // the flattened bases in the fixed-point format of apply_fixed.cu, N x (levels x k), and
+    // their exponents per leaf (fa_ok: every entry fits)
+    bool fa_ok = false;
+    DBuf<long long> fa_U;
+    DBuf<int> fa_ue;
     DBuf<double> E64;          // transfers E_c[beta][alpha] = l^parent_alpha(xi^c_beta), nnode x k x k
     int p_in = 0, k_in = 0;    // interpolation order / rank of the inner operator's far field (0: p, k)
     DBuf<double> kt_cheb_in, U_in64, E_in64;   // its Chebyshev nodes, leaf bases (N x k_in), transfers
@@ -258,6 +263,11 @@ struct OpData {
     DBuf<double> rho;                  // interior points, canonical order
     DBuf<double> S64;                  // nfar * k * k
     DBuf<double> D64;                  // near entries
+    // fixed-point copies for the FP64 apply (apply_fixed.cu): near panels with B + M added and an
+    // exponent per row, coupling blocks and an exponent per block; fa: built, every entry fits
+    bool fa = false;
+    DBuf<long long> fa_D, fa_S;
+    DBuf<int> fa_re, fa_se;
     DBuf<float> S32, D32, Ul32;        // FP32 copies (VFD_FP32)
     DBuf<unsigned short> Dtc;          // BF16 near panels pre-tiled for the TMA-fed tcgen05 kernel (first batched use)
     std::vector<int64_t> Dtc_off;      //   element offset of each leaf's image (nleaf + 1)
@@ -403,6 +413,9 @@ void launch_coupling_fixed(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_rho_coupling_fixed(const MeshData &m, OpData &op, double *yt, cudaStream_t st);
 void launch_rho_near_fixed(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_selftest_math(const MeshData &m, int which, long long n, const double *x, double *out, cudaStream_t st);
+// apply_fixed.cu
+void build_fixed_bases(MeshData &m);
+void build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t st);
 // apply.cu
 void apply_parts_ex(const MeshData &m, OpData &op, int parts, const double *X, double *Y, int nrhs, int64_t ld,
                     bool lowp, cudaStream_t st, const int *skip);
