@@ -122,30 +122,38 @@ void upload_field(const vfd_field *f, int n_vert, DBuf<double> &rows, DBuf<doubl
             if (r[j] != std::floor(r[j]) || std::fabs(r[j]) > 4.0) grouped = false;
         if (r[2] != 0.0) grouped = false;
     }
+    // Rows of equal |k_1| and |k_2| share c_1, s_1, c_2, s_2, so their coefficients
+    // add: one set of four per class (|k_1|, |k_2|), at most 25
     std::vector<int> gi;
     size_t coef_off = h.size();
     int ngrp = 0;
     if (grouped) {
+        double cls[5][5][4] = {};
+        bool has[5][5] = {};
+        for (int t = 0; t < f->n_fourier; ++t) {
+            const double *r = f->fourier + 5 * t;
+            const int m1 = (int)std::fabs(r[0]), m2 = (int)std::fabs(r[1]);
+            const double s1 = r[0] < 0 ? -1.0 : 1.0, s2 = r[1] < 0 ? -1.0 : 1.0;
+            const double ar = r[3] * std::cos(r[4]), ai = r[3] * std::sin(r[4]);
+            has[m1][m2] = true;
+            cls[m1][m2][0] += ar;
+            cls[m1][m2][1] += -ai * s2;
+            cls[m1][m2][2] += -s1 * s2 * ar;
+            cls[m1][m2][3] += -s1 * ai;
+        }
         std::vector<int> mk;
-        size_t t0 = 0;
-        while (t0 < order.size()) {
-            const double k1 = f->fourier[5 * order[t0]];
-            size_t t1 = t0;
-            while (t1 < order.size() && f->fourier[5 * order[t1]] == k1) ++t1;
-            gi.push_back((int)std::fabs(k1));
-            gi.push_back((int)(t1 - t0));
-            const double s1 = k1 < 0 ? -1.0 : 1.0;
-            for (size_t q = t0; q < t1; ++q) {
-                const double *r = f->fourier + 5 * order[q];
-                const double ar = r[3] * std::cos(r[4]), ai = r[3] * std::sin(r[4]), s2 = r[1] < 0 ? -1.0 : 1.0;
-                mk.push_back((int)std::fabs(r[1]));
-                h.push_back(ar);
-                h.push_back(-ai * s2);
-                h.push_back(-s1 * s2 * ar);
-                h.push_back(-s1 * ai);
-            }
+        for (int m1 = 0; m1 < 5; ++m1) {
+            int n = 0;
+            for (int m2 = 0; m2 < 5; ++m2)
+                if (has[m1][m2]) {
+                    mk.push_back(m2);
+                    h.insert(h.end(), cls[m1][m2], cls[m1][m2] + 4);
+                    ++n;
+                }
+            if (!n) continue;
+            gi.push_back(m1);
+            gi.push_back(n);
             ++ngrp;
-            t0 = t1;
         }
         gi.insert(gi.end(), mk.begin(), mk.end());
     }
@@ -296,10 +304,18 @@ vfd_status vfd_assemble(vfd_mesh_t mesh, const vfd_field *s, const vfd_field *lo
     // a5: singular near field
     {
         DBuf<double> Lbuf;
-        launch_singular_B(m, *op, Lbuf, st);
+        if (op->fx) op->errflag.zero(st);
+        launch_singular_B(m, *op, Lbuf, op->fx, st);
         mark();
         launch_gather_B(m, *op, Lbuf, st);
+        herr[0] = 0;
+        if (op->fx) VFD_CUDA(cudaMemcpyAsync(herr, op->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, st));
         VFD_CUDA(cudaStreamSynchronize(st));
+        if (herr[0]) {   // a mapped point's fields do not fit the fixed-point formats
+            launch_singular_B(m, *op, Lbuf, false, st);
+            launch_gather_B(m, *op, Lbuf, st);
+            VFD_CUDA(cudaStreamSynchronize(st));
+        }
     }
     // a7: weighted mass (and B + M for the apply)
     launch_gather_M(m, *op, st);

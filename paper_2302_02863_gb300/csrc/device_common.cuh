@@ -47,9 +47,9 @@ __device__ __forceinline__ void trig_table(int d, int kmax, const double *x, Tri
 // A Fourier row (k, A = amp e^{i phase}) contributes Re(A e^{i pi k.x}).  With
 // the trig table the rows are summed in groups of equal k_1:
 // Re(e^{i pi k_1 x_1} sum_group A e^{i pi (k_2 x_2 + k_3 x_3)}).  2D rows with
-// integer |k| <= 4 use the grouping prepared on the host (integer indices, the
-// signs folded into four coefficients per row: four FMAs per row); other rows
-// (sorted by k_1 on the host) are grouped on the fly.
+// integer |k| <= 4 use the classes prepared on the host (integer indices, the
+// signs folded into four coefficients per class (|k_1|, |k_2|): four FMAs per
+// class); other rows (sorted by k_1 on the host) are grouped on the fly.
 __device__ __forceinline__ double field_terms(const DField &F, int d, const double *x, const TrigTable *tab)
 {
     double v = F.c0;

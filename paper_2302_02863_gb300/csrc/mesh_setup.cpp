@@ -1138,6 +1138,7 @@ MeshData *build_mesh(int d, int64_t n_vert, const double *coords, int64_t n_cell
             gauss_legendre01(opts.n_sing, gx, gw);
             m->gl_x.upload(gx);
             m->gl_w.upload(gw);
+            m->gl_min = gx[0];
             gauss_legendre01(9, gx, gw);
             m->gl9_x.upload(gx);
             m->gl9_w.upload(gw);

@@ -8,7 +8,11 @@
 // once per distinct mapped point into shared memory, then sweeps the 4D
 // points with table lookups, so a 4D point costs one log and one exp.  The
 // per-index powers and logarithms of zeta, t and eta1 are tabulated per CTA.
+#include <algorithm>
+#include <cmath>
+
 #include "device_common.cuh"
+#include "gamma_fixed.cuh"
 
 namespace vfd {
 
@@ -252,9 +256,238 @@ __global__ void __launch_bounds__(256) k_singular2d(Sing2Params P, double *__res
     }
 }
 
+// ---------------------------------------------------------------------------
+// The same sums on the fixed-point kernel evaluations (gamma_fixed.cuh).
+//
+// What of a 4D point does not depend on the pair is tabulated once per assembly
+// (k_sing_table): the coefficients a, b of the scaled difference x - y, the
+// products w f_i f_j of rule weight, map Jacobian and basis differences, and the
+// part of the exponent that comes from zeta, t and eta1,
+//   (2 sbar - S) q + (2 - S) l = cst - (b_x + b_y) nu,   S = 2 (b_x + b_y) - 2,
+// q = ln zeta / c (+ ln t / c2) and l = ln eta1 in the identical case: nu adds to N
+// = -ln |difference|^2 and cst to the sum of the a terms.  The basis differences
+// sum to zero, so row and column 0 of a local matrix are minus the sums of the
+// others and 10, 6 or 3 products (vertex, edge, identical) are enough.
+// A 4D point then takes 10 FP64 instructions for the difference, 3 to 10 for the
+// sums, and one evaluation (FP64 kernel: about 150 in all); the fields at the
+// mapped points, about one evaluation of s and log kappa per 4D point, are as
+// before.  87.8M 4D points (27k DoFs): 48.1 -> 25.0 ms; P1 fields, 13.1M points
+// (4k DoFs): 3.3 -> 1.7 ms.
+// ---------------------------------------------------------------------------
+constexpr int ST_A = 0, ST_NU = 4, ST_CST = 5, ST_F = 6, ST_SLOTS = 16;
+
+__device__ __forceinline__ int sing_regions(int type) { return type == 1 ? 2 : (type == 2 ? 5 : 3); }
+// first table entry of a type, in units of ns^4
+__device__ __forceinline__ int sing_first(int type) { return type == 1 ? 0 : (type == 2 ? 2 : 7); }
+
+__global__ void k_sing_table(int ns, double sbar, const double *__restrict__ gx, const double *__restrict__ gw,
+                             double *__restrict__ out)
+{
+    const int per = ns * ns * ns * ns, t = blockIdx.x * blockDim.x + threadIdx.x, ne = 10 * per;
+    if (t >= ne) return;
+    const int type = t < 2 * per ? 1 : (t < 7 * per ? 2 : 3);
+    const int i = t - sing_first(type) * per, reg = i / per, r = i - reg * per;
+    const int iz = r % ns, i1 = (r / ns) % ns, i2 = (r / (ns * ns)) % ns, i3 = r / (ns * ns * ns);
+    const double c = 4.0 - 2.0 * sbar, c2 = 2.0 - 2.0 * sbar;
+    const double e1 = gx[i1], e3 = gx[i3], wq = gw[iz] * gw[i1] * gw[i2] * gw[i3], lz = log(gx[iz]);
+    double a[2], b[2], f[5] = {0, 0, 0, 0, 0}, w, q, l = 0.0;
+    if (type == 3) {
+        double dr[2];
+        const double lt = log(gx[i2]);
+        map_id(reg, e1, exp(lt / c2), e3, a, b, dr);
+        a[0] = dr[0];
+        a[1] = dr[1];
+        b[0] = b[1] = 0.0;
+        w = wq * 2.0 / (c * c2);   // the mirror regions T_I^(4..6) double the sum
+        q = lz / c + lt / c2;
+        l = log(e1);
+        f[1] = dr[0] - dr[1];
+        f[2] = dr[1];
+    } else {
+        double jac;
+        map_ve(type, reg, e1, gx[i2], e3, a, b, jac);
+        w = wq * jac / c;
+        q = lz / c;
+        if (type == 1) {
+            f[1] = a[0] - a[1]; f[2] = a[1]; f[3] = -(b[0] - b[1]); f[4] = -b[1];
+        } else {
+            f[1] = (a[0] - a[1]) - (b[0] - b[1]); f[2] = a[1]; f[3] = -b[1];
+        }
+    }
+    out[(size_t)(ST_A + 0) * ne + t] = a[0];
+    out[(size_t)(ST_A + 1) * ne + t] = a[1];
+    out[(size_t)(ST_A + 2) * ne + t] = b[0];
+    out[(size_t)(ST_A + 3) * ne + t] = b[1];
+    const double nu = -2.0 * (q + l), cst = ((2.0 * sbar + 2.0) * q + 4.0 * l) * 1.4426950408889634;
+    out[(size_t)ST_NU * ne + t] = __longlong_as_double(__double2ll_rn(nu * 72057594037927936.0));        // Q56
+    out[(size_t)ST_CST * ne + t] = __longlong_as_double(__double2ll_rn(cst * 9007199254740992.0));       // Q53
+    const int nf = type == 1 ? 4 : (type == 2 ? 3 : 2);
+    int s = ST_F;
+    for (int u = 1; u <= nf; ++u)
+        for (int v = u; v <= nf; ++v, ++s) out[(size_t)s * ne + t] = w * f[u] * f[v];
+}
+
+struct SingFx {
+    Sing2Params S;
+    int w;             // scale of the fixed-point coordinates
+    const double *st;  // k_sing_table
+    const u64 *tab;
+    int *err;
+};
+
+// sum of v[0..15] over the warp, halving the values at every step: lane 2 q and 2 q + 1 get sum q
+template <int NF>
+__device__ __forceinline__ double warp_sum16(double *v, int lane)
+{
+#pragma unroll
+    for (int q = NF; q < 16; ++q) v[q] = 0.0;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        const int o = 16 >> h, n = 8 >> h;
+        const bool up = lane & o;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (q < n && q < NF) {
+                const double send = up ? v[q] : v[q + n], keep = up ? v[q + n] : v[q];
+                v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// phase 2 of one pair with NF products
+template <int NF, bool IDENT>
+__device__ __forceinline__ void sing_sum(const SingFx &P, const FxTab &tab, int type, const double *JP, const double *JQ,
+                                         const i64 *fa, const i64 *fb, const int *xo, const int *yo, double pre,
+                                         double *__restrict__ L, int lane)
+{
+    const int ns = P.S.ns, per = ns * ns * ns * ns, tot = sing_regions(type) * per, ne = 10 * per, ti = type - 1;
+    const double *st = P.st + (size_t)sing_first(type) * per;
+    double acc[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) acc[q] = 0.0;
+    for (int idx = lane; idx < tot; idx += 32) {
+        const int reg = idx / per, r = idx - reg * per;
+        const int ind[4] = {r % ns, (r / ns) % ns, (r / (ns * ns)) % ns, r / (ns * ns * ns)};
+        const int ix = xo[reg] + tindex(c_xmask[ti][reg], ns, ind), iy = yo[reg] + tindex(c_ymask[ti][reg], ns, ind);
+        const double a0 = st[idx], a1 = st[ne + idx];
+        double dx = JP[0] * a0 + JP[1] * a1, dy = JP[2] * a0 + JP[3] * a1;
+        if (!IDENT) {
+            const double b0 = st[2 * (size_t)ne + idx], b1 = st[3 * (size_t)ne + idx];
+            dx = dx - JQ[0] * b0 - JQ[1] * b1;
+            dy = dy - JQ[2] * b0 - JQ[3] * b1;
+        }
+        u64 M;
+        int K;
+        fx_r2(dx * dx + dy * dy, P.w, M, K);
+        const u64 N = fx_neglog(tab, M, K) + (u64)__double_as_longlong(st[(size_t)ST_NU * ne + idx]);
+        const i64 A = fa[ix] + fa[iy] + __double_as_longlong(st[(size_t)ST_CST * ne + idx]);
+        const double w = fx_exp(tab, A, (u64)(fb[ix] + fb[iy]), N);
+#pragma unroll
+        for (int q = 0; q < NF; ++q) acc[q] = fma(w, st[(size_t)(ST_F + q) * ne + idx], acc[q]);
+    }
+    const double mine = pre * warp_sum16<NF>(acc, lane);   // lanes 2 q hold sum q
+    // local matrix: rows 1..nf from the sums, row and column 0 from the zero row sums
+    constexpr int nf = NF == 10 ? 4 : (NF == 6 ? 3 : 2);
+    double m[5][5] = {};
+    int s = 0;
+#pragma unroll
+    for (int u = 1; u <= nf; ++u)
+#pragma unroll
+        for (int v = u; v <= nf; ++v, ++s) m[u][v] = m[v][u] = __shfl_sync(0xffffffffu, mine, 2 * s);
+    double all = 0.0;
+#pragma unroll
+    for (int u = 1; u <= nf; ++u) {
+        double t = 0.0;
+#pragma unroll
+        for (int v = 1; v <= nf; ++v) t += m[u][v];
+        m[0][u] = m[u][0] = -t;
+        all += t;
+    }
+    m[0][0] = all;
+    double out = 0.0;   // one entry per lane
+#pragma unroll
+    for (int u = 0; u < 5; ++u)
+#pragma unroll
+        for (int v = 0; v < 5; ++v)
+            if (lane == u * 5 + v) out = m[u][v];
+    if (lane < 25) L[lane] = out;
+}
+
+__global__ void __launch_bounds__(256) k_singular2d_fx(SingFx P, double *__restrict__ Lbuf)
+{
+    extern __shared__ __align__(16) u64 sh_sing[];
+    const Sing2Params &Q = P.S;
+    const int ns = Q.ns;
+    const FxTab tab = fx_stage(P.tab, sh_sing);
+    __shared__ double txi[NSMAX], te2[NSMAX];
+    if ((int)threadIdx.x < ns) {
+        const double lg = log(Q.gx[threadIdx.x]);
+        txi[threadIdx.x] = exp(lg / (4.0 - 2.0 * Q.sbar));
+        te2[threadIdx.x] = exp(lg / (2.0 - 2.0 * Q.sbar));
+    }
+    __syncthreads();
+    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    i64 *fa = (i64 *)(sh_sing + FX_WORDS) + (size_t)wib * 2 * Q.cap, *fb = fa + Q.cap;
+    for (int pair = blockIdx.x * nw + wib; pair < Q.npairs; pair += gridDim.x * nw) {
+        const int *pi = Q.pinfo + (size_t)pair * 8;
+        const int type = pi[0], ti = type - 1, nreg = sing_regions(type);
+        int pv[3] = {pi[2], pi[3], pi[4]}, qv[3] = {pi[5], pi[6], pi[7]};
+        double Pv[6], Qv[6];
+        for (int a = 0; a < 3; ++a)
+            for (int j = 0; j < 2; ++j) {
+                Pv[a * 2 + j] = Q.vx[(size_t)j * Q.M + pv[a]];
+                Qv[a * 2 + j] = Q.vx[(size_t)j * Q.M + qv[a]];
+            }
+        const double JP[4] = {Pv[2] - Pv[0], Pv[4] - Pv[2], Pv[3] - Pv[1], Pv[5] - Pv[3]};
+        const double JQ[4] = {Qv[2] - Qv[0], Qv[4] - Qv[2], Qv[3] - Qv[1], Qv[5] - Qv[3]};
+        const double detP = fabs(JP[0] * JP[3] - JP[1] * JP[2]), detQ = fabs(JQ[0] * JQ[3] - JQ[1] * JQ[2]);
+        // phase 1: exponent terms at the distinct mapped points
+        int xo[5], yo[5], off = 0;
+        for (int reg = 0; reg < nreg; ++reg) {
+            xo[reg] = off;
+            off += ipow(ns, __popc(c_xmask[ti][reg]));
+            yo[reg] = off;
+            off += ipow(ns, __popc(c_ymask[ti][reg]));
+        }
+        bool fits = true;
+        __syncwarp();
+        for (int t = lane; t < off; t += 32) {
+            int reg = 0;
+            while (reg + 1 < nreg && t >= xo[reg + 1]) ++reg;
+            const bool second = t >= yo[reg];
+            const unsigned mask = second ? c_ymask[ti][reg] : c_xmask[ti][reg];
+            int ind[4];
+            tdecode(mask, ns, t - (second ? yo[reg] : xo[reg]), ind);
+            const double xi = txi[ind[0]], e1 = Q.gx[ind[1]], e3 = Q.gx[ind[3]];
+            double a[2], b[2], aux[2], jac;
+            if (type == 3) map_id(reg, e1, te2[ind[2]], e3, a, b, aux);
+            else map_ve(type, reg, e1, Q.gx[ind[2]], e3, a, b, jac);
+            double h[2], x[2], bary[3], sv, kv;
+            h[0] = xi * (second ? b[0] : a[0]);
+            h[1] = xi * (second ? b[1] : a[1]);
+            const bool onq = second && type != 3;
+            phys(onq ? Qv : Pv, h, x, bary);
+            fields2(Q.Fs, Q.Fk, 2, x, onq ? qv : pv, bary, sv, kv, Q.mt);
+            i64 A, B;
+            fits &= fx_terms(2, P.w, sv, kv, A, B);
+            fa[t] = A;
+            fb[t] = B;
+        }
+        if (!fits) atomicOr(P.err, 1);
+        __syncwarp();
+        // phase 2
+        const double wgt = (double)pi[1];
+        double *L = Lbuf + (size_t)pair * 25;
+        if (type == 1) sing_sum<10, false>(P, tab, 1, JP, JQ, fa, fb, xo, yo, wgt * detP * detQ, L, lane);
+        else if (type == 2) sing_sum<6, false>(P, tab, 2, JP, JQ, fa, fb, xo, yo, wgt * detP * detQ, L, lane);
+        else sing_sum<3, true>(P, tab, 3, JP, JQ, fa, fb, xo, yo, wgt * detP * detP, L, lane);
+    }
+}
+
 }  // namespace
 
-void launch_singular_B(const MeshData &m, OpData &op, DBuf<double> &Lbuf, cudaStream_t st)
+void launch_singular_B(const MeshData &m, OpData &op, DBuf<double> &Lbuf, bool fixed, cudaStream_t st)
 {
     const int ns = m.opts.n_sing;
     // largest field table: the edge case, 4 ns^4 + 4 ns^3 + 2 ns^2 points
@@ -281,6 +514,31 @@ void launch_singular_B(const MeshData &m, OpData &op, DBuf<double> &Lbuf, cudaSt
     P.mt = m.mtab.p;
     P.Fs = op.fs;
     P.Fk = op.fk;
+    // fixed point where nu and cst fit (see k_sing_table): they grow with the number of
+    // Gauss points and as s_bar nears 1
+    const double lg = std::fabs(std::log(m.gl_min)), c = 4.0 - 2.0 * op.s_bar, c2 = 2.0 - 2.0 * op.s_bar;
+    const double q = lg * (1.0 / c + 1.0 / c2);
+    wpb = 8;
+    while (wpb > 1 && FX_BYTES + per_warp * wpb > 110 * 1024) wpb /= 2;
+    if (fixed && c2 > 0.0 && 2.0 * (q + lg) < 60.0 && 1.45 * (std::fabs(2.0 * op.s_bar + 2.0) * q + 4.0 * lg) < 200.0 &&
+        FX_BYTES + per_warp * wpb <= 220 * 1024) {
+        const int ne = 10 * ns * ns * ns * ns;
+        op.sing_tab.alloc((size_t)ST_SLOTS * ne);
+        k_sing_table<<<cdiv(ne, 128), 128, 0, st>>>(ns, op.s_bar, P.gx, P.gw, op.sing_tab.p);
+        SingFx F;
+        F.S = P;
+        F.w = m.fx_w;
+        F.st = op.sing_tab.p;
+        F.tab = m.fx_tab.p;
+        F.err = op.errflag.p;
+        const size_t shm = FX_BYTES + per_warp * wpb;
+        VFD_CUDA(cudaFuncSetAttribute(k_singular2d_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+        k_singular2d_fx<<<std::min(cdiv(m.npairs, wpb), 152 * 16), 32 * wpb, shm, st>>>(F, Lbuf.p);
+        VFD_CUDA(cudaGetLastError());
+        return;
+    }
+    wpb = 8;
+    while (wpb > 1 && per_warp * wpb > 200 * 1024) wpb /= 2;
     size_t shm = per_warp * wpb;
     VFD_CUDA(cudaFuncSetAttribute(k_singular2d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
     k_singular2d<<<cdiv(m.npairs, wpb), 32 * wpb, shm, st>>>(P, Lbuf.p);

@@ -80,9 +80,9 @@ struct DField {
     double c0, lo, hi;
     const double *rows; // device, (nF + nG + nT) * 5
     const double *vals; // device, n_vert (nodal)
-    // 2D Fourier rows with integer |k| <= 4 and k_3 = 0, grouped by k_1 (0 groups
-    // otherwise): gint = per group (|k_1|, rows), then per row |k_2|; gcoef = per
-    // row four coefficients with the signs of k_1, k_2 folded in
+    // 2D Fourier rows with integer |k| <= 4 and k_3 = 0, summed per class (|k_1|, |k_2|) and
+    // grouped by |k_1| (0 groups otherwise): gint = per group (|k_1|, classes), then per class
+    // |k_2|; gcoef = per class four coefficients with the signs of k_1, k_2 folded in
     int ngrp;
     const int *gint;
     const double *gcoef;
@@ -209,6 +209,7 @@ struct MeshData {
     int64_t rnear_pairs = 0;
     DBuf<int> rnear_ptr, rnear_col;     // by target leaf
     DBuf<double> gl_x, gl_w;            // Gauss-Legendre on [0,1], n_sing points
+    double gl_min = 0.5;                // the smallest of them
     DBuf<double> gl9_x, gl9_w;          // 9-point rule for the tail
     DBuf<double> mtab;                  // tables of the table-driven FP64 log/exp
     // fixed-point kernel evaluations (gamma_fixed.cuh): scale 2^fx_w, coordinates of the
@@ -258,6 +259,7 @@ struct OpData {
     // exponent terms of the fixed-point kernel evaluations, (a, b) per point; q_ab ends with a
     // third array, a + log2 of the rule weight.  fx: every point fits the formats
     bool fx = false;
+    DBuf<double> sing_tab;             // singular rules: what of a 4D point is the same for all pairs
     DBuf<long long> q_ab, kc_ab, kc_ab_in, tc_ab, sc_ab;
     DBuf<double> valB, valM, valBM;    // CSR values
     DBuf<double> rho;                  // interior points, canonical order
@@ -398,7 +400,8 @@ void cheb_nodes_1d(int p, double lo, double hi, double *out);
 void launch_field_points(const MeshData &m, OpData &op, cudaStream_t st);
 // nearest-point location of every tree's Chebyshev nodes (mesh_setup.cpp)
 void locate_nodes(MeshData &m);
-void launch_singular_B(const MeshData &m, OpData &op, DBuf<double> &Lbuf, cudaStream_t st);
+// fixed: with the fixed-point kernel evaluations; errflag[0] is set where a point does not fit them
+void launch_singular_B(const MeshData &m, OpData &op, DBuf<double> &Lbuf, bool fixed, cudaStream_t st);
 void launch_gather_B(const MeshData &m, OpData &op, const DBuf<double> &Lbuf, cudaStream_t st);
 void launch_density(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_gather_M(const MeshData &m, OpData &op, cudaStream_t st);

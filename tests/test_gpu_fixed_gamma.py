@@ -18,9 +18,10 @@ SHIFT = 120.0
 
 # the FP64 path rounds an exponent of up to SHIFT + 60 at every operation (2^-53
 # of it, a few times: below 1e-13); the fixed path's error is below 1e-14.  Near
-# blocks and the density are sums of positive terms; the far field's bases change
-# sign, which costs another factor of 10
-TOL = {"rho": 1e-13, vfd.VFD_PART_M: 1e-13, vfd.VFD_PART_KNEAR: 1e-13, vfd.VFD_PART_KFAR: 1e-12}
+# blocks and the density are sums of positive terms; the far field's bases and the
+# singular rules' basis differences change sign, which costs another factor of 10
+TOL = {"rho": 1e-13, vfd.VFD_PART_M: 1e-13, vfd.VFD_PART_KNEAR: 1e-13, vfd.VFD_PART_KFAR: 1e-12,
+       vfd.VFD_PART_B: 1e-12}
 
 MESHES = {
     "interval": lambda: synth.interval_mesh(150),
@@ -38,11 +39,11 @@ MESHES = {
     ("interval", 16, 3), ("interval", 64, 8), ("interval_wide", 5, 2), ("disk", 64, 4), ("disk", 7, 8), ("disk", 3, 1),
     ("disk_unsplit", 64, 4), ("disk_unsplit", 33, 5), ("disk_leaf", 130, 3), ("square", 20, 7), ("graded", 16, 4),
     ("ball", 64, 4), ("ball", 10, 3)])
-@pytest.mark.parametrize("s_range", [(0.0, 0.1), (0.2, 0.89)])
-def test_fixed_point_assembly_matches_fp64(name, leaf, p, s_range):
+@pytest.mark.parametrize("s_range,n_sing", [((0.0, 0.1), 2), ((0.2, 0.89), 3)])
+def test_fixed_point_assembly_matches_fp64(name, leaf, p, s_range, n_sing):
     import torch
     m = MESHES[name]()
-    mesh = vfd.vfd_mesh(m.d, m.coords, m.cells, m.cell_is_interior, leaf_m=leaf, cheb_p=p, rho_leaf_m=leaf)
+    mesh = vfd.vfd_mesh(m.d, m.coords, m.cells, m.cell_is_interior, leaf_m=leaf, cheb_p=p, rho_leaf_m=leaf, n_sing=n_sing)
     lo, hi = s_range
     s = synth.sigmoid_field(synth.random_fourier_field(11, 1.0, d=m.d), lo, hi)
     rows = synth.random_fourier_field(12, 0.7, d=m.d).fourier
@@ -51,12 +52,12 @@ def test_fixed_point_assembly_matches_fp64(name, leaf, p, s_range):
     def parts(shift):
         op = vfd.vfd_assemble(mesh, s, SimpleNamespace(c0=shift, fourier=rows), 0.9)
         out = {"rho": vfd.vfd_op_rho(op, torch.empty(mesh.info["n_qint"], dtype=torch.float64, device="cuda"))}
-        for part in (vfd.VFD_PART_M, vfd.VFD_PART_KNEAR, vfd.VFD_PART_KFAR):
+        for part in (vfd.VFD_PART_M, vfd.VFD_PART_KNEAR, vfd.VFD_PART_KFAR, vfd.VFD_PART_B):
             out[part] = vfd.vfd_apply_parts(op, part, x, torch.empty_like(x))
         return {k: v.cpu().numpy() for k, v in out.items()}
 
     fixed, fp64 = parts(0.0), parts(SHIFT)
     for key, tol in TOL.items():
         a, b = fixed[key], fp64[key] * math.exp(-SHIFT)
-        scale = np.abs(b).max() if key == vfd.VFD_PART_KFAR else np.abs(b)
+        scale = np.abs(b).max() if key in (vfd.VFD_PART_KFAR, vfd.VFD_PART_B) else np.abs(b)
         assert np.all(np.abs(a - b) <= tol * scale), (key, float(np.max(np.abs(a - b) / (scale + 1e-300))))
