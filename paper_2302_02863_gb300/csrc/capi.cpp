@@ -311,6 +311,7 @@ vfd_status vfd_assemble(vfd_mesh_t mesh, const vfd_field *s, const vfd_field *lo
         herr[0] = 0;
         if (op->fx) VFD_CUDA(cudaMemcpyAsync(herr, op->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, st));
         VFD_CUDA(cudaStreamSynchronize(st));
+        op->sing_fx = op->sing_tab.n > 0 && herr[0] == 0;
         if (herr[0]) {   // a mapped point's fields do not fit the fixed-point formats
             launch_singular_B(m, *op, Lbuf, false, st);
             launch_gather_B(m, *op, Lbuf, st);

@@ -144,6 +144,15 @@ __device__ __forceinline__ bool fx_terms(int d, int w, double s, double lk, i64 
     return true;
 }
 
+// the same for the sums of s and of log kappa over two points that fit (2D)
+__device__ __forceinline__ void fx_sums(int w, double s, double lk, i64 &A, u64 &B)
+{
+    const u64 b = (u64)__double2ll_rn(s * 2305843009213693952.0) + (1ULL << 62);   // Q62, below 2^64
+    B = __umul64hi(b, 0xB8AA3B295C17F0BCULL);
+    const i64 l = __mul64hi(__double2ll_rn(lk * 36028797018963968.0), 0x5C551D94AE0BF85ELL);   // Q55 x Q63
+    A = ((l + 1) >> 1) - (((i64)(b >> 6) * (2 * w)) >> 3);
+}
+
 template <int D>
 __device__ __forceinline__ double fx_gamma(const FxTab &t, const i64 *x, const i64 *y, i64 A, u64 B)
 {

@@ -42,6 +42,8 @@
 #include <cmath>
 
 #include "device_common.cuh"
+#include "gamma_fixed.cuh"
+#include "sing_maps.cuh"
 
 namespace vfd {
 
@@ -99,19 +101,19 @@ struct GKN {
 
 // c_a(q) for the columns of this pass: w_q sum over the cell's vertices whose
 // DoF lies in [r0, r1) of the barycentric coordinate times x
-template <int NV>
+template <int NV, int NR = GNR>
 __device__ __forceinline__ void leaf_coef(const GKN &P, int q, int r0, int r1, double *cl, double *cu)
 {
     const int cell = P.qcell[q];
     const double w = P.qw[q];
 #pragma unroll
-    for (int r = 0; r < GNR; ++r) cl[r] = cu[r] = 0.0;
+    for (int r = 0; r < NR; ++r) cl[r] = cu[r] = 0.0;
     for (int k = 0; k < NV; ++k) {
         const int i = P.vdof[P.cells[(size_t)cell * NV + k]];
         if (i >= r0 && i < r1) {
             const double c = w * P.qbary[(size_t)q * QB + k];
 #pragma unroll
-            for (int r = 0; r < GNR; ++r)
+            for (int r = 0; r < NR; ++r)
                 if (r < P.nr) {
                     cl[r] = fma(c, P.Lam[(size_t)r * P.ld + i], cl[r]);
                     cu[r] = fma(c, P.U[(size_t)r * P.ld + i], cu[r]);
@@ -774,6 +776,459 @@ __global__ void __launch_bounds__(256) k_grad_sing(GradSing P, double *__restric
         }
 }
 
+// ---------------------------------------------------------------------------
+// The same sums on the fixed-point kernel evaluations (gamma_fixed.cuh), which
+// give gamma and N = -ln(r^2 / W^2): the logarithm of the sensitivities is
+// ln r^2 = 2 w ln 2 - N, and the constant is taken out of the sums.  Every kernel
+// spreads a target's sources over the warps of a CTA (targets in the lanes) and
+// adds the warps' results in order, so that meshes of a few thousand DoFs fill
+// the chip.  Per evaluation about 60 cycles of an SM and warp in the integer
+// pipes and 3 to 6 FP64 instructions of 16.  At 4k DoFs (disk, rank 36): K near
+// 35.7 -> 3.9 ms (231M evaluations), density near 5.0 -> 0.7, density far 2.9 -> 0.33,
+// target moments 2.4 -> 0.18, singular rules 6.4 -> 1.85; vfd_grad 52.9 -> 7.5 ms.
+// ---------------------------------------------------------------------------
+constexpr int GF_W = 8, GF_S = 128;   // warps of a CTA, sources per staged tile
+constexpr double FX_N1 = 1.3877787807814457e-17;   // 2^-56
+
+__device__ __forceinline__ double fx_n(u64 N) { return (double)(i64)N * FX_N1; }
+
+template <int D>
+__device__ __forceinline__ double fx_gamma_n(const FxTab &t, const i64 *x, const i64 *y, i64 A, u64 B, double &n)
+{
+    u64 M;
+    int K;
+    fx_r2<D>(x, y, M, K);
+    const u64 N = fx_neglog(t, M, K);
+    n = fx_n(N);
+    return fx_exp(t, A, B, N);
+}
+
+// sums of (a, b) over the CTA's warps, in warp order; the first warp's lanes get them
+__device__ __forceinline__ void gf_reduce(double &a, double &b, double (*ra)[32], double (*rb)[32])
+{
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    __syncthreads();
+    ra[w][l] = a;
+    rb[w][l] = b;
+    __syncthreads();
+    if (w == 0) {
+        a = b = 0.0;
+#pragma unroll
+        for (int q = 0; q < GF_W; ++q) {
+            a += ra[q][l];
+            b += rb[q][l];
+        }
+    }
+}
+
+struct GFx {   // element points
+    const i64 *X, *a, *b, *aw;
+    const u64 *tab;
+    double lnW2;   // 2 w ln 2
+};
+
+// NR >= P.nr columns a pass: a predicated-off FP64 instruction takes its issue slot all
+// the same, so the widths 1, 2 and 8 have their own code (8 for one column: 11.1 ms)
+template <int D, int NR>
+__global__ void __launch_bounds__(32 * GF_W) k_gh_knear_fx(GKN P, GFx F)
+{
+    constexpr int NV = D + 1;
+    extern __shared__ __align__(16) u64 sh_tab[];
+    __shared__ i64 sx[GF_S * D], sa[GF_S], sb[GF_S];
+    __shared__ double sl[NR][GF_S], su[NR][GF_S], ra[GF_W][32], rb[GF_W][32];
+    __shared__ int sv[GF_S * NV];
+    const int a = blockIdx.x, pa0 = P.lp_ptr[a], npa = P.lp_ptr[a + 1] - pa0;
+    if ((int)blockIdx.y * 32 >= npa) return;   // the whole CTA
+    const FxTab tab = fx_stage(F.tab, sh_tab);
+    const int warp = threadIdx.x >> 5, t = blockIdx.y * 32 + (threadIdx.x & 31);
+    const int q = P.lp_pts[pa0 + min(t, npa - 1)];
+    i64 x[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) x[c] = F.X[(size_t)c * P.nQ + q];
+    const i64 aq = F.a[q], bq = F.b[q];
+    int v[NV];
+    for (int k = 0; k < NV; ++k) v[k] = P.cells[(size_t)P.qcell[q] * NV + k];
+    double cl[NR], cu[NR];
+    leaf_coef<NV, NR>(P, q, P.kt_begin[P.fl + a], P.kt_end[P.fl + a], cl, cu);
+    double accn = 0.0, acc1 = 0.0;
+    for (int e = P.near_ptr[a]; e < P.near_ptr[a + 1]; ++e) {
+        const int b = P.near_col[e], pb0 = P.lp_ptr[b], npb = P.lp_ptr[b + 1] - pb0;
+        const int rb0 = P.kt_begin[P.fl + b], rb1 = P.kt_end[P.fl + b];
+        for (int j0 = 0; j0 < npb; j0 += GF_S) {
+            const int nt = min(GF_S, npb - j0);
+            __syncthreads();
+            if ((int)threadIdx.x < nt) {
+                const int id = P.lp_pts[pb0 + j0 + threadIdx.x];
+#pragma unroll
+                for (int c = 0; c < D; ++c) sx[threadIdx.x * D + c] = F.X[(size_t)c * P.nQ + id];
+                sa[threadIdx.x] = F.a[id];
+                sb[threadIdx.x] = F.b[id];
+                for (int k = 0; k < NV; ++k) sv[threadIdx.x * NV + k] = P.cells[(size_t)P.qcell[id] * NV + k];
+                double ml[NR], mu[NR];
+                leaf_coef<NV, NR>(P, id, rb0, rb1, ml, mu);
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    sl[r][threadIdx.x] = ml[r];
+                    su[r][threadIdx.x] = mu[r];
+                }
+            }
+            __syncthreads();
+#pragma unroll 2
+            for (int jj = warp; jj < nt; jj += GF_W) {
+                double n;
+                const double g = fx_gamma_n<D>(tab, x, sx + jj * D, aq + sa[jj], (u64)(bq + sb[jj]), n);
+                bool touch = false;   // touching cells belong to B
+#pragma unroll
+                for (int i = 0; i < NV; ++i)
+#pragma unroll
+                    for (int k = 0; k < NV; ++k) touch |= v[i] == sv[jj * NV + k];
+                double X = 0.0;
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    X = fma(cl[r], su[r][jj], fma(cu[r], sl[r][jj], X));
+                const double tX = touch ? 0.0 : g * X;
+                acc1 += tX;
+                accn = fma(tX, touch ? 0.0 : n, accn);
+            }
+        }
+    }
+    gf_reduce(acc1, accn, ra, rb);
+    if (warp == 0 && t < npa) {
+        // -d/ds(q) of -2 gamma X = -ln(r^2) gamma X; -d/dlogk(q) = gamma X
+        const size_t o = (size_t)pa0 + t;
+        const double accs = fma(F.lnW2, acc1, -accn);
+        P.hs[o] = P.accumulate ? P.hs[o] - accs : -accs;
+        P.hk[o] = P.accumulate ? P.hk[o] + acc1 : acc1;
+    }
+}
+
+// density near part, SRC false: target side (k_gh_rho_near_t), true: source side
+// (k_gh_rho_near_s); the roles of the two trees are swapped
+template <int D, bool SRC>
+__global__ void __launch_bounds__(32 * GF_W) k_gh_rho_near_fx(GRho P, GFx F)
+{
+    constexpr int NV = D + 1;
+    extern __shared__ __align__(16) u64 sh_tab[];
+    __shared__ i64 sx[GF_S * D], sa[GF_S], sb[GF_S];
+    __shared__ double sc[GF_S], ra[GF_W][32], rb[GF_W][32];
+    __shared__ int sv[GF_S * NV];
+    const FxTab tab = fx_stage(F.tab, sh_tab);
+    const int leaf = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int node = (SRC ? P.sfl : P.tfl) + leaf;
+    const int *tb = SRC ? P.st_begin : P.tt_begin, *te = SRC ? P.st_end : P.tt_end, *tp = SRC ? P.st_perm : P.tt_perm;
+    const int *ob = SRC ? P.tt_begin : P.st_begin, *oe = SRC ? P.tt_end : P.st_end, *op = SRC ? P.tt_perm : P.st_perm;
+    const int *lp = SRC ? P.rnearT_ptr : P.rnear_ptr, *lc = SRC ? P.rnearT_col : P.rnear_col;
+    const int b = tb[node], e = te[node];
+    for (int i0 = b; i0 < e; i0 += 32) {
+        const int id = tp[min(i0 + lane, e - 1)];
+        i64 x[D];
+#pragma unroll
+        for (int c = 0; c < D; ++c) x[c] = F.X[(size_t)c * P.nQ + id];
+        const i64 a_ = F.a[id], b_ = F.b[id];
+        int cv[NV];
+        for (int k = 0; k < NV; ++k) cv[k] = P.cells[(size_t)P.qcell[id] * NV + k];
+        double accn = 0.0, acc1 = 0.0;
+        for (int ne = lp[leaf]; ne < lp[leaf + 1]; ++ne) {
+            const int on = SRC ? P.tfl + lc[ne] : lc[ne], o0 = ob[on], o1 = oe[on];
+            for (int j0 = o0; j0 < o1; j0 += GF_S) {
+                const int nj = min(GF_S, o1 - j0);
+                __syncthreads();
+                if ((int)threadIdx.x < nj) {
+                    const int jd = op[j0 + threadIdx.x];
+#pragma unroll
+                    for (int c = 0; c < D; ++c) sx[threadIdx.x * D + c] = F.X[(size_t)c * P.nQ + jd];
+                    sa[threadIdx.x] = SRC ? F.a[jd] : F.aw[jd];   // the source weight in the exponent
+                    sb[threadIdx.x] = F.b[jd];
+                    if (SRC) sc[threadIdx.x] = P.cq[jd];
+                    for (int k = 0; k < NV; ++k) sv[threadIdx.x * NV + k] = P.cells[(size_t)P.qcell[jd] * NV + k];
+                }
+                __syncthreads();
+#pragma unroll 2
+                for (int jj = warp; jj < nj; jj += GF_W) {
+                    double n;
+                    double g = fx_gamma_n<D>(tab, x, sx + jj * D, a_ + sa[jj], (u64)(b_ + sb[jj]), n);
+                    bool touch = false;
+#pragma unroll
+                    for (int i = 0; i < NV; ++i)
+#pragma unroll
+                        for (int k = 0; k < NV; ++k) touch |= cv[i] == sv[jj * NV + k];
+                    if (SRC) g *= sc[jj];
+                    if (touch) g = n = 0.0;
+                    acc1 += g;
+                    accn = fma(g, n, accn);
+                }
+            }
+        }
+        gf_reduce(acc1, accn, ra, rb);
+        if (warp == 0 && i0 + lane < e) {
+            const double accs = fma(F.lnW2, acc1, -accn), c = SRC ? P.qw[id] : P.cq[id];
+            if (SRC) {
+                P.hs[id] += 0.5 * c * accs;
+                P.hk[id] -= 0.5 * c * acc1;
+            } else {
+                P.hs[id] = 0.5 * c * accs;
+                P.hk[id] = -0.5 * c * acc1;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// density far part: node i = (n, alpha) of one tree over the nodes of its list in
+// the other, whose points carry the weights ow; the result times iw[i] / 2
+template <int D>
+__global__ void __launch_bounds__(128)
+k_gh_rho_far_fx(int k, int nnode, int nother, const int *__restrict__ ptr, const int *__restrict__ col,
+                const i64 *__restrict__ X, const i64 *__restrict__ ab, const i64 *__restrict__ oX,
+                const i64 *__restrict__ oab, const double *__restrict__ iw, const double *__restrict__ ow, GFx F,
+                double *__restrict__ Gs, double *__restrict__ Gk)
+{
+    extern __shared__ __align__(16) u64 sh_tab[];
+    const FxTab tab = fx_stage(F.tab, sh_tab);
+    __syncthreads();
+    // four lanes share a node's point: every fourth point of the other nodes
+    const size_t nn = (size_t)nnode * k, no = (size_t)nother * k, th = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    const size_t i = th >> 2;
+    const int part = (int)(th & 3);
+    double accn = 0.0, acc1 = 0.0;
+    if (i < nn) {
+        const int n = (int)(i / k), e0 = ptr[n], e1 = ptr[n + 1];
+        i64 x[D];
+#pragma unroll
+        for (int c = 0; c < D; ++c) x[c] = X[i * D + c];
+        const i64 a = ab[i], b = ab[nn + i];
+        for (int e = e0; e < e1; ++e)
+#pragma unroll 2
+            for (int be = part; be < k; be += 4) {
+                const size_t j = (size_t)col[e] * k + be;
+                double ln;
+                const double g = fx_gamma_n<D>(tab, x, oX + j * D, a + oab[j], (u64)(b + oab[no + j]), ln) * ow[j];
+                acc1 += g;
+                accn = fma(g, ln, accn);
+            }
+    }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        acc1 += __shfl_xor_sync(0xffffffffu, acc1, o);
+        accn += __shfl_xor_sync(0xffffffffu, accn, o);
+    }
+    if (i < nn && part == 0) {
+        Gs[i] = 0.5 * iw[i] * fma(F.lnW2, acc1, -accn);
+        Gk[i] = -0.5 * iw[i] * acc1;
+    }
+}
+
+// target moments chat[t][alpha] as k_gh_rho_moments, with Lagrange values by prefix
+// and suffix products from the reference points of the box, and the points spread
+// over the CTA's thread groups of k
+struct GMom {
+    int p, k, nQ;
+    const int *fptr, *tb, *te, *perm;
+    const double *lo, *hi, *qx, *cq;
+    double tref[PMAX], wref[PMAX];
+    double *chat;
+};
+
+template <int D>
+__global__ void __launch_bounds__(256) k_gh_rho_moments2(GMom P)
+{
+    __shared__ double l1[D][PMAX][MCH + 1], red[256];
+    const int t = blockIdx.x, k = P.k, p = P.p;
+    if (P.fptr[t + 1] == P.fptr[t]) return;
+    const int b = P.tb[t], e = P.te[t], grp = threadIdx.x / k, ng = 256 / k, al = threadIdx.x - grp * k;
+    const int a0 = al % p, a1 = D > 1 ? al / p : 0;
+    double acc = 0.0;
+    for (int i0 = b; i0 < e; i0 += MCH) {
+        const int n = min(MCH, e - i0);
+        __syncthreads();
+        for (int u = threadIdx.x; u < n * D; u += blockDim.x) {
+            const int c = u / n, pt = u - c * n, id = P.perm[i0 + pt];
+            const double lo = P.lo[(size_t)t * D + c], hi = P.hi[(size_t)t * D + c];
+            const double x = (P.qx[(size_t)c * P.nQ + id] - 0.5 * (lo + hi)) / (0.5 * (hi - lo));
+            double pre = c == 0 ? P.cq[id] : 1.0, suf = 1.0;   // c_q goes with the first axis
+            for (int a = 0; a < p; ++a) {
+                l1[c][a][pt] = pre;
+                pre *= x - P.tref[a];
+            }
+            for (int a = p - 1; a >= 0; --a) {
+                l1[c][a][pt] *= suf * P.wref[a];
+                suf *= x - P.tref[a];
+            }
+        }
+        __syncthreads();
+        if (grp < ng)
+            for (int pt = grp; pt < n; pt += ng)
+                acc = D > 1 ? fma(l1[0][a0][pt], l1[D - 1][a1][pt], acc) : acc + l1[0][a0][pt];
+    }
+    __syncthreads();
+    red[threadIdx.x] = acc;
+    __syncthreads();
+    if ((int)threadIdx.x < k) {
+        double v = 0.0;
+        for (int g = 0; g < ng; ++g) v += red[g * k + threadIdx.x];
+        P.chat[(size_t)t * k + threadIdx.x] = v;
+    }
+}
+
+// touching pairs in 2D.  Tabulated per 4D point (k_gs_table): the coefficients of
+// the scaled difference, nu and cst of the exponent (singular.cu), the rule weight,
+// the basis differences f_1.. (f_0 is minus their sum) and the mapped reference
+// points xh, yh.  With P1 fields s(x) + s(y) and log kappa are linear in xh, yh, and
+// the barycentric sums of the sensitivities come from the sums of c, c xh, c yh.
+constexpr int GT_D = 0, GT_NU = 4, GT_CST = 5, GT_W = 6, GT_F = 7, GT_XY = 11, GT_SLOTS = 15;
+
+__global__ void k_gs_table(int ns, double sbar, const double *__restrict__ gx, const double *__restrict__ gw,
+                           double *__restrict__ out)
+{
+    const int per = ns * ns * ns * ns, t = blockIdx.x * blockDim.x + threadIdx.x, ne = 10 * per;
+    if (t >= ne) return;
+    const int type = t < 2 * per ? 1 : (t < 7 * per ? 2 : 3);
+    const int i = t - sing_first(type) * per, reg = i / per, r = i - reg * per;
+    const int iz = r % ns, i1 = (r / ns) % ns, i2 = (r / (ns * ns)) % ns, i3 = r / (ns * ns * ns);
+    double a[2], b[2], d[4];
+    const SingPoint p = sing_point(type, reg, sbar, gx[iz], gx[i1], gx[i2], gx[i3], a, b, d);
+    const double v[GT_SLOTS] = {d[0], d[1], d[2], d[3], fx_bits(p.nu, 56), fx_bits(p.cst, 53),
+                                p.w * gw[iz] * gw[i1] * gw[i2] * gw[i3], p.f[1], p.f[2], p.f[3], p.f[4],
+                                p.xi * a[0], p.xi * a[1], p.xi * b[0], p.xi * b[1]};
+    for (int q = 0; q < GT_SLOTS; ++q) out[(size_t)q * ne + t] = v[q];
+}
+
+template <int NF>
+__device__ __forceinline__ void gs_sum(const GradSing &P, const GFx &F, int w, const FxTab &tab, const double *st, int ne,
+                                       int tot, bool ident, const double *JP, const double *JQ, const double *s,
+                                       const double *k, double pre, const int *loc, int lane, double *out)
+{
+    // per column the differences to vertex 0 of U and Lam
+    double du[2][NF], dl[2][NF];
+    auto load = [&](int r, int h) {
+        auto val = [&](const double *v, int q) {
+            const int j = P.vdof[loc[q]];
+            return j >= 0 ? v[(size_t)r * P.ld + j] : 0.0;
+        };
+        const double u0 = val(P.U, 0), l0 = val(P.Lam, 0);
+#pragma unroll
+        for (int q = 0; q < NF; ++q) {
+            du[h][q] = val(P.U, q + 1) - u0;
+            dl[h][q] = val(P.Lam, q + 1) - l0;
+        }
+    };
+    const int nr = P.nrhs;
+    load(0, 0);
+    if (nr > 1) load(1, 1);
+    double S[10];
+#pragma unroll
+    for (int q = 0; q < 10; ++q) S[q] = 0.0;
+    for (int idx = lane; idx < tot; idx += 32) {
+        const double *e = st + idx;
+        auto slot = [&](int q) { return e[(size_t)q * ne]; };
+        double dx = JP[0] * slot(0) + JP[1] * slot(1), dy = JP[2] * slot(0) + JP[3] * slot(1);
+        if (!ident) {
+            dx = dx - JQ[0] * slot(2) - JQ[1] * slot(3);
+            dy = dy - JQ[2] * slot(2) - JQ[3] * slot(3);
+        }
+        u64 M;
+        int K;
+        fx_r2(dx * dx + dy * dy, w, M, K);
+        const u64 N = fx_neglog(tab, M, K) + (u64)__double_as_longlong(slot(GT_NU));
+        const double x0 = slot(GT_XY), x1 = slot(GT_XY + 1), y0 = slot(GT_XY + 2), y1 = slot(GT_XY + 3);
+        const double ss = fma(y1, s[4], fma(y0, s[3], fma(x1, s[2], fma(x0, s[1], s[0]))));
+        const double kk = fma(y1, k[4], fma(y0, k[3], fma(x1, k[2], fma(x0, k[1], k[0]))));
+        i64 A;
+        u64 B;
+        fx_sums(w, ss, kk, A, B);
+        const double g = fx_exp(tab, A + __double_as_longlong(slot(GT_CST)), B, N) * slot(GT_W);
+        double f[NF], ul = 0.0;
+#pragma unroll
+        for (int q = 0; q < NF; ++q) f[q] = slot(GT_F + q);
+        for (int r = 0; r < nr; ++r) {
+            if (nr > 2 && r > 0) load(r, 1);   // one column more than the registers hold
+            double u = 0.0, l = 0.0;
+#pragma unroll
+            for (int q = 0; q < NF; ++q) {
+                u = fma(r ? du[1][q] : du[0][q], f[q], u);
+                l = fma(r ? dl[1][q] : dl[0][q], f[q], l);
+            }
+            ul = fma(u, l, ul);
+        }
+        const double c = g * ul, h = c * fx_n(N);   // d ln(w) / dS = (N + nu - ln W^2) / 2
+        S[0] += c;
+        S[1] = fma(c, x0, S[1]);
+        S[2] = fma(c, x1, S[2]);
+        S[3] = fma(c, y0, S[3]);
+        S[4] = fma(c, y1, S[4]);
+        S[5] += h;
+        S[6] = fma(h, x0, S[6]);
+        S[7] = fma(h, x1, S[7]);
+        S[8] = fma(h, y0, S[8]);
+        S[9] = fma(h, y1, S[9]);
+    }
+#pragma unroll
+    for (int q = 0; q < 10; ++q) S[q] = pre * warp_sum(S[q]);
+    if (lane == 0) {
+        double z[5];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) z[q] = 0.5 * (S[5 + q] - F.lnW2 * S[q]);
+        out[0] = -(z[0] - z[1]);
+        out[1] = -(z[1] - z[2]);
+        out[2] = -z[2];
+        out[3] = -(z[0] - z[3]);
+        out[4] = -(z[3] - z[4]);
+        out[5] = -z[4];
+        out[6] = -0.5 * (S[0] - S[1]);
+        out[7] = -0.5 * (S[1] - S[2]);
+        out[8] = -0.5 * S[2];
+        out[9] = -0.5 * (S[0] - S[3]);
+        out[10] = -0.5 * (S[3] - S[4]);
+        out[11] = -0.5 * S[4];
+    }
+}
+
+__global__ void __launch_bounds__(256)
+k_grad_sing2d_fx(GradSing P, GFx F, int w, const double *__restrict__ st, double *__restrict__ pg)
+{
+    extern __shared__ __align__(16) u64 sh_tab[];
+    const FxTab tab = fx_stage(F.tab, sh_tab);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5, per = P.ns * P.ns * P.ns * P.ns, ne = 10 * per;
+    for (int pair = blockIdx.x * nw + (threadIdx.x >> 5); pair < P.npairs; pair += gridDim.x * nw) {
+        const int *pi = P.pinfo + (size_t)pair * 8;
+        const int type = pi[0], pv[3] = {pi[2], pi[3], pi[4]}, qv[3] = {pi[5], pi[6], pi[7]};
+        double Pv[6], Qv[6];
+        for (int a = 0; a < 3; ++a)
+            for (int j = 0; j < 2; ++j) {
+                Pv[a * 2 + j] = P.vx[(size_t)j * P.M + pv[a]];
+                Qv[a * 2 + j] = P.vx[(size_t)j * P.M + qv[a]];
+            }
+        const double JP[4] = {Pv[2] - Pv[0], Pv[4] - Pv[2], Pv[3] - Pv[1], Pv[5] - Pv[3]};
+        const double JQ[4] = {Qv[2] - Qv[0], Qv[4] - Qv[2], Qv[3] - Qv[1], Qv[5] - Qv[3]};
+        const double detP = fabs(JP[0] * JP[3] - JP[1] * JP[2]), detQ = fabs(JQ[0] * JQ[3] - JQ[1] * JQ[2]);
+        // field sums over both points: value at vertices 0, then the coefficients of x0, x1, y0, y1
+        auto lin = [&](const double *f, double *o) {
+            o[0] = f[pv[0]] + f[qv[0]];
+            o[1] = f[pv[1]] - f[pv[0]];
+            o[2] = f[pv[2]] - f[pv[1]];
+            o[3] = f[qv[1]] - f[qv[0]];
+            o[4] = f[qv[2]] - f[qv[1]];
+        };
+        double s[5], k[5];
+        lin(P.s, s);
+        lin(P.lk, k);
+        const double wgt = (double)pi[1];
+        const double *t = st + (size_t)sing_first(type) * per;
+        const int tot = sing_regions(type) * per;
+        double *out = pg + (size_t)pair * 12;
+        if (type == 1) {
+            const int loc[5] = {pv[0], pv[1], pv[2], qv[1], qv[2]};
+            gs_sum<4>(P, F, w, tab, t, ne, tot, false, JP, JQ, s, k, wgt * detP * detQ, loc, lane, out);
+        } else if (type == 2) {
+            const int loc[4] = {pv[0], pv[1], pv[2], qv[2]};
+            gs_sum<3>(P, F, w, tab, t, ne, tot, false, JP, JQ, s, k, wgt * detP * detQ, loc, lane, out);
+        } else {
+            gs_sum<2>(P, F, w, tab, t, ne, tot, true, JP, JQ, s, k, wgt * detP * detP, pv, lane, out);
+        }
+    }
+}
+
 // per vertex: the point sensitivities (density), the K-near leaf-point
 // sensitivities, the node sensitivities (K, target, source nodes) and the
 // touching pairs' slots, each times the barycentric coordinate of the vertex
@@ -934,6 +1389,15 @@ void grad_adjoint(MeshData &m, OpData &op, const double *U, const double *Lam, i
     VFD_CUDA(cudaGetLastError());
     VFD_CUDA(cudaMemsetAsync(op.gr_Gs.p, 0, sizeof(double) * std::max<int64_t>(nn, 1), st));
     VFD_CUDA(cudaMemsetAsync(op.gr_Gk.p, 0, sizeof(double) * std::max<int64_t>(nn, 1), st));
+    GFx F{};
+    if (op.fx) {
+        F.X = m.fx_qX.p;
+        F.a = op.q_ab.p;
+        F.b = op.q_ab.p + m.nQ;
+        F.aw = op.q_ab.p + 2 * (size_t)m.nQ;
+        F.tab = m.fx_tab.p;
+        F.lnW2 = 2.0 * m.fx_w * 0.6931471805599453;
+    }
     // K: near blocks and admissible blocks, GNR columns per pass
     const int fl = m.kt.first_leaf();
     const size_t hsz = (size_t)m.kt.nnode * k;
@@ -974,7 +1438,13 @@ void grad_adjoint(MeshData &m, OpData &op, const double *U, const double *Lam, i
             P.hs = op.gr_hKs.p;
             P.hk = op.gr_hKk.p;
             dim3 g(m.kt.nleaf, cdiv(m.max_leaf_pts, GT));
-            if (m.d == 2) k_gh_knear<2><<<g, GT, 0, st>>>(P);
+            if (op.fx) {
+                auto f = nr == 1   ? (m.d == 2 ? k_gh_knear_fx<2, 1> : k_gh_knear_fx<1, 1>)
+                         : nr == 2 ? (m.d == 2 ? k_gh_knear_fx<2, 2> : k_gh_knear_fx<1, 2>)
+                                   : (m.d == 2 ? k_gh_knear_fx<2, GNR> : k_gh_knear_fx<1, GNR>);
+                VFD_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_BYTES));
+                f<<<dim3(m.kt.nleaf, cdiv(m.max_leaf_pts, 32)), 32 * GF_W, FX_BYTES, st>>>(P, F);
+            } else if (m.d == 2) k_gh_knear<2><<<g, GT, 0, st>>>(P);
             else k_gh_knear<1><<<g, GT, 0, st>>>(P);
             VFD_CUDA(cudaGetLastError());
         }
@@ -1020,22 +1490,64 @@ void grad_adjoint(MeshData &m, OpData &op, const double *U, const double *Lam, i
         P.hk = op.gr_h1.p;
         VFD_CUDA(cudaMemsetAsync(op.gr_hs.p, 0, sizeof(double) * nq, st));
         VFD_CUDA(cudaMemsetAsync(op.gr_h1.p, 0, sizeof(double) * nq, st));
-        k_gh_rho_near_t<<<m.tt.nleaf, RCH, 0, st>>>(P);
-        k_gh_rho_near_s<<<m.st.nleaf, RCH, 0, st>>>(P);
+        if (op.fx) {
+            auto ft = m.d == 2 ? k_gh_rho_near_fx<2, false> : k_gh_rho_near_fx<1, false>;
+            auto fs = m.d == 2 ? k_gh_rho_near_fx<2, true> : k_gh_rho_near_fx<1, true>;
+            VFD_CUDA(cudaFuncSetAttribute(ft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_BYTES));
+            VFD_CUDA(cudaFuncSetAttribute(fs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_BYTES));
+            ft<<<m.tt.nleaf, 32 * GF_W, FX_BYTES, st>>>(P, F);
+            fs<<<m.st.nleaf, 32 * GF_W, FX_BYTES, st>>>(P, F);
+        } else {
+            k_gh_rho_near_t<<<m.tt.nleaf, RCH, 0, st>>>(P);
+            k_gh_rho_near_s<<<m.st.nleaf, RCH, 0, st>>>(P);
+        }
         VFD_CUDA(cudaGetLastError());
     }
     if (m.nrfar > 0) {
         const size_t nt = (size_t)m.tt.nnode * k;
         if (op.gr_ct.n < nt) op.gr_ct.alloc(nt);
         VFD_CUDA(cudaMemsetAsync(op.gr_ct.p, 0, sizeof(double) * nt, st));
-        k_gh_rho_moments<<<m.tt.nnode, 128, 0, st>>>(m.d, m.p, k, m.nQ, m.rfar_ptr.p, m.tt_begin.p, m.tt_end.p,
-                                                     m.tt_perm.p, m.tt_cheb.p, m.qx.p, op.gr_cq.p, op.gr_ct.p);
-        k_gh_rho_far_t<<<cdiv((long long)m.tt.nnode * k, 128), 128, 0, st>>>(
-            m.d, k, m.tt.nnode, m.rfar_ptr.p, m.rfar_col.p, m.tt_cheb.p, op.tc_s.p, op.tc_lk.p, m.st_cheb.p,
-            op.sc_s.p, op.sc_lk.p, m.st_xhat.p, op.gr_ct.p, m.mtab.p, op.gr_Gs.p + oT, op.gr_Gk.p + oT);
-        k_gh_rho_far_s<<<cdiv((long long)m.st.nnode * k, 128), 128, 0, st>>>(
-            m.d, k, m.st.nnode, m.rfarT_ptr.p, m.rfarT_col.p, m.tt_cheb.p, op.tc_s.p, op.tc_lk.p, m.st_cheb.p,
-            op.sc_s.p, op.sc_lk.p, m.st_xhat.p, op.gr_ct.p, m.mtab.p, op.gr_Gs.p + oS, op.gr_Gk.p + oS);
+        if (op.fx) {
+            GMom G;
+            G.p = m.p;
+            G.k = k;
+            G.nQ = m.nQ;
+            G.fptr = m.rfar_ptr.p;
+            G.tb = m.tt_begin.p;
+            G.te = m.tt_end.p;
+            G.perm = m.tt_perm.p;
+            G.lo = m.tt_lo.p;
+            G.hi = m.tt_hi.p;
+            G.qx = m.qx.p;
+            G.cq = op.gr_cq.p;
+            for (int a = 0; a < m.p; ++a) G.tref[a] = std::cos((2.0 * a + 1.0) * M_PI / (2.0 * m.p));
+            for (int a = 0; a < m.p; ++a) {
+                double w = 1.0;
+                for (int b = 0; b < m.p; ++b)
+                    if (b != a) w *= G.tref[a] - G.tref[b];
+                G.wref[a] = 1.0 / w;
+            }
+            G.chat = op.gr_ct.p;
+            auto fm = m.d == 2 ? k_gh_rho_moments2<2> : k_gh_rho_moments2<1>;
+            auto ff = m.d == 2 ? k_gh_rho_far_fx<2> : k_gh_rho_far_fx<1>;
+            VFD_CUDA(cudaFuncSetAttribute(ff, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_BYTES));
+            fm<<<m.tt.nnode, 256, 0, st>>>(G);
+            ff<<<cdiv((long long)m.tt.nnode * k * 4, 128), 128, FX_BYTES, st>>>(
+                k, m.tt.nnode, m.st.nnode, m.rfar_ptr.p, m.rfar_col.p, m.fx_ttX.p, op.tc_ab.p, m.fx_stX.p, op.sc_ab.p,
+                op.gr_ct.p, m.st_xhat.p, F, op.gr_Gs.p + oT, op.gr_Gk.p + oT);
+            ff<<<cdiv((long long)m.st.nnode * k * 4, 128), 128, FX_BYTES, st>>>(
+                k, m.st.nnode, m.tt.nnode, m.rfarT_ptr.p, m.rfarT_col.p, m.fx_stX.p, op.sc_ab.p, m.fx_ttX.p, op.tc_ab.p,
+                m.st_xhat.p, op.gr_ct.p, F, op.gr_Gs.p + oS, op.gr_Gk.p + oS);
+        } else {
+            k_gh_rho_moments<<<m.tt.nnode, 128, 0, st>>>(m.d, m.p, k, m.nQ, m.rfar_ptr.p, m.tt_begin.p, m.tt_end.p,
+                                                         m.tt_perm.p, m.tt_cheb.p, m.qx.p, op.gr_cq.p, op.gr_ct.p);
+            k_gh_rho_far_t<<<cdiv((long long)m.tt.nnode * k, 128), 128, 0, st>>>(
+                m.d, k, m.tt.nnode, m.rfar_ptr.p, m.rfar_col.p, m.tt_cheb.p, op.tc_s.p, op.tc_lk.p, m.st_cheb.p,
+                op.sc_s.p, op.sc_lk.p, m.st_xhat.p, op.gr_ct.p, m.mtab.p, op.gr_Gs.p + oT, op.gr_Gk.p + oT);
+            k_gh_rho_far_s<<<cdiv((long long)m.st.nnode * k, 128), 128, 0, st>>>(
+                m.d, k, m.st.nnode, m.rfarT_ptr.p, m.rfarT_col.p, m.tt_cheb.p, op.tc_s.p, op.tc_lk.p, m.st_cheb.p,
+                op.sc_s.p, op.sc_lk.p, m.st_xhat.p, op.gr_ct.p, m.mtab.p, op.gr_Gs.p + oS, op.gr_Gk.p + oS);
+        }
         VFD_CUDA(cudaGetLastError());
     }
     if (m.npairs > 0) {
@@ -1056,7 +1568,16 @@ void grad_adjoint(MeshData &m, OpData &op, const double *U, const double *Lam, i
         P.lk = op.fk.vals;
         P.U = U;
         P.Lam = Lam;
-        k_grad_sing<<<cdiv((long long)m.npairs * 32, 256), 256, 0, st>>>(P, op.gr_pg.p);
+        if (op.sing_fx) {
+            const int ne = 10 * P.ns * P.ns * P.ns * P.ns;
+            if (op.gr_st.n < (size_t)GT_SLOTS * ne) op.gr_st.alloc((size_t)GT_SLOTS * ne);
+            k_gs_table<<<cdiv(ne, 128), 128, 0, st>>>(P.ns, P.sbar, P.gx, P.gw, op.gr_st.p);
+            VFD_CUDA(cudaFuncSetAttribute(k_grad_sing2d_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_BYTES));
+            k_grad_sing2d_fx<<<std::min(cdiv(m.npairs, 8), 152 * 8), 256, FX_BYTES, st>>>(P, F, m.fx_w, op.gr_st.p,
+                                                                                          op.gr_pg.p);
+        } else {
+            k_grad_sing<<<cdiv((long long)m.npairs * 32, 256), 256, 0, st>>>(P, op.gr_pg.p);
+        }
         VFD_CUDA(cudaGetLastError());
     }
     k_gh_gather<<<cdiv(m.M, 256), 256, 0, st>>>(m.M, m.gq_ptr.p, m.gq_idx.p, m.qbary.p, op.gr_hs.p, op.gr_h1.p,

@@ -256,7 +256,8 @@ namespace {
 
 std::vector<unsigned long long> make_fixed_tables()
 {
-    // layout and formats in gamma_fixed.cuh, computed in extended precision
+    // layout and formats in gamma_fixed.cuh, computed in extended precision (in software
+    // on some hosts)
     std::vector<unsigned long long> t(FX_WORDS);
     for (int j = 0; j < FX_LOGN; ++j) {
         const long double one = 2147483648.0L;   // 2^31
@@ -317,11 +318,14 @@ void setup_fixed(MeshData &m, const std::vector<double> &qx, const std::vector<d
     for (size_t i = 0; i < qw.size(); ++i) {
         const double l = std::log2(qw[i]);
         if (!(std::fabs(l) < 100.0)) return;
-        lw[i] = (long long)std::llround(std::ldexp(std::log2((long double)qw[i]), 53));
+        // the points of a cell share their weight in 2D and 3D
+        lw[i] = i && qw[i] == qw[i - 1] ? lw[i - 1]
+                                        : (long long)std::llround(std::ldexp(std::log2((long double)qw[i]), 53));
     }
     m.fx_w = w;
     m.fx_lw.upload(lw);
-    m.fx_tab.upload(make_fixed_tables());
+    static const std::vector<unsigned long long> tab = make_fixed_tables();
+    m.fx_tab.upload(tab);
     fixed_coords(qx, d, true, o, w, m.fx_qX);
     fixed_coords(m.kt_cheb_h, d, false, o, w, m.fx_ktX);
     fixed_coords(m.kt_cheb_in_h, d, false, o, w, m.fx_ktX_in);

@@ -13,6 +13,7 @@
 
 #include "device_common.cuh"
 #include "gamma_fixed.cuh"
+#include "sing_maps.cuh"
 
 namespace vfd {
 
@@ -56,42 +57,6 @@ __device__ __forceinline__ void tdecode(unsigned mask, int ns, int t, int *ind)
             ind[j] = t % ns;
             t /= ns;
         }
-    }
-}
-
-// region maps divided by xi: xhat = xi a, yhat = xi b (vertex: T_V^(1,2)
-// eq. e:map-v; edge: T_E^(1..5) Sec. 4.2), with the eta-Jacobian factor
-__device__ __forceinline__ void map_ve(int type, int reg, double e1, double e2, double e3, double *a, double *b,
-                                       double &jac)
-{
-    if (type == 1) {
-        if (reg == 0) { a[0] = 1.0; a[1] = e1; b[0] = e2; b[1] = e2 * e3; }
-        else { a[0] = e2; a[1] = e2 * e3; b[0] = 1.0; b[1] = e1; }
-        jac = e2;
-        return;
-    }
-    switch (reg) {
-    case 0: a[0] = 1.0; a[1] = e1 * e3; b[0] = 1.0 - e1 * e2; b[1] = e1 * (1.0 - e2); jac = e1 * e1; break;
-    case 1: a[0] = 1.0; a[1] = e1; b[0] = 1.0 - e1 * e2 * e3; b[1] = e1 * e2 * (1.0 - e3); jac = e1 * e1 * e2; break;
-    case 2: a[0] = 1.0 - e1 * e2; a[1] = e1 * (1.0 - e2); b[0] = 1.0; b[1] = e1 * e2 * e3; jac = e1 * e1 * e2; break;
-    case 3: a[0] = 1.0 - e1 * e2 * e3; a[1] = e1 * e2 * (1.0 - e3); b[0] = 1.0; b[1] = e1; jac = e1 * e1 * e2; break;
-    default: a[0] = 1.0 - e1 * e2 * e3; a[1] = e1 * (1.0 - e2 * e3); b[0] = 1.0; b[1] = e1 * e2; jac = e1 * e1 * e2; break;
-    }
-}
-
-// identical maps T_I^(1..3) (Sec. 4.3; region 2 with the factor eta1 on
-// xhat_2, region 3 scaled difference (-eta3, 1-eta3)); dr = (xhat - yhat)/(xi eta1 eta2)
-__device__ __forceinline__ void map_id(int reg, double e1, double e2, double e3, double *a, double *b, double *dr)
-{
-    if (reg == 0) {
-        a[0] = 1.0; a[1] = 1.0 - e1 + e1 * e2; b[0] = 1.0 - e1 * e2 * e3; b[1] = 1.0 - e1;
-        dr[0] = e3; dr[1] = 1.0;
-    } else if (reg == 1) {
-        a[0] = 1.0; a[1] = e1 * (1.0 - e2 + e2 * e3); b[0] = 1.0 - e1 * e2; b[1] = e1 * (1.0 - e2);
-        dr[0] = 1.0; dr[1] = e3;
-    } else {
-        a[0] = 1.0 - e1 * e2 * e3; a[1] = e1 * (1.0 - e2 * e3); b[0] = 1.0; b[1] = e1 * (1.0 - e2);
-        dr[0] = -e3; dr[1] = 1.0 - e3;
     }
 }
 
@@ -276,10 +241,6 @@ __global__ void __launch_bounds__(256) k_singular2d(Sing2Params P, double *__res
 // ---------------------------------------------------------------------------
 constexpr int ST_A = 0, ST_NU = 4, ST_CST = 5, ST_F = 6, ST_SLOTS = 16;
 
-__device__ __forceinline__ int sing_regions(int type) { return type == 1 ? 2 : (type == 2 ? 5 : 3); }
-// first table entry of a type, in units of ns^4
-__device__ __forceinline__ int sing_first(int type) { return type == 1 ? 0 : (type == 2 ? 2 : 7); }
-
 __global__ void k_sing_table(int ns, double sbar, const double *__restrict__ gx, const double *__restrict__ gw,
                              double *__restrict__ out)
 {
@@ -288,43 +249,16 @@ __global__ void k_sing_table(int ns, double sbar, const double *__restrict__ gx,
     const int type = t < 2 * per ? 1 : (t < 7 * per ? 2 : 3);
     const int i = t - sing_first(type) * per, reg = i / per, r = i - reg * per;
     const int iz = r % ns, i1 = (r / ns) % ns, i2 = (r / (ns * ns)) % ns, i3 = r / (ns * ns * ns);
-    const double c = 4.0 - 2.0 * sbar, c2 = 2.0 - 2.0 * sbar;
-    const double e1 = gx[i1], e3 = gx[i3], wq = gw[iz] * gw[i1] * gw[i2] * gw[i3], lz = log(gx[iz]);
-    double a[2], b[2], f[5] = {0, 0, 0, 0, 0}, w, q, l = 0.0;
-    if (type == 3) {
-        double dr[2];
-        const double lt = log(gx[i2]);
-        map_id(reg, e1, exp(lt / c2), e3, a, b, dr);
-        a[0] = dr[0];
-        a[1] = dr[1];
-        b[0] = b[1] = 0.0;
-        w = wq * 2.0 / (c * c2);   // the mirror regions T_I^(4..6) double the sum
-        q = lz / c + lt / c2;
-        l = log(e1);
-        f[1] = dr[0] - dr[1];
-        f[2] = dr[1];
-    } else {
-        double jac;
-        map_ve(type, reg, e1, gx[i2], e3, a, b, jac);
-        w = wq * jac / c;
-        q = lz / c;
-        if (type == 1) {
-            f[1] = a[0] - a[1]; f[2] = a[1]; f[3] = -(b[0] - b[1]); f[4] = -b[1];
-        } else {
-            f[1] = (a[0] - a[1]) - (b[0] - b[1]); f[2] = a[1]; f[3] = -b[1];
-        }
-    }
-    out[(size_t)(ST_A + 0) * ne + t] = a[0];
-    out[(size_t)(ST_A + 1) * ne + t] = a[1];
-    out[(size_t)(ST_A + 2) * ne + t] = b[0];
-    out[(size_t)(ST_A + 3) * ne + t] = b[1];
-    const double nu = -2.0 * (q + l), cst = ((2.0 * sbar + 2.0) * q + 4.0 * l) * 1.4426950408889634;
-    out[(size_t)ST_NU * ne + t] = __longlong_as_double(__double2ll_rn(nu * 72057594037927936.0));        // Q56
-    out[(size_t)ST_CST * ne + t] = __longlong_as_double(__double2ll_rn(cst * 9007199254740992.0));       // Q53
+    double a[2], b[2], d[4];
+    const SingPoint p = sing_point(type, reg, sbar, gx[iz], gx[i1], gx[i2], gx[i3], a, b, d);
+    const double w = p.w * gw[iz] * gw[i1] * gw[i2] * gw[i3];
+    for (int q = 0; q < 4; ++q) out[(size_t)(ST_A + q) * ne + t] = d[q];
+    out[(size_t)ST_NU * ne + t] = fx_bits(p.nu, 56);
+    out[(size_t)ST_CST * ne + t] = fx_bits(p.cst, 53);
     const int nf = type == 1 ? 4 : (type == 2 ? 3 : 2);
     int s = ST_F;
     for (int u = 1; u <= nf; ++u)
-        for (int v = u; v <= nf; ++v, ++s) out[(size_t)s * ne + t] = w * f[u] * f[v];
+        for (int v = u; v <= nf; ++v, ++s) out[(size_t)s * ne + t] = w * p.f[u] * p.f[v];
 }
 
 struct SingFx {
@@ -514,14 +448,9 @@ void launch_singular_B(const MeshData &m, OpData &op, DBuf<double> &Lbuf, bool f
     P.mt = m.mtab.p;
     P.Fs = op.fs;
     P.Fk = op.fk;
-    // fixed point where nu and cst fit (see k_sing_table): they grow with the number of
-    // Gauss points and as s_bar nears 1
-    const double lg = std::fabs(std::log(m.gl_min)), c = 4.0 - 2.0 * op.s_bar, c2 = 2.0 - 2.0 * op.s_bar;
-    const double q = lg * (1.0 / c + 1.0 / c2);
     wpb = 8;
     while (wpb > 1 && FX_BYTES + per_warp * wpb > 110 * 1024) wpb /= 2;
-    if (fixed && c2 > 0.0 && 2.0 * (q + lg) < 60.0 && 1.45 * (std::fabs(2.0 * op.s_bar + 2.0) * q + 4.0 * lg) < 200.0 &&
-        FX_BYTES + per_warp * wpb <= 220 * 1024) {
+    if (fixed && sing_fixed_fits(m, op.s_bar) && FX_BYTES + per_warp * wpb <= 220 * 1024) {
         const int ne = 10 * ns * ns * ns * ns;
         op.sing_tab.alloc((size_t)ST_SLOTS * ne);
         k_sing_table<<<cdiv(ne, 128), 128, 0, st>>>(ns, op.s_bar, P.gx, P.gw, op.sing_tab.p);

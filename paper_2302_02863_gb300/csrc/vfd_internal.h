@@ -258,7 +258,7 @@ struct OpData {
     DBuf<double> tc_s, tc_lk, sc_s, sc_lk;  // density trees' Chebyshev nodes
     // exponent terms of the fixed-point kernel evaluations, (a, b) per point; q_ab ends with a
     // third array, a + log2 of the rule weight.  fx: every point fits the formats
-    bool fx = false;
+    bool fx = false, sing_fx = false;   // sing_fx: so do those of the singular rules (2D)
     DBuf<double> sing_tab;             // singular rules: what of a 4D point is the same for all pairs
     DBuf<long long> q_ab, kc_ab, kc_ab_in, tc_ab, sc_ab;
     DBuf<double> valB, valM, valBM;    // CSR values
@@ -287,6 +287,7 @@ struct OpData {
     struct BatchData *self = nullptr;
     // adjoint gradient workspaces
     DBuf<double> gr_uq, gr_lq, gr_hs, gr_h1, gr_pg;   // point values, point sensitivities, pair slots
+    DBuf<double> gr_st;                                // singular rules' table
     DBuf<double> gr_cq, gr_hKs, gr_hKk;                // c_q; K-near leaf-point sensitivities
     DBuf<double> gr_Gs, gr_Gk, gr_xU, gr_xL, gr_ct;    // node sensitivities; K far moments; target moments
     // apply workspace

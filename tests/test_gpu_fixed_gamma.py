@@ -61,3 +61,29 @@ def test_fixed_point_assembly_matches_fp64(name, leaf, p, s_range, n_sing):
         a, b = fixed[key], fp64[key] * math.exp(-SHIFT)
         scale = np.abs(b).max() if key in (vfd.VFD_PART_KFAR, vfd.VFD_PART_B) else np.abs(b)
         assert np.all(np.abs(a - b) <= tol * scale), (key, float(np.max(np.abs(a - b) / (scale + 1e-300))))
+
+
+@pytest.mark.parametrize("name,leaf,p,n_sing", [("interval", 16, 4, 3), ("disk", 16, 4, 3), ("disk", 9, 7, 2),
+                                                ("square", 64, 6, 3), ("disk_unsplit", 64, 5, 3)])
+@pytest.mark.parametrize("nrhs", [1, 2, 3, 10])
+def test_fixed_point_gradient_matches_fp64(name, leaf, p, n_sing, nrhs):
+    """vfd_grad at fixed U and Lam scales by e^c with A; the sums change sign, so the
+    1e-13 of their terms is left to grow by the cancellation of random U and Lam."""
+    import torch
+    m = MESHES[name]()
+    mesh = vfd.vfd_mesh(m.d, m.coords, m.cells, m.cell_is_interior, leaf_m=leaf, cheb_p=p, rho_leaf_m=leaf, n_sing=n_sing)
+    x = m.coords
+    s = 0.45 + 0.3 * np.sin(2.0 * x[:, 0]) * np.cos(1.3 * x[:, -1])
+    lk = 0.3 * np.cos(1.5 * x[:, -1])
+    g = torch.Generator("cuda").manual_seed(3)
+    U, Lam = (torch.randn(nrhs, mesh.n_dof, dtype=torch.float64, device="cuda", generator=g) for _ in range(2))
+
+    def grads(shift):
+        op = vfd.vfd_assemble(mesh, synth.nodal_field(s), synth.nodal_field(lk + shift), 0.9)
+        out = [torch.empty(m.n_vert, dtype=torch.float64, device="cuda") for _ in range(2)]
+        vfd.vfd_grad(op, U, Lam, *out)
+        return [o.cpu().numpy() for o in out]
+
+    for a, b in zip(grads(0.0), grads(SHIFT)):
+        b = b * math.exp(-SHIFT)
+        assert np.abs(a - b).max() <= 1e-11 * np.abs(b).max()
