@@ -512,8 +512,9 @@ void release_streams(OpData &op)
 
 // parts: VFD_PART_* mask; lowp: use the FP32 copies of K (VFD_FP32 and VFD_BF16 operators)
 void apply_parts_ex(const MeshData &m, OpData &op, int parts, const double *X, double *Y, int nrhs, int64_t ld,
-                    bool lowp, cudaStream_t st, const int *skip)
+                    bool lowp, cudaStream_t st, const int *skip, ApplyDot *dot)
 {
+    if (dot) dot->n = 0;
     ensure_streams(op);
     const int nlev = m.nfar > 0 ? m.kt.L - m.far_lmin + 1 : 0;
     const size_t need = (size_t)m.kt.nnode * m.k * nrhs;
@@ -538,7 +539,7 @@ void apply_parts_ex(const MeshData &m, OpData &op, int parts, const double *X, d
             op.ye64.alloc(needy);
         }
         if (parts == VFD_PART_ALL && op.fa && m.nnear > 0) {
-            apply_fixed(m, op, X, Y, nrhs, ld, st, skip);
+            apply_fixed(m, op, X, Y, nrhs, ld, st, skip, dot);
             return;
         }
         const bool rc = op.rc_on;   // the recompressed far field of the FP64 operator

@@ -11,6 +11,6 @@ void launch_far_sum(const MeshData &m, OpData &op, int c0, int cols, cudaStream_
 void launch_far_couple_sum(const MeshData &m, OpData &op, int c0, int cols, cudaStream_t st, const int *skip);
 // apply_fixed.cu: Y = A X with the FP64 operator (OpData::fa)
 void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st,
-                 const int *skip);
+                 const int *skip, ApplyDot *dot);
 
 }  // namespace vfd

@@ -707,15 +707,30 @@ __device__ __forceinline__ bool fa_piece(unsigned char *sm, int W, unsigned mk, 
     return slow;
 }
 
-// 16 rows a CTA, 4 a warp, 8 lanes a row
+// partial of X . Y over the rows of this CTA (CG's p . A p comes with the apply): v the
+// product of a row in the lanes with l8 = 0, zero in the others
+__device__ __forceinline__ void fa_dot(double v, double *dot)
+{
+    __shared__ double sh[4];
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) dot[blockIdx.x * gridDim.y + blockIdx.y] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
+}
+
+// 16 rows a CTA, 4 a warp, 8 lanes a row; dot: see fa_dot, or null
 __global__ void __launch_bounds__(128)
-k_fa_near1(FaNear P, const double *__restrict__ X, double *__restrict__ Y, const int *skip)
+k_fa_near1(FaNear P, const double *__restrict__ X, double *__restrict__ Y, double *__restrict__ dot, const int *skip)
 {
     extern __shared__ __align__(16) unsigned char fa_sm[];
     __shared__ unsigned key;
     if (skip && *skip) return;
     const int lf = blockIdx.x, b_leaf = P.kb[P.fl + lf], b = b_leaf + blockIdx.y * 16, e = min(P.ke[P.fl + lf], b + 16);
-    if (b >= e) return;
+    if (b >= e) {
+        if (dot && threadIdx.x == 0) dot[blockIdx.x * gridDim.y + blockIdx.y] = 0.0;
+        return;
+    }
     const int W = P.pw[lf], lane = threadIdx.x & 31, l8 = lane & 7, i = b + 4 * (threadIdx.x >> 5) + (lane >> 3);
     const size_t ro = P.poff[lf] + (size_t)(min(i, e - 1) - b_leaf) * W;
     const int4 *row = (const int4 *)(P.D + ro) + l8;
@@ -747,27 +762,34 @@ k_fa_near1(FaNear P, const double *__restrict__ X, double *__restrict__ Y, const
                 [&] { s.carry(); });
     s.fold();
     fa_sum8<1>(&s, l8);
-    if (i >= e || l8) return;
-    double v = s.value() * fa_pow2(P.re[i] - 30) * fa_scale(ky);
-    if (slow) {
-        v = 0.0;
-        for (int j = 0; j < W; ++j) v = fma(P.Dd[ro + j], raw[j], v);
+    double xy = 0.0;
+    if (i < e && !l8) {
+        double v = s.value() * fa_pow2(P.re[i] - 30) * fa_scale(ky);
+        if (slow) {
+            v = 0.0;
+            for (int j = 0; j < W; ++j) v = fma(P.Dd[ro + j], raw[j], v);
+        }
+        if (slow || !P.folded)
+            for (int q = P.rowptr[i]; q < P.rowptr[i + 1]; ++q) v = fma(P.val[q], X[P.colidx[q]], v);
+        Y[i] = v;
+        if (dot) xy = X[i] * v;
     }
-    if (slow || !P.folded)
-        for (int q = P.rowptr[i]; q < P.rowptr[i + 1]; ++q) v = fma(P.val[q], X[P.colidx[q]], v);
-    Y[i] = v;
+    if (dot) fa_dot(xy, dot);
 }
 
 __global__ void __launch_bounds__(128)
 k_fa_expand1(FaFar P, const double *__restrict__ ye, const double *__restrict__ yhat, double *__restrict__ Y,
-             const int *skip)
+             const double *__restrict__ X, double *__restrict__ dot, const int *skip)
 {
     extern __shared__ __align__(16) unsigned char fa_sm[];
     __shared__ unsigned key;
     if (skip && *skip) return;
     const int lf = blockIdx.x, k = P.k, w = P.nlev * k, b0 = P.kb[P.fl + lf];
     const int b = b0 + blockIdx.y * 16, e = min(P.ke[P.fl + lf], b + 16);
-    if (b >= e) return;
+    if (b >= e) {
+        if (dot && threadIdx.x == 0) dot[blockIdx.x * gridDim.y + blockIdx.y] = 0.0;
+        return;
+    }
     const int lane = threadIdx.x & 31, l8 = lane & 7, i = b + 4 * (threadIdx.x >> 5) + (lane >> 3);
     const int nv = P.wp >> 1, n = (nv + 7) >> 3;
     const int4 *row = (const int4 *)P.U + (size_t)min(i, e - 1) * nv + l8;
@@ -806,14 +828,20 @@ k_fa_expand1(FaFar P, const double *__restrict__ ye, const double *__restrict__ 
                 [&] { s.carry(); });
     s.fold();
     fa_sum8<1>(&s, l8);
-    if (i >= e || l8) return;
-    double v = s.value() * fa_pow2(P.ue[lf] - 30) * fa_scale(ky);
-    if (slow) {
-        v = 0.0;
-        for (int j = 0; j < w; ++j) v = fma(P.Ud[((size_t)(j / k) * P.N + i) * k + j % k], raw[j], v);
+    double xy = 0.0;
+    if (i < e && !l8) {
+        double v = s.value() * fa_pow2(P.ue[lf] - 30) * fa_scale(ky);
+        if (slow) {
+            v = 0.0;
+            for (int j = 0; j < w; ++j) v = fma(P.Ud[((size_t)(j / k) * P.N + i) * k + j % k], raw[j], v);
+        }
+        v += Y[i];
+        Y[i] = v;
+        if (dot) xy = X[i] * v;
     }
-    Y[i] += v;
+    if (dot) fa_dot(xy, dot);
 }
+
 
 // ---------------------------------------------------------------------------
 // the operands
@@ -951,7 +979,7 @@ namespace {
 // one launch of every kernel for ng groups of NC columns from column c0
 template <int NC>
 void apply_group(const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int nrhs, int64_t ld,
-                 bool summed, cudaStream_t st, const int *skip)
+                 bool summed, cudaStream_t st, const int *skip, ApplyDot *dot)
 {
     const int k = m.k, nleaf = m.kt.nleaf, nnode = m.kt.nnode;
     const bool far = m.nfar > 0;
@@ -1023,7 +1051,7 @@ void apply_group(const MeshData &m, OpData &op, const double *X, double *Y, int 
     if (NC == 1) {
         if (shm > 47 * 1024)
             VFD_CUDA(cudaFuncSetAttribute(k_fa_near1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-        k_fa_near1<<<dim3(nleaf, cdiv(m.max_leaf_size, 16)), 128, shm, st>>>(R, X1, Y1, skip);
+        k_fa_near1<<<dim3(nleaf, cdiv(m.max_leaf_size, 16)), 128, shm, st>>>(R, X1, Y1, dot && !far ? dot->part : nullptr, skip);
     } else {
         if (shm > 47 * 1024)
             VFD_CUDA(cudaFuncSetAttribute(k_fa_near<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
@@ -1035,7 +1063,7 @@ void apply_group(const MeshData &m, OpData &op, const double *X, double *Y, int 
         const size_t she = (size_t)P.wp * NC * 8;
         if (NC == 1) {
             k_fa_expand1<<<dim3(nleaf, cdiv(m.max_leaf_size, 16)), 128, she, st>>>(
-                P, op.ye64.p + c0 * ys, summed ? op.yhat.p + c0 * hs : nullptr, Y1, skip);
+                P, op.ye64.p + c0 * ys, summed ? op.yhat.p + c0 * hs : nullptr, Y1, X1, dot ? dot->part : nullptr, skip);
         } else {
             if (she > 47 * 1024)
                 VFD_CUDA(cudaFuncSetAttribute(k_fa_expand<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)she));
@@ -1050,8 +1078,10 @@ void apply_group(const MeshData &m, OpData &op, const double *X, double *Y, int 
 
 // Y = A X with the FP64 operator (all parts); the workspaces are those of the FP64 apply
 void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st,
-                 const int *skip)
+                 const int *skip, ApplyDot *dot)
 {
+    if (dot) dot->n = nrhs == 1 ? m.kt.nleaf * cdiv(m.max_leaf_size, 16) : 0;
+    if (dot && !dot->n) dot = nullptr;
     // the node sums inside the gathers pay for few columns and short spans
     const bool summed = nrhs >= 4 || m.kt.L - m.far_lmin > 7;
     // widest group whose panel piece leaves room for two CTAs an SM
@@ -1059,10 +1089,10 @@ void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int 
     while (nc > 1 && (size_t)m.max_panel_w * nc * 8 > 100 * 1024) nc >>= 1;
     int c0 = 0;
     auto go = [&](int NC, int ng) {
-        if (NC == 8) apply_group<8>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip);
-        else if (NC == 4) apply_group<4>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip);
-        else if (NC == 2) apply_group<2>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip);
-        else apply_group<1>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip);
+        if (NC == 8) apply_group<8>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip, dot);
+        else if (NC == 4) apply_group<4>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip, dot);
+        else if (NC == 2) apply_group<2>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip, dot);
+        else apply_group<1>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip, dot);
         c0 += NC * ng;
     };
     if (nrhs / nc) go(nc, nrhs / nc);

@@ -721,9 +721,6 @@ __global__ void __launch_bounds__(BT) k_bp_zr(Seg S, const int *__restrict__ row
 
 }  // namespace
 
-void apply_parts_ex(const MeshData &m, OpData &op, int parts, const double *X, double *Y, int nrhs, int64_t ld,
-                    bool lowp, cudaStream_t st, const int *skip);
-
 // reduction blocks: per mesh a share of one block per SM proportional to its
 // rows (at least one); vectors, partials, scalars and flags for Rp columns
 static void ensure_solve(BatchData &b, int Rp)

@@ -1,8 +1,8 @@
 // Conjugate gradients on the device (the paper solves with CG, Sec. 7), with
-// deterministic reductions (block partials summed in a fixed order by the
-// last block to finish; no float atomics, no spin-wait) and a device-side
-// convergence flag that turns the remaining kernels of a captured chunk of
-// iterations into no-ops.  The host replays one captured CUDA graph per
+// deterministic reductions (a kernel writes one partial per block, every block
+// of the next kernel sums them in the same order; no float atomics, no
+// spin-wait) and a device-side convergence flag that turns the remaining
+// kernels of a captured chunk of iterations into no-ops.  The host replays one captured CUDA graph per
 // chunk and reads the flag once per chunk.
 //
 // For VFD_FP32 and VFD_BF16 operators the single-column solve is iterative
@@ -15,14 +15,11 @@
 
 namespace vfd {
 
-void apply_parts_ex(const MeshData &m, OpData &op, int parts, const double *X, double *Y, int nrhs, int64_t ld,
-                    bool lowp, cudaStream_t st, const int *skip);
-
 namespace {
 
 constexpr int RB = 256;        // reduction block size
 constexpr int CHUNK = 8;       // CG iterations per captured graph
-enum { S_RR = 0, S_PQ = 1, S_BB = 2, S_TOL2 = 3, S_BETA = 4, S_TMP = 5 };   // 6, 7: PCG (r.z)
+enum { S_RR = 0, S_PQ = 1, S_BB = 2, S_TOL2 = 3, S_OLD = 4, S_TMP = 5, S_RZ = 6, S_RZOLD = 7 };   // r.z: PCG
 enum { F_DONE = 0, F_ITERS = 1, F_MAXIT = 2, F_CNT = 4 };  // F_CNT..F_CNT+3: block counters
 
 int red_blocks(int n) { return std::max(1, std::min(cdiv(n, RB * 4), 264)); }
@@ -97,38 +94,94 @@ __global__ void k_init_flag(int *flag, double *scal, double rtol, int max_it)
     if (max_it <= 0) flag[F_DONE] = 1;
 }
 
-// alpha = rr / pq; x += alpha p; r -= alpha q; rr_new = r.r; convergence test
-__global__ void __launch_bounds__(RB) k_cg_xr(int n, double *__restrict__ x, double *__restrict__ r,
-                                              const double *__restrict__ p, const double *__restrict__ q,
-                                              double *part, unsigned *cnt, double *scal, int *flag)
+// sum of n partials, the same in every block (all threads get it)
+__device__ double sum_partials(const double *__restrict__ part, int n, double *sh)
+{
+    double v = 0.0;
+    for (int i = threadIdx.x; i < n; i += RB) v += part[i];
+    v = block_sum(v, sh);
+    if (threadIdx.x == 0) sh[0] = v;
+    __syncthreads();
+    v = sh[0];
+    __syncthreads();
+    return v;
+}
+
+// partials of a . b (where the apply does not bring them)
+__global__ void __launch_bounds__(RB) k_dot_part(int n, const double *__restrict__ a, const double *__restrict__ b,
+                                                 double *__restrict__ part, const int *flag)
 {
     __shared__ double sh[32];
     if (flag[F_DONE]) return;
-    const double rr = scal[S_RR], pq = scal[S_PQ];
+    double v = 0.0;
+    for (int i = blockIdx.x * RB + threadIdx.x; i < n; i += gridDim.x * RB) v += a[i] * b[i];
+    v = block_sum(v, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = v;
+}
+
+// One iteration after q = A p is two launches: k_cg_xr needs p.q whole, k_cg_p needs
+// r.r whole.  Both are latency (16k to 27k entries): one entry a thread, the sums of
+// the partials in every block instead of a last block's.  With the dot product out of
+// the apply this took 22 us of an iteration in three launches (16,129 DoFs: 7.4 +
+// 11.7 + 3.1), now 12.5 us in two; the solve of 16,129 DoFs 24.9 -> 22.9 ms.
+//
+// alpha = rr / pq; x += alpha p; r -= alpha q; partials of r.r
+__global__ void __launch_bounds__(RB) k_cg_xr(int n, int npq, const double *__restrict__ pq_part, double *__restrict__ x,
+                                              double *__restrict__ r, const double *__restrict__ p,
+                                              const double *__restrict__ q, double *__restrict__ rr_part, double *scal,
+                                              const int *flag)
+{
+    __shared__ double sh[32];
+    if (flag[F_DONE]) return;
+    const double rr = scal[S_RR], pq = sum_partials(pq_part, npq, sh);
     const double alpha = (pq != 0.0) ? rr / pq : 0.0;
     double v = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (int i = blockIdx.x * RB + threadIdx.x; i < n; i += gridDim.x * RB) {
         x[i] += alpha * p[i];
-        double ri = r[i] - alpha * q[i];
+        const double ri = r[i] - alpha * q[i];
         r[i] = ri;
         v += ri * ri;
     }
-    double rrn;
-    if (last_block_sum(v, part, cnt, &rrn, sh) && threadIdx.x == 0) {
-        int it = flag[F_ITERS] + 1;
-        flag[F_ITERS] = it;
-        scal[S_BETA] = (rr != 0.0) ? rrn / rr : 0.0;
-        scal[S_RR] = rrn;
-        if (rrn <= scal[S_TOL2] || it >= flag[F_MAXIT] || !(pq > 0.0)) flag[F_DONE] = 1;
+    v = block_sum(v, sh);
+    if (threadIdx.x == 0) {
+        rr_part[blockIdx.x] = v;
+        if (blockIdx.x == 0) {   // for k_cg_p, which overwrites S_RR
+            scal[S_OLD] = rr;
+            scal[S_PQ] = pq;
+        }
     }
 }
 
-__global__ void k_cg_p(int n, const double *__restrict__ r, double *__restrict__ p, const double *scal,
-                       const int *flag)
+// the end of an iteration, in one thread: count it, test the recursive residual
+__device__ __forceinline__ void end_iteration(double rrn, double *scal, int *flag)
 {
-    if (flag[F_DONE]) return;
-    const double beta = scal[S_BETA];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = r[i] + beta * p[i];
+    const int it = flag[F_ITERS] + 1;
+    flag[F_ITERS] = it;
+    scal[S_RR] = rrn;
+    if (rrn <= scal[S_TOL2] || it >= flag[F_MAXIT] || !(scal[S_PQ] > 0.0)) flag[F_DONE] = 1;
+}
+
+// whether the solve is done, the same for the whole block: k_cg_p and k_pcg_p set the
+// flag while other blocks start (a block that finds it set leaves its part of p, which
+// nothing reads any more)
+__device__ __forceinline__ bool block_done(const int *flag)
+{
+    __shared__ int done;
+    if (threadIdx.x == 0) done = *(volatile const int *)(flag + F_DONE);
+    __syncthreads();
+    return done != 0;
+}
+
+// beta = rr_new / rr; p = r + beta p; convergence test
+__global__ void __launch_bounds__(RB) k_cg_p(int n, int nrr, const double *__restrict__ rr_part,
+                                             const double *__restrict__ r, double *__restrict__ p, double *scal, int *flag)
+{
+    __shared__ double sh[32];
+    if (block_done(flag)) return;
+    const double rr = scal[S_OLD], rrn = sum_partials(rr_part, nrr, sh);
+    const double beta = (rr != 0.0) ? rrn / rr : 0.0;
+    for (int i = blockIdx.x * RB + threadIdx.x; i < n; i += gridDim.x * RB) p[i] = r[i] + beta * p[i];
+    if (blockIdx.x == 0 && threadIdx.x == 0) end_iteration(rrn, scal, flag);
 }
 
 __global__ void k_axpy(int n, double a, const double *__restrict__ x, double *__restrict__ y)
@@ -156,6 +209,19 @@ void release_graphs(OpData &op)
         op.pcg_exec = nullptr;
         op.pcg_key = nullptr;
     }
+}
+
+// q = A p with the partials of p . q in cg_pq; returns their number
+static int apply_with_dot(const MeshData &m, OpData &op, bool lowp, cudaStream_t st)
+{
+    const int n = m.N, NB = red_blocks(n), *flag = op.cg_flag.p;
+    ApplyDot dot;
+    dot.part = op.cg_pq.p;
+    apply_parts_ex(m, op, VFD_PART_ALL, op.cg_p.p, op.cg_q.p, 1, n, lowp, st, flag, &dot);
+    if (dot.n) return dot.n;
+    k_dot_part<<<NB, RB, 0, st>>>(n, op.cg_p.p, op.cg_q.p, op.cg_pq.p, flag);
+    VFD_CUDA(cudaGetLastError());
+    return NB;
 }
 
 // CG on (lowp ? A32 : A64) z = b, b and z in op.cg_b / op.cg_x (device, n).
@@ -186,10 +252,10 @@ static int run_cg(const MeshData &m, OpData &op, bool lowp, double rtol, int max
         VFD_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
         try {
             for (int it = 0; it < CHUNK; ++it) {
-                apply_parts_ex(m, op, VFD_PART_ALL, op.cg_p.p, op.cg_q.p, 1, n, lowp, cs, flag);
-                k_dot<<<NB, RB, 0, cs>>>(n, op.cg_p.p, op.cg_q.p, part, cnt, scal, S_PQ, flag);
-                k_cg_xr<<<NB, RB, 0, cs>>>(n, op.cg_x.p, op.cg_r.p, op.cg_p.p, op.cg_q.p, part, cnt, scal, flag);
-                k_cg_p<<<VB, RB, 0, cs>>>(n, op.cg_r.p, op.cg_p.p, scal, flag);
+                const int npq = apply_with_dot(m, op, lowp, cs);
+                k_cg_xr<<<VB, RB, 0, cs>>>(n, npq, op.cg_pq.p, op.cg_x.p, op.cg_r.p, op.cg_p.p, op.cg_q.p, part, scal,
+                                           flag);
+                k_cg_p<<<VB, RB, 0, cs>>>(n, VB, part, op.cg_r.p, op.cg_p.p, scal, flag);
             }
         } catch (...) {
             cudaStreamEndCapture(cs, &graph);
@@ -227,7 +293,8 @@ static void ensure_ws(const MeshData &m, OpData &op)
         op.cg_x.alloc(n);
         op.cg_b.alloc(n);
         op.cg_z.alloc(n);
-        op.cg_red.alloc(1024);
+        op.cg_red.alloc(std::max(2048, m.kt.nleaf));
+        op.cg_pq.alloc(std::max(dot_partials(m), 264));
         op.cg_scal.alloc(8);
         op.cg_flag.alloc(8);
         VFD_CUDA(cudaMemset(op.cg_flag.p, 0, 8 * sizeof(int)));
@@ -247,56 +314,40 @@ static double dev_dot(const MeshData &m, OpData &op, const double *a, const doub
 
 // ---------------------------------------------------------------------------
 // preconditioned CG (two-level preconditioner of precond.cu):
-//   z = M^-1 r = (block inverse of the leaf's diagonal block) r + R^T A_c^-1 R r
-// with R the leaf-indicator restriction.  Scalars: S_RZ = r.z, S_RZN = the new
-// r.z, S_RR = r.r (the stopping test is on the true recursive residual r).
+//   z = M^-1 r = (block inverse of the leaf's diagonal block) r + R^T A_c^-1 R r,
+// with R the leaf-indicator restriction.  The stopping test is on the recursive
+// residual r.  One iteration after q = A p: precond_step (x, r, the local solves and
+// the leaf sums of r, a CTA per leaf), the coarse product, and k_pcg_p, which adds
+// the coarse correction where it reads z; r.z comes as partials of the first two.
 // ---------------------------------------------------------------------------
 namespace {
-enum { S_RZ = 6, S_RZN = 7 };
-
-// alpha = rz / pq; x += alpha p; r -= alpha q; rr = r.r; convergence test
-__global__ void __launch_bounds__(RB) k_pcg_xr(int n, double *__restrict__ x, double *__restrict__ r,
-                                               const double *__restrict__ p, const double *__restrict__ q,
-                                               double *part, unsigned *cnt, double *scal, int *flag)
+// beta = rz_new / rz; p = z + R^T zc + beta p; convergence test
+__global__ void __launch_bounds__(RB)
+k_pcg_p(int n, int nrr, const double *__restrict__ rr_part, int nrz, const double *__restrict__ rz_part,
+        const double *__restrict__ z, const double *__restrict__ zc, const int *__restrict__ cidx,
+        double *__restrict__ p, double *scal, int *flag)
 {
     __shared__ double sh[32];
-    if (flag[F_DONE]) return;
-    const double rz = scal[S_RZ], pq = scal[S_PQ];
-    const double alpha = (pq != 0.0) ? rz / pq : 0.0;
-    double v = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        x[i] += alpha * p[i];
-        const double ri = r[i] - alpha * q[i];
-        r[i] = ri;
-        v += ri * ri;
-    }
-    double rrn;
-    if (last_block_sum(v, part, cnt, &rrn, sh) && threadIdx.x == 0) {
-        const int it = flag[F_ITERS] + 1;
-        flag[F_ITERS] = it;
-        scal[S_RR] = rrn;
-        if (rrn <= scal[S_TOL2] || it >= flag[F_MAXIT] || !(pq > 0.0)) flag[F_DONE] = 1;
-    }
-}
-
-// p = z + (rz_new / rz) p; rz = rz_new
-__global__ void k_pcg_p(int n, const double *__restrict__ z, double *__restrict__ p, double *scal, const int *flag)
-{
-    if (flag[F_DONE]) return;
-    const double rzn = scal[S_RZN], rz = scal[S_RZ];
+    if (block_done(flag)) return;
+    const double rz = scal[S_RZOLD], rzn = sum_partials(rz_part, nrz, sh);
     const double beta = rz != 0.0 ? rzn / rz : 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = z[i] + beta * p[i];
-}
-
-__global__ void k_pcg_rz_commit(double *scal, const int *flag)
-{
-    if (flag && flag[F_DONE]) return;
-    scal[S_RZ] = scal[S_RZN];
+    for (int i = blockIdx.x * RB + threadIdx.x; i < n; i += gridDim.x * RB)
+        p[i] = (zc ? z[i] + zc[cidx[i]] : z[i]) + beta * p[i];
+    if (blockIdx.x == 0) {
+        const double rrn = sum_partials(rr_part, nrr, sh);
+        if (threadIdx.x == 0) {
+            scal[S_RZ] = rzn;
+            end_iteration(rrn, scal, flag);
+        }
+    }
 }
 }  // namespace
 
-// z = M^-1 r (precond.cu)
+// precond.cu: z = M^-1 r; and one PCG iteration up to the coarse product
 void precond_apply(const MeshData &m, const OpData &op, const double *r, double *z, cudaStream_t st, const int *skip);
+void precond_step(const MeshData &m, OpData &op, int npq, double *rr_part, double *rz_part, double *scal, int s_rz,
+                  int s_rzold, int s_pq, const int *flag, cudaStream_t st);
+int precond_rz_partials(const MeshData &m, const OpData &op);
 
 static int run_pcg(const MeshData &m, OpData &op, double rtol, int max_it, cudaStream_t st, double *rr_out,
                    double *bb_out)
@@ -326,13 +377,10 @@ static int run_pcg(const MeshData &m, OpData &op, double rtol, int max_it, cudaS
         VFD_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
         try {
             for (int it = 0; it < CHUNK; ++it) {
-                apply_parts_ex(m, op, VFD_PART_ALL, op.cg_p.p, op.cg_q.p, 1, n, false, cs, flag);
-                k_dot<<<NB, RB, 0, cs>>>(n, op.cg_p.p, op.cg_q.p, part, cnt, scal, S_PQ, flag);
-                k_pcg_xr<<<NB, RB, 0, cs>>>(n, op.cg_x.p, op.cg_r.p, op.cg_p.p, op.cg_q.p, part, cnt, scal, flag);
-                precond_apply(m, op, op.cg_r.p, op.cg_z.p, cs, flag);
-                k_dot<<<NB, RB, 0, cs>>>(n, op.cg_r.p, op.cg_z.p, part, cnt, scal, S_RZN, flag);
-                k_pcg_p<<<VB, RB, 0, cs>>>(n, op.cg_z.p, op.cg_p.p, scal, flag);
-                k_pcg_rz_commit<<<1, 1, 0, cs>>>(scal, flag);
+                const int npq = apply_with_dot(m, op, false, cs), nrz = precond_rz_partials(m, op);
+                precond_step(m, op, npq, part, op.prec_rz.p, scal, S_RZ, S_RZOLD, S_PQ, flag, cs);
+                k_pcg_p<<<VB, RB, 0, cs>>>(n, m.kt.nleaf, part, nrz, op.prec_rz.p, op.cg_z.p,
+                                           op.prec_nc ? op.prec_zc.p : nullptr, op.prec_cidx.p, op.cg_p.p, scal, flag);
             }
         } catch (...) {
             cudaStreamEndCapture(cs, &graph);

@@ -311,6 +311,7 @@ struct OpData {
     // solver workspace
     DBuf<double> cg_r, cg_p, cg_q, cg_x, cg_b, cg_z;
     DBuf<double> cg_red;               // reduction partials
+    DBuf<double> cg_pq;                // partials of p . A p
     DBuf<double> cg_scal;              // device scalars (8)
     DBuf<int> cg_flag;
     DBuf<int> errflag;
@@ -329,6 +330,7 @@ struct OpData {
     DBuf<double> prec_coarse;          // nc x nc (inverse of R A R^T)
     DBuf<float> prec_coarse32;         //   FP32 copy
     DBuf<int> prec_cidx;               // coarse cluster of every DoF
+    DBuf<double> prec_rz;              // partials of r . z per leaf and coarse cluster
     DBuf<double> prec_rl, prec_zc;     // leaf sums of the residual (nleaf), coarse correction (nc)
 };
 
@@ -421,8 +423,15 @@ void launch_selftest_math(const MeshData &m, int which, long long n, const doubl
 void build_fixed_bases(MeshData &m);
 void build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t st);
 // apply.cu
+// partial sums of X . Y, written by the apply of one column where it can (n of them; part
+// holds at least dot_partials(m)), else n = 0
+struct ApplyDot {
+    double *part = nullptr;
+    int n = 0;
+};
+inline int dot_partials(const MeshData &m) { return m.kt.nleaf * ((m.max_leaf_size + 15) / 16); }
 void apply_parts_ex(const MeshData &m, OpData &op, int parts, const double *X, double *Y, int nrhs, int64_t ld,
-                    bool lowp, cudaStream_t st, const int *skip);
+                    bool lowp, cudaStream_t st, const int *skip, ApplyDot *dot = nullptr);
 void apply_parts(const MeshData &m, OpData &op, int parts, const double *X, double *Y, int nrhs, int64_t ld,
                  cudaStream_t st);
 void recompress_far(MeshData &m, OpData &op, double tol, cudaStream_t st);
