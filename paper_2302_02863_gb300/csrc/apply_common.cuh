@@ -12,5 +12,9 @@ void launch_far_couple_sum(const MeshData &m, OpData &op, int c0, int cols, cuda
 // apply_fixed.cu: Y = A X with the FP64 operator (OpData::fa)
 void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st,
                  const int *skip, ApplyDot *dot);
+// apply_tensor.cu: the same for many columns
+bool apply_tensor_fits(const MeshData &m, int nrhs);
+void apply_tensor_alloc(const MeshData &m, OpData &op);   // its workspace, on first use
+const int *apply_tensor(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st);
 
 }  // namespace vfd

@@ -41,69 +41,11 @@
 #include <algorithm>
 
 #include "apply_common.cuh"
+#include "apply_fixed.cuh"
 
 namespace vfd {
 
-typedef long long i64;
-typedef unsigned long long u64;
-
 namespace {
-
-constexpr int FA_LO = 30, FA_TOP = 40;
-
-// exponent key of a value: 0 for zero, else its biased exponent (denormals 1)
-__device__ __forceinline__ unsigned fa_key(double v)
-{
-    // the exponent field is masked after the shift: a mask of the sign bit alone becomes
-    // an FP64 absolute value, which leaves the sign of a NaN
-    const unsigned h = (unsigned)__double2hiint(v);
-    return (h << 1 | (unsigned)__double2loint(v)) == 0 ? 0u : max(1u, (h >> 20) & 0x7ffu);
-}
-// keys of a piece that the fixed-point products cannot take
-__device__ __forceinline__ bool fa_slow(unsigned key) { return key == 0x7ffu || (key && key < 128u); }
-
-// v 2^(60 - E) rounded, E = key - 1022 with key the largest of the piece
-__device__ __forceinline__ i64 fa_round(double v, int key)
-{
-    const u64 b = (u64)__double_as_longlong(v);
-    const int e = (int)((b >> 52) & 0x7ff), s = e - key + 7;
-    const u64 m = (b & 0xfffffffffffffULL) | (e ? 1ULL << 52 : 0ULL);
-    const u64 r = s >= 0 ? m << s : (s > -64 ? (m + (1ULL << (-s - 1))) >> -s : 0ULL);
-    return (i64)b < 0 ? -(i64)r : (i64)r;
-}
-__device__ __forceinline__ int2 fa_split(i64 v)
-{
-    const int lo = (int)((unsigned)v << (32 - FA_LO)) >> (32 - FA_LO);
-    return make_int2(lo, (int)((v - lo) >> FA_LO));
-}
-// 2^k as FP64, -1022 <= k <= 1023
-__device__ __forceinline__ double fa_pow2(int k) { return __longlong_as_double((i64)(k + 1023) << 52); }
-// scale of a piece: 2^(E - 30), E = key - 1022 (any for a piece of zeros)
-__device__ __forceinline__ double fa_scale(unsigned key) { return fa_pow2(key ? (int)key - 1022 - 30 : 0); }
-// sums of products: carry() after every fourth mac at most (seven fit)
-struct FaAcc {
-    i64 hh = 0, mid = 0;
-    int th = 0, tm = 0;   // what hh and mid have passed on, weight 2^FA_TOP
-    __device__ __forceinline__ void mac(int2 a, int2 x)
-    {
-        hh += (i64)a.y * x.y;
-        mid += (i64)a.y * x.x;
-        mid += (i64)a.x * x.y;
-    }
-    __device__ __forceinline__ void carry()
-    {
-        th += (int)(hh >> FA_TOP);
-        hh &= (1LL << FA_TOP) - 1;
-        tm += (int)(mid >> FA_TOP);
-        mid &= (1LL << FA_TOP) - 1;
-    }
-    // after carry: hh takes mid, rounded (the sum is th 2^FA_TOP + hh in units of 2^60)
-    __device__ __forceinline__ void fold()
-    {
-        hh += ((mid + (1LL << (FA_LO - 1))) >> FA_LO) + ((i64)tm << (FA_TOP - FA_LO));
-    }
-    __device__ __forceinline__ double value() const { return fma((double)th, 1099511627776.0, (double)hh); }
-};
 
 // products of a column: out_a = sum_b M[b stride + a] x[b], thread per a, x in
 // shared memory [b][NC]
@@ -141,16 +83,6 @@ __device__ __forceinline__ void fa_column(const int2 *__restrict__ M, size_t str
 // ---------------------------------------------------------------------------
 // 1. projections: CTA per (leaf, 128 of the nlev k columns, group of columns)
 // ---------------------------------------------------------------------------
-struct FaFar {
-    int fl, nleaf, lmin, L, nlev, k, nnode, nfar, nrhs, c0;   // c0: first column of this launch
-    int kp, wp;   // row strides of a coupling block and of the bases (even: 16-byte rows)
-    const int *kb, *ke, *fptr, *fcol;
-    const int2 *U, *S;
-    const int *ue, *se;
-    const double *Ud, *Sd;   // FP64: [level][N][k], blocks
-    int N;
-};
-
 template <int NC>
 __global__ void __launch_bounds__(128) k_fa_proj(FaFar P, const double *__restrict__ X, int64_t ld,
                                                  double *__restrict__ part, const int *skip)
@@ -388,17 +320,6 @@ __device__ __forceinline__ int fa_slot(int j, int c, int ws)   // of column c's 
 // ---------------------------------------------------------------------------
 // 3. near rows: CTA per (leaf, slice of NR rows, group of columns)
 // ---------------------------------------------------------------------------
-struct FaNear {
-    int fl, NR, nrhs, c0;
-    const int *kb, *ke, *pw, *gcol, *goff, *rowptr, *colidx;
-    const int64_t *poff;
-    const double *val;   // B + M
-    int folded;          // B + M are in the fixed-point panels
-    const int2 *D;
-    const int *re;
-    const double *Dd;    // FP64 panels
-};
-
 template <int NC>
 __global__ void __launch_bounds__(128) k_fa_near(FaNear P, const double *__restrict__ X, int64_t ld,
                                                  double *__restrict__ Y, const int *skip)
@@ -884,22 +805,34 @@ __global__ void k_fa_build_near(int N, int fl, const int *__restrict__ vleaf, co
     if (lane == 0) re[i] = E;
 }
 
-// coupling blocks, a warp each; rows padded to an even length
-__global__ void k_fa_build_S(int nfar, int k, int kp, const double *__restrict__ S, int2 *__restrict__ out,
-                             int *__restrict__ se, int *err)
+// coupling blocks, a CTA per row node: one exponent for its blocks, so that their sums add
+// up as integers; rows padded to an even length
+__global__ void __launch_bounds__(256)
+k_fa_build_S(const int *__restrict__ fptr, int k, int kp, const double *__restrict__ S, int2 *__restrict__ out,
+             int *__restrict__ se, int *err)
 {
-    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (e >= nfar) return;
-    const double *in = S + (size_t)e * k * k;
-    int2 *o = out + (size_t)e * k * kp;
-    unsigned key = 0;
-    for (int j = lane; j < k * k; j += 32) key = max(key, fa_key(in[j]));
-    const int E = fa_exponent(key, err);
-    for (int j = lane; j < k * kp; j += 32) {
-        const int b = j / kp, a = j - b * kp;
-        o[j] = a < k ? fa_split(fa_round(in[b * k + a], E + 1022)) : make_int2(0, 0);
+    __shared__ unsigned key;
+    __shared__ int E;
+    const int e0 = fptr[blockIdx.x], ne = fptr[blockIdx.x + 1] - e0;
+    if (ne == 0) return;
+    const double *in = S + (size_t)e0 * k * k;
+    int2 *o = out + (size_t)e0 * k * kp;
+    if (threadIdx.x == 0) key = 0;
+    __syncthreads();
+    unsigned mk = 0;
+    for (int j = threadIdx.x; j < ne * k * k; j += 256) mk = max(mk, fa_key(in[j]));
+    atomicMax(&key, mk);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int e = fa_exponent(key, err);
+        if (threadIdx.x == 0) E = e;
     }
-    if (lane == 0) se[e] = E;
+    __syncthreads();
+    for (int j = threadIdx.x; j < ne * k * kp; j += 256) {
+        const int b = j / kp, a = j - b * kp;
+        o[j] = a < k ? fa_split(fa_round(in[(size_t)b * k + a], E + 1022)) : make_int2(0, 0);
+    }
+    for (int e = threadIdx.x; e < ne; e += 256) se[e0 + e] = E;
 }
 
 // flattened bases, CTA per leaf: [level][N][k] -> [N][level k], rows padded to an even length
@@ -968,8 +901,7 @@ void build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t 
         const int kp = (m.k + 1) & ~1;
         op.fa_S.alloc((size_t)m.nfar * m.k * kp);
         op.fa_se.alloc(m.nfar);
-        k_fa_build_S<<<cdiv((long long)m.nfar * 32, 256), 256, 0, st>>>(m.nfar, m.k, kp, op.S64.p, (int2 *)op.fa_S.p,
-                                                                        op.fa_se.p, err);
+        k_fa_build_S<<<m.kt.nnode, 256, 0, st>>>(m.far_ptr.p, m.k, kp, op.S64.p, (int2 *)op.fa_S.p, op.fa_se.p, err);
     }
     VFD_CUDA(cudaGetLastError());
 }
@@ -983,30 +915,9 @@ void apply_group(const MeshData &m, OpData &op, const double *X, double *Y, int 
 {
     const int k = m.k, nleaf = m.kt.nleaf, nnode = m.kt.nnode;
     const bool far = m.nfar > 0;
-    FaFar P;
-    P.fl = m.kt.first_leaf();
-    P.nleaf = nleaf;
-    P.lmin = m.far_lmin;
-    P.L = m.kt.L;
-    P.nlev = far ? m.kt.L - m.far_lmin + 1 : 0;
-    P.k = k;
-    P.kp = (k + 1) & ~1;
-    P.wp = (P.nlev * k + 1) & ~1;
-    P.nnode = nnode;
-    P.nfar = m.nfar;
+    FaFar P = fa_far_view(m, op);
     P.nrhs = nrhs;
     P.c0 = c0;
-    P.kb = m.kt_begin.p;
-    P.ke = m.kt_end.p;
-    P.fptr = m.far_ptr.p;
-    P.fcol = m.far_col.p;
-    P.U = (const int2 *)m.fa_U.p;
-    P.S = (const int2 *)op.fa_S.p;
-    P.ue = m.fa_ue.p;
-    P.Ud = m.Ul64.p;
-    P.Sd = op.S64.p;
-    P.N = m.N;
-    P.se = op.fa_se.p;
     const int w = P.nlev * k, cols = std::min(nrhs - c0, ng * NC);
     // one column: the kernels get its own pieces
     const size_t ps = (size_t)P.nlev * nleaf * k, hs = (size_t)nnode * k, ys = (size_t)m.nfar * k;
@@ -1027,24 +938,10 @@ void apply_group(const MeshData &m, OpData &op, const double *X, double *Y, int 
                 P, op.P64.p, summed ? op.xhat.p : nullptr, op.ye64.p, skip);
         if (summed) launch_far_couple_sum(m, op, c0, cols, op.side, skip);
     }
-    FaNear R;
-    R.fl = P.fl;
+    FaNear R = fa_near_view(m, op);
     R.NR = 64;
     R.nrhs = nrhs;
     R.c0 = c0;
-    R.kb = P.kb;
-    R.ke = P.ke;
-    R.pw = m.panel_w.p;
-    R.gcol = m.gcol.p;
-    R.goff = m.gcol_off.p;
-    R.rowptr = m.rowptr.p;
-    R.colidx = m.colidx.p;
-    R.poff = m.panel_off.p;
-    R.val = op.valBM.p;
-    R.folded = m.bm_in_panels ? 1 : 0;
-    R.Dd = op.D64.p;
-    R.D = (const int2 *)op.fa_D.p;
-    R.re = op.fa_re.p;
     const size_t shm = (size_t)m.max_panel_w * NC * 8;
     VFD_REQUIRE(shm <= 227 * 1024, VFD_EUNSUPPORTED,
                 "apply: a near panel is wider than shared memory holds (use a low-rank operator, lambda > 0)");
@@ -1067,8 +964,8 @@ void apply_group(const MeshData &m, OpData &op, const double *X, double *Y, int 
         } else {
             if (she > 47 * 1024)
                 VFD_CUDA(cudaFuncSetAttribute(k_fa_expand<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)she));
-            k_fa_expand<NC><<<dim3(nleaf, cdiv(m.max_leaf_size, 64), ng), 128, she, st>>>(
-                P, 64, op.ye64.p, summed ? op.yhat.p : nullptr, Y, ld, skip);
+            k_fa_expand<NC><<<dim3(nleaf, cdiv(m.max_leaf_size, R.NR), ng), 128, she, st>>>(
+                P, R.NR, op.ye64.p, summed ? op.yhat.p : nullptr, Y, ld, skip);
         }
     }
     VFD_CUDA(cudaGetLastError());
@@ -1082,6 +979,8 @@ void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int 
 {
     if (dot) dot->n = nrhs == 1 ? m.kt.nleaf * cdiv(m.max_leaf_size, 16) : 0;
     if (dot && !dot->n) dot = nullptr;
+    // many columns: on the tensor cores; what follows is then a fallback behind a flag
+    if (!skip && !dot && apply_tensor_fits(m, nrhs)) skip = apply_tensor(m, op, X, Y, nrhs, ld, st);
     // the node sums inside the gathers pay for few columns and short spans
     const bool summed = nrhs >= 4 || m.kt.L - m.far_lmin > 7;
     // widest group whose panel piece leaves room for two CTAs an SM

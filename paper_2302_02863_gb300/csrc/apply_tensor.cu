@@ -1,0 +1,853 @@
+// The FP64 operator apply of many columns on the tensor cores, in exact integer digits.
+//
+// The fixed-point products of apply_fixed.cu cost three 32-bit multiply-adds each,
+// about 5 cycles of an SM and warp with their carries.  Here an entry (62 bits: the
+// fixed-point integer times 4) is cut into eight digits of base 2^8 in [-128, 127],
+// exact in FP16, and the digits of the two factors are multiplied by tcgen05.mma
+// (kind::f16, FP32 accumulators in tensor memory):
+//   a x = sum_{i, j} 2^(8 (i + j)) a_i x_j,
+// the 36 products with i + j >= 7.  Products of equal i + j share an accumulator, 8 of
+// them, and after 160 products at most they move to 96-bit integers in registers: 6 pairs
+// of 160 stay below 2^24 and are exact; of the two lowest accumulators (8 and 7 pairs) a
+// sum above 2^24 is rounded by less than the dropped pairs add up to.  So the result is
+// that of integer arithmetic up to the dropped pairs.
+//
+// A CTA computes 128 rows (two halves of 64: sibling leaves, sibling nodes) of a tile
+// of NC columns.  The digit planes of the vector lie one after the other along N, so
+// one instruction multiplies plane i of the operator by planes 7 - i .. 7 of the vector
+// into neighbouring accumulators: N = NC (i + 1).  Sibling rows share most of their
+// partners, and a partner's vector digits serve both halves (records built with the
+// mesh: build_tensor_lists); a half without the partner multiplies zeros.
+//
+//   k_td_max, k_td_digits   x -> digits per leaf, in the order the instruction reads
+//   k_td<PROJ>              projections, then the node sums (apply.cu), digits per node
+//   k_td<COUPLE>            coupling blocks summed per node (one exponent a node), digits
+//   k_td<ROWS>              near panel rows and the expansion of a leaf, Y
+//
+// Warp roles of k_td, per step of 16 rows of a partner:
+//   warps 0-15 copy the operator's integers (apply_fixed.cu) two steps ahead and cut them
+//              into digit planes in shared memory; after every 10 steps at most they move
+//              the accumulators on
+//   warp 16    lane 0 issues the products (it waits where the tensor cores are behind, so
+//              it cannot also cut); the warp owns the tensor memory
+//   warp 17    lane 0 copies the vector's digits of the step (cp.async.bulk)
+// Every wait is bounded by a count of cycles; a CTA whose wait expires raises err, waits
+// (bounded again) for its copies and products, and returns.  Columns where a vector does
+// not fit (Inf, NaN, all below 2^-895) raise err too; then the kernels of apply_fixed.cu,
+// launched behind a flag, do the apply.
+//
+// What bounds it: 36 products of 128 x 64 x 16 (12 instructions) are 1152 cycles of the
+// tensor cores, cutting a step 800 to 1100 cycles of 16 warps beside them, and a move of the
+// accumulators (64 K conversions at 16 a cycle, 64-bit sums) about 6000 cycles in which
+// the tensor cores wait.  64 columns at 27361 DoFs and rank 64: 1145 us (fixed-point kernels
+// 5270, FP64 kernels 11880): rows 436, coupling 302, projections 154, node sums 56, digits
+// 100; the tensor cores are busy 36% of the coupling's time.  The same digits with
+// mma.sync m16n8k16 (600 TFLOP/s against 2.2 PFLOP/s) took 2664 us.
+// Error against extended precision (meshes of 800 to 1100 DoFs, columns of normal
+// numbers): 0.7 to 0.9e-16 of |y|, FP64 kernels 1.2 to 1.3e-16; at most 6e-16 of a
+// component of |A||x|, FP64 3.8e-16.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+#include "apply_common.cuh"
+#include "apply_fixed.cuh"
+
+namespace vfd {
+
+namespace {
+
+constexpr int TD_D = 8;                     // digits
+constexpr int TD_G = 8;                     // accumulators: i + j = 7 .. 14
+constexpr int TD_COLS = 64;                 // columns of a pass
+constexpr int TD_NST = 4;                   // stages
+constexpr int TD_MOVE = 10;                 // steps between two moves of the accumulators at most
+constexpr int TD_LAG = 3;                   // steps cut ahead of a move of the accumulators
+constexpr int TD_CW = 16;                   // cutting warps
+constexpr int TD_AHEAD = 2;                 // steps whose entries are on their way
+constexpr int TD_RAW = TD_CW * 32 * 32;     // bytes of a step's entries
+constexpr int TD_THREADS = 32 * (TD_CW + 2);
+constexpr int TD_A = 128 * 16 * TD_D * 2;   // bytes of the operator's digits of a step
+constexpr int TD_SMS = 152;                // CTAs of a launch and tile: one an SM
+constexpr long long TD_WAIT = 2000000000LL;   // cycles, about a second
+enum { TD_PROJ, TD_COUPLE, TD_ROWS };
+
+// bytes of the vector's digits of a step: [digit][column / 8][row / 8][column % 8][row % 8],
+// i.e. core matrices of 8 columns x 16 bytes
+__host__ __device__ constexpr int td_step(int nc) { return nc * 16 * TD_D * 2; }
+
+struct TdVec {          // a set of pieces of a matrix of columns
+    const double *v;
+    size_t ld, base;    // column stride; offset of piece 0 (nodes)
+    int npiece, ns, len;                 // ns: steps of a piece; len: rows of a piece (nodes)
+    const int *kb, *ke;                  // rows of a piece (leaves), or null
+    int nrhs, c0, nc;                    // columns c0 .. min(c0 + 64, nrhs) in tiles of nc
+    unsigned *key;                       // per column of the pass
+    unsigned char *out;                  // [tile][piece][step]
+    int *err;
+};
+
+__device__ __forceinline__ void td_range(const TdVec &P, int p, size_t &b, int &n)
+{
+    b = P.kb ? (size_t)P.kb[p] : P.base + (size_t)p * P.len;
+    n = P.kb ? P.ke[p] - (int)b : P.len;
+}
+
+// largest exponent of every column (grid.y) over all pieces, which are contiguous
+__global__ void __launch_bounds__(256) k_td_max(TdVec P)
+{
+    const int c = blockIdx.y;
+    size_t b, b1;
+    int n, n1;
+    td_range(P, 0, b, n);
+    td_range(P, P.npiece - 1, b1, n1);
+    const double *v = P.v + (size_t)(P.c0 + c) * P.ld + b;
+    const size_t tot = b1 + n1 - b;
+    unsigned mk = 0;
+    for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < tot; i += (size_t)gridDim.x * 256) mk = max(mk, fa_key(v[i]));
+    mk = __reduce_max_sync(0xffffffffu, mk);
+    if ((threadIdx.x & 31) == 0 && mk) atomicMax(P.key + c, mk);
+}
+
+// digits of piece blockIdx.x for tile blockIdx.y; a thread takes 8 rows of a column
+__global__ void __launch_bounds__(256) k_td_digits(TdVec P)
+{
+    const int p = blockIdx.x;
+    size_t b;
+    int n;
+    td_range(P, p, b, n);
+    unsigned char *out = P.out + ((size_t)blockIdx.y * P.npiece + p) * P.ns * td_step(P.nc);
+    for (int t = threadIdx.x; t < P.nc * 2 * P.ns; t += 256) {
+        const int ch = t / P.nc, col = t % P.nc, r = blockIdx.y * P.nc + col;
+        const bool on = P.c0 + r < P.nrhs;
+        const unsigned key = on ? P.key[r] : 0u;
+        if (fa_slow(key)) atomicOr(P.err, 1);
+        const double *v = P.v + (size_t)(P.c0 + r) * P.ld + b;
+        u64 d[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int i = ch * 8 + q;
+            const i64 x = on && i < n ? fa_round(v[i], (int)key) : 0;
+            d[q] = (u64)(x << 2) + 0x8080808080808080ULL;   // digits plus 128
+        }
+        unsigned char *o = out + (size_t)(ch >> 1) * td_step(P.nc) + (ch & 1) * 128 + (col & 7) * 16;
+#pragma unroll
+        for (int i = 0; i < TD_D; ++i) {
+            half2 h[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const unsigned u = (unsigned)(d[2 * q] >> (8 * i)) & 255u, w = (unsigned)(d[2 * q + 1] >> (8 * i)) & 255u;
+                h[q] = __halves2half2(__int2half_rn((int)u - 128), __int2half_rn((int)w - 128));
+            }
+            *(uint4 *)(o + (size_t)(i * (P.nc >> 3) + (col >> 3)) * 256) = *(const uint4 *)h;
+        }
+    }
+}
+
+struct TdP {
+    FaFar F;
+    FaNear R;
+    int nrhs, c0, nsl, nsn, node0, nnodes;   // steps of a leaf and of a node; nodes node0 .. node0 + nnodes
+    const unsigned char *dx, *dh;            // digits of the leaves' x; of the nodes' xhat or yhat
+    const unsigned *kx, *kh;                 // their column keys
+    unsigned *ko;                            // COUPLE: keys of yhat
+    const int *bin;                          // items of a CTA (build_tensor_lists)
+    const int4 *items;
+    const TdRec *rec;
+    int *err;
+};
+
+__device__ __forceinline__ unsigned td_sa(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// SM cycles (reading the global timer instead takes about a microsecond)
+__device__ __forceinline__ u64 td_timer() { return (u64)clock64(); }
+
+__device__ __forceinline__ bool td_wait(unsigned bar, unsigned parity, u64 deadline)
+{
+    while (true) {
+        unsigned done;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if (td_timer() > deadline) return false;
+    }
+}
+__device__ __forceinline__ void td_arrive(unsigned bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void td_commit(unsigned bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
+}
+
+// K-major operand without swizzle: core matrices of 8 rows x 16 bytes, the two of a
+// step's 16 rows 128 bytes apart, groups of 8 rows 256 bytes apart
+__device__ __forceinline__ u64 td_desc(unsigned a)
+{
+    return (u64)((a & 0x3FFFF) >> 4) | (u64)(128 >> 4) << 16 | (u64)(256 >> 4) << 32 | (u64)1 << 46;
+}
+// FP32 accumulator, FP16 operands, both K-major, M = 128
+__device__ __forceinline__ void td_mma(unsigned d, unsigned a, unsigned b, int n, bool acc)
+{
+    const unsigned idesc = (1u << 4) | ((unsigned)(n >> 3) << 17) | ((128u >> 4) << 24);
+    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+                 "l"(td_desc(a)), "l"(td_desc(b)), "r"(idesc), "r"((unsigned)acc));
+}
+
+// (h 2^32 + l) 2^(56 + e) rounded to FP64 with integers (two conversions, a multiply-add
+// and a scaling in FP64 would be 80 cycles of the SM a warp); bad: not a normal number
+__device__ __forceinline__ double td_value(i64 h, unsigned l, int e, bool &bad)
+{
+    const bool neg = h < 0;
+    if (neg) {
+        h = ~h + (l == 0);
+        l = 0u - l;
+    }
+    const bool big = (u64)h >> 32 != 0;
+    const u64 a = big ? (u64)h : (u64)h << 32 | l;
+    const int z = __clzll(a);
+    const u64 t = z == 64 ? 0 : a << z | (big ? l >> (32 - z) : 0u);   // leading one at 63
+    const int b = 1023 + 56 + 95 - z - (big ? 0 : 32) + e;
+    bad |= t != 0 && (b < 2 || b > 2045);
+    const u64 r = (((t >> 1) + 512) >> 10) + ((u64)(b - 1) << 52);
+    return __longlong_as_double(t ? (i64)(r | (neg ? 1ULL << 63 : 0ULL)) : 0LL);
+}
+
+// a b + c, kept a multiply-add (as shifts and 64-bit adds it takes four instructions)
+__device__ __forceinline__ i64 td_mad(int a, int b, i64 c)
+{
+    i64 r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+
+// exponent of a sum of digit products: entries below 2^ea, a column with this key
+__device__ __forceinline__ int td_exp(int ea, unsigned key) { return ea + (key ? (int)key - 1022 : 0) - 2 * 62; }
+
+// where a role stands: piece q of an item, its partner, rows and the half's offset
+struct TdIt {
+    int i, item, q, q1, q2, col, n, nrow, W;   // i: of the CTA's items
+    i64 off;
+};
+
+template <int NC, int MODE>
+__global__ void __launch_bounds__(TD_THREADS, 1)
+k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restrict__ out)
+{
+    extern __shared__ __align__(1024) unsigned char td_sm[];
+    constexpr int STAGE = TD_A + td_step(NC), NH = NC / 4;
+    u64 *bars = (u64 *)(td_sm + TD_NST * STAGE + TD_AHEAD * TD_RAW);   // A full, B full, empty [stages each], moved, drained
+    unsigned *tslot = (unsigned *)(bars + 3 * TD_NST + 2);
+    volatile int *abort_f = (volatile int *)(tslot + 1);
+    unsigned *skey = tslot + 2;   // column keys of the tile: leaves, nodes
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tile = blockIdx.y;
+    const unsigned bar0 = td_sa(bars), base = td_sa(td_sm);
+    auto fullA = [&](int s) { return bar0 + 8u * s; };
+    auto fullB = [&](int s) { return bar0 + 8u * (TD_NST + s); };
+    auto empty = [&](int s) { return bar0 + 8u * (2 * TD_NST + s); };
+    const unsigned moved = bar0 + 24u * TD_NST, drained = moved + 8u;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < TD_NST; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(fullA(s)), "r"(TD_CW));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(fullB(s)), "r"(1));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(empty(s)), "r"(1));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(moved), "r"(1));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(drained), "r"(TD_CW));
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        *abort_f = 0;
+    }
+    if (warp == TD_CW) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(td_sa(tslot)), "n"(TD_G * NC));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
+    if (threadIdx.x < 2 * NC) {
+        const unsigned *key = threadIdx.x < NC ? P.kx : P.kh;
+        skey[threadIdx.x] = key ? key[tile * NC + (int)threadIdx.x % NC] : 0u;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const unsigned taddr = *tslot;
+    const u64 deadline = td_timer() + TD_WAIT;
+
+    // Items: pairs of leaves (ROWS), of nodes (COUPLE), 128 columns of a leaf's bases (PROJ).
+    // An item's records q .. q2, the first section up to q1 (ROWS: near, then far).
+    const int k = P.F.k, half = warp >> 3 & 1, nz = (P.F.nlev * k + 127) >> 7;
+    const int ibeg = MODE == TD_PROJ ? (int)((i64)nitem * blockIdx.x / gridDim.x) : P.bin[blockIdx.x];
+    const int iend = MODE == TD_PROJ ? (int)((i64)nitem * (blockIdx.x + 1) / gridDim.x) : P.bin[blockIdx.x + 1];
+    auto record = [&](TdIt &I) {
+        if (MODE == TD_PROJ) return;
+        const TdRec r = P.rec[I.q];
+        I.col = r.col;
+        I.n = r.n;
+        I.off = r.off[half];
+    };
+    auto start = [&](TdIt &I) {   // first piece of item I.i; false: no more items
+        I.n = 0;
+        if (I.i >= iend) return false;
+        if (MODE == TD_PROJ) {
+            const int leaf = I.i / nz, c0 = (I.i - leaf * nz) * 128 + half * 64;
+            const int b = P.F.kb[P.F.fl + leaf], n = P.F.ke[P.F.fl + leaf] - b;
+            I.item = I.i;
+            I.q = 0;
+            I.q1 = I.q2 = 1;
+            I.col = leaf;
+            I.n = max(n, 1);
+            I.off = n > 0 ? (i64)b * P.F.wp + c0 : -1;
+            I.nrow = max(0, min(64, P.F.nlev * k - c0));
+        } else {
+            const int4 v = P.items[I.i];
+            I.q = v.x;
+            I.q1 = v.y;
+            I.q2 = v.z;
+            I.item = v.w;
+            I.nrow = k;
+        }
+        if (MODE == TD_ROWS) {
+            const int leaf = 2 * I.item + half;
+            I.nrow = leaf < P.F.nleaf ? P.R.ke[P.R.fl + leaf] - P.R.kb[P.R.fl + leaf] : 0;
+            I.W = leaf < P.F.nleaf ? P.R.pw[leaf] : 0;
+        }
+        record(I);
+        return true;
+    };
+    auto next = [&](TdIt &I) {
+        if (++I.q < I.q2) {
+            record(I);
+            return true;
+        }
+        ++I.i;
+        return start(I);
+    };
+    // 0: nothing after this step; 1: move the accumulators; 2, 3: and end the first, second section
+    int since = 0;
+    auto code_of = [&](int end, bool last) {
+        const int c = last ? end : 0;
+        since = c || since == TD_MOVE - 1 ? 0 : since + 1;
+        return c ? c : (since == 0 ? 1 : 0);
+    };
+    TdIt I{};
+    I.i = ibeg;
+    bool have = start(I), ok = true;
+    int issued = 0;   // steps of the products, of the copies
+    if (warp < TD_CW) {
+        // cutting: 8 rows a warp; a lane takes 4 neighbouring entries of a row
+        const int g = lane >> 1 & 7, tt = 8 * (lane >> 4) + 4 * (lane & 1);   // row, first entry
+        const int mrow = (warp & 7) * 8 + g;   // this lane's row in the half
+        // reading the accumulators: row of the tile, columns
+        const int orow = 32 * (warp & 3) + lane, ohalf = orow >> 6, om = orow & 63, oc = (warp >> 2) * NH;
+        i64 sh[NH];   // sums in units of 2^56: sh 2^32 + sl
+        unsigned sl[NH];
+#pragma unroll
+        for (int c = 0; c < NH; ++c) sh[c] = sl[c] = 0;
+        int moves = 0, m8 = 256, m16 = 65536, m24 = 16777216;
+        asm("" : "+r"(m8), "+r"(m16), "+r"(m24));   // in registers: not shifts
+        int ei = ibeg;   // the item that ends next
+        auto emit = [&](int code) {
+            int ri = 0, e = 0;   // row of out
+            bool on = false, bad = false;
+            size_t os = (size_t)ld;   // column stride
+            const int item = MODE == TD_PROJ ? ei : P.items[ei].w;
+            if (MODE != TD_ROWS || code == 3 || P.F.nlev == 0) ++ei;
+            if (MODE == TD_PROJ) {
+                const int leaf = item / nz, c = (item - leaf * nz) * 128 + orow, lv = c / k;
+                on = c < P.F.nlev * k;
+                ri = (lv * P.F.nleaf + leaf) * k + c - lv * k;
+                e = P.F.ue[leaf];
+                os = (size_t)P.F.nlev * P.F.nleaf * k;
+            }
+            if (MODE == TD_ROWS) {
+                const int leaf = 2 * item + ohalf;
+                if (leaf < P.F.nleaf) {
+                    const int b = P.R.kb[P.R.fl + leaf];
+                    ri = b + om;
+                    on = om < P.R.ke[P.R.fl + leaf] - b;
+                    if (on) e = code == 2 ? P.R.re[ri] : P.F.ue[leaf];
+                }
+            }
+            if (MODE == TD_COUPLE) {
+                const int node = P.node0 + 2 * item + ohalf;
+                on = node < P.F.nnode && om < k;
+                ri = node * k + om;
+                if (on && P.F.fptr[node] < P.F.fptr[node + 1]) e = P.F.se[P.F.fptr[node]];
+                os = (size_t)P.F.nnode * k;
+            }
+            const unsigned *key = skey + oc + (MODE == TD_PROJ || (MODE == TD_ROWS && code == 2) ? 0 : NC);
+            double *o = out + ri;
+            const int r0 = P.c0 + tile * NC + oc, nr = on ? P.nrhs - r0 : 0;   // columns 0 .. nr of this thread
+            o += (size_t)r0 * os;
+            unsigned mine = 0;
+#pragma unroll
+            for (int c0 = 0; c0 < NH; c0 += 2) {
+                double v[2], y[2];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    bool b = false;
+                    v[j] = td_value(sh[c0 + j], sl[c0 + j], td_exp(e, key[c0 + j]), b);
+                    bad |= b && c0 + j < nr;
+                    sh[c0 + j] = sl[c0 + j] = 0;
+                    if (MODE == TD_ROWS) y[j] = code == 3 && c0 + j < nr ? o[(c0 + j) * os] : 0.0;
+                    if (MODE == TD_COUPLE) {
+                        const unsigned mk = __reduce_max_sync(0xffffffffu, c0 + j < nr ? fa_key(v[j]) : 0u);
+                        if (lane == c0 + j) mine = mk;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    if (MODE == TD_ROWS) v[j] += y[j];
+                    if (c0 + j < nr) o[(c0 + j) * os] = v[j];
+                }
+            }
+            if (MODE == TD_COUPLE && mine) atomicMax(P.ko + tile * NC + oc + lane, mine);
+            if (MODE == TD_ROWS && code == 2 && !P.R.folded)   // B + M outside the panels
+                for (int c = 0; c < min(nr, NH); ++c) {
+                    double v = o[c * os];
+                    for (int s = P.R.rowptr[ri]; s < P.R.rowptr[ri + 1]; ++s)
+                        v = fma(P.R.val[s], X[(size_t)(r0 + c) * ld + P.R.colidx[s]], v);
+                    o[c * os] = v;
+                }
+            if (bad) atomicOr(P.err, 1);
+        };
+        auto move = [&](int code) {
+            if (!td_wait(moved, moves & 1, deadline)) return false;
+            ++moves;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+#pragma unroll
+            for (int c = 0; c < NH; c += 2) {
+                unsigned f[TD_G][2];
+#pragma unroll
+                for (int q = 0; q < TD_G; ++q)
+                    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];\n"
+                                 : "=r"(f[q][0]), "=r"(f[q][1])
+                                 : "r"(taddr + ((unsigned)(32 * (warp & 3)) << 16) + (unsigned)(q * NC + oc + c)));
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    int v[TD_G];
+#pragma unroll
+                    for (int q = 0; q < TD_G; ++q) v[q] = __float2int_rn(__uint_as_float(f[q][j]));
+                    i64 lo = td_mad(v[1], m8, (i64)v[0]);
+                    lo = td_mad(v[3], m24, td_mad(v[2], m16, lo));
+                    i64 hi = td_mad(v[5], m8, (lo >> 32) + v[4]);
+                    hi = td_mad(v[7], m24, td_mad(v[6], m16, hi));
+                    const u64 x = (u64)sl[c + j] + (unsigned)lo;
+                    sl[c + j] = (unsigned)x;
+                    sh[c + j] += hi + (i64)(x >> 32);
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+            __syncwarp();
+            if (lane == 0) td_arrive(drained);
+            if (code > 1) emit(code);
+            return true;
+        };
+        auto matrix = [&](const TdIt &J, int &sm, int &sk) {
+            const bool far = MODE == TD_ROWS && J.q >= J.q1;
+            sm = MODE == TD_ROWS ? (far ? P.F.wp : J.W) : 1;
+            sk = MODE == TD_ROWS ? 1 : (MODE == TD_COUPLE ? P.F.kp : P.F.wp);
+            return (MODE == TD_COUPLE ? P.F.S : (MODE == TD_PROJ || far ? P.F.U : P.R.D)) + J.off;
+        };
+        // copies the entries of the next step to the lane's place, and puts its code to hist
+        int2 *const raw = (int2 *)(td_sm + TD_NST * STAGE) + warp * 128 + lane;
+        const int2 *p = nullptr;
+        int left = 0, steps = 0, np = 0, end = 0, pulled = 0;   // of the piece: rows and steps that are left
+        unsigned hist = 0;
+        auto pull = [&]() {
+            if (steps == 0) {
+                if (!have) {
+                    hist <<= 2;
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                    return false;
+                }
+                int sm, sk;
+                p = matrix(I, sm, sk) + (mrow * sm + tt * sk);
+                left = I.off >= 0 && mrow < I.nrow ? I.n - tt : 0;
+                np = I.n;
+                steps = (np + 15) >> 4;
+                end = I.q + 1 == I.q1 ? 2 : (I.q + 1 == I.q2 ? 3 : 0);
+                have = next(I);   // I: the piece after this one
+            }
+            const int sk = MODE == TD_ROWS ? 1 : (MODE == TD_COUPLE ? P.F.kp : P.F.wp);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)   // zeros outside (nothing is read)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
+                                 td_sa(raw + (pulled % TD_AHEAD) * (TD_RAW / 8) + 32 * j)),
+                             "l"(j < left ? p + j * sk : (const int2 *)P.F.U), "r"(j < left ? 8 : 0)
+                             : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            p += 16 * sk;
+            left -= 16;
+            ++pulled;
+            --steps;
+            hist = hist << 2 | (unsigned)code_of(end, steps == 0);
+            if (have && steps + 2 == (np + 15) >> 4) {
+                // in the piece's second step (its record has come): the warp's entries of the next piece to L2
+                int sm, sq;
+                const int2 *A = matrix(I, sm, sq);
+                const int m = (warp & 7) * 8;
+                if (MODE == TD_ROWS) {   // 8 rows of 64 entries
+                    if (I.off >= 0 && m + (lane >> 2) < I.nrow && 16 * (lane & 3) < I.n)
+                        asm volatile("prefetch.global.L2 [%0];\n" ::"l"(A + ((m + (lane >> 2)) * sm + 16 * (lane & 3))));
+                } else {                 // 8 entries of 64 rows
+#pragma unroll
+                    for (int h = 0; h < 64; h += 32)
+                        if (I.off >= 0 && m < I.nrow && h + lane < I.n)
+                            asm volatile("prefetch.global.L2 [%0];\n" ::"l"(A + (m + (h + lane) * sq)));
+                }
+            }
+            return true;
+        };
+        static_assert(TD_AHEAD == 2, "v0, v1");
+        bool v0 = pull(), v1 = pull();
+        int cut = 0;   // steps cut
+#pragma unroll 1
+        for (int t = 0; v0 || t < cut + TD_LAG; ++t) {
+            const bool now = v0;
+            unsigned wl[4], wh[4];   // low and high words of the digits plus 128
+            asm volatile("cp.async.wait_group %0;" ::"n"(TD_AHEAD - 1) : "memory");
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int2 a = raw[(t % TD_AHEAD) * (TD_RAW / 8) + 32 * j];
+                const u64 v = ((u64)(unsigned)a.y << 32) + (u64)((i64)a.x << 2) + 0x8080808080808080ULL;
+                wl[j] = (unsigned)v;
+                wh[j] = (unsigned)(v >> 32);
+            }
+            v0 = v1;
+            v1 = pull();
+            if (now) {
+                const int st = t % TD_NST;
+                if (t >= TD_NST && !td_wait(empty(st), (t / TD_NST - 1) & 1, deadline)) {
+                    ok = false;
+                    break;
+                }
+                unsigned char *sa = td_sm + st * STAGE + warp * 256 + lane * 8;
+#pragma unroll
+                for (int i = 0; i < TD_D; i += 2) {
+                    const unsigned *w = i < 4 ? wl : wh;
+                    unsigned d[2][2];   // [digit i, i + 1][pair of entries]
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        // digits i (bytes 0, 1) and i + 1 (bytes 2, 3) of two entries
+                        const unsigned b = __byte_perm(w[2 * j], w[2 * j + 1], i & 2 ? 0x7362 : 0x5140);
+                        // 0x64dd is 1024 + dd in FP16; less 1152
+                        const unsigned h0 = __byte_perm(b, 0x64646464u, 0x4140), h1 = __byte_perm(b, 0x64646464u, 0x4342);
+                        const half2 off2 = __half2half2(__ushort_as_half(0x6480));
+                        const half2 d0 = __hsub2(*(const half2 *)&h0, off2), d1 = __hsub2(*(const half2 *)&h1, off2);
+                        d[0][j] = *(const unsigned *)&d0;
+                        d[1][j] = *(const unsigned *)&d1;
+                    }
+                    *(uint2 *)(sa + i * 4096) = make_uint2(d[0][0], d[0][1]);
+                    *(uint2 *)(sa + i * 4096 + 4096) = make_uint2(d[1][0], d[1][1]);
+                }
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) td_arrive(fullA(st));
+                ++cut;
+            }
+            const int c = (hist >> (2 * (TD_AHEAD + TD_LAG))) & 3;   // of step t - LAG
+            if (c && !move(c)) {
+                ok = false;
+                break;
+            }
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+    } else if (lane == 0) {
+        int moves = 0;
+        bool first = true;
+        while (have && ok) {
+            TdIt J = I;   // its record comes while this piece is worked on
+            const bool more = next(J);
+            const int ns = (I.n + 15) >> 4, end = I.q + 1 == I.q1 ? 2 : (I.q + 1 == I.q2 ? 3 : 0);
+            const bool leaf = MODE == TD_PROJ || (MODE == TD_ROWS && I.q < I.q1);
+            const unsigned char *src = leaf ? P.dx + ((size_t)tile * P.F.nleaf + I.col) * P.nsl * td_step(NC)
+                                            : P.dh + ((size_t)tile * P.nnodes + I.col) * P.nsn * td_step(NC);
+            for (int s = 0; s < ns && ok; ++s) {
+                const int st = issued % TD_NST;
+                const unsigned par = (issued / TD_NST) & 1;
+                if (warp == TD_CW) {
+                    // ---- products
+                    if (!td_wait(fullA(st), par, deadline) || !td_wait(fullB(st), par, deadline)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    const unsigned sa = base + st * STAGE, sb = sa + TD_A;
+#pragma unroll
+                    for (int i = TD_D - 1; i >= 0; --i) {
+                        // accumulators 0 .. i, in instructions of at most 256 columns; i = 7 first: it clears all
+                        constexpr int GM = 256 / NC < 8 ? 256 / NC : 8;
+#pragma unroll
+                        for (int g0 = 0; g0 <= i; g0 += GM) {
+                            const int ng = i + 1 - g0 < GM ? i + 1 - g0 : GM;
+                            td_mma(taddr + g0 * NC, sa + i * 4096, sb + (7 - i + g0) * (NC * 32), ng * NC, !(first && i == 7));
+                        }
+                    }
+                    td_commit(empty(st));
+                    ++issued;
+                    first = false;
+                    if (code_of(end, s + 1 == ns)) {
+                        td_commit(moved);
+                        ok = td_wait(drained, moves & 1, deadline);
+                        ++moves;
+                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        first = true;
+                    }
+                } else {
+                    // ---- the vector's digits
+                    if (issued >= TD_NST && !td_wait(empty(st), par ^ 1, deadline)) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fullB(st)), "r"(td_step(NC))
+                                 : "memory");
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                            base + st * STAGE + TD_A),
+                        "l"(src + (size_t)s * td_step(NC)), "r"(td_step(NC)), "r"(fullB(st))
+                        : "memory");
+                    ++issued;
+                }
+            }
+            I = J;
+            have = more;
+        }
+    }
+    if (!ok) *abort_f = 1;
+    __syncwarp();
+    __syncthreads();
+    if (*abort_f) {
+        // wait for what is in flight: the copies, then the products
+        const u64 dl = td_timer() + TD_WAIT;
+        if (warp >= TD_CW && lane == 0)
+            for (int i = max(0, issued - TD_NST); i < issued; ++i)
+                td_wait(warp == TD_CW ? empty(i % TD_NST) : fullB(i % TD_NST), (i / TD_NST) & 1, dl);
+        if (threadIdx.x == 0) atomicOr(P.err, 1);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == TD_CW)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "n"(TD_G * NC));
+}
+
+__global__ void k_td_good(const int *err, int *good) { *good = *err == 0; }
+
+template <int NC, int MODE>
+void launch_td(const TdP &P, int nitem, int nt, const double *X, int64_t ld, double *out, cudaStream_t st)
+{
+    constexpr int shm = TD_NST * (TD_A + td_step(NC)) + TD_AHEAD * TD_RAW + (3 * TD_NST + 2) * 8 + 8 + 2 * NC * 4;
+    VFD_CUDA(cudaFuncSetAttribute(k_td<NC, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, shm));
+    k_td<NC, MODE><<<dim3(std::min(nitem, TD_SMS), nt), TD_THREADS, shm, st>>>(P, nitem, X, ld, out);
+    VFD_CUDA(cudaGetLastError());
+}
+template <int MODE>
+void launch_td(int nc, const TdP &P, int nitem, int nt, const double *X, int64_t ld, double *out, cudaStream_t st)
+{
+    if (nc == 16) launch_td<16, MODE>(P, nitem, nt, X, ld, out, st);
+    else if (nc == 32) launch_td<32, MODE>(P, nitem, nt, X, ld, out, st);
+    else launch_td<64, MODE>(P, nitem, nt, X, ld, out, st);
+}
+
+}  // namespace
+
+// Records of k_td, geometry only (end of the mesh setup).  A record: partner (leaf, or node
+// less the first far node), its rows (> 0), offsets of the two halves' entries (-1: none).
+// td_rows: pairs of leaves (2 p, 2 p + 1): near partners (offsets in the panels), then the
+// ancestors of the far levels (offsets in the flattened bases).
+// td_couple: pairs of nodes from the first far node on (offsets in the coupling blocks).
+// Items (first record, second section, end, pair) in the order of the CTAs that take them.
+void build_tensor_lists(MeshData &m)
+{
+    if (m.max_leaf_size > 64 || !m.nnear) return;
+    const int nleaf = m.kt.nleaf, fl = m.kt.first_leaf(), nlev = m.nfar > 0 ? m.kt.L - m.far_lmin + 1 : 0;
+    const int k = m.k, kp = (k + 1) & ~1, wp = (nlev * k + 1) & ~1, node0 = nlev ? (1 << m.far_lmin) - 1 : 0;
+    std::vector<TdRec> rec;
+    std::vector<int4> items;
+    auto add = [&](int col, int n, int64_t a, int64_t b) { if (n > 0) rec.push_back({col, n, {a, b}}); };
+    // merge of two sorted lists [a0, a1) and [b0, b1) of partners
+    auto merge = [&](const std::vector<int> &list, int a0, int a1, int b0, int b1, auto f) {
+        while (a0 < a1 || b0 < b1) {
+            const int c = std::min(a0 < a1 ? list[a0] : list[b0], b0 < b1 ? list[b0] : list[a0]);
+            const int ea = a0 < a1 && list[a0] == c ? a0++ : -1, eb = b0 < b1 && list[b0] == c ? b0++ : -1;
+            f(c, ea, eb);
+        }
+    };
+    // the largest items first, each to the CTA with the fewest steps so far
+    auto upload = [&](DBuf<TdRec> &dr, DBuf<int4> &di, DBuf<int> &db) {
+        const int n = (int)items.size(), nb = std::min(n, TD_SMS);
+        std::vector<int64_t> steps(n, 2), load(nb, 0);   // and 2 for an item's end
+        std::vector<int> ord(n), bin(1, 0);
+        std::vector<std::vector<int>> of(nb);
+        for (int i = 0; i < n; ++i) {
+            ord[i] = i;
+            for (int q = items[i].x; q < items[i].z; ++q) steps[i] += (rec[q].n + 15) >> 4;
+        }
+        std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return steps[a] > steps[b]; });
+        for (int i : ord) {
+            const int b = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+            load[b] += steps[i];
+            of[b].push_back(i);
+        }
+        std::vector<int4> out;
+        for (auto &l : of) {
+            for (int i : l) out.push_back(items[i]);
+            bin.push_back((int)out.size());
+        }
+        dr.upload(rec);
+        di.upload(out);
+        db.upload(bin);
+        rec.clear();
+        items.clear();
+    };
+    for (int a = 0; a < nleaf; a += 2) {
+        const int b = a + 1 < nleaf ? a + 1 : -1, q0 = (int)rec.size();
+        merge(m.near_col_h, m.near_ptr_h[a], m.near_ptr_h[a + 1], b < 0 ? 0 : m.near_ptr_h[b], b < 0 ? 0 : m.near_ptr_h[b + 1],
+              [&](int c, int ea, int eb) {
+                  add(c, m.kt.end[fl + c] - m.kt.begin[fl + c], ea < 0 ? -1 : m.near_off_h[ea], eb < 0 ? -1 : m.near_off_h[eb]);
+              });
+        const int q1 = (int)rec.size();
+        for (int lv = 0; lv < nlev; ++lv) {
+            const int na = ((fl + a + 1) >> (nlev - 1 - lv)) - 1, nb = b < 0 ? -1 : ((fl + b + 1) >> (nlev - 1 - lv)) - 1;
+            const int64_t oa = (int64_t)m.kt.begin[fl + a] * wp + lv * k;
+            const int64_t ob = b < 0 ? -1 : (int64_t)m.kt.begin[fl + b] * wp + lv * k;
+            if (na == nb || b < 0) {
+                add(na - node0, k, oa, ob);
+            } else {
+                add(na - node0, k, oa, -1);
+                add(nb - node0, k, -1, ob);
+            }
+        }
+        if (q0 < (int)rec.size()) items.push_back({q0, q1, (int)rec.size(), a / 2});
+    }
+    upload(m.td_rows, m.td_rows_item, m.td_rows_bin);
+    if (!nlev) return;
+    const int64_t blk = (int64_t)k * kp;
+    for (int a = node0; a < m.kt.nnode; a += 2) {
+        const bool two = a + 1 < m.kt.nnode;
+        const int q0 = (int)rec.size();
+        merge(m.far_col_h, m.far_ptr_h[a], m.far_ptr_h[a + 1], two ? m.far_ptr_h[a + 1] : 0, two ? m.far_ptr_h[a + 2] : 0,
+              [&](int c, int ea, int eb) { add(c - node0, k, ea < 0 ? -1 : ea * blk, eb < 0 ? -1 : eb * blk); });
+        if (q0 == (int)rec.size()) add(0, k, -1, -1);   // no blocks: zeros
+        items.push_back({q0, (int)rec.size(), (int)rec.size(), (a - node0) / 2});
+    }
+    upload(m.td_couple, m.td_couple_item, m.td_couple_bin);
+}
+
+// Where the digits pay.  The fixed-point kernels take groups of 8 columns, 7.6 us for each
+// 10^6 entries and group once the chip is full; the digits up to 64 columns at a time, but
+// a CTA walks all partners of its rows, 150 to 280 us even for small meshes.  Measured, 10^6
+// entries x groups: fixed point / digits in us: 9 (9025 DoFs, rank 16, 8 columns) 127 / 200,
+// 18 (16 columns) 213 / 208, 27 (24) 328 / 231; 19 (10267 DoFs, rank 36, 8) 234 / 279, 38
+// (12) 364 / 304; 28 (3997 DoFs, rank 64, 24) 289 / 300, 37 (32) 328 / 303; 97 (27361 DoFs,
+// rank 64, 5) 700 / 590, 776 (64) 5269 / 1143.  Up to 4 columns go as one narrow group
+// (97: 395 / 590).
+bool apply_tensor_fits(const MeshData &m, int nrhs)
+{
+    const int nlev = m.nfar > 0 ? m.kt.L - m.far_lmin + 1 : 0;
+    const double entries = (double)m.near_entries + (double)m.nfar * m.k * m.k + 2.0 * nlev * m.k * m.N;
+    return nrhs >= 5 && m.td_rows.n > 0 && entries * cdiv(nrhs, 8) >= 2.2e7;
+}
+
+// Columns of a tile: the time of a wave of CTAs is 1, 1.07 and 1.6 for 16, 32 and 64
+// columns (27361 DoFs: 625, 685 and 996 us for 16 columns; 817 DoFs: 171, 183, 255)
+static int td_tile(const MeshData &m, int cols)
+{
+    const double cost[3] = {1.0, 1.07, 1.6};
+    int best = 0;
+    double tb = 0;
+    for (int i = 0; i < 3; ++i) {
+        const double t = cost[i] * std::max(1.0, (double)m.td_rows_item.n * cdiv(cols, 16 << i) / TD_SMS);
+        if (i == 0 || t < tb) {
+            best = i;
+            tb = t;
+        }
+    }
+    return 16 << best;
+}
+
+// workspace: the digits of 64 columns per leaf and per node, column keys and flags
+void apply_tensor_alloc(const MeshData &m, OpData &op)
+{
+    if (op.td_key.p) return;
+    const int node0 = m.nfar > 0 ? (1 << m.far_lmin) - 1 : m.kt.nnode;
+    op.td_x.alloc((size_t)m.kt.nleaf * ((m.max_leaf_size + 15) >> 4) * td_step(TD_COLS));
+    op.td_h.alloc((size_t)(m.kt.nnode - node0) * ((m.k + 15) >> 4) * td_step(TD_COLS));
+    op.td_key.alloc(3 * TD_COLS + 2);
+}
+
+// Y = A X for all columns, and the flag behind which the fixed-point kernels redo it
+const int *apply_tensor(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st)
+{
+    const bool far = m.nfar > 0;
+    const int k = m.k, nleaf = m.kt.nleaf, node0 = far ? (1 << m.far_lmin) - 1 : m.kt.nnode, nnodes = m.kt.nnode - node0;
+    TdP P{};
+    P.F = fa_far_view(m, op);
+    P.R = fa_near_view(m, op);
+    P.nrhs = nrhs;
+    P.nsl = (m.max_leaf_size + 15) >> 4;
+    P.nsn = (k + 15) >> 4;
+    P.node0 = node0;
+    P.nnodes = nnodes;
+    int *err = (int *)op.td_key.p + 3 * TD_COLS, *good = err + 1;
+    VFD_CUDA(cudaMemsetAsync(err, 0, 2 * sizeof(int), st));
+    P.err = err;
+    P.dx = op.td_x.p;
+    P.dh = op.td_h.p;
+    P.kx = op.td_key.p;
+    P.ko = op.td_key.p + 2 * TD_COLS;
+    for (int c0 = 0; c0 < nrhs; c0 += TD_COLS) {
+        const int cols = std::min(TD_COLS, nrhs - c0);
+        const int nc = td_tile(m, cols), nt = cdiv(cols, nc);
+        auto digits = [&](const double *v, size_t vld, size_t base, bool leaves, bool max, unsigned *key, unsigned char *out) {
+            TdVec V{};
+            V.v = v;
+            V.ld = vld;
+            V.base = base;
+            V.npiece = leaves ? nleaf : nnodes;
+            V.ns = leaves ? P.nsl : P.nsn;
+            V.len = k;
+            V.kb = leaves ? P.F.kb + P.F.fl : nullptr;
+            V.ke = leaves ? P.F.ke + P.F.fl : nullptr;
+            V.nrhs = nrhs;
+            V.c0 = c0;
+            V.nc = nc;
+            V.key = key;
+            V.out = out;
+            V.err = err;
+            const size_t tot = leaves ? (size_t)m.N : (size_t)nnodes * k;
+            if (max) k_td_max<<<dim3(std::max(1, std::min(cdiv((long long)tot, 1024), 32)), cols), 256, 0, st>>>(V);
+            k_td_digits<<<dim3(V.npiece, nt), 256, 0, st>>>(V);
+            VFD_CUDA(cudaGetLastError());
+        };
+        VFD_CUDA(cudaMemsetAsync(op.td_key.p, 0, 3 * TD_COLS * sizeof(unsigned), st));
+        P.c0 = c0;
+        digits(X, ld, 0, true, true, op.td_key.p, op.td_x.p);
+        if (far) {
+            const size_t hs = (size_t)m.kt.nnode * k;
+            launch_td<TD_PROJ>(nc, P, nleaf * cdiv(P.F.nlev * k, 128), nt, X, ld, op.P64.p, st);
+            launch_far_sum(m, op, c0, cols, st, nullptr);
+            digits(op.xhat.p, hs, (size_t)node0 * k, false, true, op.td_key.p + TD_COLS, op.td_h.p);
+            P.kh = op.td_key.p + TD_COLS;
+            P.items = m.td_couple_item.p;
+            P.bin = m.td_couple_bin.p;
+            P.rec = m.td_couple.p;
+            launch_td<TD_COUPLE>(nc, P, (int)m.td_couple_item.n, nt, X, ld, op.yhat.p, st);
+            digits(op.yhat.p, hs, (size_t)node0 * k, false, false, P.ko, op.td_h.p);
+            P.kh = P.ko;
+        }
+        P.items = m.td_rows_item.p;
+        P.bin = m.td_rows_bin.p;
+        P.rec = m.td_rows.p;
+        launch_td<TD_ROWS>(nc, P, (int)m.td_rows_item.n, nt, X, ld, Y, st);
+    }
+    k_td_good<<<1, 1, 0, st>>>(err, good);
+    VFD_CUDA(cudaGetLastError());
+    return good;
+}
+
+}  // namespace vfd

@@ -1075,7 +1075,7 @@ __global__ void __launch_bounds__(256) k_gh_rho_moments2(GMom P)
 // the basis differences f_1.. (f_0 is minus their sum) and the mapped reference
 // points xh, yh.  With P1 fields s(x) + s(y) and log kappa are linear in xh, yh, and
 // the barycentric sums of the sensitivities come from the sums of c, c xh, c yh.
-constexpr int GT_D = 0, GT_NU = 4, GT_CST = 5, GT_W = 6, GT_F = 7, GT_XY = 11, GT_SLOTS = 15;
+constexpr int GT_NU = 4, GT_CST = 5, GT_W = 6, GT_F = 7, GT_XY = 11, GT_SLOTS = 15;
 
 __global__ void k_gs_table(int ns, double sbar, const double *__restrict__ gx, const double *__restrict__ gw,
                            double *__restrict__ out)

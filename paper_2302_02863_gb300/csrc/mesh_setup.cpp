@@ -1149,6 +1149,7 @@ MeshData *build_mesh(int d, int64_t n_vert, const double *coords, int64_t n_cell
             m->mtab.upload(make_math_tables());
             setup_fixed(*m, qx, qw, meas, cdiam);
             build_fixed_bases(*m);
+            build_tensor_lists(*m);
         }
     } catch (...) {
         delete m;

@@ -114,6 +114,13 @@ struct NodeLoc {
 // ---------------------------------------------------------------------------
 // mesh handle: geometry-only data, built once per mesh
 // ---------------------------------------------------------------------------
+// a partner of a pair of leaves or nodes (apply_tensor.cu): its index and rows, offsets of
+// the two halves' entries (-1: none)
+struct TdRec {
+    int col, n;
+    long long off[2];
+};
+
 struct MeshData {
     int d = 2, M = 0, C = 0, N = 0;
     int nQ = 0, nQint = 0;
@@ -165,6 +172,10 @@ struct MeshData {
     bool fa_ok = false;
     DBuf<long long> fa_U;
     DBuf<int> fa_ue;
+    // partners of pairs of leaves and of nodes for the tensor-core apply (apply_tensor.cu)
+    DBuf<TdRec> td_rows, td_couple;
+    DBuf<int4> td_rows_item, td_couple_item;
+    DBuf<int> td_rows_bin, td_couple_bin;
     DBuf<double> E64;          // transfers E_c[beta][alpha] = l^parent_alpha(xi^c_beta), nnode x k x k
     int p_in = 0, k_in = 0;    // interpolation order / rank of the inner operator's far field (0: p, k)
     DBuf<double> kt_cheb_in, U_in64, E_in64;   // its Chebyshev nodes, leaf bases (N x k_in), transfers
@@ -266,10 +277,13 @@ struct OpData {
     DBuf<double> S64;                  // nfar * k * k
     DBuf<double> D64;                  // near entries
     // fixed-point copies for the FP64 apply (apply_fixed.cu): near panels with B + M added and an
-    // exponent per row, coupling blocks and an exponent per block; fa: built, every entry fits
+    // exponent per row, coupling blocks and an exponent per row node; fa: built, every entry fits
     bool fa = false;
     DBuf<long long> fa_D, fa_S;
     DBuf<int> fa_re, fa_se;
+    // digits of a vector's leaf and node pieces, column keys and flags (apply_tensor.cu)
+    DBuf<unsigned char> td_x, td_h;
+    DBuf<unsigned> td_key;
     DBuf<float> S32, D32, Ul32;        // FP32 copies (VFD_FP32)
     DBuf<unsigned short> Dtc;          // BF16 near panels pre-tiled for the TMA-fed tcgen05 kernel (first batched use)
     std::vector<int64_t> Dtc_off;      //   element offset of each leaf's image (nleaf + 1)
@@ -421,6 +435,8 @@ void launch_rho_near_fixed(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_selftest_math(const MeshData &m, int which, long long n, const double *x, double *out, cudaStream_t st);
 // apply_fixed.cu
 void build_fixed_bases(MeshData &m);
+// apply_tensor.cu
+void build_tensor_lists(MeshData &m);
 void build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t st);
 // apply.cu
 // partial sums of X . Y, written by the apply of one column where it can (n of them; part

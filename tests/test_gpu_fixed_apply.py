@@ -1,7 +1,8 @@
 """The fixed-point FP64 apply (vfd_apply) against the FP64 kernels, which
 vfd_apply_noalloc still runs, over the forms that change its launches: one to
-many columns (groups of 8, 4, 2, 1), odd ranks, ragged leaves, wide panels, deep
-trees, leading dimensions, and vectors that its formats do not hold.
+many columns (groups of 8, 4, 2, 1; digits on the tensor cores from a few hundred
+columns on for meshes this small), odd ranks, ragged leaves, wide panels, deep trees,
+leading dimensions, and vectors that its formats do not hold.
 """
 import pytest
 
@@ -19,6 +20,7 @@ MESHES = {
     "interval_long": lambda: synth.interval_mesh(2100),
     "disk": lambda: synth.disk_mesh(13, seed=3),
     "disk_mid": lambda: synth.disk_mesh(26, seed=4),
+    "square_fine": lambda: synth.square_mesh(72, jitter=0.2, seed=6),
     "square": lambda: synth.square_mesh(30, jitter=0.2, seed=5),
     "ball": lambda: synth.kuhn_ball_mesh(9),
 }
@@ -35,13 +37,13 @@ def _op(name, leaf, p, lam=0.75, **kw):
     ("interval", 16, 5, 0.75), ("interval", 64, 8, 0.75), ("interval_long", 2, 3, 0.75), ("disk", 64, 4, 0.75),
     ("disk", 11, 5, 0.75), ("disk", 7, 1, 0.75), ("disk_mid", 33, 7, 0.75), ("disk_mid", 64, 8, 0.75),
     ("disk_mid", 64, 4, 0.0), ("square", 40, 3, 0.75), ("square", 130, 6, 0.75), ("ball", 24, 3, 1.2),
-    ("ball", 64, 2, 0.75)])
+    ("ball", 64, 2, 0.75), ("square_fine", 60, 4, 0.75), ("square_fine", 28, 5, 0.75), ("square_fine", 13, 3, 0.75)])
 def test_fixed_point_apply_matches_fp64(name, leaf, p, lam):
     import torch
     mesh, op = _op(name, leaf, p, lam)
     n = mesh.n_dof
     g = torch.Generator("cuda").manual_seed(7)
-    for nrhs, ld in ((1, n), (1, n + 3), (2, n), (3, n + 1), (5, n), (8, n), (11, n + 5), (64, n)):
+    for nrhs, ld in ((1, n), (1, n + 3), (2, n), (3, n + 1), (5, n), (8, n), (11, n + 5), (64, n), (449, n + 1)):
         X = torch.randn(nrhs, ld, dtype=torch.float64, device="cuda", generator=g)
         X *= 10.0 ** torch.randint(-3, 4, (nrhs, 1), device="cuda", generator=g)   # columns of their own scale
         Y, R = torch.full_like(X, 7.0), torch.full_like(X, 7.0)
@@ -54,7 +56,7 @@ def test_fixed_point_apply_matches_fp64(name, leaf, p, lam):
 
 
 @pytest.mark.parametrize("name,leaf,p", [("disk", 20, 4), ("square", 64, 3), ("interval", 16, 5)])
-@pytest.mark.parametrize("nrhs", [1, 9])
+@pytest.mark.parametrize("nrhs", [1, 9, 1000])
 def test_fixed_point_apply_special_values(name, leaf, p, nrhs):
     import torch
     mesh, op = _op(name, leaf, p)
@@ -69,7 +71,8 @@ def test_fixed_point_apply_special_values(name, leaf, p, nrhs):
     for v, X in cases.items():
         Y, R = torch.empty_like(X), torch.empty_like(X)
         vfd.vfd_apply(op, X, Y)
-        vfd.vfd_apply_noalloc(op, X, R)
+        for r in range(0, nrhs, 8):
+            vfd.vfd_apply_noalloc(op, X[r:r + 8], R[r:r + 8])
         assert torch.equal(torch.isnan(Y), torch.isnan(R)), v
         inf = torch.isinf(R)
         assert torch.equal(torch.isinf(Y), inf) and torch.equal(Y[inf], R[inf]), v
