@@ -939,7 +939,15 @@ void apply_group(const MeshData &m, OpData &op, const double *X, double *Y, int 
         if (summed) launch_far_couple_sum(m, op, c0, cols, op.side, skip);
     }
     FaNear R = fa_near_view(m, op);
-    R.NR = 64;
+    // rows of a CTA: the whole leaf, or down to 16 rows where that leaves SMs idle, although each
+    // CTA rounds the columns again (the apply, 64 rows / this rule: 5 columns at 9025 DoFs and rank 16
+    // 106 / 73 us, 8 columns at 3997 DoFs and rank 64 235 / 116, 64 columns at 817 DoFs 128 / 83)
+    auto rows = [&](int ctas) {
+        int nr = 64;
+        while (nr > 16 && (long long)ctas * cdiv(m.max_leaf_size, nr) < 304) nr >>= 1;
+        return nr;
+    };
+    R.NR = rows(nleaf * ng);
     R.nrhs = nrhs;
     R.c0 = c0;
     const size_t shm = (size_t)m.max_panel_w * NC * 8;
