@@ -54,7 +54,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "H^2 stiffness matvec DOF*RHS/s and CG time-to-tolerance (assemble + solve step)"
 UNIT = "DOF*RHS/s"
-FP64_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12   # GB300: 2 FP64 FMA per clock per SM at 2.07 GHz
+FX_GEVALS = 163.0   # kernel evaluations in fixed point, 10^9/s with all SMs busy (measured)
 
 
 def _args():
@@ -336,52 +336,50 @@ def main():
         pass
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     if prec == vfd.VFD_FP64:
-        # FP64 FMA rate bounds this kernel on GB300 (1 FMA per 8 bytes of the
-        # streamed matrix > 1.25 TFLOP/s / 6.8 TB/s); nominal FP64 peak
-        roof = {"bound": "alu", "achieved": leaf_flops / t_leaf / 1e12, "peak": FP64_TFLOPS, "unit": "TFLOP/s",
-                "frac": leaf_flops / t_leaf / 1e12 / FP64_TFLOPS, "traffic": None,
-                "kernel": "k_near_csr<double,double> (near panels + B+M CSR rows)",
-                "peak_source": "152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz",
-                "hbm_frac": leaf_bytes / t_leaf / 1e9 / hbm}
+        # the FP64 apply runs on 61-bit integers, 8 bytes an entry: near panels and
+        # coupling blocks once, the bases twice (projection, expansion)
+        leaf_bytes = 8 * (info["near_entries"] + info["far_blocks"] * info["rank"] ** 2) + 2 * n * 8
+        roof = {"bound": "hbm", "achieved": leaf_bytes / t_apply / 1e9, "peak": hbm, "unit": "GB/s",
+                "frac": leaf_bytes / t_apply / 1e9 / hbm, "traffic": None,
+                "kernel": "vfd_apply, one column (k_fa_proj1, k_fa_couple1, k_fa_near1, k_fa_expand1; "
+                          "bytes of near panels and coupling blocks only)",
+                "peak_source": "MEASURED_PEAKS.json hbm_gbs"}
+        t_leaf = t_apply
     else:
         roof = {"bound": "hbm", "achieved": leaf_bytes / t_leaf / 1e9, "peak": hbm, "unit": "GB/s",
                 "frac": leaf_bytes / t_leaf / 1e9 / hbm, "traffic": None,
                 "kernel": "k_near_csr<float,float> (near panels + B+M CSR rows)", "peak_source": "MEASURED_PEAKS.json hbm_gbs"}
     roof["algorithmic_bytes"] = leaf_bytes
     roof["launch_us"] = t_leaf * 1e6
-    roof["traffic"] = _traffic_from_profile(args.workload, args.precision)
+    if prec != vfd.VFD_FP64:
+        roof["traffic"] = _traffic_from_profile(args.workload, args.precision)
     roof_apply = roof
-    # the assembly's two largest kernels: FP64-pipe bound (their DRAM traffic is
-    # negligible); throughput in kernel evaluations per second from the live
-    # phase timings (mean over the timed assemblies)
+    # the assembly's two largest kernels: bound by instruction issue (their DRAM
+    # traffic is negligible); throughput in kernel evaluations per second from the
+    # live phase timings (mean over the timed assemblies)
     asm_k = {}
-    for name, key, ev in (("k_singular2d", "singular", "sing_points"), ("k_near_build", "near", "near_point_pairs")):
+    for name, key, ev in (("k_singular2d_fx", "singular", "sing_points"), ("k_near_fx", "near", "near_point_pairs")):
         if info.get(ev) and ph.get(key):
-            asm_k[name] = {"bound": "alu (FP64 pipe)", "unit": "Geval/s", "evals": info[ev], "ms": round(ph[key], 3),
+            asm_k[name] = {"bound": "alu", "unit": "Geval/s", "evals": info[ev], "ms": round(ph[key], 3),
                            "achieved": info[ev] / (ph[key] / 1e3) / 1e9}
-    # the step's largest kernel (launch list share) is the near-block build: an
-    # FP64-ALU roofline in kernel evaluations per second, peak = the FP64 issue
-    # rate of the part (152 SMs x 2 FP64 instructions/clk x 2.07 GHz = 0.629e12/s,
-    # which the measured FMA rate matches) divided by the FP64 instructions of one
-    # evaluation as implemented (2D: r^2 4, exponent 3, table-driven log 11, exp
-    # 12 = 30; the leaf contractions come on top)
-    if prec == vfd.VFD_FP64 and "k_near_build" in asm_k:
-        peak_ev = FP64_TFLOPS / 2 * 1e12 / 30 / 1e9
-        nb = asm_k["k_near_build"]
-        roof = {"bound": "alu", "kernel": "k_near_build (dense inadmissible leaf blocks, Sec. 5.2)",
+    # the near-block build: kernel evaluations in 64-bit fixed point; peak = the rate
+    # of the evaluation alone with all SMs busy, measured (the leaf contractions come
+    # on top)
+    if prec == vfd.VFD_FP64 and "k_near_fx" in asm_k:
+        peak_ev = FX_GEVALS
+        nb = asm_k["k_near_fx"]
+        roof = {"bound": "alu", "kernel": "k_near_fx (dense inadmissible leaf blocks, Sec. 5.2)",
                 "achieved": nb["achieved"], "peak": peak_ev, "unit": "Geval/s", "frac": nb["achieved"] / peak_ev,
-                "traffic": _profile_value("k_near_build", args.workload, args.precision, "dram_bytes_per_launch"),
-                "fp64_pipe_active_ncu": _profile_value("k_near_build", args.workload, args.precision,
-                                                       "fp64_pipe_active"),
-                "evals_per_launch": nb["evals"], "fp64_inst_per_eval": 30, "launch_ms": nb["ms"],
-                "peak_source": "FP64 issue rate from unit counts and clock (0.629e12/s) / 30 FP64 instructions"}
+                "traffic": None, "evals_per_launch": nb["evals"], "launch_ms": nb["ms"],
+                "peak_source": "measured rate of the fixed-point kernel evaluation alone"}
 
-    # apply: far projections, node sums, coupling, row kernel, far expansion
-    apply_kernels = 5 if info["far_blocks"] > 0 else 1
+    # launches, from the structure (a list of the step's launches agrees): FP64 apply =
+    # projections, coupling, near rows, expansion; FP32 also the two node sums
     mean_it = statistics.mean(iters)
     replays = math.ceil(mean_it / 8)
-    per_solve = apply_kernels + 4 + replays * 8 * (apply_kernels + 3) + apply_kernels + 2
-    per_assemble = 4 + 1 + 2 + 2 + 1 + 1 + 1 + (4 if prec == vfd.VFD_FP32 else 0)
+    apply_kernels = (4 if prec == vfd.VFD_FP64 else 5) if info["far_blocks"] > 0 else 1
+    per_solve = 2 * apply_kernels + 6 + replays * 8 * (apply_kernels + 2)
+    per_assemble = 16 if prec == vfd.VFD_FP64 else 18
     gpu_launches = args.steps * (per_assemble + per_solve)
 
     # ---- the same step with rank 16 (p = 4): throughput and error of the lower order
@@ -1130,15 +1128,6 @@ def apply_mode(args, mesh, s, k, prm, prec, torch, vfd):
     print(json.dumps({"mode": "apply", "parts": args.parts, "precision": args.precision, "nrhs": args.nrhs,
                       "near_config": args.near_config,
                       "us_per_apply": 1000 * e0.elapsed_time(e1) / args.steps}), flush=True)
-
-
-def _profile_value(kernel, workload, precision, key):
-    """A figure from the committed ncu summary of a kernel (else null)."""
-    p = os.path.join(ROOT, "profiles", f"{kernel}_{workload}_{precision}.json")
-    try:
-        return json.load(open(p)).get(key)
-    except Exception:
-        return None
 
 
 def _traffic_from_profile(workload, precision):
