@@ -466,7 +466,8 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
                     return false;
                 }
                 int sm, sk;
-                p = matrix(I, sm, sk) + (mrow * sm + tt * sk);
+                p = matrix(I, sm, sk);   // sets the strides
+                p += mrow * sm + tt * sk;
                 left = I.off >= 0 && mrow < I.nrow ? I.n - tt : 0;
                 np = I.n;
                 steps = (np + 15) >> 4;
