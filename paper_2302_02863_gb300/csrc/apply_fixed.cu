@@ -1,21 +1,33 @@
-// The FP64 operator apply in fixed-point arithmetic.
+// The FP64 operator apply with its far field in fixed-point arithmetic.
 //
 // One FP64 multiply-add takes a warp 16 cycles of an SM on this part, so the
 // FP64 kernels of apply.cu are bound by the FP64 pipe at any number of columns
 // (98M multiply-adds a column at 27k DoFs and rank 64: 156 us at the pipe's
 // rate, against 115 us for the bytes of one pass over the operator).  Here the
-// operator's entries and the vectors are 61-bit integers, scaled by a power of
-// two per panel row (near entries, B + M added to them), coupling block or leaf
-// (flattened bases), and per gathered piece of a vector:
+// far field's entries (three quarters of the products) and its vectors are
+// 61-bit integers, scaled by a power of two per row of a coupling block or per
+// leaf (flattened bases), and per leaf's or node's piece of a vector:
 //   v = (hi 2^30 + lo) 2^(E - 60), |v| < 2^E, lo in [-2^29, 2^29), |hi| <= 2^30
 // and a product takes three 32 x 32 + 64 bit multiply-adds,
 //   hh += a.hi x.hi,   mid += a.hi x.lo + a.lo x.hi
 // (3 cycles a warp; a.lo x.lo is below the last place kept).  Every fourth product
-// the bits of hh and mid from 2^40 on move to 32-bit counters, so that nothing
-// overflows (2^60 a product).  Rounding to 2^-61 of the largest entry of a row or
-// block replaces rounding to 2^-53 of every partial sum: measured errors are at
-// the end of the comment.  The sums are exact in the integers, so their order
+// the bits of hh and mid from 2^40 on move to 32-bit counters (2^20 a full-scale
+// product, at most 64 levels x KMAX / 8 of them in a lane), so that nothing
+// overflows (2^60 a product).  The sums are exact in the integers, so their order
 // does not matter.
+//
+// What is rounded, and why it is no more than FP64 loses.  An entry of at least
+// 2^-8 of the largest of its row of a block has all 53 bits of its FP64 value in
+// 61; blocks with a smaller entry (fields that jump inside a box) stay FP64
+// (OpData::fa_hard).  The bases and the vectors are rounded to 2^-61 of the
+// largest entry of their leaf's or node's piece.  A basis row sums to its DoF's
+// weight (Lagrange functions sum to one) and a block's entries are positive and of one size, so
+// the largest entry of a piece is a part of every sum |U||S||U^T||x| that the
+// piece goes into, and 2^-61 of it is below the 2^-53 by which FP64 rounds that
+// sum.  Near rows have no such bound: their entries span up to 2^24 from the
+// diagonal to the panel's far end, and a row scale would cut the small ones.
+// They are FP64 products, which the FP64 pipe does beside the integer work of the
+// far chain.
 //
 // Non-finite or nearly denormal vectors (a piece whose largest entry is Inf,
 // NaN or below 2^-895) take plain FP64 sums over the FP64 operator instead, so
@@ -24,21 +36,24 @@
 //   1. k_fa_proj    per leaf: Ul^T x of every far level
 //   2. k_fa_couple  a warp per admissible block: S_e xhat, xhat summed over the
 //                   column node's leaves while it is gathered
-//   3. k_fa_near    per row, the near panel row (concurrently with 1-2)
+//   3. k_fa_near    per row, the near panel row and the B + M row, FP64
+//                   (concurrently with 1-2)
 //   4. k_fa_expand  Y[i] += sum over levels of Ul[i] . yhat, yhat summed over the
 //                   node's blocks while it is gathered
-// With 4 or more columns the two sums are kernels of their own (apply.cu): a
+// With 3 or more columns the two sums are kernels of their own (apply.cu): a
 // gather that repeats them for every block or leaf then costs more than it saves.
-// Columns go in groups of NC = 8 (4, 2, 1 for the remainder): an entry is loaded
-// once for NC products.
+// Columns of the far chain go in groups of NC = 8 (4, 2, 1 for the remainder): an
+// entry is loaded once for NC products.  The near rows take the remainder as it is:
+// a column that is not there would cost FP64 time.
 //
-// Measured at 27k DoFs, rank 64 (FP64 kernels first): one column 243 -> 150 us,
-// 64 columns 11.87 -> 5.27 ms.  Error against extended precision with the same
-// FP64 operator, relative 2-norm, normal x on 400 to 1000 DoFs: 1.2e-16 to
-// 1.3e-16 (FP64 kernels), 5.8e-17 to 7.8e-17 here; x = 1: 5.9e-16 to 3.3e-15 and
-// 1.5e-16 to 6.3e-16; x spread over six decades: 1.1e-16 to 1.4e-16 and 5.9e-17
-// to 7.8e-17.
+// Measured (FP64 kernels first): one column at 27k DoFs and rank 64 243 -> 170 us, at
+// 16129 DoFs and rank 16 74 -> 65.  Errors in units of |A||x| on 900 DoFs, against extended
+// precision with the FP64 operator's columns, FP64 kernels and here: normal x 6.4e-17
+// and 5.8e-17 rms, x over six decades 8.8e-17 and 9.7e-17, x falling by 14 decades across
+// the mesh 5.4e-17 and 5.0e-17, a Gaussian of width 0.1 1.0e-16 both.  A unit vector
+// gives the near entries as they are stored.
 #include <algorithm>
+#include <type_traits>
 
 #include "apply_common.cuh"
 #include "apply_fixed.cuh"
@@ -153,6 +168,7 @@ k_fa_couple(FaFar P, const double *__restrict__ part, const double *__restrict__
     double *raw = (double *)xs;
     const int node = P.fcol[e], l = 31 - __clz(node + 1), sh = P.L - l;
     const int leaf0 = ((node + 1) << sh) - (1 << P.L);
+    const bool hard = P.hard[e];
     unsigned key[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -179,8 +195,7 @@ k_fa_couple(FaFar P, const double *__restrict__ part, const double *__restrict__
     for (int c = 0; c < NC; ++c) slow |= fa_slow(key[c]);
     __syncwarp();
     const int2 *S = P.S + (size_t)e * k * P.kp;
-    const int es = P.se[e];
-    if (slow) {
+    if (slow || hard) {
         for (int a = lane; a < k; a += 32)
             for (int c = 0; c < NC && r0 + c < P.nrhs; ++c) {
                 double v = 0.0;
@@ -196,7 +211,7 @@ k_fa_couple(FaFar P, const double *__restrict__ part, const double *__restrict__
     // lanes over a; with k <= 16 the groups of ga lanes take every (32 / ga)-th row
     const int ga = k > 16 ? 32 : k > 8 ? 16 : 8, gb = 32 / ga, la = lane & (ga - 1), lb = lane / ga;
     for (int a0 = 0; a0 < k; a0 += ga) {
-        const int a = a0 + la;
+        const int a = a0 + la, es = a < k ? P.se[(size_t)e * k + a] : 0;
         double out[NC];
         if (a < k) {
             fa_column<NC>(S + a + (size_t)lb * P.kp, P.kp, max(0, k - lb), gb, xs + lb * NC, out);
@@ -220,51 +235,31 @@ k_fa_couple(FaFar P, const double *__restrict__ part, const double *__restrict__
 
 // ---------------------------------------------------------------------------
 // rows: sums over the entries of matrix rows, 8 lanes to a row and four rows to
-// a warp, x in shared memory: [j] for one column, else [pair of columns][j]
+// a warp, x in shared memory: [pair of columns][j]
 // ---------------------------------------------------------------------------
 template <int NC>
 __device__ __forceinline__ void fa_row(const int2 *__restrict__ row, int w, int l8, const int4 *xs, int ws, FaAcc *s)
 {
-    if (NC == 1) {
-        const int4 *r4 = (const int4 *)row, *x4 = xs;
-        const int nv = w >> 1;
-        int v = l8;
-#pragma unroll 2
-        for (; v + 8 < nv; v += 16) {
-            const int4 a = r4[v], b = r4[v + 8], x = x4[v], y = x4[v + 8];
-            s[0].mac(make_int2(a.x, a.y), make_int2(x.x, x.y));
-            s[0].mac(make_int2(a.z, a.w), make_int2(x.z, x.w));
-            s[0].mac(make_int2(b.x, b.y), make_int2(y.x, y.y));
-            s[0].mac(make_int2(b.z, b.w), make_int2(y.z, y.w));
-            s[0].carry();
-        }
-        if (v < nv) {
-            const int4 a = r4[v], x = x4[v];
-            s[0].mac(make_int2(a.x, a.y), make_int2(x.x, x.y));
-            s[0].mac(make_int2(a.z, a.w), make_int2(x.z, x.w));
-        }
-    } else {
-        auto term = [&](int2 a, int j) {
+    auto term = [&](int2 a, int j) {
 #pragma unroll
-            for (int p = 0; p < NC / 2; ++p) {
-                const int4 x = xs[(size_t)p * ws + j];
-                s[2 * p].mac(a, make_int2(x.x, x.y));
-                s[2 * p + 1].mac(a, make_int2(x.z, x.w));
-            }
-        };
-        int j = l8;
+        for (int p = 0; p < NC / 2; ++p) {
+            const int4 x = xs[(size_t)p * ws + j];
+            s[2 * p].mac(a, make_int2(x.x, x.y));
+            s[2 * p + 1].mac(a, make_int2(x.z, x.w));
+        }
+    };
+    int j = l8;
 #pragma unroll 1
-        for (; j + 24 < w; j += 32) {
-            int2 a[4];
+    for (; j + 24 < w; j += 32) {
+        int2 a[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) a[q] = row[j + 8 * q];
+        for (int q = 0; q < 4; ++q) a[q] = row[j + 8 * q];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) term(a[q], j + 8 * q);
+        for (int q = 0; q < 4; ++q) term(a[q], j + 8 * q);
 #pragma unroll
-            for (int c = 0; c < NC; ++c) s[c].carry();
-        }
-        for (; j < w; j += 8) term(row[j], j);
+        for (int c = 0; c < NC; ++c) s[c].carry();
     }
+    for (; j < w; j += 8) term(row[j], j);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         s[c].carry();
@@ -318,69 +313,96 @@ __device__ __forceinline__ int fa_slot(int j, int c, int ws)   // of column c's 
 }
 
 // ---------------------------------------------------------------------------
-// 3. near rows: CTA per (leaf, slice of NR rows, group of columns)
+// 3. near rows, FP64: CTA per (leaf, slice of NR rows, group of NC columns), 8 lanes to a
+// row; x in shared memory as [pair of columns][j].  Bound by the FP64 pipe (16 cycles of
+// an SM a warp and multiply-add), so that a group has no more columns than there are and
+// an entry is loaded once for all of them.  (The next four entries loaded ahead cost more
+// registers than they hide: 5 columns at 3721 DoFs 91 us instead of 76, 8 at 9025 202 / 165.)
 // ---------------------------------------------------------------------------
+// sum over the 8 lanes of a row; every lane ends with one column, returned, and its sum in s[0]
+template <int NC>
+__device__ __forceinline__ int fa_sum8(double *s, int l8)
+{
+    int n = NC, col = 0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = l8 & o;
+#pragma unroll
+            for (int q = 0; q < NC / 2; ++q)
+                if (q < n) {
+                    const double send = up ? s[q] : s[q + n], keep = up ? s[q + n] : s[q];
+                    s[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            col += up ? n : 0;
+        } else {
+            s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+        }
+    }
+    return col;
+}
+
 template <int NC>
 __global__ void __launch_bounds__(128) k_fa_near(FaNear P, const double *__restrict__ X, int64_t ld,
                                                  double *__restrict__ Y, const int *skip)
 {
     extern __shared__ __align__(16) unsigned char fa_sm[];
-    __shared__ unsigned key[NC];
     if (skip && *skip) return;
     const int lf = blockIdx.x, r0 = P.c0 + blockIdx.z * NC;
     const int b_leaf = P.kb[P.fl + lf], b = b_leaf + blockIdx.y * P.NR, e = min(P.ke[P.fl + lf], b + P.NR);
     if (b >= e) return;
     const int W = P.pw[lf];
     const int *gc = P.gcol + P.goff[lf];
-    double *raw = (double *)fa_sm;
-    if (threadIdx.x < NC) key[threadIdx.x] = 0;
-    __syncthreads();
+    const double *x0 = X + (size_t)r0 * ld;
+    constexpr int NP = NC > 4 ? 8 : NC > 2 ? 4 : 2;   // lanes of a row with a column
+    double *xs = (double *)fa_sm;
+#pragma unroll 4
+    for (int t = threadIdx.x; t < W; t += blockDim.x) {
+        const int j = gc[t];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        unsigned mk = 0;
-        const double *x = X + (size_t)(r0 + c) * ld;
-        for (int t = threadIdx.x; t < W; t += blockDim.x) {
-            const int j = gc[t];
-            const double v = j >= 0 && r0 + c < P.nrhs ? x[j] : 0.0;
-            raw[fa_slot<NC>(t, c, W)] = v;
-            mk = max(mk, fa_key(v));
-        }
-        mk = __reduce_max_sync(0xffffffffu, mk);
-        if ((threadIdx.x & 31) == 0) atomicMax(&key[c], mk);
+        for (int c = 0; c < ((NC + 1) & ~1); ++c)
+            xs[(c >> 1) * 2 * W + 2 * t + (c & 1)] = j >= 0 && c < NC ? x0[(size_t)c * ld + j] : 0.0;
     }
-    __syncthreads();
-    bool slow = false;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) slow |= fa_slow(key[c]);
-    if (!slow) fa_convert<NC>(fa_sm, W, key);
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l8 = lane & 7, nw = blockDim.x >> 5;
     for (int g0 = b + 4 * warp; g0 < e; g0 += 4 * nw) {
         const int i = g0 + (lane >> 3);
         const bool on = i < e;
-        const int2 *row = P.D + P.poff[lf] + (size_t)(i - b_leaf) * W;
-        if (!slow) {
-            FaAcc s[NC];
-            if (on) fa_row<NC>(row, W, l8, (const int4 *)fa_sm, W, s);
-            const int c = fa_sum8<NC>(s, l8), r = r0 + c;
-            if (on && (l8 & (8 / NC - 1)) == 0 && r < P.nrhs) {
-                double v = s[0].value() * fa_pow2(P.re[i] - 30) *
-                           fa_scale(key[c]);
-                if (!P.folded)
-                    for (int q = P.rowptr[i]; q < P.rowptr[i + 1]; ++q)
-                    v = fma(P.val[q], X[(size_t)r * ld + P.colidx[q]], v);
-                Y[(size_t)r * ld + i] = v;
+        double s[NP];
+#pragma unroll
+        for (int c = 0; c < NP; ++c) s[c] = 0.0;
+        if (on) {
+            const double *row = P.Dd + P.poff[lf] + (size_t)(i - b_leaf) * W + l8;
+            auto term = [&](double a, int j) {
+#pragma unroll
+                for (int p = 0; p < (NC + 1) / 2; ++p) {
+                    const double2 x = *(const double2 *)(xs + (size_t)p * 2 * W + 2 * j);
+                    s[2 * p] = fma(a, x.x, s[2 * p]);
+                    if (2 * p + 1 < NC) s[2 * p + 1] = fma(a, x.y, s[2 * p + 1]);
+                }
+            };
+            int j = l8;
+#pragma unroll 1
+            for (; j + 24 < W; j += 32) {
+                double a[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) a[q] = row[j - l8 + 8 * q];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) term(a[q], j + 8 * q);
             }
-        } else if (on) {
-            for (int c = l8; c < NC && r0 + c < P.nrhs; c += 8) {
-                double v = 0.0;
-                for (int j = 0; j < W; ++j)
-                    v = fma(P.Dd[(row - P.D) + j], raw[fa_slot<NC>(j, c, W)], v);
-                for (int q = P.rowptr[i]; q < P.rowptr[i + 1]; ++q)
-                    v = fma(P.val[q], X[(size_t)(r0 + c) * ld + P.colidx[q]], v);
-                Y[(size_t)(r0 + c) * ld + i] = v;
+#pragma unroll 1
+            for (; j < W; j += 8) term(row[j - l8], j);
+#pragma unroll 1
+            for (int q = P.rowptr[i] + l8; q < P.rowptr[i + 1]; q += 8) {
+                const double *xj = x0 + P.colidx[q];
+                const double v = P.val[q];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) s[c] = fma(v, xj[(size_t)c * ld], s[c]);
             }
         }
+        const int c = fa_sum8<NP>(s, l8);
+        if (on && (l8 & (8 / NP - 1)) == 0 && c < NC) Y[(size_t)(r0 + c) * ld + i] = s[0];
     }
 }
 
@@ -566,6 +588,9 @@ k_fa_couple1(FaFar P, const double *__restrict__ part, const double *__restrict_
     fa_batch(a, 0, n, load);
     int2 *xs = xs_[warp];
     double *raw = (double *)xs;
+    const bool hard = P.hard[e];
+    const short *se = P.se + (size_t)e * k + 2 * min(pr, np - 1);
+    const int es0 = se[0], es1 = 2 * min(pr, np - 1) + 1 < k ? se[1] : 0;
     const int node = P.fcol[e], l = 31 - __clz(node + 1), sh = P.L - l, leaf0 = ((node + 1) << sh) - (1 << P.L);
     unsigned ky = 0;
     for (int b = lane; b < k; b += 32) {
@@ -583,9 +608,10 @@ k_fa_couple1(FaFar P, const double *__restrict__ part, const double *__restrict_
     ky = __reduce_max_sync(0xffffffffu, ky);
     __syncwarp();
     double *out = ye + (size_t)e * k;
-    if (fa_slow(ky)) {
+    if (fa_slow(ky) || hard) {
         for (int al = lane; al < k; al += 32) {
             double v = 0.0;
+#pragma unroll 8
             for (int b = 0; b < k; ++b) v = fma(P.Sd[((size_t)e * k + b) * k + al], raw[b], v);
             out[al] = v;
         }
@@ -609,9 +635,9 @@ k_fa_couple1(FaFar P, const double *__restrict__ part, const double *__restrict_
         v1 += __shfl_xor_sync(0xffffffffu, v1, o);
     }
     if (lb == 0 && pr < np) {
-        const double sc = fa_pow2(P.se[e] - 30), sx = fa_scale(ky);
-        out[2 * pr] = v0 * sc * sx;
-        if (2 * pr + 1 < k) out[2 * pr + 1] = v1 * sc * sx;
+        const double sx = fa_scale(ky);
+        out[2 * pr] = v0 * fa_pow2(es0 - 30) * sx;
+        if (2 * pr + 1 < k) out[2 * pr + 1] = v1 * fa_pow2(es1 - 30) * sx;
     }
 }
 
@@ -640,12 +666,14 @@ __device__ __forceinline__ void fa_dot(double v, double *dot)
     if (threadIdx.x == 0) dot[blockIdx.x * gridDim.y + blockIdx.y] = (sh[0] + sh[1]) + (sh[2] + sh[3]);
 }
 
-// 16 rows a CTA, 4 a warp, 8 lanes a row; dot: see fa_dot, or null
-__global__ void __launch_bounds__(128)
+// 16 rows a CTA, 4 a warp, 8 lanes a row, FP64; dot: see fa_dot, or null.  What bounds it is
+// the FP64 pipe (26M multiply-adds at 27k DoFs: 42 us at its rate), so batches of four loads
+// and more CTAs: one column at 16129 DoFs and rank 16 / at 27k and rank 64, batches of eight
+// 73 / 181 us, of four and at least 8 CTAs an SM 66 / 171, of two and 16 CTAs 71 / 171.
+__global__ void __launch_bounds__(128, 8)
 k_fa_near1(FaNear P, const double *__restrict__ X, double *__restrict__ Y, double *__restrict__ dot, const int *skip)
 {
     extern __shared__ __align__(16) unsigned char fa_sm[];
-    __shared__ unsigned key;
     if (skip && *skip) return;
     const int lf = blockIdx.x, b_leaf = P.kb[P.fl + lf], b = b_leaf + blockIdx.y * 16, e = min(P.ke[P.fl + lf], b + 16);
     if (b >= e) {
@@ -653,47 +681,51 @@ k_fa_near1(FaNear P, const double *__restrict__ X, double *__restrict__ Y, doubl
         return;
     }
     const int W = P.pw[lf], lane = threadIdx.x & 31, l8 = lane & 7, i = b + 4 * (threadIdx.x >> 5) + (lane >> 3);
-    const size_t ro = P.poff[lf] + (size_t)(min(i, e - 1) - b_leaf) * W;
-    const int4 *row = (const int4 *)(P.D + ro) + l8;
+    const double2 *row = (const double2 *)(P.Dd + P.poff[lf] + (size_t)(min(i, e - 1) - b_leaf) * W);
     const int nv = W >> 1, n = (nv + 7) >> 3;
-    auto load = [&](int t) { return l8 + 8 * t < nv ? fa_ld(row + 8 * t) : make_int4(0, 0, 0, 0); };
-    int4 a[FA_B];
-    fa_batch(a, 0, n, load);
+    auto fill = [&](double2 *a, int t0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int v = l8 + 8 * (t0 + q);
+            a[q] = v < nv ? __ldcs(row + v) : make_double2(0.0, 0.0);
+        }
+    };
+    double2 a[4];
+    fill(a, 0);
     const int *gc = P.gcol + P.goff[lf];
-    double *raw = (double *)fa_sm;
-    if (threadIdx.x == 0) key = 0;
-    __syncthreads();
-    unsigned mk = 0, ky;
+    double *xs = (double *)fa_sm;
 #pragma unroll 4
     for (int t = threadIdx.x; t < W; t += blockDim.x) {
         const int j = gc[t];
-        const double v = j >= 0 ? X[j] : 0.0;
-        raw[t] = v;
-        mk = max(mk, fa_key(v));
+        xs[t] = j >= 0 ? X[j] : 0.0;
     }
-    const bool slow = fa_piece(fa_sm, W, mk, &key, ky);
-    FaAcc s;
-    if (!slow)
-        fa_pipe<2>(a, n, load,
-                [&](int4 m, int t) {
-                    const int4 x = ((const int4 *)fa_sm)[min(l8 + 8 * t, nv - 1)];
-                    s.mac(make_int2(m.x, m.y), make_int2(x.x, x.y));
-                    s.mac(make_int2(m.z, m.w), make_int2(x.z, x.w));
-                },
-                [&] { s.carry(); });
-    s.fold();
-    fa_sum8<1>(&s, l8);
+    double bm = 0.0, s0 = 0.0, s1 = 0.0;
+    if (i < e)
+        for (int q = P.rowptr[i] + l8; q < P.rowptr[i + 1]; q += 8) bm = fma(P.val[q], X[P.colidx[q]], bm);
+    __syncthreads();
+    const double2 *x2 = (const double2 *)xs;
+#pragma unroll 1
+    for (int t0 = 0; t0 < n; t0 += 4) {
+        double2 next[4];
+        fill(next, t0 + 4);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (t0 + q >= n) break;   // the same for the CTA: a product of zeros would take its FP64 time
+            const int v = l8 + 8 * (t0 + q);
+            const double2 x = v < nv ? x2[v] : make_double2(0.0, 0.0);   // (an Inf times the zero entry past the end)
+            s0 = fma(a[q].x, x.x, s0);
+            s1 = fma(a[q].y, x.y, s1);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] = next[q];
+    }
+    // B + M last: the diagonal's product is the largest term of a row
+    s0 = (s0 + s1) + bm;
+    fa_sum8<1>(&s0, l8);
     double xy = 0.0;
     if (i < e && !l8) {
-        double v = s.value() * fa_pow2(P.re[i] - 30) * fa_scale(ky);
-        if (slow) {
-            v = 0.0;
-            for (int j = 0; j < W; ++j) v = fma(P.Dd[ro + j], raw[j], v);
-        }
-        if (slow || !P.folded)
-            for (int q = P.rowptr[i]; q < P.rowptr[i + 1]; ++q) v = fma(P.val[q], X[P.colidx[q]], v);
-        Y[i] = v;
-        if (dot) xy = X[i] * v;
+        Y[i] = s0;
+        if (dot) xy = X[i] * s0;
     }
     if (dot) fa_dot(xy, dot);
 }
@@ -767,12 +799,15 @@ k_fa_expand1(FaFar P, const double *__restrict__ ye, const double *__restrict__ 
 // ---------------------------------------------------------------------------
 // the operands
 // ---------------------------------------------------------------------------
+// whether a piece with this largest key is in the format's range
+__device__ __forceinline__ bool fa_fits(unsigned key) { return !key || (key >= 200u && key <= 1900u); }
+
 // largest exponent key of n values (warp), as the exponent E with |v| < 2^E;
 // flags what the format cannot hold
 __device__ __forceinline__ int fa_exponent(unsigned key, int *err)
 {
     key = __reduce_max_sync(0xffffffffu, key);
-    if (key == 0x7ffu || (key && key < 200u) || key > 1900u) {
+    if (!fa_fits(key)) {
         if ((threadIdx.x & 31) == 0) atomicOr(err, 4);
         return 0;
     }
@@ -805,34 +840,48 @@ __global__ void k_fa_build_near(int N, int fl, const int *__restrict__ vleaf, co
     if (lane == 0) re[i] = E;
 }
 
-// coupling blocks, a CTA per row node: one exponent for its blocks, so that their sums add
-// up as integers; rows padded to an even length
+// coupling blocks, a CTA per row node, rows padded to an even length.  An exponent per row
+// of a block; sn, the largest of the node's blocks, and sh = sn - se align the blocks of a
+// node where their digits are summed (apply_tensor.cu).  Entries down to 2^-8 of their
+// row's largest keep all their bits; a block with a smaller one is marked hard.
 __global__ void __launch_bounds__(256)
 k_fa_build_S(const int *__restrict__ fptr, int k, int kp, const double *__restrict__ S, int2 *__restrict__ out,
-             int *__restrict__ se, int *err)
+             short *__restrict__ se, short *__restrict__ sn, unsigned char *__restrict__ sh,
+             unsigned char *__restrict__ hard, int *err)
 {
-    __shared__ unsigned key;
-    __shared__ int E;
-    const int e0 = fptr[blockIdx.x], ne = fptr[blockIdx.x + 1] - e0;
-    if (ne == 0) return;
-    const double *in = S + (size_t)e0 * k * k;
-    int2 *o = out + (size_t)e0 * k * kp;
-    if (threadIdx.x == 0) key = 0;
+    constexpr int NONE = -32768;
+    __shared__ int top[KMAX];
+    const int node = blockIdx.x, e0 = fptr[node], ne = fptr[node + 1] - e0;
+    if (threadIdx.x < k) top[threadIdx.x] = NONE;
+    for (int e = threadIdx.x; e < ne; e += 256) hard[e0 + e] = 0;
     __syncthreads();
-    unsigned mk = 0;
-    for (int j = threadIdx.x; j < ne * k * k; j += 256) mk = max(mk, fa_key(in[j]));
-    atomicMax(&key, mk);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        const int e = fa_exponent(key, err);
-        if (threadIdx.x == 0) E = e;
+    for (int t = threadIdx.x; t < ne * k; t += 256) {
+        const int e = t / k, a = t - e * k;
+        const double *in = S + (size_t)(e0 + e) * k * k + a;
+        unsigned key = 0, least = 0x7ffu;
+        for (int b = 0; b < k; ++b) {
+            const unsigned q = fa_key(in[(size_t)b * k]);
+            key = max(key, q);
+            if (q) least = min(least, q);
+        }
+        if (!fa_fits(key)) atomicOr(err, 4);
+        if (key > least + 7) hard[e0 + e] = 1;
+        const int E = (int)key - 1022;
+        if (key) atomicMax(&top[a], E);
+        se[(size_t)(e0 + e) * k + a] = (short)(key ? E : NONE);
+        int2 *o = out + (size_t)(e0 + e) * k * kp + a;
+        for (int b = 0; b < k; ++b) o[(size_t)b * kp] = fa_split(fa_round(in[(size_t)b * k], (int)key));
+        if (a == k - 1 && kp > k)
+            for (int b = 0; b < k; ++b) o[(size_t)b * kp + 1] = make_int2(0, 0);
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < ne * k * kp; j += 256) {
-        const int b = j / kp, a = j - b * kp;
-        o[j] = a < k ? fa_split(fa_round(in[(size_t)b * k + a], E + 1022)) : make_int2(0, 0);
+    for (int t = threadIdx.x; t < ne * k; t += 256) {   // the entries that this thread wrote
+        const size_t i = (size_t)e0 * k + t;
+        const int a = t % k, E = se[i];
+        if (E == NONE) se[i] = (short)(top[a] == NONE ? 0 : top[a]);   // a row of zeros
+        sh[i] = (unsigned char)(E == NONE ? 0 : min(top[a] - E, 63));
     }
-    for (int e = threadIdx.x; e < ne; e += 256) se[e0 + e] = E;
+    if (threadIdx.x < k) sn[(size_t)node * k + threadIdx.x] = (short)(top[threadIdx.x] == NONE ? 0 : top[threadIdx.x]);
 }
 
 // flattened bases, CTA per leaf: [level][N][k] -> [N][level k], rows padded to an even length
@@ -900,83 +949,119 @@ void build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t 
     if (m.nfar) {
         const int kp = (m.k + 1) & ~1;
         op.fa_S.alloc((size_t)m.nfar * m.k * kp);
-        op.fa_se.alloc(m.nfar);
-        k_fa_build_S<<<m.kt.nnode, 256, 0, st>>>(m.far_ptr.p, m.k, kp, op.S64.p, (int2 *)op.fa_S.p, op.fa_se.p, err);
+        op.fa_se.alloc((size_t)m.nfar * m.k);
+        op.fa_sh.alloc((size_t)m.nfar * m.k);
+        op.fa_hard.alloc(m.nfar);
+        op.fa_sn.alloc((size_t)m.kt.nnode * m.k);
+        k_fa_build_S<<<m.kt.nnode, 256, 0, st>>>(m.far_ptr.p, m.k, kp, op.S64.p, (int2 *)op.fa_S.p, op.fa_se.p, op.fa_sn.p,
+                                                 op.fa_sh.p, op.fa_hard.p, err);
     }
     VFD_CUDA(cudaGetLastError());
 }
 
 namespace {
 
-// one launch of every kernel for ng groups of NC columns from column c0
-template <int NC>
-void apply_group(const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int nrhs, int64_t ld,
-                 bool summed, cudaStream_t st, const int *skip, ApplyDot *dot)
+// rows of a CTA: the whole leaf, or down to 16 rows where that leaves SMs idle, although each
+// CTA gathers the columns again (the apply, 64 rows / this rule: 5 columns at 9025 DoFs and rank 16
+// 106 / 73 us, 8 columns at 3997 DoFs and rank 64 235 / 116, 64 columns at 817 DoFs 128 / 83)
+int rows_of(const MeshData &m, int ctas)
 {
-    const int k = m.k, nleaf = m.kt.nleaf, nnode = m.kt.nnode;
-    const bool far = m.nfar > 0;
+    int nr = 64;
+    while (nr > 16 && (long long)ctas * cdiv(m.max_leaf_size, nr) < 304) nr >>= 1;
+    return nr;
+}
+
+template <class K>
+void allow_shared(K kernel, size_t shm)
+{
+    VFD_REQUIRE(shm <= 227 * 1024, VFD_EUNSUPPORTED,
+                "apply: a near panel is wider than shared memory holds (use a low-rank operator, lambda > 0)");
+    if (shm > 47 * 1024)
+        VFD_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+}
+
+// the far field's kernels up to the expansion, on the side stream, for ng groups of NC columns from column c0
+template <int NC>
+void far_group(const MeshData &m, OpData &op, const double *X, int c0, int ng, int nrhs, int64_t ld, bool summed,
+               const int *skip)
+{
+    const int k = m.k, nleaf = m.kt.nleaf;
     FaFar P = fa_far_view(m, op);
     P.nrhs = nrhs;
     P.c0 = c0;
     const int w = P.nlev * k, cols = std::min(nrhs - c0, ng * NC);
     // one column: the kernels get its own pieces
-    const size_t ps = (size_t)P.nlev * nleaf * k, hs = (size_t)nnode * k, ys = (size_t)m.nfar * k;
-    const double *X1 = X + (size_t)c0 * ld;
-    double *Y1 = Y + (size_t)c0 * ld;
-    if (far) {
-        VFD_CUDA(cudaEventRecord(op.ev_fork, st));
-        VFD_CUDA(cudaStreamWaitEvent(op.side, op.ev_fork, 0));
-        const size_t shp = (size_t)m.max_leaf_size * NC * 8;
-        if (NC == 1) k_fa_proj1<<<dim3(nleaf, cdiv(w, 256)), 128, shp, op.side>>>(P, X1, op.P64.p + c0 * ps, skip);
-        else k_fa_proj<NC><<<dim3(nleaf, cdiv(w, 128), ng), 128, shp, op.side>>>(P, X, ld, op.P64.p, skip);
-        if (summed) launch_far_sum(m, op, c0, cols, op.side, skip);
-        if (NC == 1)
-            k_fa_couple1<<<cdiv(m.nfar, FC_WARPS), 32 * FC_WARPS, 0, op.side>>>(
-                P, op.P64.p + c0 * ps, summed ? op.xhat.p + c0 * hs : nullptr, op.ye64.p + c0 * ys, skip);
-        else
-            k_fa_couple<NC><<<dim3(cdiv(m.nfar, FC_WARPS), ng), 32 * FC_WARPS, 0, op.side>>>(
-                P, op.P64.p, summed ? op.xhat.p : nullptr, op.ye64.p, skip);
-        if (summed) launch_far_couple_sum(m, op, c0, cols, op.side, skip);
-    }
-    FaNear R = fa_near_view(m, op);
-    // rows of a CTA: the whole leaf, or down to 16 rows where that leaves SMs idle, although each
-    // CTA rounds the columns again (the apply, 64 rows / this rule: 5 columns at 9025 DoFs and rank 16
-    // 106 / 73 us, 8 columns at 3997 DoFs and rank 64 235 / 116, 64 columns at 817 DoFs 128 / 83)
-    auto rows = [&](int ctas) {
-        int nr = 64;
-        while (nr > 16 && (long long)ctas * cdiv(m.max_leaf_size, nr) < 304) nr >>= 1;
-        return nr;
-    };
-    R.NR = rows(nleaf * ng);
-    R.nrhs = nrhs;
-    R.c0 = c0;
-    const size_t shm = (size_t)m.max_panel_w * NC * 8;
-    VFD_REQUIRE(shm <= 227 * 1024, VFD_EUNSUPPORTED,
-                "apply: a near panel is wider than shared memory holds (use a low-rank operator, lambda > 0)");
-    if (NC == 1) {
-        if (shm > 47 * 1024)
-            VFD_CUDA(cudaFuncSetAttribute(k_fa_near1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-        k_fa_near1<<<dim3(nleaf, cdiv(m.max_leaf_size, 16)), 128, shm, st>>>(R, X1, Y1, dot && !far ? dot->part : nullptr, skip);
+    const size_t ps = (size_t)P.nlev * nleaf * k, hs = (size_t)m.kt.nnode * k, ys = (size_t)m.nfar * k;
+    const size_t shp = (size_t)m.max_leaf_size * NC * 8;
+    if constexpr (NC == 1)
+        k_fa_proj1<<<dim3(nleaf, cdiv(w, 256)), 128, shp, op.side>>>(P, X + (size_t)c0 * ld, op.P64.p + c0 * ps, skip);
+    else
+        k_fa_proj<NC><<<dim3(nleaf, cdiv(w, 128), ng), 128, shp, op.side>>>(P, X, ld, op.P64.p, skip);
+    if (summed) launch_far_sum(m, op, c0, cols, op.side, skip);
+    if constexpr (NC == 1)
+        k_fa_couple1<<<cdiv(m.nfar, FC_WARPS), 32 * FC_WARPS, 0, op.side>>>(
+            P, op.P64.p + c0 * ps, summed ? op.xhat.p + c0 * hs : nullptr, op.ye64.p + c0 * ys, skip);
+    else
+        k_fa_couple<NC><<<dim3(cdiv(m.nfar, FC_WARPS), ng), 32 * FC_WARPS, 0, op.side>>>(
+            P, op.P64.p, summed ? op.xhat.p : nullptr, op.ye64.p, skip);
+    if (summed) launch_far_couple_sum(m, op, c0, cols, op.side, skip);
+    VFD_CUDA(cudaGetLastError());
+}
+
+template <int NC>
+void expand_group(const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int nrhs, int64_t ld,
+                  bool summed, cudaStream_t st, const int *skip, ApplyDot *dot)
+{
+    FaFar P = fa_far_view(m, op);
+    P.nrhs = nrhs;
+    P.c0 = c0;
+    const size_t hs = (size_t)m.kt.nnode * m.k, ys = (size_t)m.nfar * m.k, shm = (size_t)P.wp * NC * 8;
+    if constexpr (NC == 1) {
+        k_fa_expand1<<<dim3(m.kt.nleaf, cdiv(m.max_leaf_size, 16)), 128, shm, st>>>(
+            P, op.ye64.p + c0 * ys, summed ? op.yhat.p + c0 * hs : nullptr, Y + (size_t)c0 * ld, X + (size_t)c0 * ld,
+            dot ? dot->part : nullptr, skip);
     } else {
-        if (shm > 47 * 1024)
-            VFD_CUDA(cudaFuncSetAttribute(k_fa_near<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-        k_fa_near<NC><<<dim3(nleaf, cdiv(m.max_leaf_size, R.NR), ng), 128, shm, st>>>(R, X, ld, Y, skip);
-    }
-    if (far) {
-        VFD_CUDA(cudaEventRecord(op.ev_join, op.side));
-        VFD_CUDA(cudaStreamWaitEvent(st, op.ev_join, 0));
-        const size_t she = (size_t)P.wp * NC * 8;
-        if (NC == 1) {
-            k_fa_expand1<<<dim3(nleaf, cdiv(m.max_leaf_size, 16)), 128, she, st>>>(
-                P, op.ye64.p + c0 * ys, summed ? op.yhat.p + c0 * hs : nullptr, Y1, X1, dot ? dot->part : nullptr, skip);
-        } else {
-            if (she > 47 * 1024)
-                VFD_CUDA(cudaFuncSetAttribute(k_fa_expand<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)she));
-            k_fa_expand<NC><<<dim3(nleaf, cdiv(m.max_leaf_size, R.NR), ng), 128, she, st>>>(
-                P, R.NR, op.ye64.p, summed ? op.yhat.p : nullptr, Y, ld, skip);
-        }
+        allow_shared(k_fa_expand<NC>, shm);
+        const int nr = rows_of(m, m.kt.nleaf * ng);
+        k_fa_expand<NC><<<dim3(m.kt.nleaf, cdiv(m.max_leaf_size, nr), ng), 128, shm, st>>>(
+            P, nr, op.ye64.p, summed ? op.yhat.p : nullptr, Y, ld, skip);
     }
     VFD_CUDA(cudaGetLastError());
+}
+
+template <int NC>
+void near_group(const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int64_t ld, cudaStream_t st,
+                const int *skip, double *dot)
+{
+    FaNear R = fa_near_view(m, op);
+    R.c0 = c0;
+    const size_t shm = (size_t)m.max_panel_w * (NC == 1 ? 1 : (NC + 1) & ~1) * 8;
+    if constexpr (NC == 1) {
+        allow_shared(k_fa_near1, shm);
+        k_fa_near1<<<dim3(m.kt.nleaf, cdiv(m.max_leaf_size, 16)), 128, shm, st>>>(R, X + (size_t)c0 * ld,
+                                                                                 Y + (size_t)c0 * ld, dot, skip);
+    } else {
+        allow_shared(k_fa_near<NC>, shm);
+        R.NR = rows_of(m, m.kt.nleaf * ng);
+        k_fa_near<NC><<<dim3(m.kt.nleaf, cdiv(m.max_leaf_size, R.NR), ng), 128, shm, st>>>(R, X, ld, Y, skip);
+    }
+    VFD_CUDA(cudaGetLastError());
+}
+
+// f(NC) with the number of columns of a group as a constant, 1 .. 8
+template <class F>
+void with_columns(int n, F f)
+{
+    switch (n) {
+    case 1: f(std::integral_constant<int, 1>()); break;
+    case 2: f(std::integral_constant<int, 2>()); break;
+    case 3: f(std::integral_constant<int, 3>()); break;
+    case 4: f(std::integral_constant<int, 4>()); break;
+    case 5: f(std::integral_constant<int, 5>()); break;
+    case 6: f(std::integral_constant<int, 6>()); break;
+    case 7: f(std::integral_constant<int, 7>()); break;
+    default: f(std::integral_constant<int, 8>());
+    }
 }
 
 }  // namespace
@@ -989,24 +1074,47 @@ void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int 
     if (dot && !dot->n) dot = nullptr;
     // many columns: on the tensor cores; what follows is then a fallback behind a flag
     if (!skip && !dot && apply_tensor_fits(m, nrhs)) skip = apply_tensor(m, op, X, Y, nrhs, ld, st);
-    // the node sums inside the gathers pay for few columns and short spans
-    const bool summed = nrhs >= 4 || m.kt.L - m.far_lmin > 7;
-    // widest group whose panel piece leaves room for two CTAs an SM
+    // the node sums inside the gathers pay for few columns and short spans (3 columns, sums inside /
+    // of their own: 27361 DoFs 432 / 395 us, 16129 182 / 171, 3721 61 / 59; 2 columns at 10267 97 / 125)
+    const bool summed = nrhs >= 3 || m.kt.L - m.far_lmin > 7, far = m.nfar > 0;
+    // far groups: of 8, the remainder in one group of the next power of two
+    auto far_groups = [&](auto f) {
+        int c0 = 0;
+        auto go = [&](int n, int ng) {
+            with_columns(n, [&](auto NC) {
+                if constexpr ((NC & (NC - 1)) == 0) f(NC, c0, ng);
+            });
+            c0 += n * ng;
+        };
+        if (nrhs / 8) go(8, nrhs / 8);
+        if (c0 < nrhs) {
+            int r = 1;
+            while (r < nrhs - c0) r <<= 1;
+            go(r, 1);
+        }
+    };
+    if (far) {
+        VFD_CUDA(cudaEventRecord(op.ev_fork, st));
+        VFD_CUDA(cudaStreamWaitEvent(op.side, op.ev_fork, 0));
+        far_groups([&](auto NC, int c0, int ng) { far_group<NC>(m, op, X, c0, ng, nrhs, ld, summed, skip); });
+    }
+    // near groups: the widest whose panel piece leaves room for two CTAs an SM
     int nc = 8;
     while (nc > 1 && (size_t)m.max_panel_w * nc * 8 > 100 * 1024) nc >>= 1;
-    int c0 = 0;
-    auto go = [&](int NC, int ng) {
-        if (NC == 8) apply_group<8>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip, dot);
-        else if (NC == 4) apply_group<4>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip, dot);
-        else if (NC == 2) apply_group<2>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip, dot);
-        else apply_group<1>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip, dot);
-        c0 += NC * ng;
+    auto near = [&](int n, int c0, int ng) {
+        with_columns(n, [&](auto NC) {
+            near_group<NC>(m, op, X, Y, c0, ng, ld, st, skip, dot && !far ? dot->part : nullptr);
+        });
     };
-    if (nrhs / nc) go(nc, nrhs / nc);
-    while (c0 < nrhs) {   // the remainder in one group of the next size
-        int r = 1;
-        while (r < std::min(nc, nrhs - c0)) r <<= 1;
-        go(r, 1);
+    if (nc == 1)
+        for (int c = 0; c < nrhs; ++c) near(1, c, 1);
+    else if (nrhs / nc)
+        near(nc, 0, nrhs / nc);
+    if (nc > 1 && nrhs % nc) near(nrhs % nc, nrhs / nc * nc, 1);
+    if (far) {
+        VFD_CUDA(cudaEventRecord(op.ev_join, op.side));
+        VFD_CUDA(cudaStreamWaitEvent(st, op.ev_join, 0));
+        far_groups([&](auto NC, int c0, int ng) { expand_group<NC>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip, dot); });
     }
 }
 

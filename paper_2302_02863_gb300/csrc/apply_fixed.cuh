@@ -70,7 +70,9 @@ struct FaFar {
     int kp, wp;   // row strides of a coupling block and of the bases (even: 16-byte rows)
     const int *kb, *ke, *fptr, *fcol;
     const int2 *U, *S;
-    const int *ue, *se;
+    const int *ue;
+    const short *se, *sn;    // exponents: of a block's row, the largest of a node's row
+    const unsigned char *hard, *sh;   // per block: stays FP64; per block's row: sn - se
     const double *Ud, *Sd;   // FP64: [level][N][k], blocks
     int N;
 };
@@ -108,6 +110,9 @@ inline FaFar fa_far_view(const MeshData &m, const OpData &op)
     P.S = (const int2 *)op.fa_S.p;
     P.ue = m.fa_ue.p;
     P.se = op.fa_se.p;
+    P.sn = op.fa_sn.p;
+    P.hard = op.fa_hard.p;
+    P.sh = op.fa_sh.p;
     P.Ud = m.Ul64.p;
     P.Sd = op.S64.p;
     P.N = m.N;

@@ -375,7 +375,7 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
                 const int node = P.node0 + 2 * item + ohalf;
                 on = node < P.F.nnode && om < k;
                 ri = node * k + om;
-                if (on && P.F.fptr[node] < P.F.fptr[node + 1]) e = P.F.se[P.F.fptr[node]];
+                if (on) e = P.F.sn[ri];
                 os = (size_t)P.F.nnode * k;
             }
             const unsigned *key = skey + oc + (MODE == TD_PROJ || (MODE == TD_ROWS && code == 2) ? 0 : NC);
@@ -451,12 +451,14 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
             const bool far = MODE == TD_ROWS && J.q >= J.q1;
             sm = MODE == TD_ROWS ? (far ? P.F.wp : J.W) : 1;
             sk = MODE == TD_ROWS ? 1 : (MODE == TD_COUPLE ? P.F.kp : P.F.wp);
-            return (MODE == TD_COUPLE ? P.F.S : (MODE == TD_PROJ || far ? P.F.U : P.R.D)) + J.off;
+            if (MODE == TD_COUPLE) return P.F.S + J.off * (k * sk);   // off: the block
+            return (MODE == TD_PROJ || far ? P.F.U : P.R.D) + J.off;
         };
         // copies the entries of the next step to the lane's place, and puts its code to hist
         int2 *const raw = (int2 *)(td_sm + TD_NST * STAGE) + warp * 128 + lane;
         const int2 *p = nullptr;
         int left = 0, steps = 0, np = 0, end = 0, pulled = 0;   // of the piece: rows and steps that are left
+        int shift = 0;   // COUPLE: the block's rows to the node's exponents
         unsigned hist = 0;
         auto pull = [&]() {
             if (steps == 0) {
@@ -469,6 +471,7 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
                 p = matrix(I, sm, sk);   // sets the strides
                 p += mrow * sm + tt * sk;
                 left = I.off >= 0 && mrow < I.nrow ? I.n - tt : 0;
+                if (MODE == TD_COUPLE) shift = left > 0 ? P.F.sh[I.off * k + mrow] : 0;
                 np = I.n;
                 steps = (np + 15) >> 4;
                 end = I.q + 1 == I.q1 ? 2 : (I.q + 1 == I.q2 ? 3 : 0);
@@ -505,7 +508,10 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
             return true;
         };
         static_assert(TD_AHEAD == 2, "v0, v1");
-        bool v0 = pull(), v1 = pull();
+        bool v0 = pull();
+        int s0 = shift;
+        bool v1 = pull();
+        int s1 = shift;
         int cut = 0;   // steps cut
 #pragma unroll 1
         for (int t = 0; v0 || t < cut + TD_LAG; ++t) {
@@ -515,12 +521,16 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int2 a = raw[(t % TD_AHEAD) * (TD_RAW / 8) + 32 * j];
-                const u64 v = ((u64)(unsigned)a.y << 32) + (u64)((i64)a.x << 2) + 0x8080808080808080ULL;
+                u64 v = ((u64)(unsigned)a.y << 32) + (u64)((i64)a.x << 2);
+                if (MODE == TD_COUPLE) v = (u64)(((i64)v + ((1LL << s0) >> 1)) >> s0);
+                v += 0x8080808080808080ULL;
                 wl[j] = (unsigned)v;
                 wh[j] = (unsigned)(v >> 32);
             }
             v0 = v1;
+            s0 = s1;
             v1 = pull();
+            s1 = shift;
             if (now) {
                 const int st = t % TD_NST;
                 if (t >= TD_NST && !td_wait(empty(st), (t / TD_NST - 1) & 1, deadline)) {
@@ -660,13 +670,13 @@ void launch_td(int nc, const TdP &P, int nitem, int nt, const double *X, int64_t
 // less the first far node), its rows (> 0), offsets of the two halves' entries (-1: none).
 // td_rows: pairs of leaves (2 p, 2 p + 1): near partners (offsets in the panels), then the
 // ancestors of the far levels (offsets in the flattened bases).
-// td_couple: pairs of nodes from the first far node on (offsets in the coupling blocks).
+// td_couple: pairs of nodes from the first far node on (offsets: the coupling blocks).
 // Items (first record, second section, end, pair) in the order of the CTAs that take them.
 void build_tensor_lists(MeshData &m)
 {
     if (m.max_leaf_size > 64 || !m.nnear) return;
     const int nleaf = m.kt.nleaf, fl = m.kt.first_leaf(), nlev = m.nfar > 0 ? m.kt.L - m.far_lmin + 1 : 0;
-    const int k = m.k, kp = (k + 1) & ~1, wp = (nlev * k + 1) & ~1, node0 = nlev ? (1 << m.far_lmin) - 1 : 0;
+    const int k = m.k, wp = (nlev * k + 1) & ~1, node0 = nlev ? (1 << m.far_lmin) - 1 : 0;
     std::vector<TdRec> rec;
     std::vector<int4> items;
     auto add = [&](int col, int n, int64_t a, int64_t b) { if (n > 0) rec.push_back({col, n, {a, b}}); };
@@ -727,12 +737,11 @@ void build_tensor_lists(MeshData &m)
     }
     upload(m.td_rows, m.td_rows_item, m.td_rows_bin);
     if (!nlev) return;
-    const int64_t blk = (int64_t)k * kp;
     for (int a = node0; a < m.kt.nnode; a += 2) {
         const bool two = a + 1 < m.kt.nnode;
         const int q0 = (int)rec.size();
         merge(m.far_col_h, m.far_ptr_h[a], m.far_ptr_h[a + 1], two ? m.far_ptr_h[a + 1] : 0, two ? m.far_ptr_h[a + 2] : 0,
-              [&](int c, int ea, int eb) { add(c - node0, k, ea < 0 ? -1 : ea * blk, eb < 0 ? -1 : eb * blk); });
+              [&](int c, int ea, int eb) { add(c - node0, k, ea, eb); });
         if (q0 == (int)rec.size()) add(0, k, -1, -1);   // no blocks: zeros
         items.push_back({q0, (int)rec.size(), (int)rec.size(), (a - node0) / 2});
     }

@@ -276,11 +276,15 @@ struct OpData {
     DBuf<double> rho;                  // interior points, canonical order
     DBuf<double> S64;                  // nfar * k * k
     DBuf<double> D64;                  // near entries
-    // fixed-point copies for the FP64 apply (apply_fixed.cu): near panels with B + M added and an
-    // exponent per row, coupling blocks and an exponent per row node; fa: built, every entry fits
+    // fixed-point copies for the FP64 apply: coupling blocks, an exponent per row of a block, the
+    // largest of a node's row, their difference, and the blocks that stay FP64 (apply_fixed.cu);
+    // near panels with B + M added and an exponent per row (apply_tensor.cu); fa: built, every
+    // entry is in range
     bool fa = false;
     DBuf<long long> fa_D, fa_S;
-    DBuf<int> fa_re, fa_se;
+    DBuf<int> fa_re;
+    DBuf<short> fa_se, fa_sn;
+    DBuf<unsigned char> fa_sh, fa_hard;
     // digits of a vector's leaf and node pieces, column keys and flags (apply_tensor.cu)
     DBuf<unsigned char> td_x, td_h;
     DBuf<unsigned> td_key;

@@ -1,0 +1,79 @@
+"""Precision of the FP64 apply (vfd_apply) row by row: columns of the operator (unit
+vectors) and vectors that span many decades, against the FP64 kernels, which
+vfd_apply_noalloc runs, in units of |A||x|.
+"""
+import numpy as np
+import pytest
+
+import synth
+from paper_2302_02863_gb300 import vfd
+
+pytestmark = pytest.mark.gpu
+
+# A row is a sum of up to 1200 products, of which a lane adds an eighth one after another:
+# at most some 150 roundings of 2^-53 of its part of |A||x|, about their square root as
+# roundings fall; the far field's three sums behave alike.  64 lies between.
+TOL = 64 * 2.0 ** -53
+
+
+def _setup(name, leaf, p, lam):
+    m = synth.disk_mesh(18, seed=3) if name == "disk" else synth.square_mesh(30, jitter=0.2, seed=5)
+    mesh = vfd.vfd_mesh(m.d, m.coords, m.cells, m.cell_is_interior, leaf_m=leaf, cheb_p=p, lam=lam)
+    s = synth.sigmoid_field(synth.random_fourier_field(21, 1.0), 0.1, 0.9)
+    op = vfd.vfd_assemble(mesh, s, synth.random_fourier_field(22, 0.5), 0.95)
+    dof = vfd.vfd_mesh_dofs(mesh)[0]
+    x = np.zeros((mesh.n_dof, 2))
+    x[dof[dof >= 0]] = np.asarray(m.coords).reshape(-1, 2)[dof >= 0]
+    return op, mesh.n_dof, x
+
+
+def _apply(f, op, X, width):
+    import torch
+    Y = torch.empty_like(X)
+    for i in range(0, len(X), width):
+        f(op, X[i:i + width], Y[i:i + width])
+    return Y
+
+
+def _columns(op, n, f, width):
+    import torch
+    return _apply(f, op, torch.eye(n, dtype=torch.float64, device="cuda"), width)   # row j: A e_j
+
+
+def _vectors(x, rows):
+    """name -> (rows, n): magnitudes that vary along the mesh, from row to row of it, or in one place."""
+    rng = np.random.default_rng(1)
+    n, at = len(x), rng.uniform(-0.5, 0.5, (rows, 1, 2))
+    sign = rng.choice([-1.0, 1.0], (rows, n))
+    spike = np.zeros((rows, n))
+    spike[np.arange(rows), rng.integers(0, n, rows)] = 1.0
+    return {"normal": rng.standard_normal((rows, n)), "ones": np.ones((rows, n)),
+            "six decades": sign * 10.0 ** (-6.0 * rng.random((rows, n))),
+            "14 decades across": sign * 10.0 ** (-7.0 * (x[:, 0] + 1.0)),
+            "local": np.exp(-((x - at) ** 2).sum(-1) / 0.02), "spike on 1e-18": spike + 1e-18 * sign}
+
+
+SETUPS = [("disk", 64, 4, 0.0), ("disk", 32, 6, 0.75), ("square", 40, 8, 0.75), ("square", 16, 3, 0.75)]
+
+
+@pytest.mark.parametrize("name,leaf,p,lam", SETUPS)
+@pytest.mark.parametrize("width", [1, 5, 8])
+def test_unit_vectors_give_the_entries(name, leaf, p, lam, width):
+    op, n, _ = _setup(name, leaf, p, lam)
+    A, B = _columns(op, n, vfd.vfd_apply_noalloc, 8), _columns(op, n, vfd.vfd_apply, width)
+    if lam == 0.0:   # no far field: a panel entry plus a B + M entry, one rounding in any order
+        assert bool((A == B).all())
+    assert bool(((B - A).abs() <= TOL * A.abs()).all()), float(((B - A).abs() / A.abs().clamp_min(1e-300)).max())
+
+
+@pytest.mark.parametrize("name,leaf,p,lam", SETUPS)
+@pytest.mark.parametrize("width", [1, 3, 8])
+def test_rows_keep_fp64_precision(name, leaf, p, lam, width):
+    import torch
+    op, n, x = _setup(name, leaf, p, lam)
+    A = _columns(op, n, vfd.vfd_apply_noalloc, 8).abs()
+    for kind, v in _vectors(x, 9).items():
+        X = torch.tensor(v, device="cuda")
+        R, Y = _apply(vfd.vfd_apply_noalloc, op, X, 3), _apply(vfd.vfd_apply, op, X, width)
+        err = (Y - R).abs() / (X.abs() @ A)
+        assert float(err.max()) <= TOL, (kind, float(err.max()))
