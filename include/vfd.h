@@ -401,6 +401,16 @@ vfd_status vfd_op_rho(vfd_op_t op, double *rho, void *stream);
  * admissible blocks); ranks (may be null) receives min(n, *nlev) entries. */
 vfd_status vfd_op_far_ranks(vfd_op_t op, int *ranks, int n, int *nlev);
 
+/* How the operator's last FP64 apply (vfd_apply, or the residuals of a solve)
+ * was computed; waits for the device.  stats receives n entries:
+ *  [0] its columns if they went to the tensor cores (many columns), else 0;
+ *  [1] 1 if a bounded wait there ran out and the apply was redone without them;
+ *  [2] near rows, [3] projections, [4] tree nodes and [5] leaves, each counted
+ *      once per group of 8 columns, whose sums the tensor cores' digits could
+ *      not hold to FP64's precision and which were computed without them;
+ *  zeros from there on. */
+vfd_status vfd_op_apply_stats(vfd_op_t op, int64_t *stats, int n);
+
 /* Device time per assembly phase (VFD_T_* order) of the vfd_assemble call
  * that created op, if it was given VFD_ASSEMBLE_TIMED; ms: host, n entries
  * (at most VFD_T_COUNT are written).  Returns VFD_EINVAL if not recorded. */

@@ -12,9 +12,14 @@ void launch_far_couple_sum(const MeshData &m, OpData &op, int c0, int cols, cuda
 // apply_fixed.cu: Y = A X with the FP64 operator (OpData::fa)
 void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st,
                  const int *skip, ApplyDot *dot);
+// its kernels for groups of 8 columns from c0 on, ng groups, where `when` says so
+struct FaWhen;
+enum FaStep { FA_PROJ, FA_COUPLE, FA_NEAR, FA_EXPAND };
+void apply_fixed_redo(FaStep step, const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int nrhs,
+                      int64_t ld, cudaStream_t st, const FaWhen &when);
 // apply_tensor.cu: the same for many columns
 bool apply_tensor_fits(const MeshData &m, int nrhs);
 void apply_tensor_alloc(const MeshData &m, OpData &op);   // its workspace, on first use
-const int *apply_tensor(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st);
+void apply_tensor(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st);
 
 }  // namespace vfd

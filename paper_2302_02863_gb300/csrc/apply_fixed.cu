@@ -100,52 +100,56 @@ __device__ __forceinline__ void fa_column(const int2 *__restrict__ M, size_t str
 // ---------------------------------------------------------------------------
 template <int NC>
 __global__ void __launch_bounds__(128) k_fa_proj(FaFar P, const double *__restrict__ X, int64_t ld,
-                                                 double *__restrict__ part, const int *skip)
+                                                 double *__restrict__ part, FaWhen when)
 {
     extern __shared__ __align__(16) unsigned char fa_sm[];
     __shared__ unsigned key[NC];
-    if (skip && *skip) return;
-    const int leaf = blockIdx.x, w = P.nlev * P.k, r0 = P.c0 + blockIdx.z * NC;
-    const int b = P.kb[P.fl + leaf], n = P.ke[P.fl + leaf] - b;
+    const int w = P.nlev * P.k, r0 = P.c0 + blockIdx.z * NC;
+    if (fa_none(when)) return;
     double *raw = (double *)fa_sm;   // [i][NC]
     int2 *xs = (int2 *)fa_sm;
-    if (threadIdx.x < NC) key[threadIdx.x] = 0;
-    __syncthreads();
-    for (int t = threadIdx.x; t < n * NC; t += blockDim.x) {
-        const int c = t / n, i = t - c * n;
-        const double v = r0 + c < P.nrhs ? X[(size_t)(r0 + c) * ld + b + i] : 0.0;
-        raw[i * NC + c] = v;
-        atomicMax(&key[c], fa_key(v));
-    }
-    __syncthreads();
-    bool slow = false;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) slow |= fa_slow(key[c]);
-    if (!slow) {
-        for (int t = threadIdx.x; t < n * NC; t += blockDim.x) xs[t] = fa_split(fa_round(raw[t], key[t % NC]));
-        __syncthreads();
-    }
     const int col = blockIdx.y * blockDim.x + threadIdx.x;
-    if (col >= w) return;
-    const int2 *M = P.U + (size_t)b * P.wp + col;
-    const int eu = P.ue[leaf], lv = col / P.k, a = col - lv * P.k;
-    double out[NC];
-    if (!slow) {
-        fa_column<NC>(M, P.wp, n, 1, xs, out);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) out[c] = out[c] * fa_pow2(eu - 30) * fa_scale(key[c]);
-    } else {
-#pragma unroll
-        for (int c = 0; c < NC; ++c) out[c] = 0.0;
-        for (int i = 0; i < n; ++i) {
-            const double m = P.Ud[((size_t)lv * P.N + b + i) * P.k + a];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) out[c] = fma(m, raw[i * NC + c], out[c]);
+    for (int leaf = blockIdx.x; leaf < P.nleaf; leaf += gridDim.x) {
+        if (fa_off(when, leaf, r0)) continue;
+        const int b = P.kb[P.fl + leaf], n = P.ke[P.fl + leaf] - b;
+        __syncthreads();
+        if (threadIdx.x < NC) key[threadIdx.x] = 0;
+        __syncthreads();
+        for (int t = threadIdx.x; t < n * NC; t += blockDim.x) {
+            const int c = t / n, i = t - c * n;
+            const double v = r0 + c < P.nrhs ? X[(size_t)(r0 + c) * ld + b + i] : 0.0;
+            raw[i * NC + c] = v;
+            atomicMax(&key[c], fa_key(v));
         }
-    }
+        __syncthreads();
+        bool slow = false;
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
-        if (r0 + c < P.nrhs) part[(((size_t)(r0 + c) * P.nlev + lv) * P.nleaf + leaf) * P.k + a] = out[c];
+        for (int c = 0; c < NC; ++c) slow |= fa_slow(key[c]);
+        if (!slow) {
+            for (int t = threadIdx.x; t < n * NC; t += blockDim.x) xs[t] = fa_split(fa_round(raw[t], key[t % NC]));
+            __syncthreads();
+        }
+        if (col >= w) continue;
+        const int2 *M = P.U + (size_t)b * P.wp + col;
+        const int eu = P.ue[leaf], lv = col / P.k, a = col - lv * P.k;
+        double out[NC];
+        if (!slow) {
+            fa_column<NC>(M, P.wp, n, 1, xs, out);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) out[c] = out[c] * fa_pow2(eu - 30) * fa_scale(key[c]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) out[c] = 0.0;
+            for (int i = 0; i < n; ++i) {
+                const double m = P.Ud[((size_t)lv * P.N + b + i) * P.k + a];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) out[c] = fma(m, raw[i * NC + c], out[c]);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (r0 + c < P.nrhs) part[(((size_t)(r0 + c) * P.nlev + lv) * P.nleaf + leaf) * P.k + a] = out[c];
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -157,78 +161,81 @@ constexpr int FC_WARPS = 4;
 template <int NC>
 __global__ void __launch_bounds__(32 * FC_WARPS)
 k_fa_couple(FaFar P, const double *__restrict__ part, const double *__restrict__ xhat, double *__restrict__ ye,
-            const int *skip)
+            FaWhen when)
 {
     __shared__ int2 xs_[FC_WARPS][KMAX * NC];
-    if (skip && *skip) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int e = blockIdx.x * FC_WARPS + warp, r0 = P.c0 + blockIdx.y * NC, k = P.k;
-    if (e >= P.nfar) return;
-    int2 *xs = xs_[warp];
-    double *raw = (double *)xs;
-    const int node = P.fcol[e], l = 31 - __clz(node + 1), sh = P.L - l;
-    const int leaf0 = ((node + 1) << sh) - (1 << P.L);
-    const bool hard = P.hard[e];
-    unsigned key[NC];
+    const int r0 = P.c0 + blockIdx.y * NC, k = P.k;
+    if (fa_none(when)) return;
+    for (int e = blockIdx.x * FC_WARPS + warp; e < P.nfar; e += gridDim.x * FC_WARPS) {
+        if (fa_off(when, when.mask ? P.row[e] : 0, r0)) continue;
+        __syncwarp();
+        int2 *xs = xs_[warp];
+        double *raw = (double *)xs;
+        const int node = P.fcol[e], l = 31 - __clz(node + 1), sh = P.L - l;
+        const int leaf0 = ((node + 1) << sh) - (1 << P.L);
+        const bool hard = P.hard[e];
+        unsigned key[NC];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        const int r = r0 + c;
-        unsigned mk = 0;
-        for (int b = lane; b < k; b += 32) {
-            double v = 0.0;
-            if (r < P.nrhs) {
-                if (xhat) {
-                    v = xhat[((size_t)r * P.nnode + node) * k + b];
-                } else {
-                    const double *p = part + (((size_t)r * P.nlev + l - P.lmin) * P.nleaf + leaf0) * k + b;
-#pragma unroll 8
-                    for (int j = 0; j < (1 << sh); ++j) v += p[(size_t)j * k];
-                }
-            }
-            raw[b * NC + c] = v;
-            mk = max(mk, fa_key(v));
-        }
-        key[c] = __reduce_max_sync(0xffffffffu, mk);
-    }
-    bool slow = false;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) slow |= fa_slow(key[c]);
-    __syncwarp();
-    const int2 *S = P.S + (size_t)e * k * P.kp;
-    if (slow || hard) {
-        for (int a = lane; a < k; a += 32)
-            for (int c = 0; c < NC && r0 + c < P.nrhs; ++c) {
+        for (int c = 0; c < NC; ++c) {
+            const int r = r0 + c;
+            unsigned mk = 0;
+            for (int b = lane; b < k; b += 32) {
                 double v = 0.0;
-                for (int b = 0; b < k; ++b) v = fma(P.Sd[((size_t)e * k + b) * k + a], raw[b * NC + c], v);
-                ye[((size_t)(r0 + c) * P.nfar + e) * k + a] = v;
+                if (r < P.nrhs) {
+                    if (xhat) {
+                        v = xhat[((size_t)r * P.nnode + node) * k + b];
+                    } else {
+                        const double *p = part + (((size_t)r * P.nlev + l - P.lmin) * P.nleaf + leaf0) * k + b;
+#pragma unroll 8
+                        for (int j = 0; j < (1 << sh); ++j) v += p[(size_t)j * k];
+                    }
+                }
+                raw[b * NC + c] = v;
+                mk = max(mk, fa_key(v));
             }
-        return;
-    }
-#pragma unroll
-    for (int c = 0; c < NC; ++c)
-        for (int b = lane; b < k; b += 32) xs[b * NC + c] = fa_split(fa_round(raw[b * NC + c], key[c]));
-    __syncwarp();
-    // lanes over a; with k <= 16 the groups of ga lanes take every (32 / ga)-th row
-    const int ga = k > 16 ? 32 : k > 8 ? 16 : 8, gb = 32 / ga, la = lane & (ga - 1), lb = lane / ga;
-    for (int a0 = 0; a0 < k; a0 += ga) {
-        const int a = a0 + la, es = a < k ? P.se[(size_t)e * k + a] : 0;
-        double out[NC];
-        if (a < k) {
-            fa_column<NC>(S + a + (size_t)lb * P.kp, P.kp, max(0, k - lb), gb, xs + lb * NC, out);
-        } else {
-#pragma unroll
-            for (int c = 0; c < NC; ++c) out[c] = 0.0;
+            key[c] = __reduce_max_sync(0xffffffffu, mk);
         }
-        for (int o = ga; o < 32; o <<= 1) {
+        bool slow = false;
 #pragma unroll
-            for (int c = 0; c < NC; ++c) out[c] += __shfl_xor_sync(0xffffffffu, out[c], o);
+        for (int c = 0; c < NC; ++c) slow |= fa_slow(key[c]);
+        __syncwarp();
+        const int2 *S = P.S + (size_t)e * k * P.kp;
+        if (slow || hard) {
+            for (int a = lane; a < k; a += 32)
+                for (int c = 0; c < NC && r0 + c < P.nrhs; ++c) {
+                    double v = 0.0;
+                    for (int b = 0; b < k; ++b) v = fma(P.Sd[((size_t)e * k + b) * k + a], raw[b * NC + c], v);
+                    ye[((size_t)(r0 + c) * P.nfar + e) * k + a] = v;
+                }
+            continue;
         }
-        if (a < k && lb == 0) {
 #pragma unroll
-            for (int c = 0; c < NC; ++c)
-                if (r0 + c < P.nrhs)
-                    ye[((size_t)(r0 + c) * P.nfar + e) * k + a] =
-                        out[c] * fa_pow2(es - 30) * fa_scale(key[c]);
+        for (int c = 0; c < NC; ++c)
+            for (int b = lane; b < k; b += 32) xs[b * NC + c] = fa_split(fa_round(raw[b * NC + c], key[c]));
+        __syncwarp();
+        // lanes over a; with k <= 16 the groups of ga lanes take every (32 / ga)-th row
+        const int ga = k > 16 ? 32 : k > 8 ? 16 : 8, gb = 32 / ga, la = lane & (ga - 1), lb = lane / ga;
+        for (int a0 = 0; a0 < k; a0 += ga) {
+            const int a = a0 + la, es = a < k ? P.se[(size_t)e * k + a] : 0;
+            double out[NC];
+            if (a < k) {
+                fa_column<NC>(S + a + (size_t)lb * P.kp, P.kp, max(0, k - lb), gb, xs + lb * NC, out);
+            } else {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) out[c] = 0.0;
+            }
+            for (int o = ga; o < 32; o <<= 1) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) out[c] += __shfl_xor_sync(0xffffffffu, out[c], o);
+            }
+            if (a < k && lb == 0) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c)
+                    if (r0 + c < P.nrhs)
+                        ye[((size_t)(r0 + c) * P.nfar + e) * k + a] =
+                            out[c] * fa_pow2(max(es, -900) - 30) * fa_scale(key[c]);
+            }
         }
     }
 }
@@ -319,42 +326,19 @@ __device__ __forceinline__ int fa_slot(int j, int c, int ws)   // of column c's 
 // an entry is loaded once for all of them.  (The next four entries loaded ahead cost more
 // registers than they hide: 5 columns at 3721 DoFs 91 us instead of 76, 8 at 9025 202 / 165.)
 // ---------------------------------------------------------------------------
-// sum over the 8 lanes of a row; every lane ends with one column, returned, and its sum in s[0]
-template <int NC>
-__device__ __forceinline__ int fa_sum8(double *s, int l8)
-{
-    int n = NC, col = 0;
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) {
-        if (n > 1) {
-            n >>= 1;
-            const bool up = l8 & o;
-#pragma unroll
-            for (int q = 0; q < NC / 2; ++q)
-                if (q < n) {
-                    const double send = up ? s[q] : s[q + n], keep = up ? s[q + n] : s[q];
-                    s[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-                }
-            col += up ? n : 0;
-        } else {
-            s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
-        }
-    }
-    return col;
-}
-
 template <int NC>
 __global__ void __launch_bounds__(128) k_fa_near(FaNear P, const double *__restrict__ X, int64_t ld,
-                                                 double *__restrict__ Y, const int *skip)
+                                                 double *__restrict__ Y, FaWhen when)
 {
     extern __shared__ __align__(16) unsigned char fa_sm[];
-    if (skip && *skip) return;
     const int lf = blockIdx.x, r0 = P.c0 + blockIdx.z * NC;
+    if (fa_none(when) || fa_off(when, 0, r0)) return;
     const int b_leaf = P.kb[P.fl + lf], b = b_leaf + blockIdx.y * P.NR, e = min(P.ke[P.fl + lf], b + P.NR);
     if (b >= e) return;
     const int W = P.pw[lf];
     const int *gc = P.gcol + P.goff[lf];
     const double *x0 = X + (size_t)r0 * ld;
+    const int nc = min(NC, P.nrhs - r0);              // columns of the group (fewer than NC where it is redone)
     constexpr int NP = NC > 4 ? 8 : NC > 2 ? 4 : 2;   // lanes of a row with a column
     double *xs = (double *)fa_sm;
 #pragma unroll 4
@@ -362,7 +346,7 @@ __global__ void __launch_bounds__(128) k_fa_near(FaNear P, const double *__restr
         const int j = gc[t];
 #pragma unroll
         for (int c = 0; c < ((NC + 1) & ~1); ++c)
-            xs[(c >> 1) * 2 * W + 2 * t + (c & 1)] = j >= 0 && c < NC ? x0[(size_t)c * ld + j] : 0.0;
+            xs[(c >> 1) * 2 * W + 2 * t + (c & 1)] = j >= 0 && c < nc ? x0[(size_t)c * ld + j] : 0.0;
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l8 = lane & 7, nw = blockDim.x >> 5;
@@ -398,11 +382,12 @@ __global__ void __launch_bounds__(128) k_fa_near(FaNear P, const double *__restr
                 const double *xj = x0 + P.colidx[q];
                 const double v = P.val[q];
 #pragma unroll
-                for (int c = 0; c < NC; ++c) s[c] = fma(v, xj[(size_t)c * ld], s[c]);
+                for (int c = 0; c < NC; ++c)
+                    if (c < nc) s[c] = fma(v, xj[(size_t)c * ld], s[c]);
             }
         }
-        const int c = fa_sum8<NP>(s, l8);
-        if (on && (l8 & (8 / NP - 1)) == 0 && c < NC) Y[(size_t)(r0 + c) * ld + i] = s[0];
+        const int c = fa_sum8d<NP>(s, l8);
+        if (on && (l8 & (8 / NP - 1)) == 0 && c < nc) Y[(size_t)(r0 + c) * ld + i] = s[0];
     }
 }
 
@@ -412,12 +397,12 @@ __global__ void __launch_bounds__(128) k_fa_near(FaNear P, const double *__restr
 template <int NC>
 __global__ void __launch_bounds__(128)
 k_fa_expand(FaFar P, int NR, const double *__restrict__ ye, const double *__restrict__ yhat, double *__restrict__ Y,
-            int64_t ld, const int *skip)
+            int64_t ld, FaWhen when)
 {
     extern __shared__ __align__(16) unsigned char fa_sm[];
     __shared__ unsigned key[NC];
-    if (skip && *skip) return;
     const int lf = blockIdx.x, r0 = P.c0 + blockIdx.z * NC, k = P.k, w = P.nlev * k, ws = P.wp;
+    if (fa_none(when) || fa_off(when, lf, r0)) return;
     const int b_leaf = P.kb[P.fl + lf], b = b_leaf + blockIdx.y * NR, e = min(P.ke[P.fl + lf], b + NR);
     if (b >= e) return;
     double *raw = (double *)fa_sm;
@@ -636,8 +621,8 @@ k_fa_couple1(FaFar P, const double *__restrict__ part, const double *__restrict_
     }
     if (lb == 0 && pr < np) {
         const double sx = fa_scale(ky);
-        out[2 * pr] = v0 * fa_pow2(es0 - 30) * sx;
-        if (2 * pr + 1 < k) out[2 * pr + 1] = v1 * fa_pow2(es1 - 30) * sx;
+        out[2 * pr] = v0 * fa_pow2(max(es0, -900) - 30) * sx;
+        if (2 * pr + 1 < k) out[2 * pr + 1] = v1 * fa_pow2(max(es1, -900) - 30) * sx;
     }
 }
 
@@ -671,10 +656,10 @@ __device__ __forceinline__ void fa_dot(double v, double *dot)
 // and more CTAs: one column at 16129 DoFs and rank 16 / at 27k and rank 64, batches of eight
 // 73 / 181 us, of four and at least 8 CTAs an SM 66 / 171, of two and 16 CTAs 71 / 171.
 __global__ void __launch_bounds__(128, 8)
-k_fa_near1(FaNear P, const double *__restrict__ X, double *__restrict__ Y, double *__restrict__ dot, const int *skip)
+k_fa_near1(FaNear P, const double *__restrict__ X, double *__restrict__ Y, double *__restrict__ dot, FaWhen when)
 {
     extern __shared__ __align__(16) unsigned char fa_sm[];
-    if (skip && *skip) return;
+    if (fa_none(when) || fa_off(when, 0, P.c0)) return;
     const int lf = blockIdx.x, b_leaf = P.kb[P.fl + lf], b = b_leaf + blockIdx.y * 16, e = min(P.ke[P.fl + lf], b + 16);
     if (b >= e) {
         if (dot && threadIdx.x == 0) dot[blockIdx.x * gridDim.y + blockIdx.y] = 0.0;
@@ -721,7 +706,7 @@ k_fa_near1(FaNear P, const double *__restrict__ X, double *__restrict__ Y, doubl
     }
     // B + M last: the diagonal's product is the largest term of a row
     s0 = (s0 + s1) + bm;
-    fa_sum8<1>(&s0, l8);
+    fa_sum8d<1>(&s0, l8);
     double xy = 0.0;
     if (i < e && !l8) {
         Y[i] = s0;
@@ -814,82 +799,85 @@ __device__ __forceinline__ int fa_exponent(unsigned key, int *err)
     return key ? (int)key - 1022 : 0;
 }
 
-// near panel rows, a warp each; B + M added at their panel positions
+// near panel rows, a warp each, for the many-column apply: the entries at the positions of B + M
+// (the row's largest, 2^5 to 2^8 above the next) go to val8 with B + M and stay FP64
 __global__ void k_fa_build_near(int N, int fl, const int *__restrict__ vleaf, const int *__restrict__ kb,
                                 const int *__restrict__ pw, const int64_t *__restrict__ poff,
                                 const double *__restrict__ D, const int *__restrict__ rowptr,
                                 const int64_t *__restrict__ bpos, const double *__restrict__ val,
-                                int2 *__restrict__ out, int *__restrict__ re, int *err)
+                                double *__restrict__ val8, int2 *__restrict__ out, int *__restrict__ re, int *err)
 {
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (i >= N) return;
     const int lf = vleaf[i], W = pw[lf];
     const size_t o = poff[lf] + (size_t)(i - kb[fl + lf]) * W;
-    unsigned key = 0;
-    for (int j = lane; j < W; j += 32) key = max(key, fa_key(D[o + j]));
-    if (val)
-        for (int q = rowptr[i] + lane; q < rowptr[i + 1]; q += 32) key = max(key, fa_key(val[q]));
-    const int E = fa_exponent(key, err) + (val ? 1 : 0);   // room for the sum of two entries
-    for (int j = lane; j < W; j += 32) out[o + j] = fa_split(fa_round(D[o + j], E + 1022));
+    for (int j = lane; j < W; j += 32) out[o + j] = make_int2(0, 0);
     __syncwarp();
-    if (val)
-        for (int q = rowptr[i] + lane; q < rowptr[i + 1]; q += 32) {   // distinct positions
-            const int2 d = out[bpos[q]];
-            out[bpos[q]] = fa_split(((i64)d.y << FA_LO) + d.x + fa_round(val[q], E + 1022));
-        }
+    for (int q = rowptr[i] + lane; q < rowptr[i + 1]; q += 32) {   // distinct positions, marked
+        const int64_t p = bpos[q];
+        val8[q] = val[q] + (p >= 0 ? D[p] : 0.0);
+        if (p >= 0) out[p] = make_int2(1, 0);
+    }
+    __syncwarp();
+    unsigned key = 0;
+    for (int j = lane; j < W; j += 32)
+        if (!out[o + j].x) key = max(key, fa_key(D[o + j]));
+    const int E = fa_exponent(key, err);
+    for (int j = lane; j < W; j += 32) out[o + j] = out[o + j].x ? make_int2(0, 0) : fa_split(fa_round(D[o + j], E + 1022));
     if (lane == 0) re[i] = E;
 }
 
-// coupling blocks, a CTA per row node, rows padded to an even length.  An exponent per row
-// of a block; sn, the largest of the node's blocks, and sh = sn - se align the blocks of a
-// node where their digits are summed (apply_tensor.cu).  Entries down to 2^-8 of their
-// row's largest keep all their bits; a block with a smaller one is marked hard.
+// coupling blocks, a CTA per row node, rows padded to an even length; an exponent per row of a
+// block.  Entries down to 2^-8 of their row's largest keep all their bits; a block with a
+// smaller one is marked hard.  low, least: smallest entry of a row (in its scale) and of the block.
 __global__ void __launch_bounds__(256)
 k_fa_build_S(const int *__restrict__ fptr, int k, int kp, const double *__restrict__ S, int2 *__restrict__ out,
-             short *__restrict__ se, short *__restrict__ sn, unsigned char *__restrict__ sh,
-             unsigned char *__restrict__ hard, int *err)
+             short *__restrict__ se, float *__restrict__ low, unsigned char *__restrict__ hard, int *__restrict__ row,
+             double *__restrict__ least, int *err)
 {
-    constexpr int NONE = -32768;
-    __shared__ int top[KMAX];
     const int node = blockIdx.x, e0 = fptr[node], ne = fptr[node + 1] - e0;
-    if (threadIdx.x < k) top[threadIdx.x] = NONE;
-    for (int e = threadIdx.x; e < ne; e += 256) hard[e0 + e] = 0;
+    for (int e = threadIdx.x; e < ne; e += 256) {
+        hard[e0 + e] = 0;
+        row[e0 + e] = node;
+    }
     __syncthreads();
     for (int t = threadIdx.x; t < ne * k; t += 256) {
         const int e = t / k, a = t - e * k;
         const double *in = S + (size_t)(e0 + e) * k * k + a;
-        unsigned key = 0, least = 0x7ffu;
+        unsigned key = 0, lk = 0x7ffu;
+        double v = INFINITY;
         for (int b = 0; b < k; ++b) {
-            const unsigned q = fa_key(in[(size_t)b * k]);
+            const double x = fabs(in[(size_t)b * k]);
+            const unsigned q = fa_key(x);
             key = max(key, q);
-            if (q) least = min(least, q);
+            if (q) lk = min(lk, q);
+            v = fmin(v, x);
         }
         if (!fa_fits(key)) atomicOr(err, 4);
-        if (key > least + 7) hard[e0 + e] = 1;
-        const int E = (int)key - 1022;
-        if (key) atomicMax(&top[a], E);
-        se[(size_t)(e0 + e) * k + a] = (short)(key ? E : NONE);
+        if (key > lk + 7) hard[e0 + e] = 1;
+        se[(size_t)(e0 + e) * k + a] = (short)(key ? (int)key - 1022 : -2000);   // a row of zeros: below all others
+        low[(size_t)(e0 + e) * k + a] = key ? (float)scalbn(v, 1022 - (int)key) : 0.0f;
         int2 *o = out + (size_t)(e0 + e) * k * kp + a;
         for (int b = 0; b < k; ++b) o[(size_t)b * kp] = fa_split(fa_round(in[(size_t)b * k], (int)key));
         if (a == k - 1 && kp > k)
             for (int b = 0; b < k; ++b) o[(size_t)b * kp + 1] = make_int2(0, 0);
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < ne * k; t += 256) {   // the entries that this thread wrote
-        const size_t i = (size_t)e0 * k + t;
-        const int a = t % k, E = se[i];
-        if (E == NONE) se[i] = (short)(top[a] == NONE ? 0 : top[a]);   // a row of zeros
-        sh[i] = (unsigned char)(E == NONE ? 0 : min(top[a] - E, 63));
+    for (int e = threadIdx.x >> 5; e < ne; e += 8) {   // a warp per block
+        double v = INFINITY;
+        for (int i = threadIdx.x & 31; i < k * k; i += 32) v = fmin(v, fabs(S[(size_t)(e0 + e) * k * k + i]));
+        for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
+        if ((threadIdx.x & 31) == 0) least[e0 + e] = v;
     }
-    if (threadIdx.x < k) sn[(size_t)node * k + threadIdx.x] = (short)(top[threadIdx.x] == NONE ? 0 : top[threadIdx.x]);
 }
 
 // flattened bases, CTA per leaf: [level][N][k] -> [N][level k], rows padded to an even length
-__global__ void k_fa_build_U(int fl, int N, int k, int nlev, const int *__restrict__ kb, const int *__restrict__ ke,
-                             const double *__restrict__ U, int2 *__restrict__ out, int *__restrict__ ue, int *err)
+__global__ void __launch_bounds__(256) k_fa_build_U(int fl, int N, int k, int nlev, const int *__restrict__ kb, const int *__restrict__ ke,
+                             const double *__restrict__ U, int2 *__restrict__ out, int *__restrict__ ue,
+                             float *__restrict__ umin, int *err)
 {
     __shared__ unsigned key;
     __shared__ int E;
+    __shared__ float least[8];
     const int b = kb[fl + blockIdx.x], n = ke[fl + blockIdx.x] - b, w = nlev * k, wp = (w + 1) & ~1;
     if (threadIdx.x == 0) key = 0;
     __syncthreads();
@@ -910,7 +898,20 @@ __global__ void k_fa_build_U(int fl, int N, int k, int nlev, const int *__restri
         out[(size_t)i * wp + q] =
             q < w ? fa_split(fa_round(U[((size_t)(q / k) * N + i) * k + q % k], E + 1022)) : make_int2(0, 0);
     }
-    if (threadIdx.x == 0) ue[blockIdx.x] = E;
+    float r = INFINITY;   // the rows sum to the DoFs' weights, the same at every level
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        double t = 0.0;
+        for (int q = 0; q < k; ++q) t += U[(size_t)(b + i) * k + q];
+        r = fminf(r, (float)(fabs(t) * fa_pow2(-E)));
+    }
+    for (int o = 16; o > 0; o >>= 1) r = fminf(r, __shfl_xor_sync(0xffffffffu, r, o));
+    if ((threadIdx.x & 31) == 0) least[threadIdx.x >> 5] = r;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < 8; ++q) r = fminf(r, least[q]);
+        ue[blockIdx.x] = E;
+        umin[blockIdx.x] = r;
+    }
 }
 
 }  // namespace
@@ -926,8 +927,9 @@ void build_fixed_bases(MeshData &m)
     err.zero(nullptr);
     m.fa_U.alloc((size_t)((nlev * m.k + 1) & ~1) * m.N);
     m.fa_ue.alloc(m.kt.nleaf);
+    m.fa_umin.alloc(m.kt.nleaf);
     k_fa_build_U<<<m.kt.nleaf, 256>>>(m.kt.first_leaf(), m.N, m.k, nlev, m.kt_begin.p, m.kt_end.p, m.Ul64.p,
-                                      (int2 *)m.fa_U.p, m.fa_ue.p, err.p);
+                                      (int2 *)m.fa_U.p, m.fa_ue.p, m.fa_umin.p, err.p);
     VFD_CUDA(cudaGetLastError());
     int h = 0;
     VFD_CUDA(cudaMemcpy(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost));
@@ -937,24 +939,25 @@ void build_fixed_bases(MeshData &m)
     }
 }
 
-// the operator's near panels (with B + M) and coupling blocks; err gets bit 2
-// where an entry does not fit
+// the operator's near panels and coupling blocks; err gets bit 2 where an entry does not fit
 void build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t st)
 {
     op.fa_D.alloc(m.near_entries);
     op.fa_re.alloc(m.N);
+    op.fa_val.alloc(m.nnz);
     k_fa_build_near<<<cdiv((long long)m.N * 32, 256), 256, 0, st>>>(
         m.N, m.kt.first_leaf(), m.vleaf.p, m.kt_begin.p, m.panel_w.p, m.panel_off.p, op.D64.p, m.rowptr.p, m.bm_pos.p,
-        m.bm_in_panels ? op.valBM.p : nullptr, (int2 *)op.fa_D.p, op.fa_re.p, err);
+        op.valBM.p, op.fa_val.p, (int2 *)op.fa_D.p, op.fa_re.p, err);
     if (m.nfar) {
         const int kp = (m.k + 1) & ~1;
         op.fa_S.alloc((size_t)m.nfar * m.k * kp);
         op.fa_se.alloc((size_t)m.nfar * m.k);
-        op.fa_sh.alloc((size_t)m.nfar * m.k);
+        op.fa_low.alloc((size_t)m.nfar * m.k);
         op.fa_hard.alloc(m.nfar);
-        op.fa_sn.alloc((size_t)m.kt.nnode * m.k);
-        k_fa_build_S<<<m.kt.nnode, 256, 0, st>>>(m.far_ptr.p, m.k, kp, op.S64.p, (int2 *)op.fa_S.p, op.fa_se.p, op.fa_sn.p,
-                                                 op.fa_sh.p, op.fa_hard.p, err);
+        op.fa_row.alloc(m.nfar);
+        op.fa_min.alloc(m.nfar);
+        k_fa_build_S<<<m.kt.nnode, 256, 0, st>>>(m.far_ptr.p, m.k, kp, op.S64.p, (int2 *)op.fa_S.p, op.fa_se.p, op.fa_low.p,
+                                                 op.fa_hard.p, op.fa_row.p, op.fa_min.p, err);
     }
     VFD_CUDA(cudaGetLastError());
 }
@@ -985,6 +988,8 @@ template <int NC>
 void far_group(const MeshData &m, OpData &op, const double *X, int c0, int ng, int nrhs, int64_t ld, bool summed,
                const int *skip)
 {
+    FaWhen when;
+    when.skip = skip;
     const int k = m.k, nleaf = m.kt.nleaf;
     FaFar P = fa_far_view(m, op);
     P.nrhs = nrhs;
@@ -996,21 +1001,21 @@ void far_group(const MeshData &m, OpData &op, const double *X, int c0, int ng, i
     if constexpr (NC == 1)
         k_fa_proj1<<<dim3(nleaf, cdiv(w, 256)), 128, shp, op.side>>>(P, X + (size_t)c0 * ld, op.P64.p + c0 * ps, skip);
     else
-        k_fa_proj<NC><<<dim3(nleaf, cdiv(w, 128), ng), 128, shp, op.side>>>(P, X, ld, op.P64.p, skip);
+        k_fa_proj<NC><<<dim3(nleaf, cdiv(w, 128), ng), 128, shp, op.side>>>(P, X, ld, op.P64.p, when);
     if (summed) launch_far_sum(m, op, c0, cols, op.side, skip);
     if constexpr (NC == 1)
         k_fa_couple1<<<cdiv(m.nfar, FC_WARPS), 32 * FC_WARPS, 0, op.side>>>(
             P, op.P64.p + c0 * ps, summed ? op.xhat.p + c0 * hs : nullptr, op.ye64.p + c0 * ys, skip);
     else
         k_fa_couple<NC><<<dim3(cdiv(m.nfar, FC_WARPS), ng), 32 * FC_WARPS, 0, op.side>>>(
-            P, op.P64.p, summed ? op.xhat.p : nullptr, op.ye64.p, skip);
+            P, op.P64.p, summed ? op.xhat.p : nullptr, op.ye64.p, when);
     if (summed) launch_far_couple_sum(m, op, c0, cols, op.side, skip);
     VFD_CUDA(cudaGetLastError());
 }
 
 template <int NC>
 void expand_group(const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int nrhs, int64_t ld,
-                  bool summed, cudaStream_t st, const int *skip, ApplyDot *dot)
+                  bool summed, cudaStream_t st, const FaWhen &when, ApplyDot *dot)
 {
     FaFar P = fa_far_view(m, op);
     P.nrhs = nrhs;
@@ -1019,31 +1024,32 @@ void expand_group(const MeshData &m, OpData &op, const double *X, double *Y, int
     if constexpr (NC == 1) {
         k_fa_expand1<<<dim3(m.kt.nleaf, cdiv(m.max_leaf_size, 16)), 128, shm, st>>>(
             P, op.ye64.p + c0 * ys, summed ? op.yhat.p + c0 * hs : nullptr, Y + (size_t)c0 * ld, X + (size_t)c0 * ld,
-            dot ? dot->part : nullptr, skip);
+            dot ? dot->part : nullptr, when.skip);
     } else {
         allow_shared(k_fa_expand<NC>, shm);
         const int nr = rows_of(m, m.kt.nleaf * ng);
         k_fa_expand<NC><<<dim3(m.kt.nleaf, cdiv(m.max_leaf_size, nr), ng), 128, shm, st>>>(
-            P, nr, op.ye64.p, summed ? op.yhat.p : nullptr, Y, ld, skip);
+            P, nr, op.ye64.p, summed ? op.yhat.p : nullptr, Y, ld, when);
     }
     VFD_CUDA(cudaGetLastError());
 }
 
 template <int NC>
-void near_group(const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int64_t ld, cudaStream_t st,
-                const int *skip, double *dot)
+void near_group(const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int nrhs, int64_t ld,
+                cudaStream_t st, const FaWhen &when, double *dot)
 {
     FaNear R = fa_near_view(m, op);
+    R.nrhs = nrhs;
     R.c0 = c0;
     const size_t shm = (size_t)m.max_panel_w * (NC == 1 ? 1 : (NC + 1) & ~1) * 8;
     if constexpr (NC == 1) {
         allow_shared(k_fa_near1, shm);
         k_fa_near1<<<dim3(m.kt.nleaf, cdiv(m.max_leaf_size, 16)), 128, shm, st>>>(R, X + (size_t)c0 * ld,
-                                                                                 Y + (size_t)c0 * ld, dot, skip);
+                                                                                 Y + (size_t)c0 * ld, dot, when);
     } else {
         allow_shared(k_fa_near<NC>, shm);
         R.NR = rows_of(m, m.kt.nleaf * ng);
-        k_fa_near<NC><<<dim3(m.kt.nleaf, cdiv(m.max_leaf_size, R.NR), ng), 128, shm, st>>>(R, X, ld, Y, skip);
+        k_fa_near<NC><<<dim3(m.kt.nleaf, cdiv(m.max_leaf_size, R.NR), ng), 128, shm, st>>>(R, X, ld, Y, when);
     }
     VFD_CUDA(cudaGetLastError());
 }
@@ -1064,6 +1070,14 @@ void with_columns(int n, F f)
     }
 }
 
+// widest near group: its panel piece leaves room for two CTAs an SM
+int near_columns(const MeshData &m)
+{
+    int nc = 8;
+    while (nc > 1 && (size_t)m.max_panel_w * nc * 8 > 100 * 1024) nc >>= 1;
+    return nc;
+}
+
 }  // namespace
 
 // Y = A X with the FP64 operator (all parts); the workspaces are those of the FP64 apply
@@ -1072,8 +1086,9 @@ void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int 
 {
     if (dot) dot->n = nrhs == 1 ? m.kt.nleaf * cdiv(m.max_leaf_size, 16) : 0;
     if (dot && !dot->n) dot = nullptr;
-    // many columns: on the tensor cores; what follows is then a fallback behind a flag
-    if (!skip && !dot && apply_tensor_fits(m, nrhs)) skip = apply_tensor(m, op, X, Y, nrhs, ld, st);
+    if (!skip && !dot && apply_tensor_fits(m, nrhs)) return apply_tensor(m, op, X, Y, nrhs, ld, st);
+    FaWhen when;
+    when.skip = skip;
     // the node sums inside the gathers pay for few columns and short spans (3 columns, sums inside /
     // of their own: 27361 DoFs 432 / 395 us, 16129 182 / 171, 3721 61 / 59; 2 columns at 10267 97 / 125)
     const bool summed = nrhs >= 3 || m.kt.L - m.far_lmin > 7, far = m.nfar > 0;
@@ -1098,12 +1113,10 @@ void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int 
         VFD_CUDA(cudaStreamWaitEvent(op.side, op.ev_fork, 0));
         far_groups([&](auto NC, int c0, int ng) { far_group<NC>(m, op, X, c0, ng, nrhs, ld, summed, skip); });
     }
-    // near groups: the widest whose panel piece leaves room for two CTAs an SM
-    int nc = 8;
-    while (nc > 1 && (size_t)m.max_panel_w * nc * 8 > 100 * 1024) nc >>= 1;
+    const int nc = near_columns(m);
     auto near = [&](int n, int c0, int ng) {
         with_columns(n, [&](auto NC) {
-            near_group<NC>(m, op, X, Y, c0, ng, ld, st, skip, dot && !far ? dot->part : nullptr);
+            near_group<NC>(m, op, X, Y, c0, ng, nrhs, ld, st, when, dot && !far ? dot->part : nullptr);
         });
     };
     if (nc == 1)
@@ -1114,8 +1127,37 @@ void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int 
     if (far) {
         VFD_CUDA(cudaEventRecord(op.ev_join, op.side));
         VFD_CUDA(cudaStreamWaitEvent(st, op.ev_join, 0));
-        far_groups([&](auto NC, int c0, int ng) { expand_group<NC>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, skip, dot); });
+        far_groups([&](auto NC, int c0, int ng) { expand_group<NC>(m, op, X, Y, c0, ng, nrhs, ld, summed, st, when, dot); });
     }
+}
+
+// the kernels above with the sums as kernels of their own, on st, for what the many-column apply
+// leaves to them
+void apply_fixed_redo(FaStep step, const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int nrhs,
+                      int64_t ld, cudaStream_t st, const FaWhen &when)
+{
+    FaFar P = fa_far_view(m, op);
+    P.nrhs = nrhs;
+    P.c0 = c0;
+    // (grids of a size at which a launch with nothing to do costs a few microseconds)
+    const int nc = near_columns(m);
+    if (step == FA_PROJ)
+        k_fa_proj<8><<<dim3(std::min(m.kt.nleaf, 64), cdiv(P.nlev * m.k, 128), ng), 128, (size_t)m.max_leaf_size * 64, st>>>(
+            P, X, ld, op.P64.p, when);
+    else if (step == FA_COUPLE)
+        k_fa_couple<8><<<dim3(std::min(cdiv(m.nfar, FC_WARPS), 608), ng), 32 * FC_WARPS, 0, st>>>(P, op.P64.p, op.xhat.p,
+                                                                                                op.ye64.p, when);
+    else if (step == FA_EXPAND)
+        expand_group<8>(m, op, X, Y, c0, ng, nrhs, ld, true, st, when, nullptr);
+    else
+        with_columns(nc, [&](auto NC) {
+            const int cols = std::min(nrhs - c0, 8 * ng);
+            if constexpr (NC == 1)
+                for (int c = c0; c < c0 + cols; ++c) near_group<1>(m, op, X, Y, c, 1, nrhs, ld, st, when, nullptr);
+            else
+                near_group<NC>(m, op, X, Y, c0, cdiv(cols, (int)NC), nrhs, ld, st, when, nullptr);
+        });
+    VFD_CUDA(cudaGetLastError());
 }
 
 }  // namespace vfd

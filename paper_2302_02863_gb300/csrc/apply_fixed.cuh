@@ -65,14 +65,58 @@ struct FaAcc {
     __device__ __forceinline__ double value() const { return fma((double)th, 1099511627776.0, (double)hh); }
 };
 
+// Which of a kernel's items run: none where *skip is set; with a mask those whose bit of this
+// group of columns is set (item 0 of near), or all where *err is set
+struct FaWhen {
+    const int *skip = nullptr;
+    const unsigned *mask = nullptr;
+    const int *any = nullptr;   // 0: no item's bit is set
+    const int *err = nullptr;
+    int c0 = 0;   // first column of the mask's bit 0
+};
+// nothing to do at all; nothing for this item
+__device__ __forceinline__ bool fa_none(const FaWhen &w)
+{
+    return (w.skip && *w.skip) || (w.mask && !*w.any && !*w.err);
+}
+__device__ __forceinline__ bool fa_off(const FaWhen &w, int item, int r0)
+{
+    return w.mask && !*w.err && !(w.mask[item] >> ((r0 - w.c0) >> 3) & 1u);
+}
+
+// sum over the 8 lanes of a row; every lane ends with one column, returned, and its sum in s[0]
+template <int NC>
+__device__ __forceinline__ int fa_sum8d(double *s, int l8)
+{
+    int n = NC, col = 0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = l8 & o;
+#pragma unroll
+            for (int q = 0; q < NC / 2; ++q)
+                if (q < n) {
+                    const double send = up ? s[q] : s[q + n], keep = up ? s[q + n] : s[q];
+                    s[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            col += up ? n : 0;
+        } else {
+            s[0] += __shfl_xor_sync(0xffffffffu, s[0], o);
+        }
+    }
+    return col;
+}
+
 struct FaFar {
     int fl, nleaf, lmin, L, nlev, k, nnode, nfar, nrhs, c0;   // c0: first column of this launch
     int kp, wp;   // row strides of a coupling block and of the bases (even: 16-byte rows)
     const int *kb, *ke, *fptr, *fcol;
     const int2 *U, *S;
     const int *ue;
-    const short *se, *sn;    // exponents: of a block's row, the largest of a node's row
-    const unsigned char *hard, *sh;   // per block: stays FP64; per block's row: sn - se
+    const short *se;         // exponents of a block's rows
+    const unsigned char *hard;   // blocks that stay FP64
+    const int *row;          // row node of a block
     const double *Ud, *Sd;   // FP64: [level][N][k], blocks
     int N;
 };
@@ -82,7 +126,7 @@ struct FaNear {
     const int *kb, *ke, *pw, *gcol, *goff, *rowptr, *colidx;
     const int64_t *poff;
     const double *val;   // B + M
-    int folded;          // B + M are in the fixed-point panels
+    const double *val8;  // B + M plus the panel entries at its positions, which D leaves out
     const int2 *D;
     const int *re;
     const double *Dd;    // FP64 panels
@@ -110,9 +154,8 @@ inline FaFar fa_far_view(const MeshData &m, const OpData &op)
     P.S = (const int2 *)op.fa_S.p;
     P.ue = m.fa_ue.p;
     P.se = op.fa_se.p;
-    P.sn = op.fa_sn.p;
     P.hard = op.fa_hard.p;
-    P.sh = op.fa_sh.p;
+    P.row = op.fa_row.p;
     P.Ud = m.Ul64.p;
     P.Sd = op.S64.p;
     P.N = m.N;
@@ -133,7 +176,7 @@ inline FaNear fa_near_view(const MeshData &m, const OpData &op)
     R.colidx = m.colidx.p;
     R.poff = m.panel_off.p;
     R.val = op.valBM.p;
-    R.folded = m.bm_in_panels ? 1 : 0;
+    R.val8 = op.fa_val.p;
     R.D = (const int2 *)op.fa_D.p;
     R.re = op.fa_re.p;
     R.Dd = op.D64.p;

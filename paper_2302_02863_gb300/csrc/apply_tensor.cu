@@ -10,7 +10,14 @@
 // them, and after 160 products at most they move to 96-bit integers in registers: 6 pairs
 // of 160 stay below 2^24 and are exact; of the two lowest accumulators (8 and 7 pairs) a
 // sum above 2^24 is rounded by less than the dropped pairs add up to.  So the result is
-// that of integer arithmetic up to the dropped pairs.
+// that of integer arithmetic up to the dropped pairs, about 2^-62 of the two scales a product.
+//
+// Scales.  A row of the operator has one (near panel rows, rows of a coupling block, bases of
+// a leaf), and so has a leaf's or node's piece of the columns of a tile; the cutting warps
+// shift the entries of a piece to the largest scale of the sum.  The diagonal and the other
+// entries at B + M's positions, 2^5 to 2^8 above the next, are left out of the near
+// panels and summed in FP64 (k_td_csr).  Sums that a scale would still cost precision are
+// found before they are used and done without digits ("What the digits cannot hold").
 //
 // A CTA computes 128 rows (two halves of 64: sibling leaves, sibling nodes) of a tile
 // of NC columns.  The digit planes of the vector lie one after the other along N, so
@@ -20,9 +27,10 @@
 // mesh: build_tensor_lists); a half without the partner multiplies zeros.
 //
 //   k_td_max, k_td_digits   x -> digits per leaf, in the order the instruction reads
+//   k_td_csr, k_td_near     Y = B + M and the large entries, FP64; rows that stay FP64
 //   k_td<PROJ>              projections, then the node sums (apply.cu), digits per node
-//   k_td<COUPLE>            coupling blocks summed per node (one exponent a node), digits
-//   k_td<ROWS>              near panel rows and the expansion of a leaf, Y
+//   k_td<COUPLE>            coupling blocks summed per node, digits per node
+//   k_td<ROWS>              near panel rows and the expansion of a leaf, added to Y
 //
 // Warp roles of k_td, per step of 16 rows of a partner:
 //   warps 0-15 copy the operator's integers (apply_fixed.cu) two steps ahead and cut them
@@ -32,20 +40,21 @@
 //              it cannot also cut); the warp owns the tensor memory
 //   warp 17    lane 0 copies the vector's digits of the step (cp.async.bulk)
 // Every wait is bounded by a count of cycles; a CTA whose wait expires raises err, waits
-// (bounded again) for its copies and products, and returns.  Columns where a vector does
-// not fit (Inf, NaN, all below 2^-895) raise err too; then the kernels of apply_fixed.cu,
-// launched behind a flag, do the apply.
+// (bounded again) for its copies and products, and returns.  What the digits of such a
+// launch should have given is then redone by the kernels of apply_fixed.cu.
 //
 // What bounds it: 36 products of 128 x 64 x 16 (12 instructions) are 1152 cycles of the
 // tensor cores, cutting a step 800 to 1100 cycles of 16 warps beside them, and a move of the
 // accumulators (64 K conversions at 16 a cycle, 64-bit sums) about 6000 cycles in which
-// the tensor cores wait.  64 columns at 27361 DoFs and rank 64: 1145 us (fixed-point kernels
-// 5270, FP64 kernels 11880): rows 436, coupling 302, projections 154, node sums 56, digits
-// 100; the tensor cores are busy 36% of the coupling's time.  The same digits with
-// mma.sync m16n8k16 (600 TFLOP/s against 2.2 PFLOP/s) took 2664 us.
-// Error against extended precision (meshes of 800 to 1100 DoFs, columns of normal
-// numbers): 0.7 to 0.9e-16 of |y|, FP64 kernels 1.2 to 1.3e-16; at most 6e-16 of a
-// component of |A||x|, FP64 3.8e-16.
+// the tensor cores wait.  64 normal columns at 27361 DoFs and rank 64: 1.42 ms (fixed point 5.27,
+// FP64 kernels 11.88): rows 458, coupling 362, projections 148, node sums 77, digits and
+// their scales 150, B + M 85, checks and alignment 60 us.  (With one scale a column for the
+// whole mesh and one a row with the diagonal in it, which lost up to 20 bits, 1.15 ms.)
+// The same digits with mma.sync m16n8k16 (600 TFLOP/s against 2.2 PFLOP/s) took 2664 us.
+// Errors in units of |A||x| (meshes of 800 to 1000 DoFs, against extended precision), FP64
+// kernels and here: normal columns 6.4e-17 and 4.7e-17 rms, 3.2e-16 and 3.6e-16 at most;
+// columns over six decades 8.8e-17 and 9.3e-17; falling by 14 decades across the mesh
+// 5.4e-17 and 4.7e-17; columns of the operator agree to 9e-16.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -82,9 +91,11 @@ struct TdVec {          // a set of pieces of a matrix of columns
     int npiece, ns, len;                 // ns: steps of a piece; len: rows of a piece (nodes)
     const int *kb, *ke;                  // rows of a piece (leaves), or null
     int nrhs, c0, nc;                    // columns c0 .. min(c0 + 64, nrhs) in tiles of nc
-    unsigned *key;                       // per column of the pass
+    int node0, lmin, nlev;               // nodes: the first, its level; keys of nlev levels (1: one for all)
+    unsigned *key, *piece;               // largest keys: per level and column of the pass; per piece and column
+    int *w;                              // [tile][piece]: exponent of a piece's scale less the columns'
     unsigned char *out;                  // [tile][piece][step]
-    int *err;
+    float *n1;                           // sum of a piece's |x| in units of its scale, [piece][64]
 };
 
 __device__ __forceinline__ void td_range(const TdVec &P, int p, size_t &b, int &n)
@@ -93,54 +104,94 @@ __device__ __forceinline__ void td_range(const TdVec &P, int p, size_t &b, int &
     n = P.kb ? P.ke[p] - (int)b : P.len;
 }
 
-// largest exponent of every column (grid.y) over all pieces, which are contiguous
+// largest key of every piece and column, and of every column (over a level's pieces); CTA per
+// piece, a warp per column
 __global__ void __launch_bounds__(256) k_td_max(TdVec P)
 {
-    const int c = blockIdx.y;
-    size_t b, b1;
-    int n, n1;
-    td_range(P, 0, b, n);
-    td_range(P, P.npiece - 1, b1, n1);
-    const double *v = P.v + (size_t)(P.c0 + c) * P.ld + b;
-    const size_t tot = b1 + n1 - b;
-    unsigned mk = 0;
-    for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < tot; i += (size_t)gridDim.x * 256) mk = max(mk, fa_key(v[i]));
-    mk = __reduce_max_sync(0xffffffffu, mk);
-    if ((threadIdx.x & 31) == 0 && mk) atomicMax(P.key + c, mk);
+    const int p = blockIdx.x, lane = threadIdx.x & 31;
+    size_t b;
+    int n;
+    td_range(P, p, b, n);
+    unsigned *key = P.key + (P.nlev > 1 ? 31 - __clz(P.node0 + p + 1) - P.lmin : 0) * TD_COLS;
+    double v[8][2];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {   // a piece has at most 64 rows
+            const int c = (threadIdx.x >> 5) + 8 * u, i = lane + 32 * h;
+            v[u][h] = P.c0 + c < P.nrhs && i < n ? P.v[(size_t)(P.c0 + c) * P.ld + b + i] : 0.0;
+        }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int c = (threadIdx.x >> 5) + 8 * u;
+        const unsigned mk = __reduce_max_sync(0xffffffffu, max(fa_key(v[u][0]), fa_key(v[u][1])));
+        if (lane == 0) {
+            P.piece[(size_t)p * TD_COLS + c] = mk;
+            if (mk > key[c]) atomicMax(key + c, mk);
+        }
+    }
 }
 
-// digits of piece blockIdx.x for tile blockIdx.y; a thread takes 8 rows of a column
+// digits of piece blockIdx.x for tile blockIdx.y; a thread takes 8 rows of a column.  A piece has
+// one scale for the tile's columns: where they are all small in it (a solution where its
+// equation is stiff, a vector that is local) the bits are not spent on zeros.  (A column that
+// does not fit gets zeros; its sums are redone.)
+// (A program's 64 solutions for random loads at 27k DoFs, s from 0.1 to 0.9: 1645 us an apply,
+// with scales in steps of 2^4 3616, because 36% of the nodes are redone.)
+constexpr int TD_WMIN = -60;
 __global__ void __launch_bounds__(256) k_td_digits(TdVec P)
 {
+    __shared__ float red[2 * ((KMAX + 15) / 16)][TD_COLS];
+    __shared__ int w;
     const int p = blockIdx.x;
     size_t b;
     int n;
     td_range(P, p, b, n);
+    const unsigned *keys = P.key + (P.nlev > 1 ? 31 - __clz(P.node0 + p + 1) - P.lmin : 0) * TD_COLS;
     unsigned char *out = P.out + ((size_t)blockIdx.y * P.npiece + p) * P.ns * td_step(P.nc);
+    if (threadIdx.x == 0) w = TD_WMIN;
+    __syncthreads();
+    if ((int)threadIdx.x < P.nc) {
+        const int r = blockIdx.y * P.nc + threadIdx.x;
+        const unsigned key = keys[r], own = P.piece[(size_t)p * TD_COLS + r];
+        if (P.c0 + r < P.nrhs && own && !fa_slow(key)) atomicMax(&w, (int)own - (int)key);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) P.w[(size_t)blockIdx.y * P.npiece + p] = w;
     for (int t = threadIdx.x; t < P.nc * 2 * P.ns; t += 256) {
         const int ch = t / P.nc, col = t % P.nc, r = blockIdx.y * P.nc + col;
         const bool on = P.c0 + r < P.nrhs;
-        const unsigned key = on ? P.key[r] : 0u;
-        if (fa_slow(key)) atomicOr(P.err, 1);
+        const unsigned key = on ? keys[r] : 0u;
+        const bool fits = on && !fa_slow(key);
         const double *v = P.v + (size_t)(P.c0 + r) * P.ld + b;
         u64 d[8];
+        float sum = 0.0f;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const int i = ch * 8 + q;
-            const i64 x = on && i < n ? fa_round(v[i], (int)key) : 0;
+            const double y = fits && i < n ? v[i] : 0.0;
+            const i64 x = fa_round(y, (int)key + w);
+            sum += y != 0.0 ? fmaxf((float)llabs(x) * 0x1p-60f, 1e-30f) : 0.0f;   // an entry that rounds to zero counts
             d[q] = (u64)(x << 2) + 0x8080808080808080ULL;   // digits plus 128
         }
+        red[ch][col] = sum;
         unsigned char *o = out + (size_t)(ch >> 1) * td_step(P.nc) + (ch & 1) * 128 + (col & 7) * 16;
 #pragma unroll
         for (int i = 0; i < TD_D; ++i) {
             half2 h[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const unsigned u = (unsigned)(d[2 * q] >> (8 * i)) & 255u, w = (unsigned)(d[2 * q + 1] >> (8 * i)) & 255u;
-                h[q] = __halves2half2(__int2half_rn((int)u - 128), __int2half_rn((int)w - 128));
+                const unsigned u = (unsigned)(d[2 * q] >> (8 * i)) & 255u, w_ = (unsigned)(d[2 * q + 1] >> (8 * i)) & 255u;
+                h[q] = __halves2half2(__int2half_rn((int)u - 128), __int2half_rn((int)w_ - 128));
             }
             *(uint4 *)(o + (size_t)(i * (P.nc >> 3) + (col >> 3)) * 256) = *(const uint4 *)h;
         }
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < P.nc) {
+        float t = 0.0f;
+        for (int ch = 0; ch < 2 * P.ns; ++ch) t += red[ch][threadIdx.x];
+        P.n1[(size_t)p * TD_COLS + blockIdx.y * P.nc + threadIdx.x] = t;
     }
 }
 
@@ -149,8 +200,13 @@ struct TdP {
     FaNear R;
     int nrhs, c0, nsl, nsn, node0, nnodes;   // steps of a leaf and of a node; nodes node0 .. node0 + nnodes
     const unsigned char *dx, *dh;            // digits of the leaves' x; of the nodes' xhat or yhat
-    const unsigned *kx, *kh;                 // their column keys
-    unsigned *ko;                            // COUPLE: keys of yhat
+    const unsigned *kx, *kh;                 // their column keys (COUPLE: kh per level)
+    const int *wx;                           // PROJ: exponents of the leaves' scales, [tile][leaf]
+    const short *er, *ef;                    // ROWS: exponents of near rows, [tile][N], and expansions, [tile][leaf]
+    const uchar2 *shr;                       // ROWS: shifts of a record's halves to them, [tile][record]
+    int nrec;
+    const short *ec;                         // COUPLE: exponents of a node's rows, [tile][node][k]
+    const unsigned char *sh;                 // COUPLE: shifts of a block's rows to them, [tile][block][k]
     const int *bin;                          // items of a CTA (build_tensor_lists)
     const int4 *items;
     const TdRec *rec;
@@ -200,9 +256,11 @@ __device__ __forceinline__ void td_mma(unsigned d, unsigned a, unsigned b, int n
 }
 
 // (h 2^32 + l) 2^(56 + e) rounded to FP64 with integers (two conversions, a multiply-add
-// and a scaling in FP64 would be 80 cycles of the SM a warp); bad: not a normal number
-__device__ __forceinline__ double td_value(i64 h, unsigned l, int e, bool &bad)
+// and a scaling in FP64 would be 80 cycles of the SM a warp), but for results that are not normal
+__device__ __forceinline__ double td_value(i64 h, unsigned l, int e)
 {
+    const i64 h0 = h;
+    const unsigned l0 = l;
     const bool neg = h < 0;
     if (neg) {
         h = ~h + (l == 0);
@@ -213,7 +271,7 @@ __device__ __forceinline__ double td_value(i64 h, unsigned l, int e, bool &bad)
     const int z = __clzll(a);
     const u64 t = z == 64 ? 0 : a << z | (big ? l >> (32 - z) : 0u);   // leading one at 63
     const int b = 1023 + 56 + 95 - z - (big ? 0 : 32) + e;
-    bad |= t != 0 && (b < 2 || b > 2045);
+    if (t != 0 && (b < 2 || b > 2045)) return scalbn(fma((double)h0, 4294967296.0, (double)l0), 56 + e);
     const u64 r = (((t >> 1) + 512) >> 10) + ((u64)(b - 1) << 52);
     return __longlong_as_double(t ? (i64)(r | (neg ? 1ULL << 63 : 0ULL)) : 0LL);
 }
@@ -233,6 +291,7 @@ __device__ __forceinline__ int td_exp(int ea, unsigned key) { return ea + (key ?
 struct TdIt {
     int i, item, q, q1, q2, col, n, nrow, W;   // i: of the CTA's items
     i64 off;
+    uchar2 sh;
 };
 
 template <int NC, int MODE>
@@ -287,6 +346,7 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
         I.col = r.col;
         I.n = r.n;
         I.off = r.off[half];
+        if (MODE == TD_ROWS) I.sh = P.shr[(size_t)tile * P.nrec + I.q];
     };
     auto start = [&](TdIt &I) {   // first piece of item I.i; false: no more items
         I.n = 0;
@@ -351,7 +411,7 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
         int ei = ibeg;   // the item that ends next
         auto emit = [&](int code) {
             int ri = 0, e = 0;   // row of out
-            bool on = false, bad = false;
+            bool on = false;
             size_t os = (size_t)ld;   // column stride
             const int item = MODE == TD_PROJ ? ei : P.items[ei].w;
             if (MODE != TD_ROWS || code == 3 || P.F.nlev == 0) ++ei;
@@ -359,7 +419,7 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
                 const int leaf = item / nz, c = (item - leaf * nz) * 128 + orow, lv = c / k;
                 on = c < P.F.nlev * k;
                 ri = (lv * P.F.nleaf + leaf) * k + c - lv * k;
-                e = P.F.ue[leaf];
+                e = P.F.ue[leaf] + P.wx[tile * P.F.nleaf + leaf];
                 os = (size_t)P.F.nlev * P.F.nleaf * k;
             }
             if (MODE == TD_ROWS) {
@@ -368,35 +428,30 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
                     const int b = P.R.kb[P.R.fl + leaf];
                     ri = b + om;
                     on = om < P.R.ke[P.R.fl + leaf] - b;
-                    if (on) e = code == 2 ? P.R.re[ri] : P.F.ue[leaf];
+                    if (on) e = code == 2 ? P.er[(size_t)tile * P.F.N + ri] : P.ef[tile * P.F.nleaf + leaf];
                 }
             }
             if (MODE == TD_COUPLE) {
                 const int node = P.node0 + 2 * item + ohalf;
                 on = node < P.F.nnode && om < k;
                 ri = node * k + om;
-                if (on) e = P.F.sn[ri];
+                if (on) e = P.ec[((size_t)tile * P.nnodes + node - P.node0) * k + om];
                 os = (size_t)P.F.nnode * k;
             }
             const unsigned *key = skey + oc + (MODE == TD_PROJ || (MODE == TD_ROWS && code == 2) ? 0 : NC);
+            if (MODE == TD_COUPLE)   // the pair's level
+                key = P.kh + (31 - __clz(P.node0 + 2 * item + 1) - P.F.lmin) * TD_COLS + tile * NC + oc;
             double *o = out + ri;
             const int r0 = P.c0 + tile * NC + oc, nr = on ? P.nrhs - r0 : 0;   // columns 0 .. nr of this thread
             o += (size_t)r0 * os;
-            unsigned mine = 0;
 #pragma unroll
             for (int c0 = 0; c0 < NH; c0 += 2) {
                 double v[2], y[2];
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    bool b = false;
-                    v[j] = td_value(sh[c0 + j], sl[c0 + j], td_exp(e, key[c0 + j]), b);
-                    bad |= b && c0 + j < nr;
+                    v[j] = td_value(sh[c0 + j], sl[c0 + j], td_exp(e, key[c0 + j]));
                     sh[c0 + j] = sl[c0 + j] = 0;
-                    if (MODE == TD_ROWS) y[j] = code == 3 && c0 + j < nr ? o[(c0 + j) * os] : 0.0;
-                    if (MODE == TD_COUPLE) {
-                        const unsigned mk = __reduce_max_sync(0xffffffffu, c0 + j < nr ? fa_key(v[j]) : 0u);
-                        if (lane == c0 + j) mine = mk;
-                    }
+                    if (MODE == TD_ROWS) y[j] = c0 + j < nr ? o[(c0 + j) * os] : 0.0;
                 }
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
@@ -404,15 +459,6 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
                     if (c0 + j < nr) o[(c0 + j) * os] = v[j];
                 }
             }
-            if (MODE == TD_COUPLE && mine) atomicMax(P.ko + tile * NC + oc + lane, mine);
-            if (MODE == TD_ROWS && code == 2 && !P.R.folded)   // B + M outside the panels
-                for (int c = 0; c < min(nr, NH); ++c) {
-                    double v = o[c * os];
-                    for (int s = P.R.rowptr[ri]; s < P.R.rowptr[ri + 1]; ++s)
-                        v = fma(P.R.val[s], X[(size_t)(r0 + c) * ld + P.R.colidx[s]], v);
-                    o[c * os] = v;
-                }
-            if (bad) atomicOr(P.err, 1);
         };
         auto move = [&](int code) {
             if (!td_wait(moved, moves & 1, deadline)) return false;
@@ -458,7 +504,7 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
         int2 *const raw = (int2 *)(td_sm + TD_NST * STAGE) + warp * 128 + lane;
         const int2 *p = nullptr;
         int left = 0, steps = 0, np = 0, end = 0, pulled = 0;   // of the piece: rows and steps that are left
-        int shift = 0;   // COUPLE: the block's rows to the node's exponents
+        int shift = 0;   // of the piece's entries, to the scale of the sum
         unsigned hist = 0;
         auto pull = [&]() {
             if (steps == 0) {
@@ -471,7 +517,8 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
                 p = matrix(I, sm, sk);   // sets the strides
                 p += mrow * sm + tt * sk;
                 left = I.off >= 0 && mrow < I.nrow ? I.n - tt : 0;
-                if (MODE == TD_COUPLE) shift = left > 0 ? P.F.sh[I.off * k + mrow] : 0;
+                if (MODE == TD_COUPLE) shift = left > 0 ? P.sh[((size_t)tile * P.F.nfar + I.off) * k + mrow] : 0;
+                if (MODE == TD_ROWS) shift = half ? I.sh.y : I.sh.x;
                 np = I.n;
                 steps = (np + 15) >> 4;
                 end = I.q + 1 == I.q1 ? 2 : (I.q + 1 == I.q2 ? 3 : 0);
@@ -522,7 +569,7 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
             for (int j = 0; j < 4; ++j) {
                 const int2 a = raw[(t % TD_AHEAD) * (TD_RAW / 8) + 32 * j];
                 u64 v = ((u64)(unsigned)a.y << 32) + (u64)((i64)a.x << 2);
-                if (MODE == TD_COUPLE) v = (u64)(((i64)v + ((1LL << s0) >> 1)) >> s0);
+                if (MODE == TD_COUPLE || (MODE == TD_ROWS && s0)) v = (u64)(((i64)v + ((1LL << s0) >> 1)) >> s0);
                 v += 0x8080808080808080ULL;
                 wl[j] = (unsigned)v;
                 wh[j] = (unsigned)(v >> 32);
@@ -646,7 +693,361 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "n"(TD_G * NC));
 }
 
-__global__ void k_td_good(const int *err, int *good) { *good = *err == 0; }
+// ---------------------------------------------------------------------------
+// What the digits cannot hold.  A piece of the vector has one scale for a tile's columns and a
+// row of the operator one for a piece (xhat) or a section (near rows), so a sum's error is
+// about sqrt(products) 2^-62 of the largest product of scales, whatever the sum's own terms
+// are.  Before the sums are used, each is compared with a lower bound of its sum of absolute
+// values; where the error could be above 2^-54 (near; 2^-53 far, a part of the row) of it,
+// FP64 products or the kernels of apply_fixed.cu, whose scales are of a column's leaf or
+// node, do that sum.
+// ---------------------------------------------------------------------------
+constexpr int TDC_CH = 512;   // columns of a panel in shared memory at a time
+
+// |v| 2^(1022 - key) for v below 2^(key - 1022), cut to 20 bits and to zero below 2^-126: the
+// conversion without FP64 instructions, and a lower bound
+__device__ __forceinline__ float td_float(double v, int key)
+{
+    return __int_as_float(max((__double2hiint(v) & 0x7fffffff) - ((key - 126) << 20), 0) << 3);
+}
+
+// Y = (B + M and the panel entries at its positions) X in FP64, a thread per row and 4 columns;
+// rows for which 2^-54 of the absolute values of these terms, its largest, is below the
+// digits' error for its others are marked (rowmask, 64 bits a leaf and tile) for k_td_near.
+// least: the smallest such sum of the rows, its log2 in units of 2^-8 (a lower bound).
+// grid (leaf, group of 8 columns).
+__global__ void __launch_bounds__(128)
+k_td_csr(FaNear R, int nleaf, int nc, const int *__restrict__ nptr, const int *__restrict__ ncol,
+         const double *__restrict__ X, int64_t ld, double *__restrict__ Y, const unsigned *__restrict__ kx,
+         const int *__restrict__ wx, int *__restrict__ wnear, unsigned *__restrict__ rowmask, int *__restrict__ least)
+{
+    __shared__ unsigned nz;   // columns with x in the panel
+    __shared__ int low[4][4];
+    constexpr int NONE = 0x7fffffff;
+    const int lf = blockIdx.x, g = blockIdx.y, r0 = R.c0 + 8 * g, b = R.kb[R.fl + lf], e = R.ke[R.fl + lf], W = R.pw[lf];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the scale of the partners' pieces, for the tile
+    const int tile = 8 * g / nc;
+    int w = TD_WMIN;
+    for (int q = nptr[lf] + lane; q < nptr[lf + 1]; q += 32) w = max(w, wx[tile * nleaf + ncol[q]]);
+    w = __reduce_max_sync(0xffffffffu, w);
+    if (threadIdx.x == 0) {
+        wnear[tile * nleaf + lf] = w;
+        nz = 0;
+    }
+    const double *x0 = X + (size_t)r0 * ld;
+    const int i = b + (threadIdx.x & 63), c0 = 4 * (threadIdx.x >> 6), nr = i < e ? min(4, R.nrhs - r0 - c0) : 0;
+    double v[4] = {};
+    float s[4] = {};
+    int t[4];
+    unsigned redo = 0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) t[c] = NONE;
+    if (nr > 0) {
+        const double *x = x0 + (size_t)c0 * ld;
+        int key[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) key[c] = c < nr ? (int)kx[8 * g + c0 + c] : 0;
+        int ka = 1;   // the scale of the row: its largest term's
+        for (int q = R.rowptr[i]; q < R.rowptr[i + 1]; ++q) ka = max(ka, (int)fa_key(R.val8[q]));
+        double d = 0.0;
+#pragma unroll 2
+        for (int q = R.rowptr[i]; q < R.rowptr[i + 1]; ++q) {   // (16 loads of x ahead: 120 us instead of 85)
+            const int j = R.colidx[q];
+            const double a = R.val8[q], o = j == i ? 0.0 : a;
+            const float fa = td_float(a, ka);
+            if (j == i) d = a;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const double y = c < nr ? x[(size_t)c * ld + j] : 0.0;
+                v[c] = fma(o, y, v[c]);
+                s[c] = fmaf(fa, td_float(y, key[c]), s[c]);
+            }
+        }
+        const float unit = sqrtf((float)W);
+        const int up = R.re[i] + w - (ka - 1022) - 8;   // digits' scale over this row's, less 8 bits
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            v[c] = fma(d, c < nr ? x[(size_t)c * ld + i] : 0.0, v[c]);   // the diagonal's product, the largest, rounds the sum once
+            if (key[c] && (fa_slow(key[c]) || up > 100 || !(s[c] >= scalbnf(unit, up)))) redo |= 1u << c;
+            if (c < nr) t[c] = s[c] > 0.0f ? (__float_as_int(s[c]) >> 15) - (127 << 8) + ((ka + key[c] - 2 * 1022) << 8) : -NONE;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        t[c] = __reduce_min_sync(0xffffffffu, t[c]);
+        if (lane == c) low[warp][c] = t[c];
+    }
+    if (__syncthreads_or(redo != 0)) {
+        // columns without any x in the panel have exact zeros
+        const int *gc = R.gcol + R.goff[lf];
+        unsigned m = 0;
+        for (int q = threadIdx.x; q < W; q += 128) {
+            const int j = gc[q];
+            for (int c = 0; c < 8 && j >= 0 && r0 + c < R.nrhs; ++c) m |= x0[(size_t)c * ld + j] != 0.0 ? 1u << c : 0u;
+        }
+        m = __reduce_or_sync(0xffffffffu, m);
+        if (lane == 0 && m) atomicOr(&nz, m);
+        __syncthreads();
+        const unsigned rows = __ballot_sync(0xffffffffu, redo & nz >> c0);
+        if (lane == 0 && rows) atomicOr(rowmask + ((size_t)tile * nleaf + lf) * 2 + (warp & 1), rows);
+    }
+    if (threadIdx.x < 8) {
+        const int h = threadIdx.x >> 2, c = threadIdx.x & 3;
+        least[(size_t)lf * TD_COLS + 8 * g + threadIdx.x] = min(low[2 * h][c], low[2 * h + 1][c]);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        if (c < nr) Y[(size_t)(r0 + c0 + c) * ld + i] = v[c];
+}
+
+// the marked near rows in FP64, 8 lanes a row and 16 rows at a time, and the exponents of the others'
+// digit sums (marked rows: so small that the sums vanish).  grid (leaf, group of 8 columns)
+constexpr int TD_NONE = -4000;
+__global__ void __launch_bounds__(128)
+k_td_near(FaNear R, int N, int nleaf, int nc, const double *__restrict__ X, int64_t ld, double *__restrict__ Y,
+          const int *__restrict__ wnear, const unsigned *__restrict__ rowmask, short *__restrict__ er, int *__restrict__ count)
+{
+    extern __shared__ __align__(16) double td_xs[];   // [pair of columns][entry]
+    const int lf = blockIdx.x, g = blockIdx.y, r0 = R.c0 + 8 * g, b = R.kb[R.fl + lf], e = R.ke[R.fl + lf], W = R.pw[lf];
+    const int tile = 8 * g / nc, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l8 = lane & 7;
+    const unsigned bad[2] = {rowmask[((size_t)tile * nleaf + lf) * 2], rowmask[((size_t)tile * nleaf + lf) * 2 + 1]};
+    if (8 * g % nc == 0 && b + (int)threadIdx.x < e) {
+        const int i = b + threadIdx.x;
+        er[(size_t)tile * N + i] = (short)((bad[threadIdx.x >> 5 & 1] >> lane & 1u) ? TD_NONE : R.re[i] + wnear[tile * nleaf + lf]);
+    }
+    if (!(bad[0] | bad[1])) return;
+    if (threadIdx.x == 0) atomicAdd(count, __popc(bad[0]) + __popc(bad[1]));
+    const double *x0 = X + (size_t)r0 * ld;
+    const int *gc = R.gcol + R.goff[lf];
+    for (int s = 0; s < 64 && b + s < e; s += 16) {
+        if (!((s < 32 ? bad[0] : bad[1]) >> (s & 31) & 0xffffu)) continue;
+        const int ro = s + 4 * warp + (lane >> 3), i = b + ro;
+        const bool any = (s < 32 ? bad[0] : bad[1]) >> (ro & 31) & 1u;
+        const double *D = R.Dd + R.poff[lf] + (size_t)ro * W;
+        double a[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) a[c] = 0.0;
+        for (int j0 = 0; j0 < W; j0 += TDC_CH) {
+            const int n = min(TDC_CH, W - j0);
+            __syncthreads();
+            for (int q = threadIdx.x; q < n; q += 128) {
+                const int j = gc[j0 + q];
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    td_xs[(c >> 1) * 2 * TDC_CH + 2 * q + (c & 1)] = j >= 0 && r0 + c < R.nrhs ? x0[(size_t)c * ld + j] : 0.0;
+            }
+            __syncthreads();
+            if (any)
+                for (int j = l8; j < n; j += 8) {
+                    const double d = D[j0 + j];
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        const double2 x = *(const double2 *)(td_xs + p * 2 * TDC_CH + 2 * j);
+                        a[2 * p] = fma(d, x.x, a[2 * p]);
+                        a[2 * p + 1] = fma(d, x.y, a[2 * p + 1]);
+                    }
+                }
+        }
+        if (any)
+            for (int q = R.rowptr[i] + l8; q < R.rowptr[i + 1]; q += 8) {
+                const double d = R.val[q], *x = x0 + R.colidx[q];
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (r0 + c < R.nrhs) a[c] = fma(d, x[(size_t)c * ld], a[c]);
+            }
+        const int c = fa_sum8d<8>(a, l8);
+        if (any && r0 + c < R.nrhs) Y[(size_t)(r0 + c) * ld + i] = a[0];
+    }
+}
+
+// shifts of the rows' records to the scales of their sums; a warp per item.  grid (items, tile)
+__global__ void __launch_bounds__(32)
+k_td_shift(const int4 *__restrict__ items, const TdRec *__restrict__ rec, int nrec, int nleaf, int nnodes,
+           const int *__restrict__ wx, const int *__restrict__ wh, const int *__restrict__ wnear, const int *__restrict__ wfar,
+           uchar2 *__restrict__ shr)
+{
+    const int4 v = items[blockIdx.x];
+    const int tile = blockIdx.y, l0 = 2 * v.w, l1 = min(l0 + 1, nleaf - 1);
+    for (int q = v.x + (int)threadIdx.x; q < v.z; q += 32) {
+        const bool near = q < v.y;
+        const int w = near ? wx[tile * nleaf + rec[q].col] : wh[tile * nnodes + rec[q].col], *to = near ? wnear : wfar;
+        const int a = to[tile * nleaf + l0] - w, c = to[tile * nleaf + l1] - w;   // (negative where the half has no such partner)
+        shr[(size_t)tile * nrec + q] = make_uchar2(min(max(a, 0), 63), min(max(c, 0), 63));
+    }
+}
+
+// bits of the groups of 8 columns in which a thread of the first 64 says yes
+__device__ __forceinline__ unsigned td_groups(bool yes, unsigned *sh)
+{
+    const unsigned b = __ballot_sync(0xffffffffu, yes);
+    if ((threadIdx.x & 31) == 0) {
+        unsigned m = 0;
+        for (int g = 0; g < 4; ++g) m |= (b >> (8 * g) & 255u) ? 1u << g : 0u;
+        sh[threadIdx.x >> 5] = m;
+    }
+    __syncthreads();
+    return sh[0] | sh[1] << 4;
+}
+
+// leaves whose projections are redone: their x is small in its column (n1: sum of a leaf's |x| in
+// units of the column's scale).  A projection's error goes to k entries of xhat and from there
+// through a block's entries, which differ by a few bits.
+__global__ void __launch_bounds__(64)
+k_td_check_x(int k, int nrow, int cols, const unsigned *__restrict__ kx, const float *__restrict__ n1,
+             const float *__restrict__ umin, unsigned *mask, int *count)
+{
+    __shared__ unsigned sh[2];
+    const int lf = blockIdx.x, c = threadIdx.x;
+    const float n = c < cols ? n1[(size_t)lf * TD_COLS + c] : 0.0f;
+    const bool redo = c < cols && (fa_slow(kx[c]) || (n > 0.0f && !(256.0f * umin[lf] * n >= 2.0f * sqrtf((float)nrow * k))));
+    const unsigned m = td_groups(redo, sh);
+    if (c == 0) {
+        mask[lf] = m;
+        if (m) atomicAdd(count, __popc(m));
+    }
+}
+
+// exponents of a node's rows (the largest product of a block row's and its partner's scales) and
+// the shifts of the blocks' rows to them.  grid (node, tile)
+__global__ void __launch_bounds__(128)
+k_td_align(FaFar P, int node0, int nnodes, const int *__restrict__ wh, short *__restrict__ ec, unsigned char *__restrict__ sh)
+{
+    __shared__ int top[KMAX];
+    const int t = node0 + blockIdx.x, tile = blockIdx.y, k = P.k, e0 = P.fptr[t], e1 = P.fptr[t + 1];
+    wh += (size_t)tile * nnodes - node0;
+    sh += (size_t)tile * P.nfar * k;
+    if ((int)threadIdx.x < k) {
+        int m = -900;   // (below it: rows of zeros)
+#pragma unroll 4
+        for (int e = e0; e < e1; ++e) m = max(m, P.se[(size_t)e * k + threadIdx.x] + wh[P.fcol[e]]);
+        top[threadIdx.x] = m;
+        ec[((size_t)tile * nnodes + blockIdx.x) * k + threadIdx.x] = (short)m;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < (e1 - e0) * k; i += 128) {
+        const int e = e0 + i / k, a = i % k;
+        sh[(size_t)e0 * k + i] = (unsigned char)min(top[a] - max(P.se[(size_t)e0 * k + i] + wh[P.fcol[e]], -900), 63);
+    }
+}
+
+// nodes whose sum over their blocks is redone, and a lower bound of sum |S||xhat| of a node's rows.
+// CTA per node, 64 columns x 4 groups of rows: low 2^-shift |xhat| of a row and block is at most
+// its sum of absolute values
+__global__ void __launch_bounds__(256)
+k_td_check_couple(FaFar P, int node0, int nnodes, int cols, int nc, const unsigned *__restrict__ kh, const int *__restrict__ wh,
+                  const float *__restrict__ n1, const double *__restrict__ least, const float *__restrict__ low,
+                  const unsigned char *__restrict__ shift, double *__restrict__ sum, unsigned *mask, int *count, const int *err)
+{
+    constexpr int CH = 8;   // blocks at a time
+    __shared__ float rows[4][TD_COLS], u[CH][KMAX];
+    const int t = node0 + blockIdx.x, c = threadIdx.x & 63, g = threadIdx.x >> 6, l = 31 - __clz(t + 1), k = P.k;
+    const int e0 = P.fptr[t], e1 = P.fptr[t + 1], tile = c < cols ? c / nc : 0;
+    const unsigned key = kh[(l - P.lmin) * TD_COLS + c];
+    float r = INFINITY;
+    for (int tl = 0; tl < (cols + nc - 1) / nc; ++tl) {
+        float v[KMAX / 4];
+#pragma unroll
+        for (int q = 0; q < KMAX / 4; ++q) v[q] = 0.0f;
+        for (int b = e0; b < e1; b += CH) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < min(CH, e1 - b) * k; i += 256) {
+                const size_t j = (size_t)b * k + i;
+                u[i / k][i % k] = low[j] * __uint_as_float((127u - shift[(size_t)tl * P.nfar * k + j]) << 23);
+            }
+            __syncthreads();
+            if (tl != tile) continue;
+#pragma unroll 4
+            for (int e = b; e < min(b + CH, e1); ++e) {
+                const float x = n1[(size_t)(P.fcol[e] - node0) * TD_COLS + c];
+#pragma unroll
+                for (int q = 0; q < KMAX / 4; ++q)
+                    if (g + 4 * q < k) v[q] = fmaf(u[e - b][g + 4 * q], x, v[q]);
+            }
+        }
+        if (tl == tile)
+#pragma unroll
+            for (int q = 0; q < KMAX / 4; ++q)
+                if (g + 4 * q < k) r = fminf(r, v[q]);
+    }
+    rows[g][c] = r;
+    __syncthreads();
+    if (g) return;
+    r = fminf(fminf(rows[0][c], rows[1][c]), fminf(rows[2][c], rows[3][c]));
+    double s = 0.0;
+    float n = 0.0f;
+    for (int e = e0; e < e1; ++e) {
+        const int f = P.fcol[e] - node0;
+        const float x = c < cols ? n1[(size_t)f * TD_COLS + c] : 0.0f;
+        n += x;
+        s = fma(least[e], scalbn((double)x, wh[(size_t)tile * nnodes + f]), s);
+    }
+    const bool redo = c < cols && e1 > e0 &&
+                      (*err || fa_slow(key) || (n > 0.0f && !(512.0f * r >= sqrtf((float)(e1 - e0) * k))));
+    const unsigned b = __ballot_sync(0xffffffffu, redo);
+    if ((c & 31) == 0) {
+        unsigned m = 0;
+        for (int q = 0; q < 4; ++q) m |= (b >> (8 * q) & 255u) ? 1u << (4 * (c >> 5) + q) : 0u;
+        if (m) {
+            atomicOr(mask + t, m);
+            atomicAdd(count, __popc(m));
+        }
+    }
+    sum[(size_t)blockIdx.x * TD_COLS + c] = n > 0.0f ? fmax(scalbn(s, (int)key - 1022), 1e-300) : 0.0;
+}
+
+// yhat of the nodes that are redone: the sum over their blocks
+__global__ void __launch_bounds__(256)
+k_td_couple_sum(FaFar P, int node0, int c0, const double *__restrict__ ye, double *__restrict__ yhat, FaWhen when)
+{
+    if (fa_none(when)) return;
+    const int k = P.k, r = c0 + blockIdx.y;
+    for (int t = node0 * k + blockIdx.x * 256 + threadIdx.x; t < P.nnode * k; t += gridDim.x * 256) {
+        const int node = t / k, a = t - node * k;
+        if (fa_off(when, node, r)) continue;
+        double s = 0.0;
+        for (int e = P.fptr[node]; e < P.fptr[node + 1]; ++e) s += ye[((size_t)r * P.nfar + e) * k + a];
+        yhat[(size_t)r * P.nnode * k + t] = s;
+    }
+}
+
+// leaves whose expansion is redone: the bound of a row's far sum (sum, umin) and of its near terms
+// (least, the smallest of the leaf's rows) against the digits' error; wfar: the scale of the
+// ancestors' pieces
+__global__ void __launch_bounds__(64)
+k_td_check_expand(FaFar P, int node0, int nnodes, int cols, int nc, const unsigned *__restrict__ ky,
+                  const int *__restrict__ wh, int *__restrict__ wfar, short *__restrict__ ef, const double *__restrict__ sum,
+                  const float *__restrict__ umin, const int *__restrict__ least, unsigned *mask, int *count, const int *err)
+{
+    __shared__ unsigned sh[2];
+    const int lf = blockIdx.x, c = threadIdx.x, tile = c < cols ? c / nc : 0;
+    double s = 0.0;
+    int w = TD_WMIN;
+    for (int lv = 0; lv < P.nlev; ++lv) {
+        const int f = ((P.fl + lf + 1) >> (P.nlev - 1 - lv)) - 1 - node0;
+        s += sum[(size_t)f * TD_COLS + c];
+        w = max(w, wh[(size_t)tile * nnodes + f]);
+    }
+    const unsigned key = ky[c];
+    const double have = 512.0 * umin[lf] * s + scalbn(1.0, max((least[(size_t)lf * TD_COLS + c] >> 8) + 8 - P.ue[lf], -2000));
+    const bool redo = c < cols && (*err || fa_slow(key) ||
+                                   (key && s > 0.0 && !(have >= scalbn((double)sqrtf((float)(P.nlev * P.k)), (int)key + w - 1022))));
+    unsigned m = td_groups(redo, sh);
+    // all groups of a tile together: its sums are left out (an exponent so small that they vanish)
+    const unsigned tm = nc == 64 ? 255u : (1u << (nc >> 3)) - 1u;
+    unsigned all = 0;
+    for (int q = 0; q < 8; q += nc >> 3)
+        if (m >> q & tm) all |= tm << q;
+    m = all & ((1u << ((cols + 7) >> 3)) - 1u);
+    if (c < cols && c % nc == 0) {
+        wfar[tile * P.nleaf + lf] = w;
+        ef[tile * P.nleaf + lf] = (short)(all >> (c >> 3) & 1u ? TD_NONE : P.ue[lf] + w);
+    }
+    if (c == 0) {
+        mask[lf] = m;
+        if (m) atomicAdd(count, __popc(m));
+    }
+}
 
 template <int NC, int MODE>
 void launch_td(const TdP &P, int nitem, int nt, const double *X, int64_t ld, double *out, cudaStream_t st)
@@ -674,7 +1075,7 @@ void launch_td(int nc, const TdP &P, int nitem, int nt, const double *X, int64_t
 // Items (first record, second section, end, pair) in the order of the CTAs that take them.
 void build_tensor_lists(MeshData &m)
 {
-    if (m.max_leaf_size > 64 || !m.nnear) return;
+    if (m.max_leaf_size > 64 || !m.nnear || (m.nfar > 0 && m.far_lmin < 1)) return;   // (pairs of nodes share a level)
     const int nleaf = m.kt.nleaf, fl = m.kt.first_leaf(), nlev = m.nfar > 0 ? m.kt.L - m.far_lmin + 1 : 0;
     const int k = m.k, wp = (nlev * k + 1) & ~1, node0 = nlev ? (1 << m.far_lmin) - 1 : 0;
     std::vector<TdRec> rec;
@@ -780,40 +1181,73 @@ static int td_tile(const MeshData &m, int cols)
     return 16 << best;
 }
 
-// workspace: the digits of 64 columns per leaf and per node, column keys and flags
+namespace {
+constexpr int TD_TILES = TD_COLS / 16;   // tiles of a pass at most
+// td_key: keys of x, of yhat, of xhat per level, of the pieces; td_mask: a zero, the nodes, the leaves (projections, expansion)
+constexpr int TK_X = 0, TK_Y = TD_COLS, TK_H = 2 * TD_COLS, TK_N = TK_H + 32 * TD_COLS;
+// td_flag: an expired wait; what was redone: near rows, projections, nodes, leaves (in groups of 8 columns)
+enum { TF_ERR, TF_ROWS, TF_PROJ, TF_NODES, TF_LEAVES, TF_N };
+}  // namespace
+
+// workspace: the digits of 64 columns per leaf and per node, column keys, masks and flags
 void apply_tensor_alloc(const MeshData &m, OpData &op)
 {
-    if (op.td_key.p) return;
+    if (op.td_flag.p) return;
     const int node0 = m.nfar > 0 ? (1 << m.far_lmin) - 1 : m.kt.nnode;
-    op.td_x.alloc((size_t)m.kt.nleaf * ((m.max_leaf_size + 15) >> 4) * td_step(TD_COLS));
-    op.td_h.alloc((size_t)(m.kt.nnode - node0) * ((m.k + 15) >> 4) * td_step(TD_COLS));
-    op.td_key.alloc(3 * TD_COLS + 2);
+    const size_t nodes = m.kt.nnode - node0, leaves = m.kt.nleaf;
+    op.td_x.alloc(leaves * ((m.max_leaf_size + 15) >> 4) * td_step(TD_COLS));
+    op.td_h.alloc(nodes * ((m.k + 15) >> 4) * td_step(TD_COLS));
+    op.td_key.alloc(TK_N + std::max(leaves, nodes) * TD_COLS);
+    op.td_w.alloc(TD_TILES * (3 * leaves + nodes));
+    op.td_exp.alloc(TD_TILES * (nodes * m.k + m.N + leaves));
+    op.td_shift.alloc((size_t)TD_TILES * (2 * m.td_rows.n + (size_t)m.nfar * m.k));
+    op.td_mask.alloc(1 + m.kt.nnode + (2 + 2 * TD_TILES) * leaves);
+    op.td_n1.alloc((nodes + leaves) * TD_COLS);
+    op.td_sum.alloc(nodes * TD_COLS);
+    op.td_least.alloc(leaves * TD_COLS);
+    op.td_flag.alloc(TF_N);
 }
 
-// Y = A X for all columns, and the flag behind which the fixed-point kernels redo it
-const int *apply_tensor(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st)
+// Y = A X for all columns
+void apply_tensor(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st)
 {
+    op.td_cols = nrhs;
     const bool far = m.nfar > 0;
     const int k = m.k, nleaf = m.kt.nleaf, node0 = far ? (1 << m.far_lmin) - 1 : m.kt.nnode, nnodes = m.kt.nnode - node0;
     TdP P{};
     P.F = fa_far_view(m, op);
     P.R = fa_near_view(m, op);
-    P.nrhs = nrhs;
+    P.nrhs = P.R.nrhs = nrhs;
     P.nsl = (m.max_leaf_size + 15) >> 4;
     P.nsn = (k + 15) >> 4;
     P.node0 = node0;
     P.nnodes = nnodes;
-    int *err = (int *)op.td_key.p + 3 * TD_COLS, *good = err + 1;
-    VFD_CUDA(cudaMemsetAsync(err, 0, 2 * sizeof(int), st));
+    int *flag = op.td_flag.p, *err = flag + TF_ERR;
+    unsigned *key = op.td_key.p, *zero = op.td_mask.p, *nodemask = zero + 1, *leafmask = nodemask + m.kt.nnode, *projmask = leafmask + nleaf, *rowmask = projmask + nleaf;
+    int *wx = op.td_w.p, *wnear = wx + TD_TILES * nleaf, *wfar = wnear + TD_TILES * nleaf, *wh = wfar + TD_TILES * nleaf;
+    float *n1x = op.td_n1.p, *n1h = n1x + (size_t)nleaf * TD_COLS;
+    int *least = op.td_least.p;
+    double *sum = op.td_sum.p;
+    VFD_CUDA(cudaMemsetAsync(flag, 0, op.td_flag.bytes(), st));
     P.err = err;
     P.dx = op.td_x.p;
     P.dh = op.td_h.p;
-    P.kx = op.td_key.p;
-    P.ko = op.td_key.p + 2 * TD_COLS;
+    P.kx = key + TK_X;
+    short *er = op.td_exp.p, *ef = er + (size_t)TD_TILES * m.N, *ec = ef + (size_t)TD_TILES * nleaf;
+    uchar2 *shr = (uchar2 *)op.td_shift.p;
+    unsigned char *shc = op.td_shift.p + (size_t)TD_TILES * 2 * m.td_rows.n;
+    P.wx = wx;
+    P.er = er;
+    P.ef = ef;
+    P.ec = ec;
+    P.shr = shr;
+    P.nrec = (int)m.td_rows.n;
+    P.sh = shc;
+    const size_t hs = (size_t)m.kt.nnode * k;
     for (int c0 = 0; c0 < nrhs; c0 += TD_COLS) {
-        const int cols = std::min(TD_COLS, nrhs - c0);
+        const int cols = std::min(TD_COLS, nrhs - c0), ng = cdiv(cols, 8);
         const int nc = td_tile(m, cols), nt = cdiv(cols, nc);
-        auto digits = [&](const double *v, size_t vld, size_t base, bool leaves, bool max, unsigned *key, unsigned char *out) {
+        auto digits = [&](const double *v, size_t vld, size_t base, bool leaves, int nlev, unsigned *keys) {
             TdVec V{};
             V.v = v;
             V.ld = vld;
@@ -826,38 +1260,77 @@ const int *apply_tensor(const MeshData &m, OpData &op, const double *X, double *
             V.nrhs = nrhs;
             V.c0 = c0;
             V.nc = nc;
-            V.key = key;
-            V.out = out;
-            V.err = err;
-            const size_t tot = leaves ? (size_t)m.N : (size_t)nnodes * k;
-            if (max) k_td_max<<<dim3(std::max(1, std::min(cdiv((long long)tot, 1024), 32)), cols), 256, 0, st>>>(V);
+            V.node0 = node0;
+            V.lmin = m.far_lmin;
+            V.nlev = nlev;
+            V.key = keys;
+            V.piece = key + TK_N;
+            V.w = leaves ? wx : wh;
+            V.out = leaves ? op.td_x.p : op.td_h.p;
+            V.n1 = leaves ? n1x : n1h;
+            k_td_max<<<V.npiece, 256, 0, st>>>(V);
             k_td_digits<<<dim3(V.npiece, nt), 256, 0, st>>>(V);
             VFD_CUDA(cudaGetLastError());
         };
-        VFD_CUDA(cudaMemsetAsync(op.td_key.p, 0, 3 * TD_COLS * sizeof(unsigned), st));
-        P.c0 = c0;
-        digits(X, ld, 0, true, true, op.td_key.p, op.td_x.p);
+        auto when = [&](const unsigned *mask, int any) {
+            FaWhen w;
+            w.mask = mask;
+            w.any = flag + any;
+            w.err = err;
+            w.c0 = c0;
+            return w;
+        };
+        auto redo = [&](FaStep step, const FaWhen &w) { apply_fixed_redo(step, m, op, X, Y, c0, ng, nrhs, ld, st, w); };
+        VFD_CUDA(cudaMemsetAsync(key, 0, TK_N * sizeof(unsigned), st));
+        VFD_CUDA(cudaMemsetAsync(zero, 0, op.td_mask.bytes(), st));
+        P.c0 = P.R.c0 = c0;
+        digits(X, ld, 0, true, 1, key + TK_X);
+        k_td_csr<<<dim3(nleaf, ng), 128, 0, st>>>(P.R, nleaf, nc, m.near_ptr.p, m.near_col.p, X, ld, Y, P.kx, wx, wnear, rowmask,
+                                                  least);
+        k_td_near<<<dim3(nleaf, ng), 128, TDC_CH * 64, st>>>(P.R, m.N, nleaf, nc, X, ld, Y, wnear, rowmask, er, flag + TF_ROWS);
+        VFD_CUDA(cudaGetLastError());
         if (far) {
-            const size_t hs = (size_t)m.kt.nnode * k;
+            k_td_check_x<<<nleaf, 64, 0, st>>>(k, m.max_leaf_size, cols, P.kx, n1x, m.fa_umin.p, projmask, flag + TF_PROJ);
             launch_td<TD_PROJ>(nc, P, nleaf * cdiv(P.F.nlev * k, 128), nt, X, ld, op.P64.p, st);
+            redo(FA_PROJ, when(projmask, TF_PROJ));
             launch_far_sum(m, op, c0, cols, st, nullptr);
-            digits(op.xhat.p, hs, (size_t)node0 * k, false, true, op.td_key.p + TD_COLS, op.td_h.p);
-            P.kh = op.td_key.p + TD_COLS;
+            digits(op.xhat.p, hs, (size_t)node0 * k, false, P.F.nlev, key + TK_H);
+            k_td_align<<<dim3(nnodes, nt), 128, 0, st>>>(P.F, node0, nnodes, wh, ec, shc);
+            P.kh = key + TK_H;
             P.items = m.td_couple_item.p;
             P.bin = m.td_couple_bin.p;
             P.rec = m.td_couple.p;
             launch_td<TD_COUPLE>(nc, P, (int)m.td_couple_item.n, nt, X, ld, op.yhat.p, st);
-            digits(op.yhat.p, hs, (size_t)node0 * k, false, false, P.ko, op.td_h.p);
-            P.kh = P.ko;
+            k_td_check_couple<<<nnodes, 256, 0, st>>>(P.F, node0, nnodes, cols, nc, P.kh, wh, n1h, op.fa_min.p, op.fa_low.p, shc,
+                                                      sum, nodemask, flag + TF_NODES, err);
+            const FaWhen nodes = when(nodemask, TF_NODES);
+            redo(FA_COUPLE, nodes);
+            k_td_couple_sum<<<dim3(std::min(cdiv(hs, 256), 32), cols), 256, 0, st>>>(P.F, node0, c0, op.ye64.p, op.yhat.p, nodes);
+            digits(op.yhat.p, hs, (size_t)node0 * k, false, 1, key + TK_Y);
+            P.kh = key + TK_Y;
+            k_td_check_expand<<<nleaf, 64, 0, st>>>(P.F, node0, nnodes, cols, nc, key + TK_Y, wh, wfar, ef, sum, m.fa_umin.p,
+                                                    least, leafmask, flag + TF_LEAVES, err);
+            VFD_CUDA(cudaGetLastError());
         }
         P.items = m.td_rows_item.p;
         P.bin = m.td_rows_bin.p;
         P.rec = m.td_rows.p;
+        k_td_shift<<<dim3((int)m.td_rows_item.n, nt), 32, 0, st>>>(P.items, P.rec, P.nrec, nleaf, nnodes, wx, wh, wnear, wfar, shr);
         launch_td<TD_ROWS>(nc, P, (int)m.td_rows_item.n, nt, X, ld, Y, st);
+        redo(FA_NEAR, when(zero, TF_ERR));
+        if (far) redo(FA_EXPAND, when(leafmask, TF_LEAVES));
     }
-    k_td_good<<<1, 1, 0, st>>>(err, good);
-    VFD_CUDA(cudaGetLastError());
-    return good;
+}
+
+// vfd_op_apply_stats; waits for the device
+void apply_tensor_stats(const OpData &op, int64_t *out, int n)
+{
+    int h[1 + TF_N] = {op.td_cols};
+    if (op.td_cols) {
+        VFD_CUDA(cudaDeviceSynchronize());
+        VFD_CUDA(cudaMemcpy(h + 1, op.td_flag.p, TF_N * sizeof(int), cudaMemcpyDeviceToHost));
+    }
+    for (int i = 0; i < n; ++i) out[i] = i <= TF_N ? h[i] : 0;
 }
 
 }  // namespace vfd

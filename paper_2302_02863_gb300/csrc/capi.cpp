@@ -524,6 +524,15 @@ vfd_status vfd_selftest_math(vfd_mesh_t mesh, int which, int64_t n, const double
     VFD_API_END
 }
 
+vfd_status vfd_op_apply_stats(vfd_op_t h, int64_t *stats, int n)
+{
+    VFD_API_BEGIN
+    VFD_REQUIRE(h && stats && n >= 0, VFD_EINVAL, "null argument");
+    apply_tensor_stats(*h->op, stats, n);
+    return VFD_OK;
+    VFD_API_END
+}
+
 vfd_status vfd_op_far_ranks(vfd_op_t h, int *ranks, int n, int *nlev)
 {
     VFD_API_BEGIN

@@ -172,6 +172,7 @@ struct MeshData {
     bool fa_ok = false;
     DBuf<long long> fa_U;
     DBuf<int> fa_ue;
+    DBuf<float> fa_umin;       // smallest row sum of a leaf's bases, of the leaf's scale
     // partners of pairs of leaves and of nodes for the tensor-core apply (apply_tensor.cu)
     DBuf<TdRec> td_rows, td_couple;
     DBuf<int4> td_rows_item, td_couple_item;
@@ -276,18 +277,28 @@ struct OpData {
     DBuf<double> rho;                  // interior points, canonical order
     DBuf<double> S64;                  // nfar * k * k
     DBuf<double> D64;                  // near entries
-    // fixed-point copies for the FP64 apply: coupling blocks, an exponent per row of a block, the
-    // largest of a node's row, their difference, and the blocks that stay FP64 (apply_fixed.cu);
-    // near panels with B + M added and an exponent per row (apply_tensor.cu); fa: built, every
-    // entry is in range
+    // fixed-point copies for the FP64 apply: coupling blocks, an exponent per row of a block, its
+    // smallest entry in that scale, the blocks that stay FP64, a block's row node and smallest entry
+    // (apply_fixed.cu); near panels without the entries at B + M's positions, an exponent per row,
+    // and those entries plus B + M (apply_tensor.cu); fa: built, every entry is in range
     bool fa = false;
     DBuf<long long> fa_D, fa_S;
-    DBuf<int> fa_re;
-    DBuf<short> fa_se, fa_sn;
-    DBuf<unsigned char> fa_sh, fa_hard;
-    // digits of a vector's leaf and node pieces, column keys and flags (apply_tensor.cu)
-    DBuf<unsigned char> td_x, td_h;
-    DBuf<unsigned> td_key;
+    DBuf<int> fa_re, fa_row;
+    DBuf<double> fa_val, fa_min;
+    DBuf<short> fa_se;
+    DBuf<float> fa_low;
+    DBuf<unsigned char> fa_hard;
+    // digits of a vector's leaf and node pieces, keys, exponents and shifts that align the pieces,
+    // what is redone (rows; groups of columns of nodes and leaves) and the sizes that decide it
+    // (apply_tensor.cu)
+    DBuf<unsigned char> td_x, td_h, td_shift;
+    DBuf<unsigned> td_key, td_mask;
+    DBuf<short> td_exp;
+    DBuf<int> td_w, td_least;
+    DBuf<float> td_n1;
+    DBuf<double> td_sum;
+    DBuf<int> td_flag;
+    int td_cols = 0;                   // columns of the last apply on the tensor cores
     DBuf<float> S32, D32, Ul32;        // FP32 copies (VFD_FP32)
     DBuf<unsigned short> Dtc;          // BF16 near panels pre-tiled for the TMA-fed tcgen05 kernel (first batched use)
     std::vector<int64_t> Dtc_off;      //   element offset of each leaf's image (nleaf + 1)
@@ -441,6 +452,7 @@ void launch_selftest_math(const MeshData &m, int which, long long n, const doubl
 void build_fixed_bases(MeshData &m);
 // apply_tensor.cu
 void build_tensor_lists(MeshData &m);
+void apply_tensor_stats(const OpData &op, int64_t *out, int n);
 void build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t st);
 // apply.cu
 // partial sums of X . Y, written by the apply of one column where it can (n of them; part

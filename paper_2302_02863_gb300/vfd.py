@@ -34,7 +34,7 @@ INFO_KEYS = ["n_dof", "n_vert", "n_cell", "touching_pairs", "nnz", "levels", "no
 
 EXPORTS = ["vfd_default_mesh_opts", "vfd_mesh", "vfd_mesh_dofs", "vfd_mesh_info", "vfd_assemble",
            "vfd_apply", "vfd_apply_parts", "vfd_apply_noalloc", "vfd_solve", "vfd_precondition", "vfd_grad", "vfd_load",
-           "vfd_op_rho", "vfd_op_timings", "vfd_op_far_ranks",
+           "vfd_op_rho", "vfd_op_timings", "vfd_op_far_ranks", "vfd_op_apply_stats", "vfd_op_apply_stats",
            "vfd_selftest_math", "vfd_batch_create", "vfd_batch_apply", "vfd_batch_solve", "vfd_batch_tuning",
            "vfd_batch_set_config", "vfd_batch_set_wait_limit", "vfd_batch_set_update_drop", "vfd_batch_free",
            "vfd_free_op", "vfd_free_mesh", "vfd_last_error"]
@@ -91,6 +91,7 @@ def load():
     L.vfd_precondition.argtypes = [vp, C.c_int, vp]
     L.vfd_op_rho.argtypes = [vp, vp, vp]
     L.vfd_op_timings.argtypes = [vp, dp, C.c_int]
+    L.vfd_op_apply_stats.argtypes = [vp, C.POINTER(C.c_int64), C.c_int]
     L.vfd_op_far_ranks.argtypes = [vp, C.POINTER(C.c_int), C.c_int, C.POINTER(C.c_int)]
     L.vfd_selftest_math.argtypes = [vp, C.c_int, C.c_int64, vp, vp, vp]
     L.vfd_batch_create.argtypes = [C.POINTER(vp), C.c_int, C.POINTER(vp)]
@@ -407,6 +408,17 @@ def vfd_op_far_ranks(op):
     r = (C.c_int * max(nl.value, 1))()
     _check(load().vfd_op_far_ranks(op.handle, r, nl.value, C.byref(nl)))
     return [int(r[i]) for i in range(nl.value)]
+
+
+APPLY_STATS_KEYS = ["tensor_columns", "expired", "near_rows", "projections", "nodes", "leaves"]
+
+
+def vfd_op_apply_stats(op):
+    """How the last FP64 apply was computed: the columns that went to the tensor cores, whether a
+    wait ran out there, and the sums (per group of 8 columns) computed without them."""
+    out = (C.c_int64 * len(APPLY_STATS_KEYS))()
+    _check(load().vfd_op_apply_stats(op.handle, out, len(out)))
+    return dict(zip(APPLY_STATS_KEYS, (int(v) for v in out)))
 
 
 def vfd_selftest_math(mesh, which, x, out, stream=None):

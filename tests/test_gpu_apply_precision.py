@@ -77,3 +77,50 @@ def test_rows_keep_fp64_precision(name, leaf, p, lam, width):
         R, Y = _apply(vfd.vfd_apply_noalloc, op, X, 3), _apply(vfd.vfd_apply, op, X, width)
         err = (Y - R).abs() / (X.abs() @ A)
         assert float(err.max()) <= TOL, (kind, float(err.max()))
+
+
+@pytest.mark.parametrize("name,leaf,p,lam", SETUPS)
+def test_many_columns_keep_fp64_precision(name, leaf, p, lam):
+    """Enough columns for the tensor cores (their digits hold normal vectors, the rest is redone)."""
+    import torch
+    op, n, x = _setup(name, leaf, p, lam)
+    A = _columns(op, n, vfd.vfd_apply_noalloc, 8)
+    # |A| as the sum over the parts: a near entry and one of B + M may cancel
+    parts = sum(_columns(op, n, lambda o, X, Y, m=m: vfd.vfd_apply_parts(o, m, X, Y), 8).abs()
+                for m in (vfd.VFD_PART_B | vfd.VFD_PART_M, vfd.VFD_PART_KNEAR, vfd.VFD_PART_KFAR))
+    B = _columns(op, n, vfd.vfd_apply, n)
+    assert vfd.vfd_op_apply_stats(op)["tensor_columns"] == n
+    if lam == 0.0:
+        assert bool((A == B).all())
+    assert bool(((B - A).abs() <= TOL * A.abs()).all())
+    rows = 1003
+    for kind, v in _vectors(x, rows).items():
+        X = torch.tensor(v, device="cuda")
+        R, Y = _apply(vfd.vfd_apply_noalloc, op, X, 3), _apply(vfd.vfd_apply, op, X, rows)
+        st = vfd.vfd_op_apply_stats(op)
+        assert st["tensor_columns"] == rows and st["expired"] == 0
+        # normal and constant columns are what the digits are for
+        if kind in ("normal", "ones"):
+            assert st["near_rows"] <= 0.01 * n * rows / 8 and st["projections"] == 0, (kind, st)
+        if kind in ("14 decades across", "spike on 1e-18"):
+            assert st["near_rows"] > 0, (kind, st)
+        err = (Y - R).abs() / (X.abs() @ parts)
+        assert float(err.max()) <= TOL, (kind, float(err.max()), st)
+
+
+def test_unfit_columns_leave_the_others_alone():
+    """Columns that the digits cannot hold at all (Inf, NaN, nearly denormal) among normal ones."""
+    import torch
+    op, n, x = _setup("square", 40, 8, 0.75)
+    A = _columns(op, n, vfd.vfd_apply_noalloc, 8).abs()
+    X = torch.randn(640, n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(4))
+    X[5, n // 2], X[77, 3], X[130], X[300] = float("nan"), float("inf"), 0.0, 1e-300 * X[300]
+    R, Y = _apply(vfd.vfd_apply_noalloc, op, X, 8), torch.empty_like(X)
+    vfd.vfd_apply(op, X, Y)
+    st = vfd.vfd_op_apply_stats(op)
+    assert st["tensor_columns"] == 640 and st["projections"] > 0 and st["leaves"] > 0
+    assert torch.equal(torch.isnan(Y), torch.isnan(R)) and torch.equal(torch.isinf(Y), torch.isinf(R))
+    ok = torch.isfinite(X).all(1)
+    assert not Y[130].any()
+    err = (Y - R).abs()[ok] / (X.abs() @ A).clamp_min(5e-324 * 2.0 ** 53)[ok]
+    assert float(err.max()) <= TOL
