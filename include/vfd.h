@@ -411,6 +411,11 @@ vfd_status vfd_op_far_ranks(vfd_op_t op, int *ranks, int n, int *nlev);
  *  zeros from there on. */
 vfd_status vfd_op_apply_stats(vfd_op_t op, int64_t *stats, int n);
 
+/* Number of columns from which FP64 applies of this operator go to the tensor
+ * cores; 0 (the default): the library's rule, by the operator's size.  Meshes
+ * with leaves over 64 DoFs never do.  Errors: VFD_EINVAL (columns < 0). */
+vfd_status vfd_op_set_tensor_columns(vfd_op_t op, int64_t columns);
+
 /* Device time per assembly phase (VFD_T_* order) of the vfd_assemble call
  * that created op, if it was given VFD_ASSEMBLE_TIMED; ms: host, n entries
  * (at most VFD_T_COUNT are written).  Returns VFD_EINVAL if not recorded. */

@@ -539,7 +539,7 @@ void apply_parts_ex(const MeshData &m, OpData &op, int parts, const double *X, d
             op.ye64.alloc(needy);
         }
         op.td_cols = 0;
-        if (op.fa && apply_tensor_fits(m, nrhs)) apply_tensor_alloc(m, op);
+        if (op.fa && apply_tensor_fits(m, op, nrhs)) apply_tensor_alloc(m, op);
         if (parts == VFD_PART_ALL && op.fa && m.nnear > 0) {
             apply_fixed(m, op, X, Y, nrhs, ld, st, skip, dot);
             return;

@@ -18,7 +18,7 @@ enum FaStep { FA_PROJ, FA_COUPLE, FA_NEAR, FA_EXPAND };
 void apply_fixed_redo(FaStep step, const MeshData &m, OpData &op, const double *X, double *Y, int c0, int ng, int nrhs,
                       int64_t ld, cudaStream_t st, const FaWhen &when);
 // apply_tensor.cu: the same for many columns
-bool apply_tensor_fits(const MeshData &m, int nrhs);
+bool apply_tensor_fits(const MeshData &m, const OpData &op, int nrhs);
 void apply_tensor_alloc(const MeshData &m, OpData &op);   // its workspace, on first use
 void apply_tensor(const MeshData &m, OpData &op, const double *X, double *Y, int nrhs, int64_t ld, cudaStream_t st);
 

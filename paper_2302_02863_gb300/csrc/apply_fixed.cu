@@ -1086,7 +1086,7 @@ void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int 
 {
     if (dot) dot->n = nrhs == 1 ? m.kt.nleaf * cdiv(m.max_leaf_size, 16) : 0;
     if (dot && !dot->n) dot = nullptr;
-    if (!skip && !dot && apply_tensor_fits(m, nrhs)) return apply_tensor(m, op, X, Y, nrhs, ld, st);
+    if (!skip && !dot && apply_tensor_fits(m, op, nrhs)) return apply_tensor(m, op, X, Y, nrhs, ld, st);
     FaWhen when;
     when.skip = skip;
     // the node sums inside the gathers pay for few columns and short spans (3 columns, sums inside /

@@ -1149,19 +1149,21 @@ void build_tensor_lists(MeshData &m)
     upload(m.td_couple, m.td_couple_item, m.td_couple_bin);
 }
 
-// Where the digits pay.  The fixed-point kernels take groups of 8 columns, 7.6 us for each
-// 10^6 entries and group once the chip is full; the digits up to 64 columns at a time, but
-// a CTA walks all partners of its rows, 150 to 280 us even for small meshes.  Measured, 10^6
-// entries x groups: fixed point / digits in us: 9 (9025 DoFs, rank 16, 8 columns) 127 / 200,
-// 18 (16 columns) 213 / 208, 27 (24) 328 / 231; 19 (10267 DoFs, rank 36, 8) 234 / 279, 38
-// (12) 364 / 304; 28 (3997 DoFs, rank 64, 24) 289 / 300, 37 (32) 328 / 303; 97 (27361 DoFs,
-// rank 64, 5) 700 / 590, 776 (64) 5269 / 1143.  Up to 4 columns go as one narrow group
-// (97: 395 / 590).
-bool apply_tensor_fits(const MeshData &m, int nrhs)
+// Where the digits pay.  The kernels of few columns take groups of 8, the digits up to 64 columns
+// a pass, and a pass costs 240 to 700 us however few they are, so the columns of one pass count
+// (817 DoFs, 256 columns in 4 passes: 369 us in groups of 8, 966 with digits).  Measured,
+// 10^6 entries x groups of a pass: groups / digits in us: 9 (9025 DoFs, rank 16, 8 columns)
+// 186 / 284, 18 (16) 288 / 294, 27 (24) 566 / 337; 19 (10267 DoFs, rank 36, 8) 282 / 399, 38
+// (12) 580 / 408; 18 (3997 DoFs, rank 64, 16) 222 / 364, 28 (24) 367 / 386, 37 (32) 411 / 386;
+// 24 (16129 DoFs, rank 16, 5) 338 / 312; 97 (27361 DoFs, rank 64, 5) 719 / 718, (8) 896 / 724.
+// Up to 4 columns go as one narrow group (97: 437 / 712).
+bool apply_tensor_fits(const MeshData &m, const OpData &op, int nrhs)
 {
+    if (!m.td_rows.n) return false;
+    if (op.td_min > 0) return nrhs >= op.td_min;
     const int nlev = m.nfar > 0 ? m.kt.L - m.far_lmin + 1 : 0;
     const double entries = (double)m.near_entries + (double)m.nfar * m.k * m.k + 2.0 * nlev * m.k * m.N;
-    return nrhs >= 5 && m.td_rows.n > 0 && entries * cdiv(nrhs, 8) >= 2.2e7;
+    return nrhs >= 5 && entries * cdiv(std::min(nrhs, TD_COLS), 8) >= 2.2e7;
 }
 
 // Columns of a tile: the time of a wave of CTAs is 1, 1.07 and 1.6 for 16, 32 and 64

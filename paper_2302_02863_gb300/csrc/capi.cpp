@@ -533,6 +533,16 @@ vfd_status vfd_op_apply_stats(vfd_op_t h, int64_t *stats, int n)
     VFD_API_END
 }
 
+vfd_status vfd_op_set_tensor_columns(vfd_op_t h, int64_t columns)
+{
+    VFD_API_BEGIN
+    VFD_REQUIRE(h, VFD_EINVAL, "null operator");
+    VFD_REQUIRE(columns >= 0 && columns <= INT32_MAX, VFD_EINVAL, "negative number of columns");
+    h->op->td_min = (int)columns;
+    return VFD_OK;
+    VFD_API_END
+}
+
 vfd_status vfd_op_far_ranks(vfd_op_t h, int *ranks, int n, int *nlev)
 {
     VFD_API_BEGIN

@@ -81,9 +81,10 @@ def test_rows_keep_fp64_precision(name, leaf, p, lam, width):
 
 @pytest.mark.parametrize("name,leaf,p,lam", SETUPS)
 def test_many_columns_keep_fp64_precision(name, leaf, p, lam):
-    """Enough columns for the tensor cores (their digits hold normal vectors, the rest is redone)."""
+    """On the tensor cores (their digits hold normal vectors, the rest is redone)."""
     import torch
     op, n, x = _setup(name, leaf, p, lam)
+    vfd.vfd_op_set_tensor_columns(op, 1)
     A = _columns(op, n, vfd.vfd_apply_noalloc, 8)
     # |A| as the sum over the parts: a near entry and one of B + M may cancel
     parts = sum(_columns(op, n, lambda o, X, Y, m=m: vfd.vfd_apply_parts(o, m, X, Y), 8).abs()
@@ -112,6 +113,7 @@ def test_unfit_columns_leave_the_others_alone():
     """Columns that the digits cannot hold at all (Inf, NaN, nearly denormal) among normal ones."""
     import torch
     op, n, x = _setup("square", 40, 8, 0.75)
+    vfd.vfd_op_set_tensor_columns(op, 1)
     A = _columns(op, n, vfd.vfd_apply_noalloc, 8).abs()
     X = torch.randn(640, n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(4))
     X[5, n // 2], X[77, 3], X[130], X[300] = float("nan"), float("inf"), 0.0, 1e-300 * X[300]
@@ -124,3 +126,61 @@ def test_unfit_columns_leave_the_others_alone():
     assert not Y[130].any()
     err = (Y - R).abs()[ok] / (X.abs() @ A).clamp_min(5e-324 * 2.0 ** 53)[ok]
     assert float(err.max()) <= TOL
+
+
+FORMS = {
+    "interval": lambda: synth.interval_mesh(333),
+    "interval_long": lambda: synth.interval_mesh(2100),
+    "disk": lambda: synth.disk_mesh(13, seed=3),
+    "disk_mid": lambda: synth.disk_mesh(26, seed=4),
+    "square": lambda: synth.square_mesh(30, jitter=0.2, seed=5),
+    "graded": lambda: synth.square_mesh_graded(20, 1.5),
+    "ball": lambda: synth.kuhn_ball_mesh(9),
+}
+
+
+@pytest.mark.parametrize("name,leaf,p,lam", [
+    ("interval", 16, 5, 0.75), ("interval_long", 2, 3, 0.75), ("disk", 11, 5, 0.75), ("disk", 7, 1, 0.75),
+    ("disk_mid", 33, 7, 0.75), ("disk_mid", 64, 8, 0.75), ("disk_mid", 64, 4, 0.0), ("square", 28, 5, 0.75),
+    ("graded", 24, 4, 0.75), ("ball", 24, 3, 1.2), ("ball", 64, 2, 0.75)])
+def test_tensor_apply_over_forms(name, leaf, p, lam):
+    """Odd ranks, ragged and tiny leaves, deep trees, no far field, one to many columns in tiles of
+    16, 32 and 64 and in several passes, leading dimensions."""
+    import torch
+    m = FORMS[name]()
+    mesh = vfd.vfd_mesh(m.d, m.coords, m.cells, m.cell_is_interior, leaf_m=leaf, cheb_p=p, lam=lam)
+    s = synth.sigmoid_field(synth.random_fourier_field(21, 1.0, d=m.d), 0.1, 0.9)
+    op = vfd.vfd_assemble(mesh, s, synth.random_fourier_field(22, 0.5, d=m.d), 0.95)
+    vfd.vfd_op_set_tensor_columns(op, 1)
+    n, g = mesh.n_dof, torch.Generator("cuda").manual_seed(7)
+    for nrhs, ld in ((1, n), (3, n + 1), (8, n), (17, n + 5), (40, n), (64, n + 3), (150, n + 1)):
+        X = torch.randn(nrhs, ld, dtype=torch.float64, device="cuda", generator=g)
+        X *= 10.0 ** torch.randint(-3, 4, (nrhs, 1), device="cuda", generator=g)
+        Y, R = torch.full_like(X, 7.0), torch.full_like(X, 7.0)
+        vfd.vfd_apply(op, X, Y)
+        st = vfd.vfd_op_apply_stats(op)
+        assert st["tensor_columns"] == nrhs and st["expired"] == 0
+        for r in range(nrhs):
+            vfd.vfd_apply_noalloc(op, X[r:r + 1], R[r:r + 1])
+        assert torch.all(Y[:, n:] == 7.0)
+        # sums of a few hundred terms of one size: a row's |A||x| is below 16 times the largest |y|
+        err = (Y - R)[:, :n].abs().amax(1) / R[:, :n].abs().amax(1)
+        assert float(err.max()) <= 16 * TOL, (nrhs, ld, float(err.max()), st)
+
+
+def test_rule_counts_the_columns_of_a_pass():
+    """Several passes of a small mesh are no reason for the tensor cores; one pass of a larger one is."""
+    import torch
+    op, n, _ = _setup("disk", 64, 4, 0.75)
+    X = torch.ones(1024, n, dtype=torch.float64, device="cuda")
+    vfd.vfd_apply(op, X, torch.empty_like(X))
+    assert vfd.vfd_op_apply_stats(op)["tensor_columns"] == 0
+    vfd.vfd_op_set_tensor_columns(op, 1000)
+    vfd.vfd_apply(op, X, torch.empty_like(X))
+    assert vfd.vfd_op_apply_stats(op)["tensor_columns"] == 1024
+    m = synth.disk_mesh(37, seed=3)
+    mesh = vfd.vfd_mesh(2, m.coords, m.cells, m.cell_is_interior, leaf_m=64, cheb_p=8)
+    op = vfd.vfd_assemble(mesh, synth.config2_s_field(), synth.const_field(0.0), 0.9)
+    X = torch.ones(64, mesh.n_dof, dtype=torch.float64, device="cuda")
+    vfd.vfd_apply(op, X, torch.empty_like(X))
+    assert vfd.vfd_op_apply_stats(op)["tensor_columns"] == 64
