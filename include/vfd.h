@@ -416,6 +416,13 @@ vfd_status vfd_op_apply_stats(vfd_op_t op, int64_t *stats, int n);
  * with leaves over 64 DoFs never do.  Errors: VFD_EINVAL (columns < 0). */
 vfd_status vfd_op_set_tensor_columns(vfd_op_t op, int64_t columns);
 
+/* Upper bound on every wait of the tensor-core kernels of FP64 applies
+ * (default 1 s).  An apply in which one runs out is redone without them and
+ * gives the same results to rounding (vfd_op_apply_stats tells).  0 makes every
+ * wait that is not already satisfied give up at once (a way to exercise the
+ * failure path).  Errors: VFD_EINVAL (negative or non-finite seconds). */
+vfd_status vfd_op_set_wait_limit(vfd_op_t op, double seconds);
+
 /* Device time per assembly phase (VFD_T_* order) of the vfd_assemble call
  * that created op, if it was given VFD_ASSEMBLE_TIMED; ms: host, n entries
  * (at most VFD_T_COUNT are written).  Returns VFD_EINVAL if not recorded. */

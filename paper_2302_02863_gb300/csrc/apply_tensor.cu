@@ -78,7 +78,8 @@ constexpr int TD_RAW = TD_CW * 32 * 32;     // bytes of a step's entries
 constexpr int TD_THREADS = 32 * (TD_CW + 2);
 constexpr int TD_A = 128 * 16 * TD_D * 2;   // bytes of the operator's digits of a step
 constexpr int TD_SMS = 152;                // CTAs of a launch and tile: one an SM
-constexpr long long TD_WAIT = 2000000000LL;   // cycles, about a second
+constexpr double TD_HZ = 2e9;               // SM cycles a second, about
+constexpr long long TD_WAIT = (long long)TD_HZ;   // of an aborted CTA's waits, and the default of the others
 enum { TD_PROJ, TD_COUPLE, TD_ROWS };
 
 // bytes of the vector's digits of a step: [digit][column / 8][row / 8][column % 8][row % 8],
@@ -211,6 +212,7 @@ struct TdP {
     const int4 *items;
     const TdRec *rec;
     int *err;
+    long long wait;                          // cycles after which a wait gives up
 };
 
 __device__ __forceinline__ unsigned td_sa(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -333,7 +335,7 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const unsigned taddr = *tslot;
-    const u64 deadline = td_timer() + TD_WAIT;
+    const u64 deadline = td_timer() + P.wait;
 
     // Items: pairs of leaves (ROWS), of nodes (COUPLE), 128 columns of a leaf's bases (PROJ).
     // An item's records q .. q2, the first section up to q1 (ROWS: near, then far).
@@ -395,7 +397,7 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
     TdIt I{};
     I.i = ibeg;
     bool have = start(I), ok = true;
-    int issued = 0;   // steps of the products, of the copies
+    int issued = 0, moves = 0;   // steps of the products, of the copies; moves of the accumulators
     if (warp < TD_CW) {
         // cutting: 8 rows a warp; a lane takes 4 neighbouring entries of a row
         const int g = lane >> 1 & 7, tt = 8 * (lane >> 4) + 4 * (lane & 1);   // row, first entry
@@ -406,7 +408,7 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
         unsigned sl[NH];
 #pragma unroll
         for (int c = 0; c < NH; ++c) sh[c] = sl[c] = 0;
-        int moves = 0, m8 = 256, m16 = 65536, m24 = 16777216;
+        int m8 = 256, m16 = 65536, m24 = 16777216;
         asm("" : "+r"(m8), "+r"(m16), "+r"(m24));   // in registers: not shifts
         int ei = ibeg;   // the item that ends next
         auto emit = [&](int code) {
@@ -616,7 +618,6 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
     } else if (lane == 0) {
-        int moves = 0;
         bool first = true;
         while (have && ok) {
             TdIt J = I;   // its record comes while this piece is worked on
@@ -680,11 +681,12 @@ k_td(TdP P, int nitem, const double *__restrict__ X, int64_t ld, double *__restr
     __syncwarp();
     __syncthreads();
     if (*abort_f) {
-        // wait for what is in flight: the copies, then the products
+        // wait for what is in flight: the copies, then the products and the arrival after them
         const u64 dl = td_timer() + TD_WAIT;
         if (warp >= TD_CW && lane == 0)
             for (int i = max(0, issued - TD_NST); i < issued; ++i)
                 td_wait(warp == TD_CW ? empty(i % TD_NST) : fullB(i % TD_NST), (i / TD_NST) & 1, dl);
+        if (warp == TD_CW && lane == 0 && moves) td_wait(moved, (moves - 1) & 1, dl);
         if (threadIdx.x == 0) atomicOr(P.err, 1);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -1232,6 +1234,7 @@ void apply_tensor(const MeshData &m, OpData &op, const double *X, double *Y, int
     double *sum = op.td_sum.p;
     VFD_CUDA(cudaMemsetAsync(flag, 0, op.td_flag.bytes(), st));
     P.err = err;
+    P.wait = (long long)(op.td_wait * TD_HZ);
     P.dx = op.td_x.p;
     P.dh = op.td_h.p;
     P.kx = key + TK_X;

@@ -543,6 +543,17 @@ vfd_status vfd_op_set_tensor_columns(vfd_op_t h, int64_t columns)
     VFD_API_END
 }
 
+vfd_status vfd_op_set_wait_limit(vfd_op_t h, double seconds)
+{
+    VFD_API_BEGIN
+    VFD_REQUIRE(h, VFD_EINVAL, "null operator");
+    VFD_REQUIRE(std::isfinite(seconds) && seconds >= 0.0 && seconds < 3600.0, VFD_EINVAL,
+                "the wait limit must be in [0, 3600) seconds");
+    h->op->td_wait = seconds;
+    return VFD_OK;
+    VFD_API_END
+}
+
 vfd_status vfd_op_far_ranks(vfd_op_t h, int *ranks, int n, int *nlev)
 {
     VFD_API_BEGIN

@@ -299,6 +299,7 @@ struct OpData {
     DBuf<double> td_sum;
     DBuf<int> td_flag;
     int td_cols = 0;                   // columns of the last apply on the tensor cores
+    double td_wait = 1.0;              // seconds after which their waits give up
     int td_min = 0;                    // columns from which they are used (0: apply_tensor_fits)
     DBuf<float> S32, D32, Ul32;        // FP32 copies (VFD_FP32)
     DBuf<unsigned short> Dtc;          // BF16 near panels pre-tiled for the TMA-fed tcgen05 kernel (first batched use)

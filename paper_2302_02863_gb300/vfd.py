@@ -35,7 +35,7 @@ INFO_KEYS = ["n_dof", "n_vert", "n_cell", "touching_pairs", "nnz", "levels", "no
 EXPORTS = ["vfd_default_mesh_opts", "vfd_mesh", "vfd_mesh_dofs", "vfd_mesh_info", "vfd_assemble",
            "vfd_apply", "vfd_apply_parts", "vfd_apply_noalloc", "vfd_solve", "vfd_precondition", "vfd_grad", "vfd_load",
            "vfd_op_rho", "vfd_op_timings", "vfd_op_far_ranks", "vfd_op_apply_stats", "vfd_op_apply_stats",
-           "vfd_op_set_tensor_columns", "vfd_selftest_math", "vfd_batch_create", "vfd_batch_apply", "vfd_batch_solve", "vfd_batch_tuning",
+           "vfd_op_set_tensor_columns", "vfd_op_set_wait_limit", "vfd_selftest_math", "vfd_batch_create", "vfd_batch_apply", "vfd_batch_solve", "vfd_batch_tuning",
            "vfd_batch_set_config", "vfd_batch_set_wait_limit", "vfd_batch_set_update_drop", "vfd_batch_free",
            "vfd_free_op", "vfd_free_mesh", "vfd_last_error"]
 
@@ -93,6 +93,7 @@ def load():
     L.vfd_op_timings.argtypes = [vp, dp, C.c_int]
     L.vfd_op_apply_stats.argtypes = [vp, C.POINTER(C.c_int64), C.c_int]
     L.vfd_op_set_tensor_columns.argtypes = [vp, C.c_int64]
+    L.vfd_op_set_wait_limit.argtypes = [vp, C.c_double]
     L.vfd_op_far_ranks.argtypes = [vp, C.POINTER(C.c_int), C.c_int, C.POINTER(C.c_int)]
     L.vfd_selftest_math.argtypes = [vp, C.c_int, C.c_int64, vp, vp, vp]
     L.vfd_batch_create.argtypes = [C.POINTER(vp), C.c_int, C.POINTER(vp)]
@@ -425,6 +426,11 @@ def vfd_op_apply_stats(op):
 def vfd_op_set_tensor_columns(op, columns):
     """Columns from which FP64 applies of the operator use the tensor cores (0: the library's rule)."""
     _check(load().vfd_op_set_tensor_columns(op.handle, int(columns)))
+
+
+def vfd_op_set_wait_limit(op, seconds):
+    """Seconds after which a wait of the tensor-core kernels of the operator's FP64 applies gives up."""
+    _check(load().vfd_op_set_wait_limit(op.handle, float(seconds)))
 
 
 def vfd_selftest_math(mesh, which, x, out, stream=None):

@@ -184,3 +184,33 @@ def test_rule_counts_the_columns_of_a_pass():
     X = torch.ones(64, mesh.n_dof, dtype=torch.float64, device="cuda")
     vfd.vfd_apply(op, X, torch.empty_like(X))
     assert vfd.vfd_op_apply_stats(op)["tensor_columns"] == 64
+
+
+@pytest.mark.parametrize("name,leaf,p,lam", SETUPS)
+def test_expired_waits_are_redone(name, leaf, p, lam):
+    """A wait limit of zero: every wait of the digit kernels that is not satisfied already gives up,
+    the kernels drain and return, and the apply comes from the others."""
+    import torch
+    op, n, _ = _setup(name, leaf, p, lam)
+    vfd.vfd_op_set_tensor_columns(op, 1)
+    X = torch.randn(150, n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    R, Y, Z, W = (torch.full_like(X, 7.0) for _ in range(4))
+    vfd.vfd_apply(op, X, R)
+    assert vfd.vfd_op_apply_stats(op)["expired"] == 0
+    vfd.vfd_op_set_wait_limit(op, 0.0)
+    vfd.vfd_apply(op, X, Y)
+    assert vfd.vfd_op_apply_stats(op)["expired"] == 1
+    vfd.vfd_op_set_tensor_columns(op, 1000)   # the kernels of few columns
+    vfd.vfd_apply(op, X, Z)
+    assert vfd.vfd_op_apply_stats(op)["tensor_columns"] == 0
+    err = (Y - Z).abs().amax(1) / Z.abs().amax(1)
+    assert float(err.max()) <= 16 * TOL
+    # the default limit again: the digits as before
+    vfd.vfd_op_set_tensor_columns(op, 1)
+    vfd.vfd_op_set_wait_limit(op, 1.0)
+    vfd.vfd_apply(op, X, W)
+    assert vfd.vfd_op_apply_stats(op)["expired"] == 0 and torch.equal(W, R)
+    for bad in (-1.0, float("nan"), float("inf")):
+        with pytest.raises(vfd.VfdError) as e:
+            vfd.vfd_op_set_wait_limit(op, bad)
+        assert e.value.status == vfd.VFD_EINVAL
