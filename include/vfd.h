@@ -189,6 +189,13 @@ vfd_status vfd_mesh_info(vfd_mesh_t mesh, int64_t *info, int n_info);
  *          must hold at every evaluation point unless VFD_ASSEMBLE_UNCHECKED.
  *   precision: VFD_FP64, VFD_FP32 or VFD_BF16.  stream: cudaStream_t.
  * Blocks the host once to read the field check.
+ * Memory: the FP64 operator, and fixed-point copies of its coupling blocks and
+ * (leaves of at most 64 DoFs) near panels for the FP64 apply, as large again.
+ * The copies are left out where they would take more than half of the device
+ * memory that is left, or an entry is out of their range (beyond 2^+-800); the
+ * apply then runs in FP64 throughout, several times slower.  Operators with a
+ * recompressed far field have no copies either: recompression saves time only
+ * against that FP64 apply.
  * Errors: VFD_EINVAL (field out of range, bad s_bar), VFD_EUNSUPPORTED
  * (nodal field with a low-rank part; tail with non-constant fields),
  * VFD_ENOMEM, VFD_ECUDA. */

@@ -923,11 +923,17 @@ void build_fixed_bases(MeshData &m)
     m.fa_ok = true;
     if (!nlev) return;
     DBuf<int> err;
-    err.alloc(1);
+    m.fa_ok = if_memory([&] {
+        err.alloc(1);
+        m.fa_U.alloc((size_t)((nlev * m.k + 1) & ~1) * m.N);
+        m.fa_ue.alloc(m.kt.nleaf);
+        m.fa_umin.alloc(m.kt.nleaf);
+    });
+    if (!m.fa_ok) {
+        m.fa_U.release();
+        return;
+    }
     err.zero(nullptr);
-    m.fa_U.alloc((size_t)((nlev * m.k + 1) & ~1) * m.N);
-    m.fa_ue.alloc(m.kt.nleaf);
-    m.fa_umin.alloc(m.kt.nleaf);
     k_fa_build_U<<<m.kt.nleaf, 256>>>(m.kt.first_leaf(), m.N, m.k, nlev, m.kt_begin.p, m.kt_end.p, m.Ul64.p,
                                       (int2 *)m.fa_U.p, m.fa_ue.p, m.fa_umin.p, err.p);
     VFD_CUDA(cudaGetLastError());
@@ -939,27 +945,58 @@ void build_fixed_bases(MeshData &m)
     }
 }
 
-// the operator's near panels and coupling blocks; err gets bit 2 where an entry does not fit
-void build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t st)
+void release_fixed_operator(OpData &op)
 {
-    op.fa_D.alloc(m.near_entries);
-    op.fa_re.alloc(m.N);
-    op.fa_val.alloc(m.nnz);
-    k_fa_build_near<<<cdiv((long long)m.N * 32, 256), 256, 0, st>>>(
-        m.N, m.kt.first_leaf(), m.vleaf.p, m.kt_begin.p, m.panel_w.p, m.panel_off.p, op.D64.p, m.rowptr.p, m.bm_pos.p,
-        op.valBM.p, op.fa_val.p, (int2 *)op.fa_D.p, op.fa_re.p, err);
-    if (m.nfar) {
-        const int kp = (m.k + 1) & ~1;
-        op.fa_S.alloc((size_t)m.nfar * m.k * kp);
-        op.fa_se.alloc((size_t)m.nfar * m.k);
-        op.fa_low.alloc((size_t)m.nfar * m.k);
-        op.fa_hard.alloc(m.nfar);
-        op.fa_row.alloc(m.nfar);
-        op.fa_min.alloc(m.nfar);
+    op.fa_D.release();
+    op.fa_re.release();
+    op.fa_val.release();
+    op.fa_S.release();
+    op.fa_se.release();
+    op.fa_low.release();
+    op.fa_hard.release();
+    op.fa_row.release();
+    op.fa_min.release();
+}
+
+// The operator's coupling blocks, and its near panels where the mesh has the lists of the
+// many-column apply; err gets bit 2 where an entry does not fit.  The copies are as large as
+// the FP64 operator: they are made where they take at most half of the memory that is left
+// (false: not), so that what fits without them fits.
+bool build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t st)
+{
+    const int kp = (m.k + 1) & ~1;
+    const bool panels = m.td_rows.n > 0;
+    size_t left = 0, total = 0;
+    VFD_CUDA(cudaMemGetInfo(&left, &total));
+    const size_t need = (panels ? (size_t)m.near_entries * 8 : 0) + (size_t)m.nfar * m.k * (kp * 8 + 8);
+    const bool ok = need <= left / 2 && if_memory([&] {
+        if (panels) {
+            op.fa_D.alloc(m.near_entries);
+            op.fa_re.alloc(m.N);
+            op.fa_val.alloc(m.nnz);
+        }
+        if (m.nfar) {
+            op.fa_S.alloc((size_t)m.nfar * m.k * kp);
+            op.fa_se.alloc((size_t)m.nfar * m.k);
+            op.fa_low.alloc((size_t)m.nfar * m.k);
+            op.fa_hard.alloc(m.nfar);
+            op.fa_row.alloc(m.nfar);
+            op.fa_min.alloc(m.nfar);
+        }
+    });
+    if (!ok) {
+        release_fixed_operator(op);
+        return false;
+    }
+    if (panels)
+        k_fa_build_near<<<cdiv((long long)m.N * 32, 256), 256, 0, st>>>(
+            m.N, m.kt.first_leaf(), m.vleaf.p, m.kt_begin.p, m.panel_w.p, m.panel_off.p, op.D64.p, m.rowptr.p, m.bm_pos.p,
+            op.valBM.p, op.fa_val.p, (int2 *)op.fa_D.p, op.fa_re.p, err);
+    if (m.nfar)
         k_fa_build_S<<<m.kt.nnode, 256, 0, st>>>(m.far_ptr.p, m.k, kp, op.S64.p, (int2 *)op.fa_S.p, op.fa_se.p, op.fa_low.p,
                                                  op.fa_hard.p, op.fa_row.p, op.fa_min.p, err);
-    }
     VFD_CUDA(cudaGetLastError());
+    return true;
 }
 
 namespace {

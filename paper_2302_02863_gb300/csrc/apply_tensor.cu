@@ -1075,7 +1075,7 @@ void launch_td(int nc, const TdP &P, int nitem, int nt, const double *X, int64_t
 // ancestors of the far levels (offsets in the flattened bases).
 // td_couple: pairs of nodes from the first far node on (offsets: the coupling blocks).
 // Items (first record, second section, end, pair) in the order of the CTAs that take them.
-void build_tensor_lists(MeshData &m)
+static void build_lists(MeshData &m)
 {
     if (m.max_leaf_size > 64 || !m.nnear || (m.nfar > 0 && m.far_lmin < 1)) return;   // (pairs of nodes share a level)
     const int nleaf = m.kt.nleaf, fl = m.kt.first_leaf(), nlev = m.nfar > 0 ? m.kt.L - m.far_lmin + 1 : 0;
@@ -1150,6 +1150,10 @@ void build_tensor_lists(MeshData &m)
     }
     upload(m.td_couple, m.td_couple_item, m.td_couple_bin);
 }
+void build_tensor_lists(MeshData &m)
+{
+    if (!if_memory([&] { build_lists(m); })) m.td_rows.release();   // (no digits then)
+}
 
 // Where the digits pay.  The kernels of few columns take groups of 8, the digits up to 64 columns
 // a pass, and a pass costs 240 to 700 us however few they are, so the columns of one pass count
@@ -1161,7 +1165,7 @@ void build_tensor_lists(MeshData &m)
 // Up to 4 columns go as one narrow group (97: 437 / 712).
 bool apply_tensor_fits(const MeshData &m, const OpData &op, int nrhs)
 {
-    if (!m.td_rows.n) return false;
+    if (!m.td_rows.n || op.td_off) return false;
     if (op.td_min > 0) return nrhs >= op.td_min;
     const int nlev = m.nfar > 0 ? m.kt.L - m.far_lmin + 1 : 0;
     const double entries = (double)m.near_entries + (double)m.nfar * m.k * m.k + 2.0 * nlev * m.k * m.N;
@@ -1199,17 +1203,24 @@ void apply_tensor_alloc(const MeshData &m, OpData &op)
     if (op.td_flag.p) return;
     const int node0 = m.nfar > 0 ? (1 << m.far_lmin) - 1 : m.kt.nnode;
     const size_t nodes = m.kt.nnode - node0, leaves = m.kt.nleaf;
-    op.td_x.alloc(leaves * ((m.max_leaf_size + 15) >> 4) * td_step(TD_COLS));
-    op.td_h.alloc(nodes * ((m.k + 15) >> 4) * td_step(TD_COLS));
-    op.td_key.alloc(TK_N + std::max(leaves, nodes) * TD_COLS);
-    op.td_w.alloc(TD_TILES * (3 * leaves + nodes));
-    op.td_exp.alloc(TD_TILES * (nodes * m.k + m.N + leaves));
-    op.td_shift.alloc((size_t)TD_TILES * (2 * m.td_rows.n + (size_t)m.nfar * m.k));
-    op.td_mask.alloc(1 + m.kt.nnode + (2 + 2 * TD_TILES) * leaves);
-    op.td_n1.alloc((nodes + leaves) * TD_COLS);
-    op.td_sum.alloc(nodes * TD_COLS);
-    op.td_least.alloc(leaves * TD_COLS);
-    op.td_flag.alloc(TF_N);
+    op.td_off = !if_memory([&] {
+        op.td_x.alloc(leaves * ((m.max_leaf_size + 15) >> 4) * td_step(TD_COLS));
+        op.td_h.alloc(nodes * ((m.k + 15) >> 4) * td_step(TD_COLS));
+        op.td_key.alloc(TK_N + std::max(leaves, nodes) * TD_COLS);
+        op.td_w.alloc(TD_TILES * (3 * leaves + nodes));
+        op.td_exp.alloc(TD_TILES * (nodes * m.k + m.N + leaves));
+        op.td_shift.alloc((size_t)TD_TILES * (2 * m.td_rows.n + (size_t)m.nfar * m.k));
+        op.td_mask.alloc(1 + m.kt.nnode + (2 + 2 * TD_TILES) * leaves);
+        op.td_n1.alloc((nodes + leaves) * TD_COLS);
+        op.td_sum.alloc(nodes * TD_COLS);
+        op.td_least.alloc(leaves * TD_COLS);
+        op.td_flag.alloc(TF_N);
+    });
+    if (op.td_off) {   // the kernels of few columns do without
+        op.td_x.release();
+        op.td_h.release();
+        op.td_shift.release();
+    }
 }
 
 // Y = A X for all columns

@@ -324,14 +324,16 @@ vfd_status vfd_assemble(vfd_mesh_t mesh, const vfd_field *s, const vfd_field *lo
         launch_convert_fp32(m, *op, st);
         launch_lowp_csr(m, *op, st);
     }
+    bool fixed = false;
     if (m.fa_ok && m.nnear > 0 && !op->rc_on) {   // fixed-point copies for the FP64 apply
         op->errflag.zero(st);
-        build_fixed_operator(m, *op, op->errflag.p, st);
+        fixed = build_fixed_operator(m, *op, op->errflag.p, st);
         VFD_CUDA(cudaMemcpyAsync(herr, op->errflag.p, sizeof(int), cudaMemcpyDeviceToHost, st));
     }
     mark();
     VFD_CUDA(cudaStreamSynchronize(st));
-    op->fa = op->fa_re.n > 0 && herr[0] == 0;
+    op->fa = fixed && herr[0] == 0;
+    if (fixed && !op->fa) release_fixed_operator(*op);   // an entry is out of their range
     if (op->timed) {
         // events: 0 start, 1 fields, 2 coupling, 3 near, 4 density, 5 singular, 6 gathers
         for (int i = 0; i + 1 < nev && i < 6; ++i) {

@@ -50,8 +50,8 @@ struct DBuf {
     }
     void alloc(size_t count) {
         release();
-        n = count;
         if (count) VFD_CUDA(cudaMalloc(&p, sizeof(T) * count));
+        n = count;   // (nothing where the allocation failed)
     }
     void upload(const std::vector<T> &h) {
         alloc(h.size());
@@ -300,6 +300,7 @@ struct OpData {
     DBuf<int> td_flag;
     int td_cols = 0;                   // columns of the last apply on the tensor cores
     double td_wait = 1.0;              // seconds after which their waits give up
+    bool td_off = false;               // no memory for the workspace: not used
     int td_min = 0;                    // columns from which they are used (0: apply_tensor_fits)
     DBuf<float> S32, D32, Ul32;        // FP32 copies (VFD_FP32)
     DBuf<unsigned short> Dtc;          // BF16 near panels pre-tiled for the TMA-fed tcgen05 kernel (first batched use)
@@ -455,7 +456,21 @@ void build_fixed_bases(MeshData &m);
 // apply_tensor.cu
 void build_tensor_lists(MeshData &m);
 void apply_tensor_stats(const OpData &op, int64_t *out, int n);
-void build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t st);
+bool build_fixed_operator(const MeshData &m, OpData &op, int *err, cudaStream_t st);
+void release_fixed_operator(OpData &op);
+// f() allocates what only makes things faster: false (and the error cleared) where the device is out of memory
+template <class F>
+bool if_memory(F f)
+{
+    try {
+        f();
+        return true;
+    } catch (const Error &e) {
+        if (e.st != VFD_ENOMEM) throw;
+        cudaGetLastError();
+        return false;
+    }
+}
 // apply.cu
 // partial sums of X . Y, written by the apply of one column where it can (n of them; part
 // holds at least dot_partials(m)), else n = 0
