@@ -564,14 +564,14 @@ void precond_apply(const MeshData &m, const OpData &op, const double *r, double 
 
 int precond_rz_partials(const MeshData &m, const OpData &op) { return m.kt.nleaf + op.prec_nc; }
 
-// alpha = rz / pq (s_rz, npq partials in cg_pq), x, r, z = local part of M^-1 r, and the
+// alpha = rz / pq (s_rz, npq partials of pq), x, r, z = local part of M^-1 r, and the
 // coarse correction zc = A_c^-1 R r; partials of r.r per leaf and of r.z per leaf and cluster
-void precond_step(const MeshData &m, OpData &op, int npq, double *rr_part, double *rz_part, double *scal, int s_rz,
+void precond_step(const MeshData &m, OpData &op, int npq, const double *pq, double *rr_part, double *rz_part, double *scal, int s_rz,
                   int s_rzold, int s_pq, const int *flag, cudaStream_t st)
 {
     const int nleaf = m.kt.nleaf, mb = op.prec_mb;
     k_prec_step<<<nleaf, 256, (size_t)(mb + 256) * sizeof(double), st>>>(
-        m.kt.first_leaf(), mb, m.kt_begin.p, m.kt_end.p, op.prec_blk.p, npq, op.cg_pq.p, op.cg_x.p, op.cg_r.p, op.cg_p.p,
+        m.kt.first_leaf(), mb, m.kt_begin.p, m.kt_end.p, op.prec_blk.p, npq, pq, op.cg_x.p, op.cg_r.p, op.cg_p.p,
         op.cg_q.p, op.cg_z.p, op.prec_rl.p, rr_part, rz_part, scal, s_rz, s_rzold, s_pq, flag);
     if (op.prec_nc > 0)
         k_prec_coarse<<<cdiv((long long)op.prec_nc * 32, 256), 256, (size_t)op.prec_nc * sizeof(double), st>>>(

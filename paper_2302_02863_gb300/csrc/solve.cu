@@ -119,6 +119,22 @@ __global__ void __launch_bounds__(RB) k_dot_part(int n, const double *__restrict
     if (threadIdx.x == 0) part[blockIdx.x] = v;
 }
 
+// Every block of the next kernel sums all partials, so their number is bounded: at 27k DoFs
+// an apply leaves 2048; more than 4096 (leaves of a few DoFs, or over 60k DoFs) are summed to
+// 256 first, in order.  (PCG an iteration, without / with this stage:
+// 27k DoFs in 8192 leaves 729 / 667 us, 76k DoFs in 16384 leaves 1707 / 1291.)
+constexpr int MAXPART = 4096, NFOLD = 256;
+__global__ void __launch_bounds__(RB) k_fold(int n, const double *__restrict__ part, double *__restrict__ out, const int *flag)
+{
+    __shared__ double sh[32];
+    if (flag[F_DONE]) return;
+    const int per = (n + NFOLD - 1) / NFOLD, b = blockIdx.x * per, e = min(n, b + per);
+    double v = 0.0;
+    for (int i = b + threadIdx.x; i < e; i += RB) v += part[i];
+    v = block_sum(v, sh);
+    if (threadIdx.x == 0) out[blockIdx.x] = v;
+}
+
 // One iteration after q = A p is two launches: k_cg_xr needs p.q whole, k_cg_p needs
 // r.r whole.  Both are latency (16k to 27k entries): one entry a thread, the sums of
 // the partials in every block instead of a last block's.  With the dot product out of
@@ -211,15 +227,22 @@ void release_graphs(OpData &op)
     }
 }
 
-// q = A p with the partials of p . q in cg_pq; returns their number
-static int apply_with_dot(const MeshData &m, OpData &op, bool lowp, cudaStream_t st)
+// q = A p with the partials of p . q: their number, *pq where they are
+static int apply_with_dot(const MeshData &m, OpData &op, bool lowp, cudaStream_t st, const double **pq)
 {
     const int n = m.N, NB = red_blocks(n), *flag = op.cg_flag.p;
     ApplyDot dot;
-    dot.part = op.cg_pq.p;
+    dot.part = op.cg_pq.p + NFOLD;
     apply_parts_ex(m, op, VFD_PART_ALL, op.cg_p.p, op.cg_q.p, 1, n, lowp, st, flag, &dot);
+    *pq = dot.part;
+    if (dot.n > MAXPART) {
+        k_fold<<<NFOLD, RB, 0, st>>>(dot.n, dot.part, op.cg_pq.p, flag);
+        VFD_CUDA(cudaGetLastError());
+        *pq = op.cg_pq.p;
+        return NFOLD;
+    }
     if (dot.n) return dot.n;
-    k_dot_part<<<NB, RB, 0, st>>>(n, op.cg_p.p, op.cg_q.p, op.cg_pq.p, flag);
+    k_dot_part<<<NB, RB, 0, st>>>(n, op.cg_p.p, op.cg_q.p, dot.part, flag);
     VFD_CUDA(cudaGetLastError());
     return NB;
 }
@@ -252,8 +275,9 @@ static int run_cg(const MeshData &m, OpData &op, bool lowp, double rtol, int max
         VFD_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
         try {
             for (int it = 0; it < CHUNK; ++it) {
-                const int npq = apply_with_dot(m, op, lowp, cs);
-                k_cg_xr<<<VB, RB, 0, cs>>>(n, npq, op.cg_pq.p, op.cg_x.p, op.cg_r.p, op.cg_p.p, op.cg_q.p, part, scal,
+                const double *pq;
+                const int npq = apply_with_dot(m, op, lowp, cs, &pq);
+                k_cg_xr<<<VB, RB, 0, cs>>>(n, npq, pq, op.cg_x.p, op.cg_r.p, op.cg_p.p, op.cg_q.p, part, scal,
                                            flag);
                 k_cg_p<<<VB, RB, 0, cs>>>(n, VB, part, op.cg_r.p, op.cg_p.p, scal, flag);
             }
@@ -294,7 +318,7 @@ static void ensure_ws(const MeshData &m, OpData &op)
         op.cg_b.alloc(n);
         op.cg_z.alloc(n);
         op.cg_red.alloc(std::max(2048, m.kt.nleaf));
-        op.cg_pq.alloc(std::max(dot_partials(m), 264));
+        op.cg_pq.alloc(NFOLD + std::max(dot_partials(m), 264));
         op.cg_scal.alloc(8);
         op.cg_flag.alloc(8);
         VFD_CUDA(cudaMemset(op.cg_flag.p, 0, 8 * sizeof(int)));
@@ -345,7 +369,7 @@ k_pcg_p(int n, int nrr, const double *__restrict__ rr_part, int nrz, const doubl
 
 // precond.cu: z = M^-1 r; and one PCG iteration up to the coarse product
 void precond_apply(const MeshData &m, const OpData &op, const double *r, double *z, cudaStream_t st, const int *skip);
-void precond_step(const MeshData &m, OpData &op, int npq, double *rr_part, double *rz_part, double *scal, int s_rz,
+void precond_step(const MeshData &m, OpData &op, int npq, const double *pq, double *rr_part, double *rz_part, double *scal, int s_rz,
                   int s_rzold, int s_pq, const int *flag, cudaStream_t st);
 int precond_rz_partials(const MeshData &m, const OpData &op);
 
@@ -377,8 +401,9 @@ static int run_pcg(const MeshData &m, OpData &op, double rtol, int max_it, cudaS
         VFD_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
         try {
             for (int it = 0; it < CHUNK; ++it) {
-                const int npq = apply_with_dot(m, op, false, cs), nrz = precond_rz_partials(m, op);
-                precond_step(m, op, npq, part, op.prec_rz.p, scal, S_RZ, S_RZOLD, S_PQ, flag, cs);
+                const double *pq;
+                const int npq = apply_with_dot(m, op, false, cs, &pq), nrz = precond_rz_partials(m, op);
+                precond_step(m, op, npq, pq, part, op.prec_rz.p, scal, S_RZ, S_RZOLD, S_PQ, flag, cs);
                 k_pcg_p<<<VB, RB, 0, cs>>>(n, m.kt.nleaf, part, nrz, op.prec_rz.p, op.cg_z.p,
                                            op.prec_nc ? op.prec_zc.p : nullptr, op.prec_cidx.p, op.cg_p.p, scal, flag);
             }
