@@ -954,11 +954,9 @@ void launch_near_build(const MeshData &m, OpData &op, cudaStream_t st)
     const size_t tshm = (size_t)32 * NB_TC * 8 + (size_t)32 * P.maxleaf * 8 + (size_t)P.maxleaf * P.maxleaf * 8 +
                         (size_t)NB_TC * (m.d + 2) * 8 + (size_t)32 * (m.d + 2) * 8 + (size_t)NB_TC * 4 * 4 +
                         (size_t)32 * 4 * 4;
+    // (the same leaves are refused whether the fields fit the fixed-point kernel or not)
     VFD_REQUIRE(whole || tshm <= 220 * 1024, VFD_EUNSUPPORTED, "leaves too large for the near-block kernel");
-    if (op.fx) {
-        launch_near_build_fixed(m, op, st);
-        return;
-    }
+    if (op.fx && launch_near_build_fixed(m, op, st)) return;
     if (whole) {
         P.TQ = TQ;
         VFD_CUDA(cudaFuncSetAttribute(k_near_build, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));

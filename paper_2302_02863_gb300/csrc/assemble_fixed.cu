@@ -225,7 +225,7 @@ __global__ void k_near_reduce(int nsplit, size_t part, const double *__restrict_
 }
 
 template <int D>
-void near_fx(const MeshData &m, OpData &op, cudaStream_t st)
+bool near_fx(const MeshData &m, OpData &op, cudaStream_t st)
 {
     constexpr int NV = D + 1, NQ = D == 3 ? 4 : 3;
     NearFx P;
@@ -269,6 +269,7 @@ void near_fx(const MeshData &m, OpData &op, cudaStream_t st)
     // that one's folds and staging run under the other's evaluations
     const size_t shm = FX_BYTES + (size_t)P.maxleaf * (NF_RT + 1) * 8 +
                        (size_t)NF_CELLS * (NQ * (D + 2) * 8 + 2 * NV * 4);
+    if (shm > 227 * 1024) return false;
     // few blocks (small meshes): the row tiles of a block on several CTAs, their
     // partial results summed in order afterwards
     const int ntile = std::max(1, cdiv(m.max_leaf_pts, NF_RT)), ncomp = (m.nnear + m.kt.nleaf) / 2;
@@ -289,16 +290,16 @@ void near_fx(const MeshData &m, OpData &op, cudaStream_t st)
         VFD_CUDA(cudaGetLastError());
         VFD_CUDA(cudaStreamSynchronize(st));   // the partial results are released on return
     }
+    return true;
 }
 
 }  // namespace
 
-void launch_near_build_fixed(const MeshData &m, OpData &op, cudaStream_t st)
+bool launch_near_build_fixed(const MeshData &m, OpData &op, cudaStream_t st)
 {
-    if (m.d == 1) near_fx<1>(m, op, st);
-    else if (m.d == 2) near_fx<2>(m, op, st);
-    else near_fx<3>(m, op, st);
+    if (!(m.d == 1 ? near_fx<1>(m, op, st) : m.d == 2 ? near_fx<2>(m, op, st) : near_fx<3>(m, op, st))) return false;
     launch_near_transpose(m, op, st);
+    return true;
 }
 
 // ---------------------------------------------------------------------------

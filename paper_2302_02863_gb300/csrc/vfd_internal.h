@@ -445,7 +445,7 @@ void launch_near_build(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_convert_fp32(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_load(const MeshData &m, const double *f, double *F, cudaStream_t st);
 // assemble_fixed.cu: the same with fixed-point kernel evaluations (operators with fx set)
-void launch_near_build_fixed(const MeshData &m, OpData &op, cudaStream_t st);
+bool launch_near_build_fixed(const MeshData &m, OpData &op, cudaStream_t st);   // false: leaves too large for it
 void launch_near_transpose(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_coupling_fixed(const MeshData &m, OpData &op, cudaStream_t st);
 void launch_rho_coupling_fixed(const MeshData &m, OpData &op, double *yt, cudaStream_t st);
