@@ -1126,8 +1126,9 @@ void apply_fixed(const MeshData &m, OpData &op, const double *X, double *Y, int 
     if (!skip && !dot && apply_tensor_fits(m, op, nrhs)) return apply_tensor(m, op, X, Y, nrhs, ld, st);
     FaWhen when;
     when.skip = skip;
-    // the node sums inside the gathers pay for few columns and short spans (3 columns, sums inside /
-    // of their own: 27361 DoFs 432 / 395 us, 16129 182 / 171, 3721 61 / 59; 2 columns at 10267 97 / 125)
+    // the node sums inside the gathers pay for few columns and short spans (sums inside / of their own:
+    // 3 columns at 27361 DoFs 432 / 395 us, 16129 182 / 171, 3721 61 / 59; 2 columns at 27361 258 / 270,
+    // 10267 138 / 160, 3997 51 / 58)
     const bool summed = nrhs >= 3 || m.kt.L - m.far_lmin > 7, far = m.nfar > 0;
     // far groups: of 8, the remainder in one group of the next power of two
     auto far_groups = [&](auto f) {
