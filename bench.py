@@ -336,13 +336,14 @@ def main():
         pass
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     if prec == vfd.VFD_FP64:
-        # the FP64 apply runs on 61-bit integers, 8 bytes an entry: near panels and
-        # coupling blocks once, the bases twice (projection, expansion)
-        leaf_bytes = 8 * (info["near_entries"] + info["far_blocks"] * info["rank"] ** 2) + 2 * n * 8
+        # 8 bytes an entry: near panels and coupling blocks once, the bases of the far levels
+        # twice (projection, expansion)
+        bases = len(vfd.vfd_op_far_ranks(op)) * info["rank"] * n
+        leaf_bytes = 8 * (info["near_entries"] + info["far_blocks"] * info["rank"] ** 2 + 2 * bases) + 2 * n * 8
         roof = {"bound": "hbm", "achieved": leaf_bytes / t_apply / 1e9, "peak": hbm, "unit": "GB/s",
                 "frac": leaf_bytes / t_apply / 1e9 / hbm, "traffic": None,
                 "kernel": "vfd_apply, one column (k_fa_proj1, k_fa_couple1, k_fa_near1, k_fa_expand1; "
-                          "bytes of near panels and coupling blocks only)",
+                          "bytes of near panels, coupling blocks and, twice, the bases)",
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs"}
         t_leaf = t_apply
     else:

@@ -211,7 +211,12 @@ vfd_status vfd_assemble(vfd_mesh_t mesh, const vfd_field *s, const vfd_field *lo
  * terms hi + lo, B + M and the far field in FP32, with the diagonal of B + M
  * compensated on the first batched use so that the rounded operator is exact
  * on constant vectors -- else column by column with K in FP32 and B + M in
- * FP64. */
+ * FP64.
+ * FP64 operators: a row is off by what FP64 sums in another order may differ
+ * by, a few 2^-53 of the sum of the absolute values of its products, whatever
+ * the magnitudes in X.  The kernels depend on nrhs and, for many columns, on X
+ * (vfd_op_apply_stats), so the last bits of a column may differ between calls
+ * with other columns beside it. */
 vfd_status vfd_apply(vfd_op_t op, const double *X, double *Y, int64_t nrhs, int64_t ld, void *stream);
 
 /* Y = (sum of the selected parts) X; parts is a mask of VFD_PART_*. */
@@ -221,9 +226,10 @@ vfd_status vfd_apply_parts(vfd_op_t op, int parts, const double *X, double *Y, i
 /* Size of the fixed device scratch used by vfd_apply_noalloc (8 MiB per device). */
 #define VFD_APPLY_NOALLOC_SCRATCH_BYTES 8388608
 
-/* Y = A X for nrhs columns, as vfd_apply computes it column by column, but
- * without allocating anything during the call.  The paper has no counterpart:
- * this is a library convenience.
+/* Y = A X for nrhs columns, vfd_apply's result to rounding, without allocating
+ * anything during the call: VFD_FP64 operators by FP64 sums throughout, column by
+ * column (the same bits of a column at any nrhs), the others as vfd_apply does
+ * column by column.  The paper has no counterpart: this is a library convenience.
  *
  * Who needs it: callers that must not allocate device memory while they run,
  * e.g. a solver loop whose device memory is reserved in advance by another

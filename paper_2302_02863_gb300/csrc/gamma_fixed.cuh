@@ -55,8 +55,6 @@ __device__ __forceinline__ FxTab fx_stage(const u64 *__restrict__ g, u64 *sh)
     return {t, sh + 2 * FX_LOGN};
 }
 
-__device__ __forceinline__ FxTab fx_global(const u64 *g) { return {(const ulonglong2 *)g, g + 2 * FX_LOGN}; }
-
 __device__ __forceinline__ u64 fx_wide(unsigned a, unsigned b) { return (u64)a * b; }
 
 // r^2 / W^2 = M 2^(-K), M in [1, 2) as Q63, from the coordinate differences
