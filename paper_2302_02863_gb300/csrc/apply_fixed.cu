@@ -47,7 +47,7 @@
 // a column that is not there would cost FP64 time.
 //
 // Measured (FP64 kernels first): one column at 27k DoFs and rank 64 243 -> 170 us, at
-// 16129 DoFs and rank 16 74 -> 65.  Errors in units of |A||x| on 900 DoFs, against extended
+// 16129 DoFs and rank 16 97 -> 66.  Errors in units of |A||x| on 900 DoFs, against extended
 // precision with the FP64 operator's columns, FP64 kernels and here: normal x 6.4e-17
 // and 5.8e-17 rms, x over six decades 8.8e-17 and 9.7e-17, x falling by 14 decades across
 // the mesh 5.4e-17 and 5.0e-17, a Gaussian of width 0.1 1.0e-16 both.  A unit vector
@@ -467,8 +467,8 @@ k_fa_expand(FaFar P, int NR, const double *__restrict__ ye, const double *__rest
 // so what bounds them is the number of loads in flight.  Every lane keeps two
 // batches of eight 16-byte loads going; the first is issued before x is gathered.
 // Measured against the column kernels above with NC = 1 (four loads ahead, none
-// before the gather): coupling 94 -> 66 us, near rows 65 -> 51, expansion 46 -> 38,
-// projections 32 -> 22 us.
+// before the gather): coupling 94 -> 66 us, expansion 46 -> 38, projections 32 -> 22 us.
+// The near rows are FP64 and bound by its pipe (k_fa_near1).
 // ---------------------------------------------------------------------------
 constexpr int FA_B = 8;
 
