@@ -1200,27 +1200,32 @@ enum { TF_ERR, TF_ROWS, TF_PROJ, TF_NODES, TF_LEAVES, TF_N };
 // workspace: the digits of 64 columns per leaf and per node, column keys, masks and flags
 void apply_tensor_alloc(const MeshData &m, OpData &op)
 {
-    if (op.td_flag.p) return;
+    if (op.td_mem.p) return;
     const int node0 = m.nfar > 0 ? (1 << m.far_lmin) - 1 : m.kt.nnode;
     const size_t nodes = m.kt.nnode - node0, leaves = m.kt.nleaf;
-    op.td_off = !if_memory([&] {
-        op.td_x.alloc(leaves * ((m.max_leaf_size + 15) >> 4) * td_step(TD_COLS));
-        op.td_h.alloc(nodes * ((m.k + 15) >> 4) * td_step(TD_COLS));
-        op.td_key.alloc(TK_N + std::max(leaves, nodes) * TD_COLS);
-        op.td_w.alloc(TD_TILES * (3 * leaves + nodes));
-        op.td_exp.alloc(TD_TILES * (nodes * m.k + m.N + leaves));
-        op.td_shift.alloc((size_t)TD_TILES * (2 * m.td_rows.n + (size_t)m.nfar * m.k));
-        op.td_mask.alloc(1 + m.kt.nnode + (2 + 2 * TD_TILES) * leaves);
-        op.td_n1.alloc((nodes + leaves) * TD_COLS);
-        op.td_sum.alloc(nodes * TD_COLS);
-        op.td_least.alloc(leaves * TD_COLS);
-        op.td_flag.alloc(TF_N);
-    });
-    if (op.td_off) {   // the kernels of few columns do without
-        op.td_x.release();
-        op.td_h.release();
-        op.td_shift.release();
-    }
+    size_t total = 0;
+    auto part = [&](auto &v, size_t n) {   // sizes, then (with the memory) places
+        v.n = n;
+        if (op.td_mem.p) v.p = (decltype(v.p))(op.td_mem.p + total);
+        total += (v.bytes() + 1023) & ~(size_t)1023;
+    };
+    auto parts = [&] {
+        total = 0;
+        part(op.td_x, leaves * ((m.max_leaf_size + 15) >> 4) * td_step(TD_COLS));
+        part(op.td_h, nodes * ((m.k + 15) >> 4) * td_step(TD_COLS));
+        part(op.td_key, TK_N + std::max(leaves, nodes) * TD_COLS);
+        part(op.td_w, TD_TILES * (3 * leaves + nodes));
+        part(op.td_exp, TD_TILES * (nodes * m.k + m.N + leaves));
+        part(op.td_shift, (size_t)TD_TILES * (2 * m.td_rows.n + (size_t)m.nfar * m.k));
+        part(op.td_mask, 1 + m.kt.nnode + (2 + 2 * TD_TILES) * leaves);
+        part(op.td_n1, (nodes + leaves) * TD_COLS);
+        part(op.td_sum, nodes * TD_COLS);
+        part(op.td_least, leaves * TD_COLS);
+        part(op.td_flag, TF_N);
+    };
+    parts();
+    op.td_off = !if_memory([&] { op.td_mem.alloc(total); });   // the kernels of few columns do without
+    if (!op.td_off) parts();
 }
 
 // Y = A X for all columns

@@ -63,6 +63,14 @@ struct DBuf {
     size_t bytes() const { return sizeof(T) * n; }
 };
 
+// a part of a buffer
+template <class T>
+struct Part {
+    T *p = nullptr;
+    size_t n = 0;
+    size_t bytes() const { return sizeof(T) * n; }
+};
+
 constexpr int KMAX = 64;       // max rank p^d handled by the kernels
 constexpr int PMAX = 8;        // max Chebyshev nodes per dimension
 constexpr int NSMAX = 16;      // max Gauss points per direction of the singular rules
@@ -290,14 +298,14 @@ struct OpData {
     DBuf<unsigned char> fa_hard;
     // digits of a vector's leaf and node pieces, keys, exponents and shifts that align the pieces,
     // what is redone (rows; groups of columns of nodes and leaves) and the sizes that decide it
-    // (apply_tensor.cu)
-    DBuf<unsigned char> td_x, td_h, td_shift;
-    DBuf<unsigned> td_key, td_mask;
-    DBuf<short> td_exp;
-    DBuf<int> td_w, td_least;
-    DBuf<float> td_n1;
-    DBuf<double> td_sum;
-    DBuf<int> td_flag;
+    // (apply_tensor.cu), in one allocation
+    DBuf<unsigned char> td_mem;
+    Part<unsigned char> td_x, td_h, td_shift;
+    Part<unsigned> td_key, td_mask;
+    Part<short> td_exp;
+    Part<int> td_w, td_least, td_flag;
+    Part<float> td_n1;
+    Part<double> td_sum;
     int td_cols = 0;                   // columns of the last apply on the tensor cores
     double td_wait = 1.0;              // seconds after which their waits give up
     bool td_off = false;               // no memory for the workspace: not used
